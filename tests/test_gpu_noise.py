@@ -55,3 +55,21 @@ def test_in_place_and_argument_checks():
     for g, s in ((0.0, 1.0), (-1.0, 1.0), (10.0, -1.0), (10.0, float("nan"))):
         with pytest.raises(OsogError):
             sensor_noise(x, g, s, 3)
+
+
+# both sides of every boundary of the FP32 draw: rates at and around 10 and
+# 2^22, gains and read noises outside its range, images that are dark, far too
+# bright or not finite
+@pytest.mark.parametrize("g,sigma,level", [
+    (10.0, 1.0, 1.0), (9.999999, 0.5, 1.0), (10.0 / 3.0, 0.0, 3.0), (4194304.0, 2.0, 1.0),
+    (1e-7, 1.0, 2e8), (100.0, 1e-7, 1.0), (100.0, 2e6, 1.0), (50.0, 1.0, 0.0)])
+def test_boundaries_of_the_fp32_draw(g, sigma, level):
+    from paper_2606_21381_gb300.noise import sensor_noise
+    x = np.full(20_011, level, dtype=np.float32)
+    x[1::3] = np.nextafter(np.float32(level), np.float32(0.0))
+    x[2::3] = np.nextafter(np.float32(level), np.float32(4.0 * level + 1.0))
+    x[::1009] = 0.0
+    x[5] = np.nan  # no photons, like every value that is not above zero
+    want = oracle.sensor_noise(np.nan_to_num(x), g, sigma, 99)
+    got = sensor_noise(torch.from_numpy(x).cuda(), g, sigma, 99).cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=2e-7, atol=1e-9)
