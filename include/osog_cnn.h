@@ -52,8 +52,9 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
 /* dx = (d conv / dx)^T dy, then multiplied by the mask (x_act > 0) when
  * x_act is not NULL (the derivative of the ReLU that produced x).  dy is the
  * gradient at the convolution's output (after its own ReLU derivative).
- * w_t is a workspace of R*S*K*C bf16 holding the filters reordered to
- * [C][R][S][K] (filled by this call). */
+ * w_t is a workspace of R*S*K*C bf16 for this call's use (the warp-level MMA
+ * engine reorders the filters to [C][R][S][K] in it; the tcgen05 engine reads
+ * them as they are and leaves it untouched). */
 int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy,
                               const uint16_t *w, const uint16_t *x_act, uint16_t *dx,
                               uint16_t *w_t, osog_stream_t stream);

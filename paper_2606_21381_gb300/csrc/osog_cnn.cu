@@ -1,9 +1,8 @@
 // Convolutions of the learned warm start as implicit GEMMs on the tensor
-// cores (BF16 operands, FP32 accumulation): on tcgen05 (TMEM accumulators,
-// shared-memory descriptors, mbarrier completion) where it is faster --
-// forward and data gradients, and filter gradients with at least 128
-// output channels -- and on the warp-level MMA (mma.sync) otherwise; the
-// warp-level path stays selectable for all three.
+// cores (BF16 operands, FP32 accumulation): the C ABI, the warp-level MMA
+// kernels (mma.sync) and the filter gradients.  Forward and data gradients run
+// on tcgen05 in osog_conv_tma.cu unless the warp-level engine is selected or
+// the reduction is too short to feed it.
 //
 //   forward  Y[m = (n,p,q)][k]   = sum_{j = (r,s,c)} X(im2col)[m][j] W[k][j]
 //   data     dX[m = (n,h,w)][c]  = sum_{j = (r,s,k)} dY(gathered)[m][j] Wt[c][j]
@@ -19,6 +18,7 @@
 #include <cuda_bf16.h>
 
 #include "osog_cnn.h"
+#include "osog_conv_tma.h"
 
 namespace osog {
 namespace cnn {
@@ -32,10 +32,6 @@ constexpr int kSplitPixels = 2048;  // pixels per CTA in the filter-gradient red
 // pixels of one parity class (h mod 2, w mod 2), reduced over the taps that
 // reach them only (the other taps of that class are zero).
 enum Pass { kFwd = 0, kDgrad = 1, kWgrad = 2, kDgrad2 = 3 };
-
-struct Geo {
-    int N, H, W, C, K, R, S, stride, pad, P, Q;
-};
 
 struct Args {
     Geo g;
@@ -208,45 +204,6 @@ __device__ __forceinline__ void epilogue_pair(const Args &a, int row, int col, f
     }
 }
 
-// Output of eight consecutive columns col .. col + 7 (col a multiple of 8)
-// of GEMM row `row`, forward or data gradient, as 16-byte accesses.
-template <int PASS>
-__device__ __forceinline__ void epilogue_vec8(const Args &a, int row, int col, const float *v) {
-    size_t o = (size_t)row * a.Ncols + col;
-    if constexpr (PASS == kDgrad2) {
-        const int wi = row % a.Wc, t = row / a.Wc, hi = t % a.Hc, n = t / a.Hc;
-        o = (((size_t)n * a.g.H + 2 * hi + a.ph) * a.g.W + 2 * wi + a.pw) * a.Ncols + col;
-    }
-    float x[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = v[j];
-    if constexpr (PASS == kFwd) {
-        const float4 b0 = *reinterpret_cast<const float4 *>(a.bias + col);
-        const float4 b1 = *reinterpret_cast<const float4 *>(a.bias + col + 4);
-        const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            x[j] += bb[j];
-            if (a.relu) x[j] = fmaxf(x[j], 0.f);
-        }
-        if (a.y32) {
-            *reinterpret_cast<float4 *>(a.y32 + o) = make_float4(x[0], x[1], x[2], x[3]);
-            *reinterpret_cast<float4 *>(a.y32 + o + 4) = make_float4(x[4], x[5], x[6], x[7]);
-        }
-    } else if (a.mask) {
-        const uint4 mk = *reinterpret_cast<const uint4 *>(a.mask + o);
-        const __nv_bfloat16 *m8 = reinterpret_cast<const __nv_bfloat16 *>(&mk);
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (!(__bfloat162float(m8[j]) > 0.f)) x[j] = 0.f;
-    }
-    uint4 out;
-    __nv_bfloat162 *o2 = reinterpret_cast<__nv_bfloat162 *>(&out);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) o2[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-    *reinterpret_cast<uint4 *>(a.y + o) = out;
-}
-
 // ---------------------------------------------------------------- GEMM
 // The filter gradient reduces over pixels, the outer index of both NHWC
 // operands: its tiles are kept as [pixel][row] (16-byte vector stores) and
@@ -375,20 +332,13 @@ __global__ void __launch_bounds__(NT) k_conv_gemm(const __grid_constant__ Args a
 }
 
 // ---------------------------------------------------------------- tcgen05
-// Forward and data-gradient convolutions on the fifth-generation tensor
-// cores.  A CTA of UNT threads owns a tile of UM = 128 GEMM rows (pixels) by
-// BNU columns (output channels rounded up to 16, at most 128); the FP32
-// accumulator lives in tensor memory (TMEM, one lane per row).  Each
-// reduction slice of UBK = 64 is copied by all threads (cp.async, 16 bytes,
-// zero-filled outside the image) into one of UST shared stages in the
-// canonical K-major layout without swizzle -- 8-row x 16-byte
-// core matrices, contiguous along K (LBO = 128 bytes) and 8-row groups
-// UBK / 8 core matrices apart (SBO = 1024 bytes) -- then one thread issues
-// four tcgen05.mma (M 128, N BNU, K 16) with shared-memory descriptors and
-// commits them to the stage's mbarrier; a stage is refilled once its
-// multiplications are done, while the next stage's are already queued, so
-// copies of UST - 1 stages overlap the multiplications.  Waits are bounded: a timeout latches
-// g_cnn_status and the kernel still releases its tensor memory.
+// Staging of the tcgen05 filter gradient: reduction slices of UBK = 64 are
+// copied by all threads (cp.async, 16 bytes, zero-filled outside the image)
+// into UST shared stages of 8 x 16-byte core matrices without swizzle; one
+// thread issues the tcgen05.mma of a slice and commits them to the stage's
+// mbarrier; a stage is refilled once its multiplications are done.  Waits are
+// bounded: a timeout latches g_cnn_status and the kernel still releases its
+// tensor memory.
 constexpr int UM = 128, UBK = 64, UST = 3, UKC = UBK / 8, UNT = 256;
 constexpr int kUStage = UM * UBK * 2;   // bytes of one operand stage (B <= 128 rows)
 constexpr int kSpinLimit = 1 << 22;
@@ -398,10 +348,6 @@ __device__ int g_cnn_status;
 // tcgen05 convolution CTA also waits, for this many polls, on a barrier that
 // nothing arrives on, so the bounded wait runs out and latches g_cnn_status.
 __device__ int g_cnn_probe_polls;
-
-__device__ __forceinline__ int canon(int row, int k) {  // byte offset in a stage
-    return (row >> 3) * (UKC * 128) + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
-}
 
 __device__ __forceinline__ uint64_t umma_desc(uint32_t addr) {
     return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) |
@@ -440,227 +386,6 @@ __device__ __forceinline__ void cp16(void *dst, const __nv_bfloat16 *src, const 
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n"
                  :: "r"(smem_u32(dst)), "l"(src ? (const void *)src : any), "r"(src ? 16 : 0)
                  : "memory");
-}
-
-// The operand copies of one thread.  Thread t copies the 8-element column
-// kv = t % 8 of every slice for the A rows t / 8 + 32 i (i < 4) and the B
-// rows t / 8 + 32 i below BNU.  The pixel of each A row is decoded once; the
-// tap and channel of the reduction entry j = k0 + 8 kv advance by UBK per
-// slice without divisions.
-template <int PASS>
-struct UGather {
-    int kv;
-    int n[UM * UKC / UNT], y[UM * UKC / UNT], x[UM * UKC / UNT];  // n < 0: row past M
-    int t0, t1, ch;  // (r, s, c) forward, (r, s, k) data gradient, (ri, si, k) stride-2 class
-
-    __device__ __forceinline__ void init(const Args &a, int m0, int tid) {
-        const Geo &g = a.g;
-        kv = tid & 7;
-        const int cch = PASS == kFwd ? g.C : g.K, t1n = PASS == kDgrad2 ? a.ns : g.S;
-        const int j = kv * 8, tap = j / cch;
-        ch = j - tap * cch;
-        if (t1n > 0) {
-            t0 = tap / t1n;
-            t1 = tap - t0 * t1n;
-        } else {  // a parity class without taps: nothing to copy
-            t0 = 1 << 20;
-            t1 = 0;
-        }
-#pragma unroll
-        for (int i = 0; i < UM * UKC / UNT; ++i) {
-            const int m = m0 + (tid >> 3) + 32 * i;
-            n[i] = -1;
-            if (m >= a.M) continue;
-            if constexpr (PASS == kFwd) {
-                const int q = m % g.Q, t = m / g.Q, p = t % g.P;
-                n[i] = t / g.P;
-                y[i] = p * g.stride - g.pad;
-                x[i] = q * g.stride - g.pad;
-            } else if constexpr (PASS == kDgrad) {  // stride 1
-                const int w = m % g.W, t = m / g.W, h = t % g.H;
-                n[i] = t / g.H;
-                y[i] = h + g.pad;
-                x[i] = w + g.pad;
-            } else {
-                const int wi = m % a.Wc, t = m / a.Wc, hi = t % a.Hc;
-                n[i] = t / a.Hc;
-                y[i] = 2 * hi + a.ph + g.pad;
-                x[i] = 2 * wi + a.pw + g.pad;
-            }
-        }
-    }
-
-    __device__ __forceinline__ void advance(const Args &a) {
-        const int cch = PASS == kFwd ? a.g.C : a.g.K, t1n = PASS == kDgrad2 ? a.ns : a.g.S;
-        ch += UBK;
-        while (ch >= cch) {
-            ch -= cch;
-            if (++t1 == t1n) {
-                t1 = 0;
-                ++t0;
-            }
-        }
-    }
-
-    __device__ __forceinline__ void load(const Args &a, unsigned char *A, unsigned char *B, int n0,
-                                         int k0, int BNU, int tid) const {
-        const Geo &g = a.g;
-        const bool live = t0 < (PASS == kDgrad2 ? a.nr : g.R);  // j < Kred
-        const int r = PASS == kDgrad2 ? a.rtap[live ? t0 : 0] : t0;
-        const int sx = PASS == kDgrad2 ? a.stap[t1] : t1;
-#pragma unroll
-        for (int i = 0; i < UM * UKC / UNT; ++i) {
-            const int row = (tid >> 3) + 32 * i;
-            const __nv_bfloat16 *src = nullptr;
-            if (live && n[i] >= 0) {
-                if constexpr (PASS == kFwd) {
-                    const int h = y[i] + r, w = x[i] + sx;
-                    if (h >= 0 && h < g.H && w >= 0 && w < g.W)
-                        src = a.x + (((size_t)n[i] * g.H + h) * g.W + w) * g.C + ch;
-                } else {
-                    const int p = PASS == kDgrad ? y[i] - r : (y[i] - r) >> 1;
-                    const int q = PASS == kDgrad ? x[i] - sx : (x[i] - sx) >> 1;
-                    if (p >= 0 && p < g.P && q >= 0 && q < g.Q)
-                        src = a.x + (((size_t)n[i] * g.P + p) * g.Q + q) * g.K + ch;
-                }
-            }
-            cp16(A + canon(row, kv * 8), src, a.x);
-        }
-        for (int row = tid >> 3; row < BNU; row += UNT / 8) {
-            const int b = n0 + row;
-            const __nv_bfloat16 *src = nullptr;
-            if (live && b < a.Ncols) {
-                if constexpr (PASS == kDgrad2)
-                    src = a.w + (((size_t)b * g.R + r) * g.S + sx) * g.K + ch;
-                else
-                    src = a.w + (size_t)b * a.Kred + k0 + kv * 8;
-            }
-            cp16(B + canon(row, kv * 8), src, a.w);
-        }
-    }
-};
-
-template <int PASS>
-__global__ void __launch_bounds__(UNT) k_conv_umma(const __grid_constant__ Args a, int BNU) {
-    extern __shared__ __align__(1024) unsigned char sm[];
-    const int bstage = BNU * UBK * 2;  // bytes of one B stage
-    unsigned char *stA = sm, *stB = sm + UST * kUStage;
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(stB + UST * bstage);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + UST);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * UM, n0 = blockIdx.y * BNU;
-    const uint32_t ncols = BNU <= 32 ? 32u : BNU <= 64 ? 64u : 128u;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
-                     :: "r"(smem_u32(tslot)), "r"(ncols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int st = 0; st < UST; ++st)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_u32(mbar + st)), "r"(1));
-        // the failure-detection probe's barrier (after tslot): nothing arrives on it
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_u32(mbar + UST + 1)), "r"(1));
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    const int nk = (a.Kred + UBK - 1) / UBK;
-    UGather<PASS> ga;
-    ga.init(a, m0, tid);
-    // prologue: stages 0 .. UST-2 in flight, one commit group each
-    for (int kt = 0; kt < UST - 1; ++kt) {
-        if (kt < nk) {
-            ga.load(a, stA + kt * kUStage, stB + kt * bstage, n0, kt * UBK, BNU, tid);
-            ga.advance(a);
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t taddr = *tslot;
-    const uint32_t idesc = umma_idesc(BNU);
-    bool ok = true;
-    for (int kt = 0; kt < nk; ++kt) {
-        const int st = kt % UST;
-        // this thread's copies of stage kt have landed (UST-2 newer groups may pend)
-        asm volatile("cp.async.wait_group %0;\n" :: "n"(UST - 2) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor core
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            unsigned char *A = stA + st * kUStage, *B = stB + st * bstage;
-#pragma unroll
-            for (int s = 0; s < UBK / 16; ++s) {
-                const uint64_t ad = umma_desc(smem_u32(A) + s * 256);
-                const uint64_t bd = umma_desc(smem_u32(B) + s * 256);
-                const uint32_t acc = (kt > 0 || s > 0) ? 1u : 0u;
-                asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             :: "r"(taddr), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                         :: "r"(smem_u32(mbar + st)) : "memory");
-        }
-        // refill the stage of step kt-1 with step kt+UST-1 once its
-        // multiplications are done (those of step kt are queued behind them)
-        const int nx = kt + UST - 1;
-        if (nx < nk) {
-            const int sx = nx % UST;
-            if (kt >= 1) ok = mbar_wait(smem_u32(mbar + sx), (uint32_t)(((kt - 1) / UST) & 1)) && ok;
-            ga.load(a, stA + sx * kUStage, stB + sx * bstage, n0, nx * UBK, BNU, tid);
-            ga.advance(a);
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    // the last commit covers every multiplication issued before it (a
-    // reduction of length 0 issues none: the result is zero)
-    if (nk > 0) {
-        const int last = nk - 1;
-        ok = mbar_wait(smem_u32(mbar + last % UST), (uint32_t)((last / UST) & 1)) && ok;
-    }
-    if (tid == 0 && g_cnn_probe_polls > 0)  // a wait made to run out (test hook)
-        ok = mbar_wait(smem_u32(mbar + UST + 1), 0u, g_cnn_probe_polls) && ok;
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!ok && lane == 0) atomicExch(&g_cnn_status, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its rows) and the
-    // 32-column chunks c with c % (UNT / 128) == w / 4
-    const int quarter = warp & 3, group = warp >> 2;
-    const int row = m0 + quarter * 32 + lane;
-    for (int c0 = group * 32; c0 < BNU; c0 += 32 * (UNT / 128)) {
-        uint32_t v[32];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-            "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-              "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-              "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-              "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
-              "=r"(v[31])
-            : "r"(taddr + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-        if (nk == 0) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = 0u;
-        }
-        if (row < a.M) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-                const int col = n0 + c0 + j;
-                if (c0 + j < BNU && col < a.Ncols) {
-                    float f[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(v[j + i]);
-                    epilogue_vec8<PASS>(a, row, col, f);
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(taddr), "r"(ncols)
-                     : "memory");
 }
 
 // Filter gradient on tcgen05: dW[k][j] = sum over pixels of dY[pixel][k]
@@ -855,33 +580,14 @@ __host__ __device__ constexpr int umma_smem(int bnu) { return UST * (kUStage + b
 // One-time opt-in to the stages' dynamic shared memory.
 cudaError_t umma_prepare() {
     static const cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(k_conv_umma<kFwd>,
+        cudaError_t r = cudaFuncSetAttribute(k_wgrad_umma<false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_conv_umma<kDgrad>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_conv_umma<kDgrad2>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_wgrad_umma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kUmmaSmem);
         if (r == cudaSuccess)
             r = cudaFuncSetAttribute(k_wgrad_umma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kUmmaSmem);
         return r;
     }();
     return e;
-}
-
-template <int PASS>
-cudaError_t launch_umma(const Args &a, cudaStream_t st) {
-    cudaError_t e = umma_prepare();
-    if (e != cudaSuccess) return e;
-    const int bnu = ((a.Ncols + 15) / 16) * 16 < 128 ? ((a.Ncols + 15) / 16) * 16 : 128;
-    dim3 grid((a.M + UM - 1) / UM, (a.Ncols + bnu - 1) / bnu);
-    k_conv_umma<PASS><<<grid, UNT, umma_smem(bnu), st>>>(a, bnu);
-    return cudaGetLastError();
 }
 
 // Sum of the filter-gradient partial tiles over the pixel splits, in split
@@ -1057,7 +763,10 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // reductions shorter than two slices feed the tensor cores too little per
     // copied row (measured: the 8-channel first layer is faster on mma.sync)
-    if (g_use_tcgen05 && a.Kred >= 2 * UBK) return status_of(launch_umma<kFwd>(a, st));
+    if (g_use_tcgen05 && a.Kred >= 2 * UBK) {
+        const cudaError_t e = conv_forward_tma(a.g, x, w, bias, relu != 0, y, y_f32, st);
+        if (e != cudaErrorNotSupported) return status_of(e);
+    }
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
     k_conv_gemm<kFwd><<<grid, NT, 0, st>>>(a);
     return status_of(cudaGetLastError());
@@ -1069,6 +778,10 @@ int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy
     if (!shape_ok(shape) || !dy || !w || !dx || !w_t) return OSOG_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const Geo g = geo_of(shape);
+    if (g_use_tcgen05) {  // reads the filters in place: w_t stays untouched
+        const cudaError_t e = conv_dgrad_tma(g, dy, w, x_act, dx, st);
+        if (e != cudaErrorNotSupported) return status_of(e);
+    }
     const int64_t nw = (int64_t)g.K * g.R * g.S * g.C;
     k_filter_transpose<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(bf(w), g.K, g.R * g.S, g.C, bf(w_t));
     Args a{};
@@ -1093,11 +806,6 @@ int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy
                 a.M = g.N * a.Hc * a.Wc;
                 a.Kred = a.nr * a.ns * g.K;
                 if (a.M == 0) continue;
-                if (g_use_tcgen05) {
-                    const cudaError_t e = launch_umma<kDgrad2>(a, st);
-                    if (e != cudaSuccess) return status_of(e);
-                    continue;
-                }
                 dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
                 k_conv_gemm<kDgrad2><<<grid, NT, 0, st>>>(a);
             }
@@ -1105,7 +813,6 @@ int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy
     }
     a.M = g.N * g.H * g.W;
     a.Kred = g.R * g.S * g.K;
-    if (g_use_tcgen05) return status_of(launch_umma<kDgrad>(a, st));
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
     k_conv_gemm<kDgrad><<<grid, NT, 0, st>>>(a);
     return status_of(cudaGetLastError());
@@ -1184,14 +891,18 @@ void osog_conv_use_tcgen05(int32_t enable) { g_use_tcgen05 = enable ? 1 : 0; }
 
 int osog_conv_test_wait_limit(int32_t polls) {
     const int v = polls > 0 ? polls : 0;
-    return cudaMemcpyToSymbol(g_cnn_probe_polls, &v, sizeof v) == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA;
+    return cudaMemcpyToSymbol(g_cnn_probe_polls, &v, sizeof v) == cudaSuccess &&
+                   conv_tma_set_probe(v) == cudaSuccess
+               ? OSOG_OK
+               : OSOG_ERR_CUDA;
 }
 
 int osog_conv_sync_status(osog_stream_t stream) {
     if (cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return OSOG_ERR_CUDA;
-    int v = 0;
+    int v = 0, t = 0;
     if (cudaMemcpyFromSymbol(&v, g_cnn_status, sizeof v) != cudaSuccess) return OSOG_ERR_CUDA;
-    if (!v) return OSOG_OK;
+    if (conv_tma_take_status(&t) != cudaSuccess) return OSOG_ERR_CUDA;
+    if (!v) return t ? OSOG_ERR_TIMEOUT : OSOG_OK;
     const int zero = 0;
     if (cudaMemcpyToSymbol(g_cnn_status, &zero, sizeof zero) != cudaSuccess) return OSOG_ERR_CUDA;
     return OSOG_ERR_TIMEOUT;

@@ -1,0 +1,760 @@
+// Convolutions as implicit GEMMs on the fifth-generation tensor cores, with
+// the operands staged by the TMA unit (BF16 operands, FP32 accumulation).
+//
+// What bounds such a convolution is not the tensor pipe but the traffic into
+// shared memory: an im2col tile holds every input pixel once per filter tap
+// (nine times for 3 x 3).  Here a tile of output pixels is 8 wide and 16 high
+// and its input is loaded once, as the patch of pixels that all taps touch
+// ((8 + S - 1) x (16 + R - 1) for stride 1).  A patch row is one pixel's 64
+// channels, 128 bytes, in the TMA unit's 128-byte swizzle, which is a function
+// of the shared address alone; so the operand of a tap is the same patch read
+// from a start address shifted by the tap's rows, with the patch's pitch as
+// the stride between the groups of eight rows (one image row of the tile) that
+// the matrix descriptor describes.  Padding and ragged edges are the TMA
+// unit's zero fill.
+//
+//   forward   Y[(y, x)][k]  = sum_{r, s, c} X[(y st + r - pad, ...)][c] W[k][r, s][c]
+//   data      dX[(y, x)][c] = sum_{r, s, k} dY[(y + pad - r, ...)][k] W[k][r, s][c]
+//
+// Stride 2, forward: the taps of one row and column parity read every second
+// pixel, which the TMA unit gathers (traversal stride 2) into a patch of its
+// own, one per parity.  Stride 2, data gradient: the input pixels of one parity
+// class are reached by the taps of that parity only and form a stride-1
+// problem on dY; one CTA computes the four classes of its tile from one patch.
+// The data gradient reads the filters as they are stored ([K][R][S][C], the
+// reduction index outermost: an MN-major operand), so no transposed copy of
+// them is made.
+//
+// Measured on 64 images (us, before / now, the copies through 16-byte cp.async
+// that this replaces): 128 -> 128 channels, 32 x 32: forward 104 / 21 (925
+// TFLOP/s), data gradient 113 / 22; 32 -> 64, stride 2, 128 x 128 (100 to 167 MB
+// of activations): forward 90 / 32, data gradient 209 / 55; 64 -> 128, stride 2:
+// 59 / 20 and 132 / 23.  What bounds the wide layers now is the part of a CTA
+// that its neighbour on the SM does not cover (launch, first patch, epilogue);
+// the strided ones also write and read several HBM floors' worth of
+// activations at partial overlap.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include "osog_conv_tma.h"
+
+namespace osog {
+namespace cnn {
+namespace {
+
+constexpr int kTileW = 8, kTileH = 16;   // pixels of a sub-tile: the 128 rows of one MMA
+// A patch row is CH channels of one pixel: 64 (128 bytes, 128-byte swizzle), or
+// 32 (64 bytes, 64-byte swizzle) when the source has no more, which halves the
+// patch.
+constexpr int kMaxTaps = 64;
+constexpr int kCtaThreads = 256;
+constexpr int kSmemMax = 232448;         // shared memory a CTA may opt in to (227 KB)
+constexpr int kSpinLimit = 1 << 22;
+constexpr int kMaxRing = 4;
+
+__device__ int g_status;        // a bounded wait ran out
+__device__ int g_probe_polls;   // failure-detection hook (osog_conv_test_wait_limit)
+
+// One filter tap of a launch: the patch plane it reads, its shift inside the
+// plane, its index in the filters and the output class it adds to.
+struct Tap {
+    uint8_t plane, sy, sx, cls;
+    int16_t wt;
+    int16_t first;   // 1: the first tap of its class (overwrites the accumulator)
+};
+
+struct PatchArgs {
+    int tiles_x, tiles_y;      // CTA tiles per image
+    int tx, ty;                // sub-tiles of a CTA, across and down
+    int classes;               // 1, or 4 output parity classes (stride-2 data gradient)
+    int taps;
+    int planes, pw, ph;        // patch planes and their pixels
+    int plane_bytes;           // of one plane and chunk (1024-byte multiple)
+    int mul, off_y, off_x;     // patch origin: tile origin times mul, plus off, plus parity
+    int ch;                    // channels of a patch row: 64 or 32
+    int chunks, group;         // chunks of ch channels of the source; those held at a time
+    int src_ch;                // source channels
+    int bn, ncols;             // columns of a CTA and of the result
+    int b_bytes;               // filters of one (tap, chunk) step
+    int per, ring;             // steps of a stage, stages
+    int mn_major;              // 1: filters as [reduction][column] (data gradient)
+    uint32_t tmem_cols;
+    // result
+    int out_h, out_w;          // result image
+    int cls_mul;               // 2: class (a, b) pixel (i, j) is result pixel (2 i + a, 2 j + b)
+    const float *bias;
+    const __nv_bfloat16 *mask;
+    __nv_bfloat16 *y;
+    float *y32;
+    int relu;
+    uint32_t live;             // bit c: class c has a tap
+    Tap tap[kMaxTaps];
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, int limit = kSpinLimit) {
+    for (int it = 0; it < limit; ++it) {
+        uint32_t done;
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                     "selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+        if (it > 64) __nanosleep(32);
+    }
+    return false;
+}
+// True in one lane of the (converged) warp.  The warps that issue TMA loads and
+// matrix instructions run their loops with all lanes and issue from the elected
+// one, so that loop state and descriptors stay warp-uniform (uniform
+// registers); a loop inside a single-lane branch moves every operand there
+// first, 80 to 100 cycles a matrix instruction.
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ void expect_bytes(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void init_bar(uint32_t bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void commit_to(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+                 ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void load_4d(uint32_t dst, const CUtensorMap *m, int c, int x, int y,
+                                        int n, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+                 "[%0], [%1, {%2, %3, %4, %5}], [%6];\n"
+                 ::"r"(dst), "l"(m), "r"(c), "r"(x), "r"(y), "r"(n), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void load_3d(uint32_t dst, const CUtensorMap *m, int c, int t, int k,
+                                        uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+                 "[%0], [%1, {%2, %3, %4}], [%5];\n"
+                 ::"r"(dst), "l"(m), "r"(c), "r"(t), "r"(k), "r"(bar) : "memory");
+}
+
+// Matrix descriptor of a swizzled tile, in two words: the low one holds the
+// start address (16-byte units, so operands are moved by adding to it) and the
+// byte stride between 64-element groups of the row index (MN-major tiles only),
+// the high one the byte stride between groups of eight rows, the version and
+// the swizzle (128-byte rows, or 64-byte ones).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lead) {
+    return ((addr >> 4) & 0x3FFF) | (lead >> 4) << 16;
+}
+template <int ROW = 128>
+__device__ __forceinline__ uint32_t desc_hi(uint32_t stride) {
+    return (stride >> 4) | 1u << 14 | (ROW == 128 ? 2u : 4u) << 29;
+}
+// kind::f16 instruction descriptor: FP32 accumulator, BF16 operands, M 128.
+__device__ __forceinline__ uint32_t instr_desc(int n, bool a_mn, bool b_mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u) |
+           ((uint32_t)(n >> 3) << 17) | (8u << 24);
+}
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                    uint32_t b_hi, uint32_t idesc, uint32_t add) {
+    asm volatile("{\n.reg .pred p;\n.reg .b64 ad, bd;\nsetp.ne.b32 p, %6, 0;\n"
+                 "mov.b64 ad, {%1, %2};\nmov.b64 bd, {%3, %4};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n}\n"
+                 ::"r"(d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(add)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_load32(uint32_t addr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
+        "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+          "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
+          "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
+          "=r"(v[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+// Result columns of one pixel (this lane's), eight of them from v, as bf16.
+template <bool FWD>
+__device__ __forceinline__ uint4 finish8(const PatchArgs &a, const uint32_t *v, const float *bias,
+                                         float *y32) {
+    float x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = __uint_as_float(v[j]);
+    if constexpr (FWD) {
+        const float4 b0 = *reinterpret_cast<const float4 *>(bias);
+        const float4 b1 = *reinterpret_cast<const float4 *>(bias + 4);
+        const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            x[j] += bb[j];
+            if (a.relu) x[j] = fmaxf(x[j], 0.f);
+        }
+        if (y32) {
+            *reinterpret_cast<float4 *>(y32) = make_float4(x[0], x[1], x[2], x[3]);
+            *reinterpret_cast<float4 *>(y32 + 4) = make_float4(x[4], x[5], x[6], x[7]);
+        }
+    }
+    uint4 out;
+    __nv_bfloat162 *o2 = reinterpret_cast<__nv_bfloat162 *>(&out);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o2[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+    return out;
+}
+
+// v with the entries whose activation is not above zero cleared.
+__device__ __forceinline__ uint4 relu_mask(uint4 v, uint4 act) {
+    __nv_bfloat16 *x = reinterpret_cast<__nv_bfloat16 *>(&v);
+    const __nv_bfloat16 *m = reinterpret_cast<const __nv_bfloat16 *>(&act);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (!(__bfloat162float(m[j]) > 0.f)) x[j] = __float2bfloat16(0.f);
+    return v;
+}
+
+// Staging of one warp in the epilogue: 32 pixels x 64 columns, rows of 144
+// bytes (conflict-free for 16-byte accesses by consecutive rows).
+constexpr int kStageCols = 64;
+constexpr int kStageRow = 2 * kStageCols + 16;
+constexpr int kStageBytes = 32 * kStageRow;
+constexpr int kEpilogueSmem = kCtaThreads / 32 * kStageBytes;
+
+// A CTA owns tx x ty sub-tiles of 8 x 16 output pixels of one image and bn
+// result columns; accumulator (class, sub-tile) has bn columns of tensor
+// memory.  Warp 0 issues the TMA loads (the patch, then the filters of the
+// (tap, chunk) steps, `per` of them to a stage of the ring), warp 1 the matrix
+// instructions; the steps run over the taps, each over the channel chunks, so
+// that products are added in the order (tap, channel).  Then all eight warps
+// read the accumulators back and write the result.
+template <bool FWD, int CH>
+__global__ void __launch_bounds__(kCtaThreads, 2)
+k_conv_patch(const __grid_constant__ CUtensorMap src, const __grid_constant__ CUtensorMap flt,
+             const __grid_constant__ PatchArgs a) {
+    constexpr int kRow = 2 * CH;  // bytes of a patch row
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ uint64_t bars[2 * kMaxRing + 4];
+    __shared__ __align__(16) float bias[128];  // of this CTA's columns
+    __shared__ uint32_t tmem_slot;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const uint32_t patch = smem_addr(smem);
+    const uint32_t ring = patch + (uint32_t)(a.group * a.planes * a.plane_bytes);
+    const uint32_t full = smem_addr(bars), empty = full + 8u * kMaxRing;
+    const uint32_t patch_full = empty + 8u * kMaxRing, group_done = patch_full + 8u,
+                   all_done = patch_full + 16u, probe = patch_full + 24u;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
+                     ::"r"(smem_addr(&tmem_slot)), "r"(a.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < 2 * kMaxRing + 4; ++i) init_bar(full + 8u * i);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const int tile = blockIdx.x % (a.tiles_x * a.tiles_y), img = blockIdx.x / (a.tiles_x * a.tiles_y);
+    const int oy0 = (tile / a.tiles_x) * a.ty * kTileH, ox0 = (tile % a.tiles_x) * a.tx * kTileW;
+    const int n0 = blockIdx.y * a.bn;
+    const int subs = a.tx * a.ty;
+    const int groups = (a.chunks + a.group - 1) / a.group;
+    const int per = a.per, stages = a.ring, taps = a.taps;
+    const uint32_t stage_bytes = (uint32_t)(per * a.b_bytes);
+    bool ok = true;
+    if (warp == 0) {
+        int st = 0;
+        uint32_t ph = 0;
+        bool filled = false;  // every stage used once: waits on its consumer from then on
+        for (int g = 0; g < groups && ok; ++g) {
+            const int c0 = g * a.group, nc = min(a.group, a.chunks - c0);
+            if (g > 0) ok = wait_bar(group_done, (uint32_t)(g - 1) & 1u);
+            if (!ok) break;
+            if (elect_lane()) {
+                expect_bytes(patch_full, (uint32_t)(nc * a.planes * a.pw * a.ph * kRow));
+                for (int p = 0; p < a.planes; ++p)
+                    for (int c = 0; c < nc; ++c)
+                        load_4d(patch + (uint32_t)((c * a.planes + p) * a.plane_bytes), &src,
+                                (c0 + c) * CH, ox0 * a.mul + a.off_x + (p & 1),
+                                oy0 * a.mul + a.off_y + (p >> 1), img, patch_full);
+            }
+            __syncwarp();
+            int t = 0, c = 0;
+            for (int left = taps * nc; left > 0 && ok; left -= per) {
+                if (filled) ok = wait_bar(empty + 8u * st, ph ^ 1u);
+                if (!ok) break;
+                const int n = min(per, left);
+                const uint32_t bar = full + 8u * st;
+                uint32_t dst = ring + (uint32_t)st * stage_bytes;
+                const bool lead = elect_lane();
+                if (lead) expect_bytes(bar, (uint32_t)(n * a.b_bytes));
+                for (int i = 0; i < n; ++i) {
+                    const int wt = a.tap[t].wt;
+                    if (lead) {
+                        if (a.mn_major) {
+                            for (int b = 0; b * 64 < a.bn; ++b)
+                                load_3d(dst + (uint32_t)(b * CH * 128), &flt, n0 + b * 64, wt,
+                                        (c0 + c) * CH, bar);
+                        } else {
+                            load_3d(dst, &flt, (c0 + c) * CH, wt, n0, bar);
+                        }
+                    }
+                    dst += (uint32_t)a.b_bytes;
+                    if (++c == nc) {
+                        c = 0;
+                        ++t;
+                    }
+                }
+                __syncwarp();
+                if (++st == stages) {
+                    st = 0;
+                    ph ^= 1u;
+                    filled = true;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = instr_desc(a.bn, false, a.mn_major != 0);
+        const uint32_t pitch = (uint32_t)(a.pw * kRow);
+        // K-major filters have the patch's row width, MN-major ones rows of 64
+        // result columns
+        const uint32_t a_hi = desc_hi<kRow>(pitch),
+                       b_hi = a.mn_major ? desc_hi<128>(1024u) : desc_hi<kRow>(8u * kRow);
+        const uint32_t pitch16 = pitch >> 4, chunk16 = (uint32_t)(a.planes * a.plane_bytes) >> 4,
+                       plane16 = (uint32_t)a.plane_bytes >> 4, bn = (uint32_t)a.bn;
+        const uint32_t b_step = a.mn_major ? 2048u >> 4 : 32u >> 4;  // 16 reduction entries
+        const uint32_t b_first = desc_lo(ring, a.mn_major ? CH * 128 : 16u);
+        const uint32_t b16 = (uint32_t)a.b_bytes >> 4;
+        uint32_t sub16[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            sub16[s] = (uint32_t)(s / a.tx) * kTileH * pitch16 +
+                       (uint32_t)(s % a.tx) * (kTileW * kRow >> 4);
+        const int last_ch = a.src_ch;
+        int st = 0;
+        uint32_t ph = 0;
+        for (int g = 0; g < groups && ok; ++g) {
+            const int c0 = g * a.group, nc = min(a.group, a.chunks - c0);
+            ok = wait_bar(patch_full, (uint32_t)g & 1u);
+            int t = 0, c = 0;
+            Tap now = a.tap[0], next = a.tap[min(1, taps - 1)];
+            uint32_t a_lo = desc_lo(patch, 16u) + now.plane * plane16 + now.sy * pitch16 +
+                            now.sx * (kRow >> 4);
+            for (int left = taps * nc; left > 0 && ok; left -= per) {
+                ok = wait_bar(full + 8u * st, ph);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                uint32_t b_lo = b_first + (uint32_t)(st * per) * b16;
+                const int n = min(per, left);
+                const bool lead = elect_lane();
+                for (int i = 0; i < n; ++i) {
+                    const uint32_t add = now.first && g == 0 && c == 0 ? 0u : 1u;
+                    const int rest = last_ch - (c0 + c) * CH;
+                    const uint32_t acc = tmem + now.cls * (uint32_t)subs * bn;
+                    if (lead) {
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            if (s >= subs) break;
+                            const uint32_t as = a_lo + sub16[s], d = acc + (uint32_t)s * bn;
+                            mma(d, as, a_hi, b_lo, b_hi, idesc, add);
+                            if (rest > 16) mma(d, as + 2u, a_hi, b_lo + b_step, b_hi, idesc, 1u);
+                            if constexpr (CH == 64) {
+                                if (rest > 32) mma(d, as + 4u, a_hi, b_lo + 2u * b_step, b_hi, idesc, 1u);
+                                if (rest > 48) mma(d, as + 6u, a_hi, b_lo + 3u * b_step, b_hi, idesc, 1u);
+                            }
+                        }
+                    }
+                    b_lo += b16;
+                    a_lo += chunk16;
+                    if (++c == nc) {
+                        c = 0;
+                        ++t;
+                        now = next;
+                        next = a.tap[min(t + 1, taps - 1)];  // read ahead of its use
+                        a_lo = desc_lo(patch, 16u) + now.plane * plane16 + now.sy * pitch16 +
+                               now.sx * (kRow >> 4);
+                    }
+                }
+                if (lead) commit_to(empty + 8u * st);
+                __syncwarp();
+                if (++st == stages) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+            }
+            if (ok && g + 1 < groups && elect_lane()) commit_to(group_done);
+            __syncwarp();
+        }
+        if (ok && elect_lane()) commit_to(all_done);
+    } else if (FWD && tid >= kCtaThreads - 128) {  // meanwhile
+        const int col = tid - (kCtaThreads - 128);
+        if (col < a.bn && n0 + col < a.ncols) bias[col] = __ldg(a.bias + n0 + col);
+    }
+    __syncwarp();
+    ok = wait_bar(all_done, 0u) && ok;
+    __syncthreads();
+    if (tid == 0 && g_probe_polls > 0)  // a wait made to run out (test hook)
+        ok = wait_bar(probe, 0u, g_probe_polls) && ok;
+    if (!ok) atomicExch(&g_status, 1);
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    // Warp w reads the tensor-memory lanes 32 (w % 4) .. + 31 (pixels) of the
+    // (accumulator, 64 columns) units of its half (w / 4).  A lane holds one
+    // pixel; written from there, the 16-byte stores of a warp would fall on 32
+    // different lines, so a unit goes through the warp's own shared-memory
+    // rows (the operands are consumed by now) and leaves as whole pixels.
+    const int quarter = warp & 3, half = warp >> 2;
+    unsigned char *stage = smem + warp * kStageBytes;
+    const int units = (a.bn + kStageCols - 1) / kStageCols;
+    for (int u = half; u < a.classes * subs * units; u += 2) {
+        const int acc = u / units, cc = (u % units) * kStageCols;
+        const int cls = acc / subs, s = acc % subs;
+        const int ncol = min(kStageCols, min(a.bn - cc, a.ncols - n0 - cc));  // a multiple of 8
+        if (ncol <= 0) continue;
+        int oy = oy0 + (s / a.tx) * kTileH + quarter * 4, ox = ox0 + (s % a.tx) * kTileW;
+        if (a.cls_mul == 2) {
+            oy = 2 * oy + (cls >> 1);
+            ox = 2 * ox + (cls & 1);
+        }
+        // pixel i of the warp: (oy + (i / 8) cls_mul, ox + (i % 8) cls_mul)
+        const size_t img_row = (size_t)img * a.out_h;
+        const int my = oy + (lane >> 3) * a.cls_mul, mx = ox + (lane & 7) * a.cls_mul;
+        float *y32 = FWD && a.y32 && my < a.out_h && mx < a.out_w
+                         ? a.y32 + ((img_row + my) * a.out_w + mx) * a.ncols + n0 + cc
+                         : nullptr;
+        // this lane's 16-byte vectors of the result: pixels first + i step; the
+        // activations of the mask are read ahead of everything else
+        const int vecs = ncol >> 3;                            // of a pixel
+        const int lanes = vecs > 4 ? 8 : vecs > 2 ? 4 : vecs;  // of a pixel (1, 2, 4 or 8)
+        const int sh = lanes == 8 ? 3 : lanes == 4 ? 2 : lanes - 1;
+        const int vec = lane & (lanes - 1), first = lane >> sh, step = 32 >> sh;
+        int64_t at[8];
+        uint4 act[FWD ? 1 : 8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int p = first + i * step;
+            const int py = oy + (p >> 3) * a.cls_mul, px = ox + (p & 7) * a.cls_mul;
+            const bool in = p < 32 && vec < vecs && py < a.out_h && px < a.out_w;
+            at[i] = in ? (int64_t)(((img_row + py) * a.out_w + px) * a.ncols + n0 + cc + vec * 8) : -1;
+            if constexpr (!FWD)
+                if (a.mask && in) act[i] = __ldg(reinterpret_cast<const uint4 *>(a.mask + at[i]));
+        }
+#pragma unroll
+        for (int h = 0; h < kStageCols; h += 32) {
+            if (h >= ncol) break;
+            uint32_t v[32];
+            tmem_load32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * a.bn + cc + h), v);
+            if (!((a.live >> cls) & 1u)) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                if (h + j < ncol)
+                    *reinterpret_cast<uint4 *>(stage + lane * kStageRow + (h + j) * 2) =
+                        finish8<FWD>(a, v + j, bias + cc + h + j, y32 ? y32 + h + j : nullptr);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (at[i] >= 0) {
+                uint4 v = *reinterpret_cast<const uint4 *>(stage + (first + i * step) * kStageRow + vec * 16);
+                if (!FWD && a.mask) v = relu_mask(v, act[i]);
+                *reinterpret_cast<uint4 *>(a.y + at[i]) = v;
+            }
+        __syncwarp();
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.tmem_cols)
+                     : "memory");
+}
+
+// ------------------------------------------------------------------ host
+using EncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
+                              const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                              const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeFn encode_fn() {
+    static const EncodeFn fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                             &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<EncodeFn>(p);
+    }();
+    return fn;
+}
+
+// Tensor map of a bf16 tensor with `rank` dimensions (innermost first), boxes
+// of the given extents (the innermost 64 or 32: 128- or 64-byte swizzle),
+// traversal strides es, zero fill.
+cudaError_t encode(CUtensorMap *m, const void *base, int rank, const uint64_t *dims,
+                   const uint32_t *box, const uint32_t *es) {
+    const EncodeFn fn = encode_fn();
+    if (!fn) return cudaErrorNotSupported;
+    cuuint64_t d[5], strides[5];
+    cuuint32_t b[5], e[5];
+    uint64_t bytes = 2;
+    for (int i = 0; i < rank; ++i) {
+        d[i] = dims[i];
+        bytes *= dims[i];
+        strides[i] = bytes;  // of dimension i + 1
+        b[i] = box[i];
+        e[i] = es[i];
+    }
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank,
+                          const_cast<void *>(base), d, strides, b, e, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          box[0] == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+int round_up(int v, int m) { return (v + m - 1) / m * m; }
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+uint32_t tmem_columns(int need) {
+    uint32_t c = 32;
+    while ((int)c < need) c *= 2;
+    return c;
+}
+
+int patch_smem(const PatchArgs &a) {
+    const int operands = a.group * a.planes * a.plane_bytes + a.ring * a.per * a.b_bytes;
+    return operands > kEpilogueSmem ? operands : kEpilogueSmem;
+}
+
+// Sub-tiles per CTA and the shared-memory plan of a launch over an oh x ow
+// pixel grid of `images` images.  More sub-tiles share one stage of filters and
+// one patch, but leave fewer CTAs to fill the SMs and to hide one another's
+// fixed parts.  The choice minimises a count of cycles: the larger of what the
+// SM's rates allow (bytes into shared memory at 64 a cycle, tensor cycles at N /
+// 2 for a 128 x N x 16 product) and of the waves of CTAs times the length of one
+// (launch and allocation 1400, the patch's latency, 150 for a stage, 900 for an
+// epilogue unit of a warp; measured with clock reads on the 128 -> 128 and 32 ->
+// 64 channel layers).  False if no plan fits.
+bool conv_patch_plan(PatchArgs &a, int images, int oh, int ow, int reach_y, int reach_x) {
+    static const int shapes[3][2] = {{1, 1}, {2, 1}, {2, 2}};
+    const int col_blocks = ceil_div(a.ncols, a.bn);
+    double best = 0;
+    bool found = false;
+    PatchArgs pick = a;
+    for (const auto &sh : shapes) {
+        PatchArgs t = a;
+        t.tx = sh[0];
+        t.ty = sh[1];
+        const int subs = t.tx * t.ty;
+        if (subs > 1 && ((t.tx - 1) * kTileW >= ow || (t.ty - 1) * kTileH >= oh)) continue;
+        const int cols = (t.classes * subs - 1) * t.bn + round_up(t.bn, 32);
+        if (cols > 512) continue;
+        t.tmem_cols = tmem_columns(cols);
+        t.pw = t.tx * kTileW + reach_x;
+        t.ph = t.ty * kTileH + reach_y;
+        if ((t.pw - 1) * t.mul + 1 > 256 || (t.ph - 1) * t.mul + 1 > 256) continue;
+        t.plane_bytes = round_up(t.pw * t.ph * 2 * t.ch, 1024);
+        t.tiles_x = ceil_div(ow, t.tx * kTileW);
+        t.tiles_y = ceil_div(oh, t.ty * kTileH);
+        const double per_sm_ctas = (double)images * t.tiles_x * t.tiles_y * col_blocks / 152.0;
+        const int steps = t.taps * t.chunks;
+        const double mma = (double)steps * (t.ch / 16) * t.bn / 2.0 * subs;
+        const double units = (t.classes * subs * ceil_div(t.bn, 64) + 1) / 2;
+        for (t.ring = 2; t.ring <= 4; ++t.ring)
+            for (t.per = 1; t.per <= 9; ++t.per) {
+                if (t.per > 1 && (t.ring - 1) * t.per >= steps) continue;
+                int group = t.chunks;
+                const int stages = t.ring * t.per * t.b_bytes;
+                while (group > 1 && group * t.planes * t.plane_bytes + stages > kSmemMax - 2048)
+                    group = (group + 1) / 2;
+                if (group * t.planes * t.plane_bytes + stages > kSmemMax - 2048) continue;
+                t.group = group;
+                int co = (kSmemMax + 1024) / (patch_smem(t) + 2048);
+                co = co > 512 / (int)t.tmem_cols ? 512 / (int)t.tmem_cols : co;
+                co = co > 2 ? 2 : co;  // registers
+                const double bytes = (double)t.chunks * t.planes * t.plane_bytes +
+                                     (double)steps * t.b_bytes;
+                const double rate = per_sm_ctas * (bytes / 64.0 > mma ? bytes / 64.0 : mma);
+                // a stage's filters arrive about 1200 cycles after they are asked for
+                const double turn = 1200.0 / (t.ring - 1);
+                const double stage_mma = mma / steps * t.per + 150.0;
+                const double len = 1400.0 + 1000.0 + (double)t.chunks * t.planes * t.plane_bytes / 64.0 +
+                                   (stage_mma > turn ? stage_mma : turn) * ceil_div(steps, t.per) +
+                                   1500.0 + 900.0 * units;
+                const double waves = per_sm_ctas / co;
+                const double whole = waves < 3 ? (double)(long)(waves + 0.999) : waves + 0.5;
+                double cost = whole * len;
+                if (cost < rate) cost = rate;
+                cost += 0.2 * rate;
+                if (group < t.chunks) cost *= 1.5;
+                if (!found || cost < best) {
+                    found = true;
+                    best = cost;
+                    pick = t;
+                }
+            }
+    }
+    if (found) a = pick;
+    return found;
+}
+
+template <bool FWD, int CH>
+cudaError_t launch_patch_ch(const CUtensorMap &src, const CUtensorMap &flt, const PatchArgs &a,
+                            int images, cudaStream_t st) {
+    static const cudaError_t opt_in = cudaFuncSetAttribute(
+        k_conv_patch<FWD, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
+    if (opt_in != cudaSuccess) return opt_in;
+    const dim3 grid(images * a.tiles_x * a.tiles_y, ceil_div(a.ncols, a.bn));
+    k_conv_patch<FWD, CH><<<grid, kCtaThreads, patch_smem(a), st>>>(src, flt, a);
+    return cudaGetLastError();
+}
+
+template <bool FWD>
+cudaError_t launch_patch(const CUtensorMap &src, const CUtensorMap &flt, const PatchArgs &a,
+                         int images, cudaStream_t st) {
+    return a.ch == 64 ? launch_patch_ch<FWD, 64>(src, flt, a, images, st)
+                      : launch_patch_ch<FWD, 32>(src, flt, a, images, st);
+}
+
+}  // namespace
+
+cudaError_t conv_forward_tma(const Geo &g, const uint16_t *x, const uint16_t *w, const float *bias,
+                             bool relu, uint16_t *y, float *y32, cudaStream_t st) {
+    PatchArgs a{};
+    a.classes = 1;
+    a.live = 1u;
+    a.cls_mul = 1;
+    a.mul = g.stride;
+    a.off_y = a.off_x = -g.pad;
+    a.src_ch = g.C;
+    a.ch = g.C <= 32 ? 32 : 64;
+    a.chunks = ceil_div(g.C, a.ch);
+    a.ncols = g.K;
+    a.bn = g.K > 128 ? 128 : round_up(g.K, 16);
+    a.b_bytes = a.bn * 2 * a.ch;
+    a.planes = g.stride == 1 || (g.R == 1 && g.S == 1) ? 1 : 4;
+    for (int r = 0; r < g.R; ++r)
+        for (int s = 0; s < g.S; ++s) {
+            Tap &t = a.tap[a.taps];
+            t.plane = g.stride == 1 ? 0 : (uint8_t)((r & 1) * 2 + (s & 1));
+            t.sy = (uint8_t)(g.stride == 1 ? r : r >> 1);
+            t.sx = (uint8_t)(g.stride == 1 ? s : s >> 1);
+            t.cls = 0;
+            t.wt = (int16_t)(r * g.S + s);
+            t.first = a.taps == 0;
+            ++a.taps;
+        }
+    const int ry = g.stride == 1 ? g.R - 1 : (g.R - 1) / 2, rx = g.stride == 1 ? g.S - 1 : (g.S - 1) / 2;
+    if (!conv_patch_plan(a, g.N, g.P, g.Q, ry, rx)) return cudaErrorNotSupported;
+    a.out_h = g.P;
+    a.out_w = g.Q;
+    a.bias = bias;
+    a.relu = relu;
+    a.y = reinterpret_cast<__nv_bfloat16 *>(y);
+    a.y32 = y32;
+    CUtensorMap src, flt;
+    const uint64_t sd[4] = {(uint64_t)g.C, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.N};
+    const uint32_t sb[4] = {(uint32_t)a.ch, (uint32_t)((a.pw - 1) * g.stride + 1),
+                            (uint32_t)((a.ph - 1) * g.stride + 1), 1};
+    const uint32_t se[4] = {1, (uint32_t)g.stride, (uint32_t)g.stride, 1};
+    cudaError_t e = encode(&src, x, 4, sd, sb, se);
+    const uint64_t fd[3] = {(uint64_t)g.C, (uint64_t)(g.R * g.S), (uint64_t)g.K};
+    const uint32_t fb[3] = {(uint32_t)a.ch, 1, (uint32_t)a.bn}, fe[3] = {1, 1, 1};
+    if (e == cudaSuccess) e = encode(&flt, w, 3, fd, fb, fe);
+    return e == cudaSuccess ? launch_patch<true>(src, flt, a, g.N, st) : e;
+}
+
+cudaError_t conv_dgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *w,
+                           const uint16_t *mask, uint16_t *dx, cudaStream_t st) {
+    PatchArgs a{};
+    const bool two = g.stride == 2;
+    a.classes = two ? 4 : 1;
+    a.cls_mul = two ? 2 : 1;
+    a.mul = 1;
+    a.src_ch = g.K;
+    a.ch = g.K <= 32 ? 32 : 64;
+    a.chunks = ceil_div(g.K, a.ch);
+    a.ncols = g.C;
+    a.bn = g.C > 128 ? 128 : round_up(g.C, 16);
+    a.b_bytes = ceil_div(a.bn, 64) * a.ch * 128;
+    a.mn_major = 1;
+    a.planes = 1;
+    // tap (r, s) of class (ph, pw): dY row i + (ph + pad - r) / 2 (stride 2,
+    // matching parity) or i + pad - r; shifts are counted from the smallest
+    int lo_y = 1 << 20, hi_y = -(1 << 20), lo_x = lo_y, hi_x = hi_y;
+    auto offset = [&](int cls, int tap, int &o) {
+        if (!two) {
+            o = g.pad - tap;
+            return true;
+        }
+        if ((cls + g.pad - tap) & 1) return false;
+        o = (cls + g.pad - tap) / 2;  // exact: an even number
+        return true;
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        a.taps = 0;
+        a.live = 0;
+        for (int c = 0; c < a.classes; ++c)
+            for (int r = 0; r < g.R; ++r)
+                for (int s = 0; s < g.S; ++s) {
+                    int oy, ox;
+                    if (!offset(c >> 1, r, oy) || !offset(c & 1, s, ox)) continue;
+                    if (pass == 0) {
+                        lo_y = oy < lo_y ? oy : lo_y;
+                        hi_y = oy > hi_y ? oy : hi_y;
+                        lo_x = ox < lo_x ? ox : lo_x;
+                        hi_x = ox > hi_x ? ox : hi_x;
+                        continue;
+                    }
+                    Tap &t = a.tap[a.taps];
+                    t.plane = 0;
+                    t.sy = (uint8_t)(oy - lo_y);
+                    t.sx = (uint8_t)(ox - lo_x);
+                    t.cls = (uint8_t)c;
+                    t.wt = (int16_t)(r * g.S + s);
+                    t.first = !((a.live >> c) & 1u);
+                    a.live |= 1u << c;
+                    ++a.taps;
+                }
+    }
+    a.off_y = lo_y;
+    a.off_x = lo_x;
+    const int oh = two ? (g.H + 1) / 2 : g.H, ow = two ? (g.W + 1) / 2 : g.W;
+    if (!conv_patch_plan(a, g.N, oh, ow, hi_y - lo_y, hi_x - lo_x)) return cudaErrorNotSupported;
+    a.out_h = g.H;
+    a.out_w = g.W;
+    a.mask = reinterpret_cast<const __nv_bfloat16 *>(mask);
+    a.y = reinterpret_cast<__nv_bfloat16 *>(dx);
+    CUtensorMap src, flt;
+    const uint64_t sd[4] = {(uint64_t)g.K, (uint64_t)g.Q, (uint64_t)g.P, (uint64_t)g.N};
+    const uint32_t sb[4] = {(uint32_t)a.ch, (uint32_t)a.pw, (uint32_t)a.ph, 1}, ones[4] = {1, 1, 1, 1};
+    cudaError_t e = encode(&src, dy, 4, sd, sb, ones);
+    const uint64_t fd[3] = {(uint64_t)g.C, (uint64_t)(g.R * g.S), (uint64_t)g.K};
+    const uint32_t fb[3] = {64, 1, (uint32_t)a.ch};
+    if (e == cudaSuccess) e = encode(&flt, w, 3, fd, fb, ones);
+    return e == cudaSuccess ? launch_patch<false>(src, flt, a, g.N, st) : e;
+}
+
+cudaError_t conv_tma_take_status(int *timed_out) {
+    int v = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(&v, g_status, sizeof v);
+    if (e == cudaSuccess && v) {
+        const int zero = 0;
+        e = cudaMemcpyToSymbol(g_status, &zero, sizeof zero);
+    }
+    *timed_out = v;
+    return e;
+}
+
+cudaError_t conv_tma_set_probe(int polls) {
+    return cudaMemcpyToSymbol(g_probe_polls, &polls, sizeof polls);
+}
+
+}  // namespace cnn
+}  // namespace osog

@@ -1,0 +1,29 @@
+// Host interface of the convolution kernels whose operands the TMA unit
+// stages (osog_conv_tma.cu); the C ABI around them is in osog_cnn.cu.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace osog {
+namespace cnn {
+
+struct Geo {
+    int N, H, W, C, K, R, S, stride, pad, P, Q;
+};
+
+// Forward (y = act(conv(x, w) + bias)) and data gradient (dx, times x_act > 0
+// when mask is given) on tcgen05; cudaErrorNotSupported when a size is outside
+// the kernel's range (see conv_patch_plan).
+cudaError_t conv_forward_tma(const Geo &g, const uint16_t *x, const uint16_t *w, const float *bias,
+                             bool relu, uint16_t *y, float *y32, cudaStream_t st);
+cudaError_t conv_dgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *w,
+                           const uint16_t *mask, uint16_t *dx, cudaStream_t st);
+
+// Latched status of the bounded waits (read and cleared), and the
+// failure-detection hook (osog_conv_test_wait_limit).
+cudaError_t conv_tma_take_status(int *timed_out);
+cudaError_t conv_tma_set_probe(int polls);
+
+}  // namespace cnn
+}  // namespace osog

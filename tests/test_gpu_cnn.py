@@ -25,6 +25,22 @@ SHAPES = [
 ]
 
 
+# the edges of the patch kernels' plans: several column blocks and channel
+# chunks, more chunks than shared memory holds, wide filters on both strides,
+# padding past the filter, classes and images smaller than a tile
+PATCH_SHAPES = [
+    (1, 20, 18, 264, 136, 3, 3, 1, 1),
+    (1, 9, 9, 1032, 16, 3, 3, 1, 1),
+    (2, 40, 36, 32, 48, 5, 5, 2, 2),
+    (1, 24, 25, 16, 8, 8, 8, 1, 3),
+    (1, 37, 21, 72, 24, 7, 7, 2, 3),
+    (1, 10, 11, 64, 16, 3, 3, 1, 4),
+    (1, 13, 12, 136, 40, 1, 1, 2, 1),
+    (5, 3, 2, 24, 200, 3, 2, 2, 1),
+    (2, 70, 34, 40, 16, 3, 3, 1, 0),
+]
+
+
 def _bf16(a, dev):
     """(bf16 device tensor, the same values as float64 numpy)."""
     t = torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).to(torch.bfloat16)
@@ -54,7 +70,7 @@ def cnn(request):
     m.use_tcgen05(True)
 
 
-@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
 @pytest.mark.parametrize("relu", [False, True])
 def test_conv_forward_matches_reference(cnn, shape, relu):
     dev = torch.device("cuda")
@@ -73,7 +89,7 @@ def test_conv_forward_matches_reference(cnn, shape, relu):
     assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
 
 
-@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
 @pytest.mark.parametrize("masked", [False, True])
 def test_conv_backward_data_matches_reference(cnn, shape, masked):
     dev = torch.device("cuda")
