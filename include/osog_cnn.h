@@ -61,7 +61,8 @@ int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy
 
 /* dw = sum over pixels of dy (x) and dbias = sum of dy, by a split
  * reduction over pixel chunks followed by a fixed-order sum.  ws must hold
- * osog_conv2d_backward_filter_workspace(shape) bytes. */
+ * osog_conv2d_backward_filter_workspace(shape) bytes (enough for either
+ * engine, see osog_conv_use_tcgen05). */
 size_t osog_conv2d_backward_filter_workspace(const osog_conv_shape_t *shape);
 int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *dy,
                                 const uint16_t *x, float *dw, float *dbias, void *ws,
@@ -74,10 +75,10 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
  * MMA (mma.sync).  Both compute the same products in BF16 with FP32
  * accumulation; summation order inside the tensor core differs.  With
  * tcgen05 selected, forward convolutions whose reduction R S C is below 128
- * and filter gradients with fewer than 128 output channels and fewer than
- * 64 filter entries R S C still run on the warp-level MMA (faster there);
- * filter gradients with fewer than 128 output channels but at least 64
- * filter entries take the filter entries as the tensor cores' rows.  The
+ * still run on the warp-level MMA, and so do filter gradients whose ws, dw or
+ * dbias is not 16-byte aligned.  (tcgen05 filter gradients pair output pixels
+ * past the image, as zeros, with the activations there: an infinite activation
+ * at the image's edge can make further entries of dw NaN.)  The
  * switch also covers osog_conv2d_backward_filter. */
 void osog_conv_use_tcgen05(int32_t enable);
 

@@ -1,8 +1,8 @@
 // Convolutions of the learned warm start as implicit GEMMs on the tensor
 // cores (BF16 operands, FP32 accumulation): the C ABI, the warp-level MMA
-// kernels (mma.sync) and the filter gradients.  Forward and data gradients run
-// on tcgen05 in osog_conv_tma.cu unless the warp-level engine is selected or
-// the reduction is too short to feed it.
+// kernels (mma.sync).  The convolutions and their gradients run on tcgen05 in
+// osog_conv_tma.cu unless the warp-level engine is selected or a forward
+// reduction is too short to feed it.
 //
 //   forward  Y[m = (n,p,q)][k]   = sum_{j = (r,s,c)} X(im2col)[m][j] W[k][j]
 //   data     dX[m = (n,h,w)][c]  = sum_{j = (r,s,k)} dY(gathered)[m][j] Wt[c][j]
@@ -331,265 +331,6 @@ __global__ void __launch_bounds__(NT) k_conv_gemm(const __grid_constant__ Args a
             }
 }
 
-// ---------------------------------------------------------------- tcgen05
-// Staging of the tcgen05 filter gradient: reduction slices of UBK = 64 are
-// copied by all threads (cp.async, 16 bytes, zero-filled outside the image)
-// into UST shared stages of 8 x 16-byte core matrices without swizzle; one
-// thread issues the tcgen05.mma of a slice and commits them to the stage's
-// mbarrier; a stage is refilled once its multiplications are done.  Waits are
-// bounded: a timeout latches g_cnn_status and the kernel still releases its
-// tensor memory.
-constexpr int UM = 128, UBK = 64, UST = 3, UKC = UBK / 8, UNT = 256;
-constexpr int kUStage = UM * UBK * 2;   // bytes of one operand stage (B <= 128 rows)
-constexpr int kSpinLimit = 1 << 22;
-
-__device__ int g_cnn_status;
-// Failure-detection test (osog_conv_test_wait_limit): when positive, every
-// tcgen05 convolution CTA also waits, for this many polls, on a barrier that
-// nothing arrives on, so the bounded wait runs out and latches g_cnn_status.
-__device__ int g_cnn_probe_polls;
-
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) |
-           ((uint64_t)((UKC * 128) >> 4) << 32) | ((uint64_t)1 << 46);
-}
-
-// kind::f16 instruction descriptor: FP32 D, BF16 A and B, both K-major,
-// N >> 3 and M >> 4.
-__device__ __forceinline__ uint32_t umma_idesc(int n, bool mn_major = false) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? (1u << 15) | (1u << 16) : 0u) |
-           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(UM >> 4) << 24);
-}
-
-// MN-major canonical layout (both operands of the filter gradient): core
-// matrices of 8 reduction rows x 16 bytes (8 consecutive MN elements),
-// contiguous along the reduction (LBO 128 bytes), 8-element MN groups
-// UKC core matrices apart (SBO 1024 bytes) -- the same strides as the
-// K-major tiles, with the transpose bits of the instruction descriptor set.
-__device__ __forceinline__ int canon_mn(int mn, int k) {
-    return (mn >> 3) * (UKC * 128) + (k >> 3) * 128 + (k & 7) * 16 + (mn & 7) * 2;
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int limit = kSpinLimit) {
-    for (int it = 0; it < limit; ++it) {
-        uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     "selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-        __nanosleep(32);
-    }
-    return false;
-}
-
-// 16-byte asynchronous copy to shared memory; a NULL source writes zeros.
-__device__ __forceinline__ void cp16(void *dst, const __nv_bfloat16 *src, const void *any) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n"
-                 :: "r"(smem_u32(dst)), "l"(src ? (const void *)src : any), "r"(src ? 16 : 0)
-                 : "memory");
-}
-
-// Filter gradient on tcgen05: dW[k][j] = sum over pixels of dY[pixel][k]
-// X(im2col)[pixel][j] with the output channels k as the 128 GEMM rows
-// (zero past K), the filter entries j = (r, s, c) as up to 128 columns and
-// the pixels as the reduction, in chunks of kSplitPixels per CTA (grid.z)
-// whose partial tiles are summed in chunk order.  Both operands are copied
-// from NHWC rows as 16-byte vectors (8 channels of one pixel) into the
-// MN-major layout.  SWAP (fewer than 128 output channels): the roles are
-// exchanged, the filter entries are the 128 rows and the output channels
-// the BNU columns (K rounded up to 16), so that few output channels do not
-// pad the rows; the partial tiles are written in the same [k][j] layout.
-template <bool SWAP>
-__global__ void __launch_bounds__(UNT) k_wgrad_umma(const __grid_constant__ Args a, int BNU) {
-    extern __shared__ __align__(1024) unsigned char sm[];
-    const int bstage = BNU * UBK * 2;
-    unsigned char *stA = sm, *stB = sm + UST * kUStage;
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(stB + UST * bstage);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + UST);
-    const Geo &g = a.g;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * UM, n0 = blockIdx.y * BNU;
-    const int pbeg = blockIdx.z * kSplitPixels;
-    const int pend = min(a.Kred, pbeg + kSplitPixels);
-    const uint32_t ncols = BNU <= 32 ? 32u : BNU <= 64 ? 64u : 128u;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
-                     :: "r"(smem_u32(tslot)), "r"(ncols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int st = 0; st < UST; ++st)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_u32(mbar + st)), "r"(1));
-        // the failure-detection probe's barrier (after tslot): nothing arrives on it
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" :: "r"(smem_u32(mbar + UST + 1)), "r"(1));
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    const int nk = (pend - pbeg + UBK - 1) / UBK;
-    // Copies of slice kt.  Thread t owns channel group t % 16 of the 128
-    // rows (A: 8 output channels) and of the 128 columns (B: 8 channels of
-    // one tap, decoded once) and the pixels t / 16 + 16 i (i < 4) of every
-    // slice, whose coordinates advance by UBK per slice without divisions;
-    // consecutive threads read consecutive channel groups of one pixel.
-    constexpr int NV = UBK * 16 / UNT;  // pixels per thread and slice
-    const int grp = tid & 15, kq = tid >> 4;
-    // m: this thread's 8 output channels (of dY); j: its 8 filter entries
-    // (one tap of X); the row group is A's, the column group B's
-    const int m = SWAP ? n0 + grp * 8 : m0 + grp * 8;
-    const int j = SWAP ? m0 + grp * 8 : n0 + grp * 8;
-    const bool jok = j < a.Ncols;
-    const bool bcol = !SWAP || grp * 8 < BNU;  // B columns past BNU are not in the stage
-    int tr = 0, ts = 0, tc = 0;
-    if (jok) {
-        const int rs = j / g.C;
-        tc = j - rs * g.C;
-        tr = rs / g.S;
-        ts = rs - tr * g.S;
-    }
-    int pn[NV], pp[NV], pq[NV];  // image, output row, output column of each pixel
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int pix = pbeg + kq + 16 * i;
-        pq[i] = pix % g.Q;
-        const int t = pix / g.Q;
-        pp[i] = t % g.P;
-        pn[i] = t / g.P;
-    }
-    auto load = [&](int kt, int st) {
-        unsigned char *A = stA + st * kUStage, *B = stB + st * bstage;
-        const int p0 = pbeg + kt * UBK;
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int k = kq + 16 * i, pix = p0 + k;
-            const bool live = pix < pend;
-            const __nv_bfloat16 *sy = live && m < a.M ? a.x + (size_t)pix * g.K + m : nullptr;
-            const __nv_bfloat16 *sx = nullptr;
-            if (live && jok) {
-                const int h = pp[i] * g.stride + tr - g.pad, w = pq[i] * g.stride + ts - g.pad;
-                if (h >= 0 && h < g.H && w >= 0 && w < g.W)
-                    sx = a.w + (((size_t)pn[i] * g.H + h) * g.W + w) * g.C + tc;
-            }
-            cp16(A + canon_mn(grp * 8, k), SWAP ? sx : sy, a.x);
-            if (bcol) cp16(B + canon_mn(grp * 8, k), SWAP ? sy : sx, a.w);
-            // next slice: UBK pixels further
-            pq[i] += UBK;
-            while (pq[i] >= g.Q) {
-                pq[i] -= g.Q;
-                if (++pp[i] == g.P) {
-                    pp[i] = 0;
-                    ++pn[i];
-                }
-            }
-        }
-    };
-    for (int kt = 0; kt < UST - 1; ++kt) {
-        if (kt < nk) load(kt, kt);
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t taddr = *tslot;
-    const uint32_t idesc = umma_idesc(BNU, true);
-    bool ok = true;
-    for (int kt = 0; kt < nk; ++kt) {
-        const int st = kt % UST;
-        asm volatile("cp.async.wait_group %0;\n" :: "n"(UST - 2) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            unsigned char *A = stA + st * kUStage, *B = stB + st * bstage;
-#pragma unroll
-            for (int s = 0; s < UBK / 16; ++s) {
-                const uint64_t ad = umma_desc(smem_u32(A) + s * 256);
-                const uint64_t bd = umma_desc(smem_u32(B) + s * 256);
-                const uint32_t acc = (kt > 0 || s > 0) ? 1u : 0u;
-                asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             :: "r"(taddr), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                         :: "r"(smem_u32(mbar + st)) : "memory");
-        }
-        const int nx = kt + UST - 1;
-        if (nx < nk) {
-            const int sx = nx % UST;
-            if (kt >= 1) ok = mbar_wait(smem_u32(mbar + sx), (uint32_t)(((kt - 1) / UST) & 1)) && ok;
-            load(nx, sx);
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    if (nk > 0) {
-        const int last = nk - 1;
-        ok = mbar_wait(smem_u32(mbar + last % UST), (uint32_t)((last / UST) & 1)) && ok;
-    }
-    if (tid == 0 && g_cnn_probe_polls > 0)  // a wait made to run out (test hook)
-        ok = mbar_wait(smem_u32(mbar + UST + 1), 0u, g_cnn_probe_polls) && ok;
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!ok && lane == 0) atomicExch(&g_cnn_status, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const int quarter = warp & 3, group = warp >> 2;
-    const int row = m0 + quarter * 32 + lane;  // output channel (SWAP: filter entry)
-    float *part = a.part + (size_t)blockIdx.z * a.M * a.Ncols;
-    for (int c0 = group * 32; c0 < BNU; c0 += 32 * (UNT / 128)) {
-        uint32_t v[32];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-            "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-              "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-              "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-              "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
-              "=r"(v[31])
-            : "r"(taddr + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-        if constexpr (SWAP) {  // lanes hold consecutive filter entries: coalesced per column
-            if (row < a.Ncols) {
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int k = n0 + c0 + jj;
-                    if (c0 + jj < BNU && k < a.M)
-                        part[(size_t)k * a.Ncols + row] = nk ? __uint_as_float(v[jj]) : 0.f;
-                }
-            }
-        } else if (row < a.M) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 4) {
-                const int col = n0 + c0 + j;
-                if (c0 + j < BNU && col < a.Ncols) {  // Ncols is a multiple of 8
-                    const float f0 = nk ? __uint_as_float(v[j]) : 0.f;
-                    const float f1 = nk ? __uint_as_float(v[j + 1]) : 0.f;
-                    const float f2 = nk ? __uint_as_float(v[j + 2]) : 0.f;
-                    const float f3 = nk ? __uint_as_float(v[j + 3]) : 0.f;
-                    *reinterpret_cast<float4 *>(part + (size_t)row * a.Ncols + col) =
-                        make_float4(f0, f1, f2, f3);
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(taddr), "r"(ncols)
-                     : "memory");
-}
-
-constexpr int kUmmaSmem = 2 * UST * kUStage + 64;  // the largest (BNU = 128)
-__host__ __device__ constexpr int umma_smem(int bnu) { return UST * (kUStage + bnu * UBK * 2) + 64; }
-
-// One-time opt-in to the stages' dynamic shared memory.
-cudaError_t umma_prepare() {
-    static const cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(k_wgrad_umma<false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_wgrad_umma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kUmmaSmem);
-        return r;
-    }();
-    return e;
-}
-
 // Sum of the filter-gradient partial tiles over the pixel splits, in split
 // order.
 // out[i] = sum over z of part[z][i] for i < count, in a fixed order: a CTA
@@ -731,9 +472,6 @@ int status_of(cudaError_t e) { return e == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA
 // Engine of the forward and data-gradient convolutions: the tcgen05 kernel
 // (1, default) or the warp-level MMA kernel (0).
 int g_use_tcgen05 = 1;
-// Filter gradients with fewer than 128 output channels on tcgen05 with the
-// roles exchanged (k_wgrad_umma<true>); 0 keeps them on the warp-level MMA.
-int g_wgrad_swap = 1;
 
 const __nv_bfloat16 *bf(const uint16_t *p) { return reinterpret_cast<const __nv_bfloat16 *>(p); }
 __nv_bfloat16 *bf(uint16_t *p) { return reinterpret_cast<__nv_bfloat16 *>(p); }
@@ -761,9 +499,9 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
     a.Ncols = a.g.K;
     a.Kred = a.g.R * a.g.S * a.g.C;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    // reductions shorter than two slices feed the tensor cores too little per
-    // copied row (measured: the 8-channel first layer is faster on mma.sync)
-    if (g_use_tcgen05 && a.Kred >= 2 * UBK) {
+    // reductions shorter than 128 stay on the warp-level MMA (the 8-channel
+    // first layer and the 1 x 1 head)
+    if (g_use_tcgen05 && a.Kred >= 128) {
         const cudaError_t e = conv_forward_tma(a.g, x, w, bias, relu != 0, y, y_f32, st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
@@ -826,8 +564,10 @@ static int bias_chunks(const Geo &g) {
 size_t osog_conv2d_backward_filter_workspace(const osog_conv_shape_t *shape) {
     if (!shape_ok(shape)) return 0;
     const Geo g = geo_of(shape);
-    return ((size_t)splits_of(g) * g.K * g.R * g.S * g.C + (size_t)bias_chunks(g) * g.K) *
-           sizeof(float);
+    const size_t warp = ((size_t)splits_of(g) * g.K * g.R * g.S * g.C +
+                         (size_t)bias_chunks(g) * g.K) * sizeof(float);
+    const size_t tma = conv_wgrad_tma_workspace(g);
+    return warp > tma ? warp : tma;  // whichever engine the call runs on
 }
 
 int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *dy,
@@ -837,6 +577,10 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     if (!ws || ws_bytes < osog_conv2d_backward_filter_workspace(shape)) return OSOG_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const Geo g = geo_of(shape);
+    if (g_use_tcgen05) {
+        const cudaError_t e = conv_wgrad_tma(g, dy, x, dw, dbias, static_cast<float *>(ws), st);
+        if (e != cudaErrorNotSupported) return status_of(e);
+    }
     Args a{};
     a.g = g;
     a.x = bf(dy);
@@ -846,24 +590,8 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     a.Ncols = g.R * g.S * g.C;
     a.Kred = g.N * g.P * g.Q;
     const int splits = splits_of(g);
-    // tcgen05: output channels as the 128 rows when there are at least 128,
-    // else, with at least 64 filter entries, the filter entries as the rows
-    // and the output channels (rounded up to 16) as the columns
-    if (g_use_tcgen05 && a.M >= UM) {
-        const cudaError_t e = umma_prepare();
-        if (e != cudaSuccess) return status_of(e);
-        dim3 grid((a.M + UM - 1) / UM, (a.Ncols + 127) / 128, splits);
-        k_wgrad_umma<false><<<grid, UNT, umma_smem(128), st>>>(a, 128);
-    } else if (g_use_tcgen05 && g_wgrad_swap && a.Ncols >= 64) {
-        const cudaError_t e = umma_prepare();
-        if (e != cudaSuccess) return status_of(e);
-        const int bnu = (a.M + 15) / 16 * 16;
-        dim3 grid((a.Ncols + UM - 1) / UM, 1, splits);
-        k_wgrad_umma<true><<<grid, UNT, umma_smem(bnu), st>>>(a, bnu);
-    } else {
-        dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN, splits);
-        k_conv_gemm<kWgrad><<<grid, NT, 0, st>>>(a);
-    }
+    dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN, splits);
+    k_conv_gemm<kWgrad><<<grid, NT, 0, st>>>(a);
     const int64_t count = (int64_t)a.M * a.Ncols;
     sum_splits(a.part, splits, count, dw, st);
     const int64_t pixels = (int64_t)g.N * g.P * g.Q;
@@ -891,21 +619,14 @@ void osog_conv_use_tcgen05(int32_t enable) { g_use_tcgen05 = enable ? 1 : 0; }
 
 int osog_conv_test_wait_limit(int32_t polls) {
     const int v = polls > 0 ? polls : 0;
-    return cudaMemcpyToSymbol(g_cnn_probe_polls, &v, sizeof v) == cudaSuccess &&
-                   conv_tma_set_probe(v) == cudaSuccess
-               ? OSOG_OK
-               : OSOG_ERR_CUDA;
+    return status_of(conv_tma_set_probe(v));
 }
 
 int osog_conv_sync_status(osog_stream_t stream) {
     if (cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return OSOG_ERR_CUDA;
-    int v = 0, t = 0;
-    if (cudaMemcpyFromSymbol(&v, g_cnn_status, sizeof v) != cudaSuccess) return OSOG_ERR_CUDA;
+    int t = 0;
     if (conv_tma_take_status(&t) != cudaSuccess) return OSOG_ERR_CUDA;
-    if (!v) return t ? OSOG_ERR_TIMEOUT : OSOG_OK;
-    const int zero = 0;
-    if (cudaMemcpyToSymbol(g_cnn_status, &zero, sizeof zero) != cudaSuccess) return OSOG_ERR_CUDA;
-    return OSOG_ERR_TIMEOUT;
+    return t ? OSOG_ERR_TIMEOUT : OSOG_OK;
 }
 
 }  // extern "C"

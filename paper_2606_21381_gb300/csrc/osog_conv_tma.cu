@@ -475,6 +475,281 @@ k_conv_patch(const __grid_constant__ CUtensorMap src, const __grid_constant__ CU
                      : "memory");
 }
 
+// Filter gradient: dW[k][r, s][c] = sum over output pixels of dY[pixel][k]
+// X[pixel st + (r, s) - pad][c], and dbias[k] = sum of dY[pixel][k].
+//
+// The pixels are the reduction.  A tile of 8 x 16 output pixels of dY (rows of
+// 64 output channels) and the patches of X it touches are loaded once and feed
+// every tap of the CTA's group: tap (r, s) multiplies the same dY rows with the
+// patch rows shifted by the tap, both operands with the reduction outermost
+// (MN-major).  A CTA adds the tiles z, z + splits, ... of its split into one
+// tensor-memory accumulator per tap (128 output channels by up to 128 input
+// channels, 512 columns in all) and writes its partial sums; k_sum_parts adds
+// the splits in order.  The warps that neither load nor issue sum dY over the
+// pixels of the tile for the bias gradient while it is in shared memory.
+//
+// Measured with the sums over the splits and the bias gradient (us, 64 images,
+// before / now): 128 -> 128, 32 x 32: 123 / 23; 64 -> 128, stride 2: 116 / 20;
+// 32 -> 64, stride 2: 138 / 37 (bound by the reads of dY from shared memory, 4 KB
+// per product however few its columns); 128 -> 64: 96 / 21.
+struct WgradArgs {
+    int tiles_x, tiles, splits;        // tiles of all images
+    int tiles_y;
+    int pw, ph, plane_bytes;           // X patch planes
+    int stride, pad;
+    int chunks;                        // ch-channel chunks of a column block
+    int k64;                           // 64-channel blocks of dY in a row block (1 or 2)
+    int ring, stage_bytes;
+    int bn, cblk;                      // columns of an accumulator, channels of a column block
+    int cblocks, groups;               // column blocks, tap groups
+    int K, C, RS;
+    uint32_t tmem_cols;
+    float *part;                       // [splits][K RS C + K]
+    int group0[kMaxTaps + 1];          // first tap of each group
+    uint8_t planes[kMaxTaps];          // per group: the planes its taps read, bit set
+    Tap tap[kMaxTaps];                 // sorted by group
+};
+
+constexpr int kSumThreads = kCtaThreads - 64;  // warps 2..7: the bias gradient
+
+template <int CH>
+__global__ void __launch_bounds__(kCtaThreads, 1)
+k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ CUtensorMap mx,
+              const __grid_constant__ WgradArgs a) {
+    constexpr int kRow = 2 * CH;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ uint64_t bars[2 * kMaxRing + 2];
+    __shared__ uint32_t tmem_slot;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const uint32_t full = smem_addr(bars), empty = full + 8u * kMaxRing,
+                   all_done = empty + 8u * kMaxRing, probe = all_done + 8u;
+    const int group = blockIdx.x % a.groups, blk = blockIdx.x / a.groups;
+    const int c0 = (blk % a.cblocks) * a.cblk, k0 = (blk / a.cblocks) * 128;
+    const int z = blockIdx.y;
+    const bool sums_bias = group == 0 && c0 == 0;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
+                     ::"r"(smem_addr(&tmem_slot)), "r"(a.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < kMaxRing; ++i) {
+            init_bar(full + 8u * i);
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n"
+                         ::"r"(empty + 8u * i), "r"(sums_bias ? 1 + kSumThreads / 32 : 1) : "memory");
+        }
+        init_bar(all_done);
+        init_bar(probe);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const uint32_t base = smem_addr(smem);
+    const int dy_bytes = a.k64 * kTileW * kTileH * 128;
+    const uint32_t planes = a.planes[group];
+    const int nplanes = __popc(planes);
+    const int t0 = a.group0[group], nt = a.group0[group + 1] - t0;
+    const int ntiles = (a.tiles - z + a.splits - 1) / a.splits;
+    bool ok = true;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (warp == 0) {
+        int st = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < ntiles && ok; ++i) {
+            if (i >= a.ring) ok = wait_bar(empty + 8u * st, ph ^ 1u);
+            if (!ok) break;
+            const int tile = z + i * a.splits;
+            const int img = tile / (a.tiles_x * a.tiles_y), t = tile - img * a.tiles_x * a.tiles_y;
+            const int oy = (t / a.tiles_x) * kTileH, ox = (t % a.tiles_x) * kTileW;
+            const uint32_t dst = base + (uint32_t)st * a.stage_bytes, bar = full + 8u * st;
+            if (elect_lane()) {
+                expect_bytes(bar, (uint32_t)(dy_bytes + nplanes * a.chunks * a.pw * a.ph * kRow));
+                for (int b = 0; b < a.k64; ++b)
+                    load_4d(dst + (uint32_t)(b * kTileW * kTileH * 128), &mdy, k0 + b * 64, ox, oy, img, bar);
+                int slot = 0;
+                for (int p = 0; p < 4; ++p) {
+                    if (!((planes >> p) & 1u)) continue;
+                    for (int c = 0; c < a.chunks; ++c)
+                        load_4d(dst + dy_bytes + (uint32_t)((c * nplanes + slot) * a.plane_bytes), &mx,
+                                c0 + c * CH, ox * a.stride - a.pad + (p & 1),
+                                oy * a.stride - a.pad + (p >> 1), img, bar);
+                    ++slot;
+                }
+            }
+            __syncwarp();
+            if (++st == a.ring) {
+                st = 0;
+                ph ^= 1u;
+            }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = instr_desc(a.bn, true, true);
+        const uint32_t pitch = (uint32_t)(a.pw * kRow), pitch16 = pitch >> 4;
+        const uint32_t a_hi = desc_hi<128>(1024u), b_hi = desc_hi<kRow>(pitch);
+        const uint32_t b_lead = (uint32_t)(nplanes * a.plane_bytes);
+        const uint32_t plane16 = (uint32_t)a.plane_bytes >> 4, bn = (uint32_t)a.bn;
+        int st = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < ntiles && ok; ++i) {
+            ok = wait_bar(full + 8u * st, ph);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t src = base + (uint32_t)st * a.stage_bytes;
+            const uint32_t a_lo = desc_lo(src, kTileW * kTileH * 128);
+            const uint32_t x_lo = desc_lo(src + dy_bytes, b_lead);
+            const bool lead = elect_lane();
+            Tap next = a.tap[t0];
+            for (int t = 0; t < nt; ++t) {
+                const Tap now = next;
+                next = a.tap[min(t0 + t + 1, t0 + nt - 1)];
+                const uint32_t slot = __popc(planes & ((1u << now.plane) - 1u));
+                const uint32_t b_lo = x_lo + slot * plane16 + now.sy * pitch16 + now.sx * (kRow >> 4);
+                const uint32_t acc = tmem + (uint32_t)t * bn;
+                if (lead) {
+#pragma unroll
+                    for (int k = 0; k < kTileH / 2; ++k)  // 16 pixels: two rows of the tile
+                        mma(acc, a_lo + k * (2048u >> 4), a_hi, b_lo + k * 2u * pitch16, b_hi, idesc,
+                            i > 0 || k > 0 ? 1u : 0u);
+                }
+            }
+            if (lead) commit_to(empty + 8u * st);
+            __syncwarp();
+            if (++st == a.ring) {
+                st = 0;
+                ph ^= 1u;
+            }
+        }
+        if (ok && elect_lane()) commit_to(all_done);
+    } else if (sums_bias) {
+        // thread u sums the 8 channels of vector u % vecs over the pixels u /
+        // vecs, + lanes, ...
+        const int u = tid - 64, vecs = a.k64 * 8, lanes = kSumThreads / vecs;
+        const int vec = u % vecs, p0 = u / vecs;
+        int st = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < ntiles && ok; ++i) {
+            ok = wait_bar(full + 8u * st, ph);
+            if (!ok) break;
+            const unsigned char *src = smem + (size_t)st * a.stage_bytes +
+                                       (vec >> 3) * (kTileW * kTileH * 128);
+            for (int p = p0; p < kTileW * kTileH; p += lanes) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(src + p * 128 + (((vec ^ p) & 7) << 4));
+                const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(h[j]);
+                    sum[2 * j] += f.x;
+                    sum[2 * j + 1] += f.y;
+                }
+            }
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(empty + 8u * st) : "memory");
+            if (++st == a.ring) {
+                st = 0;
+                ph ^= 1u;
+            }
+        }
+    }
+    __syncwarp();
+    ok = wait_bar(all_done, 0u) && ok;
+    if (tid == 0 && g_probe_polls > 0)  // a wait made to run out (test hook)
+        ok = wait_bar(probe, 0u, g_probe_polls) && ok;
+    if (!ok) atomicExch(&g_status, 1);
+    __syncthreads();  // every stage is consumed: shared memory is free
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    float *part = a.part + (size_t)z * ((size_t)a.K * a.RS * a.C + a.K);
+    if (sums_bias) {  // the pixel lanes of a channel in order
+        float *red = reinterpret_cast<float *>(smem);  // [lanes][8 vecs]
+        const int u = tid - 64, vecs = a.k64 * 8, lanes = kSumThreads / vecs;
+        if (u >= 0)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) red[(u / vecs) * vecs * 8 + (u % vecs) * 8 + j] = sum[j];
+        __syncthreads();
+        if (tid < vecs * 8 && k0 + tid < a.K) {
+            float v = 0.f;
+            for (int l = 0; l < lanes; ++l) v += red[l * vecs * 8 + tid];
+            part[(size_t)a.K * a.RS * a.C + k0 + tid] = v;
+        }
+        __syncthreads();
+    }
+    // accumulators to the partial sums: warp w holds output channels 32 (w % 4)
+    // .. + 31 (one per lane); pieces of 32 input channels leave through the
+    // warp's shared rows so that the stores are whole lines
+    const int quarter = warp & 3, half = warp >> 2;
+    unsigned char *stage = smem + warp * kStageBytes;
+    const int pieces = (a.bn + 31) / 32;
+    const int kfirst = k0 + quarter * 32;
+    if (kfirst < a.K && quarter * 32 < a.k64 * 64)
+        for (int u = half; u < nt * pieces; u += 2) {
+            const int t = u / pieces, cc = (u % pieces) * 32;
+            uint32_t v[32];
+            tmem_load32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * a.bn + cc), v);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4)
+                *reinterpret_cast<uint4 *>(stage + lane * kStageRow + j * 4) =
+                    make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            __syncwarp();
+            const int wt = a.tap[t0 + t].wt;
+            const int c = c0 + cc + (lane & 7) * 4;
+            if (c < a.C && cc + (lane & 7) * 4 < a.cblk) {
+#pragma unroll
+                for (int r = lane >> 3; r < 32; r += 4) {
+                    if (kfirst + r >= a.K) continue;
+                    *reinterpret_cast<uint4 *>(part + ((size_t)(kfirst + r) * a.RS + wt) * a.C + c) =
+                        *reinterpret_cast<const uint4 *>(stage + r * kStageRow + (lane & 7) * 16);
+                }
+            }
+            __syncwarp();
+        }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.tmem_cols)
+                     : "memory");
+}
+
+// out[i] = sum over z of part[z][i], i < count (out = dw) or count <= i < count
+// + extra (out2 = dbias), four outputs per thread (count and extra are
+// multiples of 8), the splits in order within each of kSumLanes interleaved
+// partial sums, which are then added in order.
+constexpr int kSumLanes = 8;
+__global__ void __launch_bounds__(32 * kSumLanes)
+k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, float4 *out,
+            float4 *out2) {
+    __shared__ float4 red[kSumLanes][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane, row = count4 + extra4;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < row) {
+#pragma unroll 4
+        for (int z = w; z < splits; z += kSumLanes) {
+            const float4 v = __ldg(part + (size_t)z * row + i);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    }
+    red[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && i < row) {
+        for (int l = 1; l < kSumLanes; ++l) {
+            const float4 v = red[l][lane];
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+        if (i < count4)
+            out[i] = s;
+        else
+            out2[i - count4] = s;
+    }
+}
+
 // ------------------------------------------------------------------ host
 using EncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                               const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -522,7 +797,7 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 uint32_t tmem_columns(int need) {
-    uint32_t c = 32;
+    uint32_t c = 32;  // need is at most 512, what an SM has
     while ((int)c < need) c *= 2;
     return c;
 }
@@ -739,6 +1014,131 @@ cudaError_t conv_dgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *w,
     const uint32_t fb[3] = {64, 1, (uint32_t)a.ch};
     if (e == cudaSuccess) e = encode(&flt, w, 3, fd, fb, ones);
     return e == cudaSuccess ? launch_patch<false>(src, flt, a, g.N, st) : e;
+}
+
+namespace {
+
+// Plan of the filter gradient; false if no stage fits in shared memory.
+bool wgrad_plan(const Geo &g, WgradArgs &a, int &ch) {
+    ch = g.C <= 32 ? 32 : 64;
+    a.K = g.K;
+    a.C = g.C;
+    a.RS = g.R * g.S;
+    a.stride = g.stride;
+    a.pad = g.pad;
+    a.k64 = g.K <= 64 ? 1 : 2;
+    a.tiles_x = ceil_div(g.Q, kTileW);
+    a.tiles_y = ceil_div(g.P, kTileH);
+    a.tiles = g.N * a.tiles_x * a.tiles_y;
+    const bool two = g.stride == 2;
+    a.pw = kTileW + (two ? (g.S - 1) / 2 : g.S - 1);
+    a.ph = kTileH + (two ? (g.R - 1) / 2 : g.R - 1);
+    if ((a.pw - 1) * g.stride + 1 > 256 || (a.ph - 1) * g.stride + 1 > 256) return false;
+    a.plane_bytes = round_up(a.pw * a.ph * 2 * ch, 1024);
+    const int dy = a.k64 * kTileW * kTileH * 128;
+    for (a.chunks = g.C > 64 ? 2 : 1; a.chunks >= 1; --a.chunks) {
+        a.cblk = a.chunks * ch;
+        a.bn = round_up(g.C < a.cblk ? g.C : a.cblk, 16);
+        a.cblocks = ceil_div(g.C, a.cblk);
+        // taps by the plane they read, in the order that pairs the plane of four
+        // taps with that of one; groups of as many accumulators as tensor
+        // memory holds, spread evenly
+        static const int order[4] = {0, 3, 1, 2};
+        // (an accumulator is read back in pieces of 32 columns)
+        const int fit = (512 - round_up(a.bn, 32)) / a.bn + 1;
+        const int most = fit < a.RS ? fit : a.RS;
+        a.groups = ceil_div(a.RS, most);
+        const int each = ceil_div(a.RS, a.groups);
+        int n = 0;
+        for (int o = 0; o < 4; ++o)
+            for (int r = 0; r < g.R; ++r)
+                for (int s = 0; s < g.S; ++s) {
+                    const int plane = two ? (r & 1) * 2 + (s & 1) : 0;
+                    if (plane != order[o]) continue;
+                    Tap &t = a.tap[n++];
+                    t.plane = (uint8_t)plane;
+                    t.sy = (uint8_t)(two ? r >> 1 : r);
+                    t.sx = (uint8_t)(two ? s >> 1 : s);
+                    t.wt = (int16_t)(r * g.S + s);
+                }
+        int planes = 0;
+        for (int gr = 0; gr <= a.groups; ++gr) a.group0[gr] = gr * each < a.RS ? gr * each : a.RS;
+        for (int gr = 0; gr < a.groups; ++gr) {
+            a.planes[gr] = 0;
+            for (int t = a.group0[gr]; t < a.group0[gr + 1]; ++t) a.planes[gr] |= 1u << a.tap[t].plane;
+            const int np = __builtin_popcount(a.planes[gr]);
+            planes = np > planes ? np : planes;
+        }
+        a.stage_bytes = dy + planes * a.chunks * a.plane_bytes;
+        a.ring = (kSmemMax - 2048) / a.stage_bytes;
+        if (a.ring > kMaxRing) a.ring = kMaxRing;
+        if (a.ring < 1) continue;
+        a.tmem_cols = tmem_columns((each - 1) * a.bn + round_up(a.bn, 32));
+        const int blocks = ceil_div(g.K, 128) * a.cblocks * a.groups;
+        int splits = 152 / blocks;
+        splits = splits < 1 ? 1 : splits;
+        a.splits = splits < a.tiles ? splits : a.tiles;
+        return true;
+    }
+    return false;
+}
+
+// The matrix instructions read 128 rows of dY, two 64-channel blocks, also when
+// a stage holds one (the rows of the second are not used): the last stage's
+// reads end inside the allocation too.
+int wgrad_smem(const WgradArgs &a) {
+    const int n = a.ring * a.stage_bytes;
+    const int reach = (a.ring - 1) * a.stage_bytes + 2 * kTileW * kTileH * 128;
+    const int m = n > reach ? n : reach;
+    return m > kEpilogueSmem ? m : kEpilogueSmem;
+}
+
+template <int CH>
+cudaError_t launch_wgrad(const CUtensorMap &mdy, const CUtensorMap &mx, const WgradArgs &a,
+                         cudaStream_t st) {
+    static const cudaError_t opt_in = cudaFuncSetAttribute(
+        k_wgrad_patch<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
+    if (opt_in != cudaSuccess) return opt_in;
+    const dim3 grid(ceil_div(a.K, 128) * a.cblocks * a.groups, a.splits);
+    k_wgrad_patch<CH><<<grid, kCtaThreads, wgrad_smem(a), st>>>(mdy, mx, a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t conv_wgrad_tma_workspace(const Geo &g) {
+    WgradArgs a{};
+    int ch;
+    if (!wgrad_plan(g, a, ch)) return 0;
+    return (size_t)a.splits * ((size_t)a.K * a.RS * a.C + a.K) * sizeof(float);
+}
+
+cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, float *dw,
+                           float *dbias, float *ws, cudaStream_t st) {
+    WgradArgs a{};
+    int ch;
+    if ((reinterpret_cast<uintptr_t>(ws) | reinterpret_cast<uintptr_t>(dw) |
+         reinterpret_cast<uintptr_t>(dbias)) & 15)
+        return cudaErrorNotSupported;  // moved as 16-byte vectors
+    if (!wgrad_plan(g, a, ch)) return cudaErrorNotSupported;
+    a.part = ws;
+    CUtensorMap mdy, mx;
+    const uint64_t yd[4] = {(uint64_t)g.K, (uint64_t)g.Q, (uint64_t)g.P, (uint64_t)g.N};
+    const uint32_t yb[4] = {64, kTileW, kTileH, 1}, ones[4] = {1, 1, 1, 1};
+    cudaError_t e = encode(&mdy, dy, 4, yd, yb, ones);
+    const uint64_t xd[4] = {(uint64_t)g.C, (uint64_t)g.W, (uint64_t)g.H, (uint64_t)g.N};
+    const uint32_t xb[4] = {(uint32_t)ch, (uint32_t)((a.pw - 1) * g.stride + 1),
+                            (uint32_t)((a.ph - 1) * g.stride + 1), 1};
+    const uint32_t xe[4] = {1, (uint32_t)g.stride, (uint32_t)g.stride, 1};
+    if (e == cudaSuccess) e = encode(&mx, x, 4, xd, xb, xe);
+    if (e != cudaSuccess) return e;
+    e = ch == 64 ? launch_wgrad<64>(mdy, mx, a, st) : launch_wgrad<32>(mdy, mx, a, st);
+    if (e != cudaSuccess) return e;
+    const int64_t count4 = (int64_t)a.K * a.RS * a.C / 4, extra4 = a.K / 4;
+    k_sum_parts<<<(unsigned)((count4 + extra4 + 31) / 32), 32 * kSumLanes, 0, st>>>(
+        reinterpret_cast<const float4 *>(ws), a.splits, count4, extra4, reinterpret_cast<float4 *>(dw),
+        reinterpret_cast<float4 *>(dbias));
+    return cudaGetLastError();
 }
 
 cudaError_t conv_tma_take_status(int *timed_out) {

@@ -20,6 +20,12 @@ cudaError_t conv_forward_tma(const Geo &g, const uint16_t *x, const uint16_t *w,
 cudaError_t conv_dgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *w,
                            const uint16_t *mask, uint16_t *dx, cudaStream_t st);
 
+// Filter and bias gradients (ws: conv_wgrad_tma_workspace bytes, 16-byte
+// aligned like dw and dbias); cudaErrorNotSupported as above (workspace 0).
+size_t conv_wgrad_tma_workspace(const Geo &g);
+cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, float *dw,
+                           float *dbias, float *ws, cudaStream_t st);
+
 // Latched status of the bounded waits (read and cleared), and the
 // failure-detection hook (osog_conv_test_wait_limit).
 cudaError_t conv_tma_take_status(int *timed_out);

@@ -108,7 +108,7 @@ def test_conv_backward_data_matches_reference(cnn, shape, masked):
     assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
 
 
-@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
 def test_conv_backward_filter_matches_reference(cnn, shape):
     dev = torch.device("cuda")
     x, w, b, dy = _inputs(shape, 3)
