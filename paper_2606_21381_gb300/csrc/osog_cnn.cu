@@ -331,6 +331,348 @@ __global__ void __launch_bounds__(NT) k_conv_gemm(const __grid_constant__ Args a
             }
 }
 
+// ---------------------------------------------------------------- 8 channels
+// The first layer (8 input channels, nine or ten taps): its reduction is too
+// short for tcgen05, and the tiles of k_conv_gemm spend their time on gathers
+// (every pixel is fetched once per tap through L1, 120 us of a 20 us HBM floor
+// on 64 images of 256 x 256).  A pixel is one 16-byte vector, which is also one
+// row of an ldmatrix 8 x 8 block: so the input patch of a tile is copied to
+// shared memory once and every tap's fragment is read from it in place.  For
+// stride 2 the patch's even and odd columns are kept apart, so that eight
+// output pixels of one tap are 128 contiguous bytes.  The products are added in
+// the order of k_conv_gemm (two taps per k16 step): the same bits.  On those
+// images forward 120 -> 48 us, filter gradient 167 (110 by k_wgrad_patch, whose
+// products of 16 columns are bound by their reads of dY) -> 54 us, at a quarter
+// to a third of HBM: two or three CTAs of an SM do not cover the copies' latency
+// and the issue of fragments.
+constexpr int kC8Taps = 10, kC8W = 32, kC8Threads = 256;
+
+struct PatchC8 {
+    int stride, pad, S, RS;
+    int pw, ph, half, pitch;  // pixels; half: columns of one parity; pitch: pixels per row
+};
+
+__host__ __device__ inline PatchC8 patch_c8(const Geo &g, int rows) {
+    PatchC8 p;
+    p.stride = g.stride;
+    p.pad = g.pad;
+    p.S = g.S;
+    p.RS = g.R * g.S;
+    p.pw = (kC8W - 1) * g.stride + g.S;
+    p.ph = (rows - 1) * g.stride + g.R;
+    p.half = (p.pw + 1) / 2;
+    p.pitch = g.stride == 2 ? 2 * p.half : p.pw;
+    return p;
+}
+
+// 16-byte asynchronous copy to shared memory; a NULL source writes zeros.
+__device__ __forceinline__ void cp16(void *dst, const __nv_bfloat16 *src, const void *any) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n"
+                 :: "r"(smem_u32(dst)), "l"(src ? (const void *)src : any), "r"(src ? 16 : 0)
+                 : "memory");
+}
+
+// Copy of the input patch of the output tile (oy0, ox0) of image n.
+__device__ __forceinline__ void load_patch_c8(const Geo &g, const PatchC8 &p, const __nv_bfloat16 *x,
+                                              int n, int oy0, int ox0, uint4 *dst) {
+    const int h0 = oy0 * p.stride - p.pad, w0 = ox0 * p.stride - p.pad;
+    const __nv_bfloat16 *img = x + (size_t)n * g.H * g.W * 8;
+    const float inv = 1.f / (float)p.pw;
+    for (int e = threadIdx.x; e < p.ph * p.pw; e += kC8Threads) {
+        int r = (int)((float)e * inv);  // e / pw, corrected below (e < 2^24)
+        int c = e - r * p.pw;
+        if (c >= p.pw) {
+            ++r;
+            c -= p.pw;
+        } else if (c < 0) {
+            --r;
+            c += p.pw;
+        }
+        const int h = h0 + r, w = w0 + c;
+        const bool in = h >= 0 && h < g.H && w >= 0 && w < g.W;
+        const int at = p.stride == 2 ? (c & 1) * p.half + (c >> 1) : c;
+        cp16(dst + r * p.pitch + at, in ? img + ((size_t)h * g.W + w) * 8 : nullptr, x);
+    }
+}
+
+// Shared address of tap t's pixel for output pixel (row, x) of the tile.
+__device__ __forceinline__ uint32_t tap_c8(const PatchC8 &p, uint32_t patch, int t, int row, int x) {
+    const int r = t / p.S, s = t - r * p.S;
+    const int col = p.stride == 2 ? (s & 1) * p.half + x + (s >> 1) : x + s;
+    return patch + (uint32_t)((row * p.stride + r) * p.pitch + col) * 16u;
+}
+
+__device__ __forceinline__ void ldsm_x4_at(unsigned (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldsm_x4_t_at(unsigned (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+
+// Forward: a CTA computes 32 x 16 output pixels of 32 output channels, warp w
+// the rows w and w + 8, 16 pixels at a time; the filters' fragments stay in
+// registers.
+constexpr int kC8Rows = 16;
+__global__ void __launch_bounds__(kC8Threads, 3) k_conv_c8(const __grid_constant__ Args a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(16) unsigned char out[kC8Threads / 32][16 * 80];
+    __shared__ __align__(16) uint4 zero;
+    const Geo &g = a.g;
+    const PatchC8 p = patch_c8(g, kC8Rows);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tx = (g.Q + kC8W - 1) / kC8W, ty = (g.P + kC8Rows - 1) / kC8Rows;
+    const int n = blockIdx.x / (tx * ty), tile = blockIdx.x - n * tx * ty;
+    const int oy0 = tile / tx * kC8Rows, ox0 = tile % tx * kC8W, n0 = blockIdx.y * 32;
+    if (threadIdx.x == 0) zero = zero4();
+    load_patch_c8(g, p, a.x, n, oy0, ox0, reinterpret_cast<uint4 *>(smem));
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    // fragments of the filters: column n = lane / 4 of each block of 8, entries
+    // 2 (lane % 4), + 1 and those + 8 of every k16 step
+    unsigned bf[kC8Taps / 2][4][2];
+#pragma unroll
+    for (int ks = 0; ks < kC8Taps / 2; ++ks)
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int col = n0 + nt * 8 + (lane >> 2), j = ks * 16 + h * 8 + (lane & 3) * 2;
+                bf[ks][nt][h] = col < a.Ncols && j < a.Kred
+                                    ? *reinterpret_cast<const unsigned *>(a.w + (size_t)col * a.Kred + j)
+                                    : 0u;
+            }
+    float2 bias[4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const int col = n0 + nt * 8 + (lane & 3) * 2;
+        bias[nt] = col < a.Ncols ? make_float2(a.bias[col], a.bias[col + 1]) : make_float2(0.f, 0.f);
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    const uint32_t patch = smem_u32(smem), none = smem_u32(&zero);
+    const int q = lane >> 3, r8 = lane & 7;
+    // this lane's row of each k16 step's blocks (pixels 0-7 | 8-15) x (tap 2 ks
+    // | 2 ks + 1); a tap past the last reads zeros
+    uint32_t src[kC8Taps / 2];
+    bool tap[kC8Taps / 2];
+#pragma unroll
+    for (int ks = 0; ks < kC8Taps / 2; ++ks) {
+        const int t = 2 * ks + (q >> 1);
+        tap[ks] = t < p.RS;
+        src[ks] = tap[ks] ? tap_c8(p, patch, t, 0, (q & 1) * 8 + r8) : none;
+    }
+    const uint32_t row_step = (uint32_t)(p.stride * p.pitch) * 16u;
+    unsigned char *st = out[warp];
+    for (int row = warp; row < kC8Rows; row += kC8Threads / 32) {
+        const int oy = oy0 + row;
+        if (oy >= g.P) break;
+#pragma unroll
+        for (int xb = 0; xb < kC8W; xb += 16) {
+            if (ox0 + xb >= g.Q) break;
+            float acc[4][4];
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[nt][j] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < kC8Taps / 2; ++ks) {
+                unsigned af[4];
+                ldsm_x4_at(af, src[ks] + (tap[ks] ? row * row_step + xb * 16u : 0u));
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[nt], af, bf[ks][nt][0], bf[ks][nt][1]);
+            }
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float v0 = acc[nt][2 * h] + bias[nt].x, v1 = acc[nt][2 * h + 1] + bias[nt].y;
+                    if (a.relu) {
+                        v0 = fmaxf(v0, 0.f);
+                        v1 = fmaxf(v1, 0.f);
+                    }
+                    *reinterpret_cast<__nv_bfloat162 *>(st + ((lane >> 2) + 8 * h) * 80 + nt * 16 +
+                                                        (lane & 3) * 4) = __floats2bfloat162_rn(v0, v1);
+                }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int px = i * 8 + (lane >> 2), vec = lane & 3;
+                const int ox = ox0 + xb + px, col = n0 + vec * 8;
+                if (ox < g.Q && col < a.Ncols)
+                    *reinterpret_cast<uint4 *>(a.y + (((size_t)n * g.P + oy) * g.Q + ox) * a.Ncols + col) =
+                        *reinterpret_cast<const uint4 *>(st + px * 80 + vec * 16);
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// Filter and bias gradient: a CTA adds the tiles z, z + splits, ... of 32 x 8
+// output pixels; warp w takes row w, 16 pixels to a k16 step, with the output
+// channels (16 MT) as the rows and every tap's 8 channels as one block of
+// columns.  The next tile's copies run during a tile's products.  Partial sums
+// in the layout of k_sum_parts.
+constexpr int kC8GradRows = kC8Threads / 32;
+template <int MT>
+__global__ void __launch_bounds__(kC8Threads, MT == 2 ? 2 : 1)
+k_wgrad_c8(const __grid_constant__ Args a, int splits) {
+    constexpr int KP = MT * 16, VECS = KP / 8, kPix = kC8W * kC8GradRows;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(16) uint4 zero;
+    const Geo &g = a.g;
+    const PatchC8 p = patch_c8(g, kC8GradRows);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tx = (g.Q + kC8W - 1) / kC8W, ty = (g.P + kC8GradRows - 1) / kC8GradRows;
+    const int tiles = g.N * tx * ty, z = blockIdx.x;
+    const int patch_bytes = p.pitch * p.ph * 16, stage = kPix * KP * 2 + patch_bytes;
+    if (threadIdx.x == 0) zero = zero4();
+    // vector v of pixel px: rows of KP / 8 vectors, rotated so that eight
+    // consecutive pixels of one vector fall on different banks
+    auto at = [](int px, int v) { return px * VECS + (VECS == 4 ? v ^ ((px >> 1) & 3) : v ^ (px & 7)); };
+    auto load = [&](int tile, unsigned char *dst) {
+        const int n = tile / (tx * ty), t = tile - n * tx * ty;
+        const int oy0 = t / tx * kC8GradRows, ox0 = t % tx * kC8W;
+        uint4 *d = reinterpret_cast<uint4 *>(dst);
+        for (int e = threadIdx.x; e < kPix * VECS; e += kC8Threads) {
+            const int v = e % VECS, px = e / VECS, oy = oy0 + px / kC8W, ox = ox0 + px % kC8W;
+            const bool in = oy < g.P && ox < g.Q && v * 8 < g.K;
+            cp16(d + at(px, v), in ? a.x + (((size_t)n * g.P + oy) * g.Q + ox) * g.K + v * 8 : nullptr, a.x);
+        }
+        load_patch_c8(g, p, a.w, n, oy0, ox0, reinterpret_cast<uint4 *>(dst + kPix * KP * 2));
+    };
+    float acc[MT][kC8Taps][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int t = 0; t < kC8Taps; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[mt][t][j] = 0.f;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int q = lane >> 3, r8 = lane & 7;
+    // this lane's row of the blocks (tap 2 tp | 2 tp + 1) x (pixels 0-7 | 8-15)
+    // of the warp's image row, relative to a stage; a tap past the last reads
+    // zeros
+    const uint32_t none = smem_u32(&zero);
+    uint32_t src[kC8Taps / 2];
+    bool tap[kC8Taps / 2];
+#pragma unroll
+    for (int tp = 0; tp < kC8Taps / 2; ++tp) {
+        const int t = 2 * tp + (q >> 1);
+        tap[tp] = t < p.RS;
+        src[tp] = tap[tp] ? tap_c8(p, kPix * KP * 2, t, warp, (q & 1) * 8 + r8) : none;
+    }
+    load(z, smem);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    int buf = 0;
+    for (int tile = z; tile < tiles; tile += splits) {
+        if (tile + splits < tiles) load(tile + splits, smem + (buf ^ 1) * stage);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();
+        const uint32_t dy = smem_u32(smem + buf * stage);
+#pragma unroll
+        for (int xb = 0; xb < kC8W; xb += 16) {
+            unsigned af[MT][4];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)  // (channels 0-7 | 8-15) x (pixels 0-7 | 8-15)
+                ldsm_x4_t_at(af[mt], dy + 16u * at(warp * kC8W + xb + r8 + (q >> 1) * 8, mt * 2 + (q & 1)));
+#pragma unroll
+            for (int tp = 0; tp < kC8Taps / 2; ++tp) {
+                unsigned bf[4];
+                ldsm_x4_t_at(bf, src[tp] + (tap[tp] ? dy + xb * 16u : 0u));
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    mma_bf16(acc[mt][2 * tp], af[mt], bf[0], bf[1]);
+                    mma_bf16(acc[mt][2 * tp + 1], af[mt], bf[2], bf[3]);
+                }
+            }
+        }
+        // bias: thread u sums vector u % VECS over the pixels u / VECS, ...
+        const uint4 *d = reinterpret_cast<const uint4 *>(smem + buf * stage);
+#pragma unroll
+        for (int px = threadIdx.x / VECS; px < kPix; px += kC8Threads / VECS) {
+            const uint4 v = d[at(px, threadIdx.x % VECS)];
+            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 f = __bfloat1622float2(h[j]);
+                sum[2 * j] += f.x;
+                sum[2 * j + 1] += f.y;
+            }
+        }
+        __syncthreads();
+        buf ^= 1;
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    // the warps' sums in warp order, then the pixel lanes of the bias
+    float *red = reinterpret_cast<float *>(smem);          // [KP][80]
+    float *bred = red + KP * kC8Taps * 8;                  // [lanes][KP]
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        bred[(threadIdx.x / VECS) * KP + (threadIdx.x % VECS) * 8 + j] = sum[j];
+    for (int w = 0; w < kC8Threads / 32; ++w) {
+        if (warp == w) {
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int t = 0; t < kC8Taps; ++t)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        float *r = red + (mt * 16 + (lane >> 2) + (j >> 1) * 8) * (kC8Taps * 8) + t * 8 +
+                                   (lane & 3) * 2 + (j & 1);
+                        *r = w ? *r + acc[mt][t][j] : acc[mt][t][j];
+                    }
+        }
+        __syncthreads();
+    }
+    float *part = a.part + (size_t)z * ((size_t)g.K * a.Ncols + g.K);
+    for (int i = threadIdx.x; i < g.K * a.Ncols; i += kC8Threads)
+        part[i] = red[(i / a.Ncols) * (kC8Taps * 8) + i % a.Ncols];
+    if ((int)threadIdx.x < g.K) {
+        float v = 0.f;
+        for (int l = 0; l < kC8Threads / VECS; ++l) v += bred[l * KP + threadIdx.x];
+        part[(size_t)g.K * a.Ncols + threadIdx.x] = v;
+    }
+}
+
+// Both take nine or ten taps (five k16 steps); the filter gradient up to 64
+// output channels.
+bool fits_c8(const Geo &g) {
+    const PatchC8 p = patch_c8(g, kC8Rows);
+    return g.C == 8 && g.R * g.S >= 9 && g.R * g.S <= kC8Taps && p.pitch * p.ph * 16 <= 96 * 1024;
+}
+int splits_c8(const Geo &g) {
+    const int64_t tiles = (int64_t)g.N * ((g.Q + kC8W - 1) / kC8W) * ((g.P + kC8GradRows - 1) / kC8GradRows);
+    return (int)(tiles < 304 ? tiles : 304);  // two CTAs on each of 152 SMs
+}
+
+cudaError_t launch_conv_c8(const Args &a, cudaStream_t st) {
+    const Geo &g = a.g;
+    const PatchC8 p = patch_c8(g, kC8Rows);
+    static const cudaError_t opt_in =
+        cudaFuncSetAttribute(k_conv_c8, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    if (opt_in != cudaSuccess) return opt_in;
+    const dim3 grid(g.N * ((g.Q + kC8W - 1) / kC8W) * ((g.P + kC8Rows - 1) / kC8Rows), (g.K + 31) / 32);
+    k_conv_c8<<<grid, kC8Threads, p.pitch * p.ph * 16, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int MT>
+cudaError_t launch_wgrad_c8(const Args &a, cudaStream_t st) {
+    const PatchC8 p = patch_c8(a.g, kC8GradRows);
+    const int red = (MT * 16 * kC8Taps * 8 + kC8Threads * 8) * 4;
+    int smem = 2 * (kC8W * kC8GradRows * MT * 32 + p.pitch * p.ph * 16);
+    if (smem < red) smem = red;
+    static const cudaError_t opt_in =
+        cudaFuncSetAttribute(k_wgrad_c8<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (opt_in != cudaSuccess) return opt_in;
+    const int splits = splits_c8(a.g);
+    k_wgrad_c8<MT><<<splits, kC8Threads, smem, st>>>(a, splits);
+    return cudaGetLastError();
+}
+
 // Sum of the filter-gradient partial tiles over the pixel splits, in split
 // order.
 // out[i] = sum over z of part[z][i] for i < count, in a fixed order: a CTA
@@ -505,6 +847,7 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
         const cudaError_t e = conv_forward_tma(a.g, x, w, bias, relu != 0, y, y_f32, st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
+    if (!y_f32 && fits_c8(a.g)) return status_of(launch_conv_c8(a, st));
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
     k_conv_gemm<kFwd><<<grid, NT, 0, st>>>(a);
     return status_of(cudaGetLastError());
@@ -567,7 +910,11 @@ size_t osog_conv2d_backward_filter_workspace(const osog_conv_shape_t *shape) {
     const size_t warp = ((size_t)splits_of(g) * g.K * g.R * g.S * g.C +
                          (size_t)bias_chunks(g) * g.K) * sizeof(float);
     const size_t tma = conv_wgrad_tma_workspace(g);
-    return warp > tma ? warp : tma;  // whichever engine the call runs on
+    const size_t c8 = fits_c8(g) && g.K <= 64
+                          ? (size_t)splits_c8(g) * ((size_t)g.K * g.R * g.S * g.C + g.K) * sizeof(float)
+                          : 0;
+    const size_t most = warp > tma ? warp : tma;
+    return most > c8 ? most : c8;  // whichever kernel the call runs on
 }
 
 int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *dy,
@@ -577,10 +924,6 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     if (!ws || ws_bytes < osog_conv2d_backward_filter_workspace(shape)) return OSOG_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const Geo g = geo_of(shape);
-    if (g_use_tcgen05) {
-        const cudaError_t e = conv_wgrad_tma(g, dy, x, dw, dbias, static_cast<float *>(ws), st);
-        if (e != cudaErrorNotSupported) return status_of(e);
-    }
     Args a{};
     a.g = g;
     a.x = bf(dy);
@@ -589,6 +932,17 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     a.M = g.K;
     a.Ncols = g.R * g.S * g.C;
     a.Kred = g.N * g.P * g.Q;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(ws) | reinterpret_cast<uintptr_t>(dw) |
+                           reinterpret_cast<uintptr_t>(dbias)) & 15) == 0;  // of k_sum_parts
+    if (aligned && fits_c8(g) && g.K <= 64) {
+        cudaError_t e = g.K <= 32 ? launch_wgrad_c8<2>(a, st) : launch_wgrad_c8<4>(a, st);
+        if (e == cudaSuccess) e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, st);
+        return status_of(e);
+    }
+    if (g_use_tcgen05 && aligned) {
+        const cudaError_t e = conv_wgrad_tma(g, dy, x, dw, dbias, static_cast<float *>(ws), st);
+        if (e != cudaErrorNotSupported) return status_of(e);
+    }
     const int splits = splits_of(g);
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN, splits);
     k_conv_gemm<kWgrad><<<grid, NT, 0, st>>>(a);

@@ -1117,9 +1117,6 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
                            float *dbias, float *ws, cudaStream_t st) {
     WgradArgs a{};
     int ch;
-    if ((reinterpret_cast<uintptr_t>(ws) | reinterpret_cast<uintptr_t>(dw) |
-         reinterpret_cast<uintptr_t>(dbias)) & 15)
-        return cudaErrorNotSupported;  // moved as 16-byte vectors
     if (!wgrad_plan(g, a, ch)) return cudaErrorNotSupported;
     a.part = ws;
     CUtensorMap mdy, mx;
@@ -1134,9 +1131,14 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
     if (e != cudaSuccess) return e;
     e = ch == 64 ? launch_wgrad<64>(mdy, mx, a, st) : launch_wgrad<32>(mdy, mx, a, st);
     if (e != cudaSuccess) return e;
-    const int64_t count4 = (int64_t)a.K * a.RS * a.C / 4, extra4 = a.K / 4;
+    return conv_sum_parts(g, a.splits, ws, dw, dbias, st);
+}
+
+cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
+                           cudaStream_t st) {
+    const int64_t count4 = (int64_t)g.K * g.R * g.S * g.C / 4, extra4 = g.K / 4;
     k_sum_parts<<<(unsigned)((count4 + extra4 + 31) / 32), 32 * kSumLanes, 0, st>>>(
-        reinterpret_cast<const float4 *>(ws), a.splits, count4, extra4, reinterpret_cast<float4 *>(dw),
+        reinterpret_cast<const float4 *>(part), splits, count4, extra4, reinterpret_cast<float4 *>(dw),
         reinterpret_cast<float4 *>(dbias));
     return cudaGetLastError();
 }

@@ -14,17 +14,22 @@ struct Geo {
 
 // Forward (y = act(conv(x, w) + bias)) and data gradient (dx, times x_act > 0
 // when mask is given) on tcgen05; cudaErrorNotSupported when a size is outside
-// the kernel's range (see conv_patch_plan).
+// the kernel's range (see conv_patch_plan; 16-byte aligned operands).
 cudaError_t conv_forward_tma(const Geo &g, const uint16_t *x, const uint16_t *w, const float *bias,
                              bool relu, uint16_t *y, float *y32, cudaStream_t st);
 cudaError_t conv_dgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *w,
                            const uint16_t *mask, uint16_t *dx, cudaStream_t st);
 
-// Filter and bias gradients (ws: conv_wgrad_tma_workspace bytes, 16-byte
-// aligned like dw and dbias); cudaErrorNotSupported as above (workspace 0).
+// Filter and bias gradients (ws: conv_wgrad_tma_workspace bytes; ws, dw and
+// dbias 16-byte aligned); cudaErrorNotSupported as above (workspace 0).
 size_t conv_wgrad_tma_workspace(const Geo &g);
 cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, float *dw,
                            float *dbias, float *ws, cudaStream_t st);
+
+// dw, dbias = the sums over the splits of part [splits][K R S C + K], in order
+// (all 16-byte aligned).
+cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
+                           cudaStream_t st);
 
 // Latched status of the bounded waits (read and cleared), and the
 // failure-detection hook (osog_conv_test_wait_limit).

@@ -25,22 +25,6 @@ SHAPES = [
 ]
 
 
-# the edges of the patch kernels' plans: several column blocks and channel
-# chunks, more chunks than shared memory holds, wide filters on both strides,
-# padding past the filter, classes and images smaller than a tile
-PATCH_SHAPES = [
-    (1, 20, 18, 264, 136, 3, 3, 1, 1),
-    (1, 9, 9, 1032, 16, 3, 3, 1, 1),
-    (2, 40, 36, 32, 48, 5, 5, 2, 2),
-    (1, 24, 25, 16, 8, 8, 8, 1, 3),
-    (1, 37, 21, 72, 24, 7, 7, 2, 3),
-    (1, 10, 11, 64, 16, 3, 3, 1, 4),
-    (1, 13, 12, 136, 40, 1, 1, 2, 1),
-    (5, 3, 2, 24, 200, 3, 2, 2, 1),
-    (2, 70, 34, 40, 16, 3, 3, 1, 0),
-]
-
-
 def _bf16(a, dev):
     """(bf16 device tensor, the same values as float64 numpy)."""
     t = torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).to(torch.bfloat16)
@@ -70,7 +54,7 @@ def cnn(request):
     m.use_tcgen05(True)
 
 
-@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
+@pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("relu", [False, True])
 def test_conv_forward_matches_reference(cnn, shape, relu):
     dev = torch.device("cuda")
@@ -89,7 +73,7 @@ def test_conv_forward_matches_reference(cnn, shape, relu):
     assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
 
 
-@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
+@pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("masked", [False, True])
 def test_conv_backward_data_matches_reference(cnn, shape, masked):
     dev = torch.device("cuda")
@@ -108,7 +92,7 @@ def test_conv_backward_data_matches_reference(cnn, shape, masked):
     assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
 
 
-@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
+@pytest.mark.parametrize("shape", SHAPES)
 def test_conv_backward_filter_matches_reference(cnn, shape):
     dev = torch.device("cuda")
     x, w, b, dy = _inputs(shape, 3)
@@ -198,3 +182,42 @@ def test_network_gradients_match_reference(cnn):
         assert np.linalg.norm(gw - ww) <= 3e-2 * np.linalg.norm(ww), i
         gb = db.cpu().numpy().astype(np.float64)
         assert np.linalg.norm(gb - wb) <= 3e-2 * np.linalg.norm(wb) + 1e-6, i
+
+
+# the edges of the patch kernels' plans: several column blocks and channel
+# chunks, more chunks than shared memory holds, wide filters on both strides,
+# padding past the filter, classes and images smaller than a tile
+PATCH_SHAPES = [
+    (1, 20, 18, 264, 136, 3, 3, 1, 1),
+    (1, 9, 9, 1032, 16, 3, 3, 1, 1),
+    (2, 40, 36, 32, 48, 5, 5, 2, 2),
+    (1, 24, 25, 16, 8, 8, 8, 1, 3),
+    (1, 37, 21, 72, 24, 7, 7, 2, 3),
+    (1, 10, 11, 64, 16, 3, 3, 1, 4),
+    (1, 13, 12, 136, 40, 1, 1, 2, 1),
+    (5, 3, 2, 24, 200, 3, 2, 2, 1),
+    (2, 70, 34, 40, 16, 3, 3, 1, 0),
+    # eight channels, nine or ten taps
+    (2, 35, 70, 8, 40, 3, 3, 1, 1),
+    (3, 67, 41, 8, 64, 3, 3, 2, 1),
+    (1, 20, 33, 8, 8, 2, 5, 2, 2),
+    (1, 9, 100, 8, 24, 5, 2, 1, 0),
+]
+
+
+@pytest.mark.parametrize("shape", PATCH_SHAPES)
+def test_patch_kernels_match_reference(cnn, shape):
+    test_conv_forward_matches_reference(cnn, shape, True)
+    test_conv_backward_data_matches_reference(cnn, shape, True)
+    test_conv_backward_filter_matches_reference(cnn, shape)
+
+
+@pytest.mark.parametrize("shape", SHAPES + PATCH_SHAPES)
+def test_forward_without_the_fp32_copy_gives_the_same_bits(cnn, shape):
+    dev = torch.device("cuda")
+    x, w, b, _ = _inputs(shape, 1)
+    xd, _ = _bf16(x, dev)
+    wd, _ = _bf16(w, dev)
+    bd = torch.from_numpy(b).to(dev)
+    y, _ = cnn.conv2d(xd, wd, bd, shape[7], shape[8], True, want_f32=True)
+    assert torch.equal(cnn.conv2d(xd, wd, bd, shape[7], shape[8], True), y)
