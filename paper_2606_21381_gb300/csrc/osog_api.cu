@@ -81,7 +81,7 @@ constexpr size_t kMaxKept = 64;  // forward states remembered per plan
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct Layout {
-    size_t rec, rrec, rect, cnt, band_off, pairs, pair_rect, G, Q, colrange, ctr, total;
+    size_t rec, rrec, rect, cnt, band_off, pairs, pair_rect, G, Q, ctr, total;
 };
 
 // Workspace regions for a launch group of up to S scenes, n records,
@@ -108,8 +108,6 @@ Layout make_layout(const Geometry &geo, int64_t n, int64_t nchunks, int S, int K
     o = align256(o + (size_t)S * geo.H * geo.W * sizeof(float2));
     l.Q = o;
     o = align256(o + (size_t)S * K * geo.H * geo.W * sizeof(float2));
-    l.colrange = o;
-    o = align256(o + (size_t)S * sizeof(int2));
     l.ctr = o;
     o = align256(o + (size_t)(2 + 2 * S) * sizeof(int32_t));
     l.total = o;
@@ -128,7 +126,6 @@ Work carve(void *ws, const Layout &l, int32_t *status) {
     w.pair_rect = reinterpret_cast<Rect *>(b + l.pair_rect);
     w.G = reinterpret_cast<float2 *>(b + l.G);
     w.Q = reinterpret_cast<float2 *>(b + l.Q);
-    w.colrange = reinterpret_cast<int2 *>(b + l.colrange);
     w.slotmap = nullptr;
     w.slotmap_ppp = 0;
     w.status = status;
@@ -270,6 +267,7 @@ int enqueue_group(osog_plan *p, const float *soa, int64_t ld, const int32_t *cou
     const Layout l = make_layout(geo, n, chunks, S, stage == kFull || stage == kFromMap ? K : 0, pairs);
     if (l.total > ws_bytes) return fail(OSOG_ERR_WORKSPACE, "workspace too small");
     Work w = carve(ws, l, p->status);
+    for (int s = 0; s < S; ++s) w.hull[s] = column_hull(gd.md[s], K, geo.W);
     if (opt.planes) {  // the planes' pixel-affine bounds follow the regions above
         const size_t coef = align256(l.total);
         if (coef + (size_t)opt.n_planes * sizeof(float4) > ws_bytes)
@@ -290,10 +288,9 @@ int enqueue_group(osog_plan *p, const float *soa, int64_t ld, const int32_t *cou
             rc = run_kernel(p, OSOG_KERNEL_BIN_COUNT, st,
                             [&] { return launch_bin_count(soa, ld, gd, geo, w, st); });
             if (rc) return rc;
+            rc = run_kernel(p, OSOG_KERNEL_BIN_SCAN, st, [&] { return launch_bin_scan(gd, geo, w, st); });
+            if (rc) return rc;
         }
-        // The scan also bounds the columns that any pupil passes.
-        rc = run_kernel(p, OSOG_KERNEL_BIN_SCAN, st, [&] { return launch_bin_scan(gd, geo, w, st); });
-        if (rc) return rc;
         if (stage == kBinOnly) {  // autotuner dry run: the per-band pair totals only
             opt.band_off_out->resize((size_t)S * (geo.nbands + 1));
             cudaError_t e = cudaMemcpyAsync(opt.band_off_out->data(), w.band_off,
@@ -432,6 +429,7 @@ int bwd_setup(osog_plan *p, const float *soa, int64_t ld, int32_t n, const osog_
     for (int bit = 0, k = 0; bit < 3; ++bit)
         if (optics->modes & (1u << bit)) b.gd.md[0][k++] = mode_dev(*optics, 1u << bit, p->optics_dyn);
     b.w = carve(ws, b.bl.fwd, p->status);
+    b.w.hull[0] = column_hull(b.gd.md[0], b.K, p->geo.W);
     b.w.slotmap = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + b.bl.slotmap);
     b.w.slotmap_ppp = ppp;
     b.part = reinterpret_cast<float *>(static_cast<char *>(ws) + b.bl.part);
@@ -746,12 +744,12 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     ia.S = 1;
     ia.K = 1;
     // Each step bounds its modality's columns (all of them for every op but
-    // the pupil) before the render kernels run.
+    // the pupil).
     auto use_mode = [&](const ModeDev &md) {
         gd.md[0][0] = md;
         ca.md[0][0] = md;
         sa.sc[0] = gd.sc[0];
-        return run_kernel(p, OSOG_KERNEL_BIN_SCAN, st, [&] { return launch_bin_scan(gd, geo, w, st); });
+        sa.w.hull[0] = ca.w.hull[0] = ia.w.hull[0] = column_hull(&md, 1, geo.W);
     };
     auto column = [&] { return run_kernel(p, OSOG_KERNEL_COLUMN, st, [&] { return launch_column(ca, st); }); };
     auto inverse = [&] {
@@ -768,7 +766,8 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     ca.unit_input = 1;
     ia.images = J;
     ia.real_out = 0;
-    if ((rc = use_mode(bf)) || (rc = column()) || (rc = inverse())) return rc;
+    use_mode(bf);
+    if ((rc = column()) || (rc = inverse())) return rc;
     // 2. OTF = DFT2(|h|^2), kept as a table (its DC term is sum |h|^2).
     ModeDev sp{};
     sp.op = kOpSpectrum;
@@ -776,7 +775,8 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     sp.scale = 1.f;
     ca.unit_input = 0;
     sa.opd_att = reinterpret_cast<const float2 *>(J);
-    if ((rc = use_mode(sp)) || (rc = strip(kStripFromReal)) || (rc = column())) return rc;
+    use_mode(sp);
+    if ((rc = strip(kStripFromReal)) || (rc = column())) return rc;
     // 3. J = |D|^2, D = IDFT2(DFT2(U) 2i sin(k . ds + theta)) / (H W): the
     //    exit wave sheared and interfered on every frequency (Eq. 5).
     ModeDev dic = mode_dev(*optics, OSOG_MODE_DIC, p->optics_dyn);
@@ -790,7 +790,9 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     if ((rc = run_kernel(p, OSOG_KERNEL_BIN_COUNT, st,
                          [&] { return launch_bin_count(soa, ld, gd, geo, w, st); })))
         return rc;
-    if ((rc = use_mode(dic))) return rc;
+    use_mode(dic);
+    if ((rc = run_kernel(p, OSOG_KERNEL_BIN_SCAN, st, [&] { return launch_bin_scan(gd, geo, w, st); })))
+        return rc;
     if ((rc = run_kernel(p, OSOG_KERNEL_BIN_FILL, st, [&] { return launch_bin_fill(gd, geo, w, st); })))
         return rc;
     if ((rc = strip(kStripRender)) || (rc = column()) || (rc = inverse())) return rc;
@@ -805,8 +807,8 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     gd.sc[0].pair_cap = 0;
     ia.images = image;
     ia.real_out = 1;
-    if ((rc = use_mode(tb)) || (rc = strip(kStripFromReal)) || (rc = column()) || (rc = inverse()))
-        return rc;
+    use_mode(tb);
+    if ((rc = strip(kStripFromReal)) || (rc = column()) || (rc = inverse())) return rc;
     return OSOG_OK;
 }
 
@@ -1119,8 +1121,8 @@ size_t osog_loss_table_size(const osog_plan_t *p, int32_t K) {
     return loss_table_spectra(p, K) + align256((size_t)K * sizeof(float));
 }
 
-// Workspace of the loss passes: G and Q of K single-modality images, the
-// column ranges, then the per-block partial sums.
+// Workspace of the loss passes: G and Q of K single-modality images, then
+// the per-block partial sums.
 static size_t loss_ws_part(const osog_plan *p, int K) {
     return make_layout(p->geo, 0, 0, K, 1, 0).total;
 }
@@ -1131,16 +1133,13 @@ size_t osog_loss_workspace_size(const osog_plan_t *p, int32_t K) {
 }
 
 // The spectra of K real images through the strip and column passes, with
-// modality md (kOpSpectrum or kOpLoss) per image; the column ranges are
-// set by the scan kernel (every column for these operations).
+// modality md (kOpSpectrum or kOpLoss) per image (every column).
 static int loss_passes(osog_plan *p, const float *images, int K, ModeDev md, float2 *tab,
                        const LossDev *loss, float *grad, void *ws, cudaStream_t st) {
     const Geometry &geo = p->geo;
     const Layout l = make_layout(geo, 0, 0, K, 1, 0);
-    const Work w = carve(ws, l, p->status);
-    GroupDev gd{};
-    gd.S = K;
-    gd.K = 1;
+    Work w = carve(ws, l, p->status);
+    for (int s = 0; s < K; ++s) w.hull[s] = column_hull(&md, 1, geo.W);
     StripArgs sa{};
     sa.geo = geo;
     sa.w = w;
@@ -1156,12 +1155,9 @@ static int loss_passes(osog_plan *p, const float *images, int K, ModeDev md, flo
     if (loss) ca.loss = *loss;
     for (int s = 0; s < K; ++s) {
         md.tab = tab + (size_t)s * geo.H * geo.W;
-        gd.md[s][0] = md;
         ca.md[s][0] = md;
     }
-    int rc = run_kernel(p, OSOG_KERNEL_BIN_SCAN, st, [&] { return launch_bin_scan(gd, geo, w, st); });
-    if (rc) return rc;
-    rc = run_kernel(p, OSOG_KERNEL_STRIP_FORWARD, st,
+    int rc = run_kernel(p, OSOG_KERNEL_STRIP_FORWARD, st,
                     [&] { return launch_strip_forward(sa, kStripFromReal, st); });
     if (rc) return rc;
     rc = run_kernel(p, OSOG_KERNEL_COLUMN, st, [&] { return launch_column(ca, st); });

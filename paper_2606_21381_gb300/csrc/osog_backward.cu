@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_rows(const __grid_constant_
     const int y0 = blockIdx.x * geo.R;
     const int RN = geo.R * N;
     float2 *Qm = a.w.Q + (size_t)sm * geo.nblocks * geo.H * geo.B;
-    const int2 cr = a.w.colrange[sm / K];
+    const int2 cr = a.w.hull[sm / K];
     load_strip_blocked<N>(buf, Qm, geo, y0, cr);
     __syncthreads();
     fft_lines<N, L, true>(buf, a.tw);  // E_m rows
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
     const int B = geo.B, lb = ilog2(B), half = geo.W / 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float *opart = a.opart + ((size_t)s * geo.nblocks + bk) * 4;
-    const int2 cr = a.w.colrange[s];
+    const int2 cr = a.w.hull[s];
     if (!block_active(geo, bk, cr)) {  // no pupil passes these columns: no gradient
         if (threadIdx.x < 4) opart[threadIdx.x] = 0.f;
         return;
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_strip(const __grid_constant
     const int y0 = blockIdx.x * geo.R, ylast = y0 + geo.R - 1;
     const int RN = geo.R * N;
     const SceneDev &sc = a.sc[s];
-    const int2 cr = a.w.colrange[s];
+    const int2 cr = a.w.hull[s];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     load_strip_blocked<N>(bufG, a.w.G + (size_t)s * geo.H * N, geo, y0, cr);
     float4 *o4 = reinterpret_cast<float4 *>(bufO);

@@ -8,15 +8,13 @@
 // of BH rows:
 //
 //   count  (one CTA per chunk of 256 particles): per-particle setup (record,
-//          bounding rectangle, band range), then per band a warp ballot of
-//          the particles that overlap it; per-warp counts are summed into
-//          cnt[chunk][band].
+//          bounding rectangle, band range), then per warp and band a mask
+//          of the particles that overlap it; the masks' counts are summed
+//          into cnt[chunk][band].
 //   scan   (one CTA per scene): exclusive prefix of cnt over the scene's
 //          chunks for every band, then over bands, giving each band's list
 //          start in the scene's pair region.
-//          The same kernel bounds, per scene, the columns that any pupil
-//          passes (the column kernels compute the exact chords).
-//   fill   (one CTA per chunk): the ballots again; a particle's slot is the
+//   fill   (one CTA per chunk): the masks again; a particle's slot is the
 //          band start + chunk prefix + earlier warps of the chunk + the
 //          popcount of lower lanes.  Each band list is therefore in
 //          ascending particle order.
@@ -208,34 +206,20 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
     return q;
 }
 
-// Hull [lo, hi] of the signed column frequencies that any modality of scene
-// s may pass: for a pupil, the columns with (fx / (W dx) + ox)^2 <= r2,
-// widened by one column on each side (rounding); every column for the other
-// operations.  Columns outside the hull are never read or written; the
-// column kernels decide the rest from the exact chords.
-__device__ int2 column_hull(const GroupDev &gd, int s, const Geometry &geo) {
-    const double wlo = -(double)(geo.W / 2), whi = (double)(geo.W / 2 - 1);
-    int lo = INT32_MAX, hi = INT32_MIN;
-    for (int m = 0; m < gd.K; ++m) {
-        const ModeDev &md = gd.md[s][m];
-        double a = wlo, b = whi;
-        if (md.op == kOpPupil) {
-            const double r = sqrt(md.r2);
-            a = fmin(fmax(floor((-r - md.ox) / md.fx_scale) - 1.0, wlo), whi + 1.0);
-            b = fmax(fmin(ceil((r - md.ox) / md.fx_scale) + 1.0, whi), wlo - 1.0);
-        }
-        if (a <= b) {
-            lo = min(lo, (int)a);
-            hi = max(hi, (int)b);
-        }
-    }
-    return make_int2(lo, hi);
+// The lanes of this warp whose particle overlaps each band, as bits of
+// mask[band] (zeroed by the caller).  Every lane sets its own few bands (one to
+// three at ordinary sizes); the warp need not step through all the bands that
+// any of its particles meets, up to 64 ballots, in the count and again in the
+// fill.
+__device__ __forceinline__ void mark_bands(uint32_t *mask, int b0, int b1) {
+    const uint32_t bit = 1u << (threadIdx.x & 31);
+    for (int b = b0; b <= b1; ++b) atomicOr(mask + b, bit);
 }
 
 __global__ void __launch_bounds__(kChunk)
 k_bin_count(const float *__restrict__ soa, int64_t ld, const __grid_constant__ GroupDev gd,
-            Geometry geo, Work w) {
-    __shared__ int wcnt[kChunk / 32][kMaxBands];
+            Geometry geo, const __grid_constant__ Work w) {
+    __shared__ uint32_t mask[kChunk / 32][kMaxBands];
     pdl_enter();
     const int chunk = blockIdx.x;
     const int s = scene_of_chunk(gd, chunk);
@@ -243,8 +227,7 @@ k_bin_count(const float *__restrict__ soa, int64_t ld, const __grid_constant__ G
     const int local = (chunk - sc.chunk0) * kChunk + threadIdx.x;
     const bool mine = local < sc.n;
     const int p = sc.p0 + local;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&wcnt[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&mask[0][0])[i] = 0u;
     int b0 = 1, b1 = 0;
     if (mine) {
         Rect r = setup_particle(soa, ld, p, sc, geo, w);
@@ -252,18 +235,12 @@ k_bin_count(const float *__restrict__ soa, int64_t ld, const __grid_constant__ G
         band_range(r, geo.BH, b0, b1);
     }
     __syncthreads();
-    const bool any = b0 <= b1;
-    const int lo = __reduce_min_sync(0xffffffffu, any ? b0 : kMaxBands);
-    const int hi = __reduce_max_sync(0xffffffffu, any ? b1 : -1);
-    for (int b = lo; b <= hi; ++b) {
-        const unsigned m = __ballot_sync(0xffffffffu, any && b0 <= b && b <= b1);
-        if (lane == 0) wcnt[warp][b] = __popc(m);
-    }
+    mark_bands(mask[threadIdx.x >> 5], b0, b1);
     __syncthreads();
     for (int b = threadIdx.x; b < geo.nbands; b += kChunk) {
         int t = 0;
 #pragma unroll
-        for (int k = 0; k < kChunk / 32; ++k) t += wcnt[k][b];
+        for (int k = 0; k < kChunk / 32; ++k) t += __popc(mask[k][b]);
         w.cnt[(int64_t)chunk * geo.nbands + b] = t;
     }
 }
@@ -279,7 +256,7 @@ k_bin_count(const float *__restrict__ soa, int64_t ld, const __grid_constant__ G
 constexpr int kScanTile = 64;
 
 __global__ void __launch_bounds__(1024)
-k_bin_scan(const __grid_constant__ GroupDev gd, Geometry geo, Work w) {
+k_bin_scan(const __grid_constant__ GroupDev gd, Geometry geo, const __grid_constant__ Work w) {
     __shared__ int tile[kScanTile][kMaxBands + 1];  // one pad word: conflict-free columns
     __shared__ int run[kMaxBands];
     pdl_enter();
@@ -288,8 +265,6 @@ k_bin_scan(const __grid_constant__ GroupDev gd, Geometry geo, Work w) {
     const int nch = (s + 1 < gd.S ? gd.sc[s + 1].chunk0 : gd.nchunks) - sc.chunk0;
     const int nb = geo.nbands;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 992)  // lane 0 of the last warp
-        w.colrange[s] = column_hull(gd, s, geo);
     if ((int)threadIdx.x < nb) run[threadIdx.x] = 0;
     int32_t *cnt = w.cnt + (int64_t)sc.chunk0 * nb;  // [nch][nb]
     for (int t0 = 0; t0 < nch; t0 += kScanTile) {
@@ -344,9 +319,27 @@ k_bin_scan(const __grid_constant__ GroupDev gd, Geometry geo, Work w) {
     }
 }
 
+// The list slots of particle p (band range [b0, b1], rectangle pr with its
+// kind): the band's start, then the earlier warps, then the lower lanes.
+__device__ __forceinline__ void fill_slots(const Work &w, const SceneDev &sc, int p, Rect pr, int b0,
+                                           int b1, const int *start, const int *before,
+                                           const uint32_t *mask) {
+    const unsigned lt = lanemask_lt();
+    for (int b = b0; b <= b1; ++b) {
+        const int slot = start[b] + before[b] + __popc(mask[b] & lt);
+        if (slot < sc.pair_cap) {
+            w.pairs[sc.pair0 + slot] = p;
+            if (w.pair_rect) w.pair_rect[sc.pair0 + slot] = pr;
+        }
+        if (w.slotmap && b - b0 < w.slotmap_ppp)
+            w.slotmap[(size_t)p * w.slotmap_ppp + (b - b0)] = slot < sc.pair_cap ? slot : -1;
+    }
+}
+
 __global__ void __launch_bounds__(kChunk)
-k_bin_fill(const __grid_constant__ GroupDev gd, Geometry geo, Work w) {
-    __shared__ int wpre[kChunk / 32][kMaxBands];
+k_bin_fill(const __grid_constant__ GroupDev gd, Geometry geo, const __grid_constant__ Work w) {
+    __shared__ uint32_t mask[kChunk / 32][kMaxBands];
+    __shared__ int before[kChunk / 32][kMaxBands];  // entries of the chunk's earlier warps
     __shared__ int start[kMaxBands];  // band list start + this chunk's prefix
     pdl_enter();
     const int chunk = blockIdx.x;
@@ -355,61 +348,42 @@ k_bin_fill(const __grid_constant__ GroupDev gd, Geometry geo, Work w) {
     const int local = (chunk - sc.chunk0) * kChunk + threadIdx.x;
     const bool mine = local < sc.n;
     const int p = sc.p0 + local;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     const int32_t *off = w.band_off + (int64_t)s * (geo.nbands + 1);
     const int32_t *pre = w.cnt + (int64_t)chunk * geo.nbands;
-    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&wpre[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&mask[0][0])[i] = 0u;
     for (int b = threadIdx.x; b < geo.nbands; b += kChunk) start[b] = off[b] + pre[b];
     int b0 = 1, b1 = 0;
     Rect pr{};
     if (mine) {
         pr = w.rect[p];
+        const int kind = w.rrec[p].kind;  // (loaded beside the rectangle; unused when that is empty)
         band_range(pr, geo.BH, b0, b1);
-        if (b0 <= b1) pr.x1 = (int16_t)(pr.x1 | (w.rrec[p].kind << 12));
+        if (b0 <= b1) pr.x1 = (int16_t)(pr.x1 | (kind << 12));
     }
     __syncthreads();
-    const bool any = b0 <= b1;
-    const int lo = __reduce_min_sync(0xffffffffu, any ? b0 : kMaxBands);
-    const int hi = __reduce_max_sync(0xffffffffu, any ? b1 : -1);
-    for (int b = lo; b <= hi; ++b) {
-        const unsigned m = __ballot_sync(0xffffffffu, any && b0 <= b && b <= b1);
-        if (lane == 0) wpre[warp][b] = __popc(m);
-    }
+    mark_bands(mask[warp], b0, b1);
     __syncthreads();
     for (int b = threadIdx.x; b < geo.nbands; b += kChunk) {  // exclusive over warps
         int acc = 0;
 #pragma unroll
         for (int k = 0; k < kChunk / 32; ++k) {
-            const int t = wpre[k][b];
-            wpre[k][b] = acc;
-            acc += t;
+            before[k][b] = acc;
+            acc += __popc(mask[k][b]);
         }
     }
     __syncthreads();
-    const unsigned lt = lanemask_lt();
-    for (int b = lo; b <= hi; ++b) {
-        const bool in = any && b0 <= b && b <= b1;
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) {
-            const int slot = start[b] + wpre[warp][b] + __popc(m & lt);
-            if (slot < sc.pair_cap) {
-                w.pairs[sc.pair0 + slot] = p;
-                if (w.pair_rect) w.pair_rect[sc.pair0 + slot] = pr;
-            }
-            if (w.slotmap && b - b0 < w.slotmap_ppp)
-                w.slotmap[(size_t)p * w.slotmap_ppp + (b - b0)] = slot < sc.pair_cap ? slot : -1;
-        }
-    }
+    fill_slots(w, sc, p, pr, b0, b1, start, before[warp], mask[warp]);
 }
 
 // One scene of at most kChunk particles: count, scan and fill in one CTA.
 // The slots are those of the three kernels (band start, then the earlier
-// warps, then the lower lanes: ascending particle order in every band list),
-// and the scene's column hull is bounded as in the scan.
+// warps, then the lower lanes: ascending particle order in every band list).
 __global__ void __launch_bounds__(kChunk)
 k_bin_single(const float *__restrict__ soa, int64_t ld, const __grid_constant__ GroupDev gd,
-             Geometry geo, Work w) {
-    __shared__ int wpre[kChunk / 32][kMaxBands];
+             Geometry geo, const __grid_constant__ Work w) {
+    __shared__ uint32_t mask[kChunk / 32][kMaxBands];
+    __shared__ int before[kChunk / 32][kMaxBands];
     __shared__ int start[kMaxBands];
     pdl_enter();
     const SceneDev &sc = gd.sc[0];
@@ -417,7 +391,7 @@ k_bin_single(const float *__restrict__ soa, int64_t ld, const __grid_constant__ 
     const bool mine = local < sc.n;
     const int p = sc.p0 + local;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&wpre[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < (kChunk / 32) * kMaxBands; i += kChunk) (&mask[0][0])[i] = 0u;
     int b0 = 1, b1 = 0;
     Rect pr{};
     if (mine) {
@@ -428,22 +402,15 @@ k_bin_single(const float *__restrict__ soa, int64_t ld, const __grid_constant__ 
         if (b0 <= b1) pr.x1 = (int16_t)(pr.x1 | (w.rrec[p].kind << 12));
     }
     __syncthreads();
-    const bool any = b0 <= b1;
-    const int lo = __reduce_min_sync(0xffffffffu, any ? b0 : kMaxBands);
-    const int hi = __reduce_max_sync(0xffffffffu, any ? b1 : -1);
-    for (int b = lo; b <= hi; ++b) {
-        const unsigned m = __ballot_sync(0xffffffffu, any && b0 <= b && b <= b1);
-        if (lane == 0) wpre[warp][b] = __popc(m);
-    }
+    mark_bands(mask[warp], b0, b1);
     __syncthreads();
-    int total = 0;
-    if (threadIdx.x < geo.nbands) {  // exclusive over the warps, in place
+    if (threadIdx.x < geo.nbands) {  // exclusive over the warps
         const int b = threadIdx.x;
+        int total = 0;
 #pragma unroll
         for (int k = 0; k < kChunk / 32; ++k) {
-            const int t = wpre[k][b];
-            wpre[k][b] = total;
-            total += t;
+            before[k][b] = total;
+            total += __popc(mask[k][b]);
         }
         start[b] = total;
     }
@@ -471,24 +438,10 @@ k_bin_single(const float *__restrict__ soa, int64_t ld, const __grid_constant__ 
         if (lane == 0) {
             off[geo.nbands] = all;
             if (all > sc.pair_cap) latch(w.status, OSOG_ERR_BIN_OVERFLOW);
-            w.colrange[0] = column_hull(gd, 0, geo);
         }
     }
     __syncthreads();
-    const unsigned lt = lanemask_lt();
-    for (int b = lo; b <= hi; ++b) {
-        const bool in = any && b0 <= b && b <= b1;
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) {
-            const int slot = start[b] + wpre[warp][b] + __popc(m & lt);
-            if (slot < sc.pair_cap) {
-                w.pairs[sc.pair0 + slot] = p;
-                if (w.pair_rect) w.pair_rect[sc.pair0 + slot] = pr;
-            }
-            if (w.slotmap && b - b0 < w.slotmap_ppp)
-                w.slotmap[(size_t)p * w.slotmap_ppp + (b - b0)] = slot < sc.pair_cap ? slot : -1;
-        }
-    }
+    fill_slots(w, sc, p, pr, b0, b1, start, before[warp], mask[warp]);
 }
 
 }  // namespace

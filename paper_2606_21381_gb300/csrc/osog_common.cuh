@@ -6,6 +6,7 @@
 
 #include "osog.h"
 #include "osog_ff.h"
+#include "osog_pupil.h"
 
 namespace osog {
 
@@ -137,6 +138,7 @@ struct ModeDev {
     float half_dx;        // dx / 2 (um): dsx, dsy of the bound shear
     int32_t fixed_dz;     // 1: dz stays as set here whatever is bound (an operation
                           // that applies no defocus)
+    PupilFF circle;       // r2 .. fy_span as float-float (see pupil_chord)
 };
 
 // The modality with the plan's bound optics scalars applied (see
@@ -211,8 +213,6 @@ struct Work {
                         // 12-13 of x1 (null: readers gather rect[] and rrec[])
     float2 *G;          // [S][W/B][H][B] row spectra
     float2 *Q;          // [S][K][W/B][H][B] filtered columns
-    int2 *colrange;     // [S] signed column frequencies [lo, hi] outside which no
-                        // pupil passes anything (a hull, possibly wider)
     int32_t *slotmap;   // [n][pairs per particle] band-list slot of each (particle,
                         // band); written by the fill pass when not null (adjoint)
     int32_t slotmap_ppp;
@@ -224,21 +224,25 @@ struct Work {
     const int32_t *plane_off = nullptr;
     int32_t n_planes = 0;
     float4 *plane_coef = nullptr;
+    // Per scene: signed column frequencies [lo, hi] outside which no pupil passes
+    // anything (a hull, possibly wider; column_hull()).  Bounded on the host and
+    // passed by value: on the device its square root and divisions in FP64 took
+    // one thread 3.8 us of the binning, and every pass waited for a load of it.
+    int2 hull[kMaxScenes];
 };
 
 // ---------------------------------------------------------------- pupil
 // Interval [lo, hi] of signed row frequencies fy inside the (shifted) pupil
-// circle for column frequency fx, decided in double precision:
-// (fx / (W dx) + ox)^2 + (fy / (H dx) + oy)^2 <= (NA / lambda)^2.
-// An empty column returns lo > hi.
+// circle for column frequency fx, decided as in double precision
+// (osog_pupil.h): (fx / (W dx) + ox)^2 + (fy / (H dx) + oy)^2 <= (NA /
+// lambda)^2.  An empty column returns lo > hi.
+__device__ __noinline__ inline RowRange pupil_chord_slow(const ModeDev &md, int fx) {
+    return pupil_chord_exact(md.r2, md.ox, md.oy, md.fx_scale, md.fy_span, fx);
+}
 __device__ __forceinline__ int2 pupil_chord(const ModeDev &md, int fx) {
-    const double ax = (double)fx * md.fx_scale + md.ox;
-    const double rem = md.r2 - ax * ax;
-    if (rem < 0.0) return make_int2(1, 0);
-    const double root = sqrt(rem);
-    const double lo = (-root - md.oy) * md.fy_span;
-    const double hi = (root - md.oy) * md.fy_span;
-    return make_int2((int)ceil(lo), (int)floor(hi));
+    RowRange r;
+    if (!pupil_chord_ff(md.circle, fx, &r)) r = pupil_chord_slow(md, fx);
+    return make_int2(r.lo, r.hi);
 }
 
 // Rows [lo, hi] of column fx (signed) that a modality's column operation

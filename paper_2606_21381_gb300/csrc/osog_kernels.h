@@ -2,6 +2,7 @@
 #pragma once
 
 #include <math.h>
+#include <stdint.h>
 
 #include "osog_common.cuh"
 
@@ -152,7 +153,35 @@ inline ModeDev mode_dev(const osog_optics_t &o, uint32_t mode, const float *dyn)
     m.dsy1 = (float)(0.5 * o.dx_um * sin(o.shear_angle));
     m.dyn = dyn;
     m.half_dx = (float)(0.5 * o.dx_um);
+    auto split = [](double v) {
+        const float h = (float)v;
+        return ff{h, (float)(v - (double)h)};
+    };
+    m.circle = {split(m.fx_scale), split(m.ox), split(m.oy), split(m.r2), split(m.fy_span)};
     return m;
+}
+
+// Hull [lo, hi] of the signed column frequencies that any of K modalities may
+// pass: for a pupil, the columns with (fx / (W dx) + ox)^2 <= r2, widened by
+// one column on each side (rounding); every column for the other operations.
+// Columns outside the hull are never read or written; the column kernels
+// decide the rest from the exact chords.
+inline int2 column_hull(const ModeDev *md, int K, int W) {
+    const double wlo = -(double)(W / 2), whi = (double)(W / 2 - 1);
+    int lo = INT32_MAX, hi = INT32_MIN;
+    for (int m = 0; m < K; ++m) {
+        double a = wlo, b = whi;
+        if (md[m].op == kOpPupil) {
+            const double r = sqrt(md[m].r2);
+            a = fmin(fmax(floor((-r - md[m].ox) / md[m].fx_scale) - 1.0, wlo), whi + 1.0);
+            b = fmax(fmin(ceil((r - md[m].ox) / md[m].fx_scale) + 1.0, whi), wlo - 1.0);
+        }
+        if (a <= b) {
+            lo = lo < (int)a ? lo : (int)a;
+            hi = hi > (int)b ? hi : (int)b;
+        }
+    }
+    return make_int2(lo, hi);
 }
 
 cudaError_t launch_bin_count(const float *soa, int64_t ld, const GroupDev &gd,

@@ -113,8 +113,6 @@ extern "C" int osog_render_noalloc(const float *soa, int64_t ld, int32_t n,
     off = up256(off + (size_t)geo.H * geo.W * sizeof(float2));
     const size_t o_Q = off;
     off = up256(off + (size_t)K * geo.H * geo.W * sizeof(float2));
-    const size_t o_colrange = off;
-    off = up256(off + sizeof(int2));
     const size_t o_pairs = off;
     if (off > kScratchBytes || (n > 0 && kScratchBytes - off < (size_t)n * sizeof(int32_t)))
         return OSOG_ERR_WORKSPACE;  // beyond the 8 MiB static scratch
@@ -137,7 +135,6 @@ extern "C" int osog_render_noalloc(const float *soa, int64_t ld, int32_t n,
     w.pairs = reinterpret_cast<int32_t *>(st->scratch + o_pairs);
     w.G = reinterpret_cast<float2 *>(st->scratch + o_G);
     w.Q = reinterpret_cast<float2 *>(st->scratch + o_Q);
-    w.colrange = reinterpret_cast<int2 *>(st->scratch + o_colrange);
     w.slotmap = nullptr;
     w.slotmap_ppp = 0;
     w.status = st->status;
@@ -156,6 +153,7 @@ extern "C" int osog_render_noalloc(const float *soa, int64_t ld, int32_t n,
     sc.pair_cap = (int32_t)pairs;
     for (int bit = 0, k = 0; bit < 3; ++bit)
         if (o->modes & (1u << bit)) gd.md[0][k++] = mode_dev(*o, 1u << bit, nullptr);
+    w.hull[0] = column_hull(gd.md[0], K, geo.W);
 
     // Every scratch region is written in full before it is read; the status
     // word keeps what earlier calls latched until osog_noalloc_sync_status.

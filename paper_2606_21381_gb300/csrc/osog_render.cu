@@ -102,7 +102,7 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
         const int lb = SQ ? clog2(sq_rb(N)) : ilog2(B);
         const int H = SQ ? N : geo.H;
         float2 *G = a.w.G + (size_t)s * H * N;
-        const int2 cr = a.w.colrange[s];
+        const int2 cr = a.w.hull[s];
         fft_last_pass<N, L, false, false, GRP>(buf, a.tw, [&](int l, int kx, float2 v) {
             const int fx = kx < N / 2 ? kx : kx - N;
             if (l < R && fx >= cr.x && fx <= cr.y)  // columns outside every pupil are never read
@@ -142,7 +142,7 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
         const int lb = SQ ? clog2(sq_rb(N)) : ilog2(B), lr = SQ ? clog2(sq_rb(N)) : ilog2(R);
         const int H = SQ ? N : geo.H;
         float2 *G = a.w.G + (size_t)s * H * N;
-        const int2 cr = a.w.colrange[s];
+        const int2 cr = a.w.hull[s];
 #pragma unroll
         for (int i = 0; i < ept(N); ++i) {
             const int e = threadIdx.x + i * kThreads;
@@ -349,7 +349,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
     const Geometry &geo = a.geo;
     const int B = SQ ? sq_rb(N) : geo.B, lb = SQ ? clog2(sq_rb(N)) : ilog2(B), K = a.K;
     const int W = SQ ? N : geo.W;
-    const int2 cr = a.w.colrange[s];
+    const int2 cr = a.w.hull[s];
     // A block whose columns all lie outside every pupil has nothing to filter:
     // its Q block is never read.  The block's unsigned columns [u0, u1] map to
     // signed frequencies [u0, min(u1, W/2 - 1)] and [max(u0, W/2), u1] - W.
@@ -489,7 +489,7 @@ __device__ __forceinline__ void inverse_item(const InverseArgs &a, int sm, int s
     const int H = SQ ? N : geo.H;
     const int y0 = strip * R;
     const float2 *Qm = a.w.Q + (size_t)sm * geo.nblocks * H * B;
-    const int2 cr = a.w.colrange[sm / K];
+    const int2 cr = a.w.hull[sm / K];
     // the first pass reads the strip's rows of Q straight from global memory
     // (columns that no pupil passes, and lines past the strip, read as zero);
     // the last pass writes the intensity rows
