@@ -14,7 +14,6 @@ operations on device tensors.
 """
 from __future__ import annotations
 
-import ctypes
 import math
 import time
 from dataclasses import dataclass
@@ -24,6 +23,7 @@ import torch
 
 from . import _lib, scenes
 from ._lib import check
+from ._stream import raw_stream
 
 CELL = 8                # pixels per output cell (three stride-2 layers)
 IN_CHANNELS = 8         # BF, DIC, zero padding to the kernels' multiple of 8
@@ -40,11 +40,11 @@ INPUT_SCALE = 2.0
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(dev) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+def _stream(dev) -> int:
+    return raw_stream(dev.index)
 
 
 def conv_shape(x: torch.Tensor, w: torch.Tensor, stride: int, pad: int) -> _lib.ConvShape:
@@ -56,15 +56,14 @@ def conv_shape(x: torch.Tensor, w: torch.Tensor, stride: int, pad: int) -> _lib.
 
 
 def _out_hw(s: _lib.ConvShape) -> tuple[int, int]:
-    L = _lib.lib()
-    P, Q = L.osog_conv_out_h(ctypes.byref(s)), L.osog_conv_out_w(ctypes.byref(s))
-    if P <= 0 or Q <= 0:
+    P = _lib.lib().osog_conv_out_h(s)  # 0 for a shape that the library refuses
+    if P <= 0:
         raise ValueError(f"invalid convolution shape {[getattr(s, f) for f, _ in s._fields_]}")
-    return P, Q
+    return P, (s.W + 2 * s.pad - s.S) // s.stride + 1
 
 
 def _require(t: torch.Tensor, dtype, name: str):
-    if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
+    if not (t.is_cuda and t.dtype == dtype and t.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous CUDA {dtype} tensor")
 
 
@@ -75,9 +74,9 @@ def conv2d(x, w, bias, stride: int, pad: int, relu: bool, want_f32: bool = False
     _require(bias, torch.float32, "bias")
     s = conv_shape(x, w, stride, pad)
     P, Q = _out_hw(s)
-    y = torch.empty((s.N, P, Q, s.K), dtype=torch.bfloat16, device=x.device)
+    y = x.new_empty((s.N, P, Q, s.K))
     y32 = torch.empty((s.N, P, Q, s.K), dtype=torch.float32, device=x.device) if want_f32 else None
-    check(_lib.lib().osog_conv2d_forward(ctypes.byref(s), _ptr(x), _ptr(w), _ptr(bias), int(relu),
+    check(_lib.lib().osog_conv2d_forward(s, _ptr(x), _ptr(w), _ptr(bias), int(relu),
                                          _ptr(y), _ptr(y32), _stream(x.device)), "osog_conv2d_forward")
     return (y, y32) if want_f32 else y
 
@@ -94,9 +93,9 @@ def conv2d_backward_data(dy, w, x_shape, stride: int, pad: int, x_act=None):
     P, Q = _out_hw(s)
     if tuple(dy.shape) != (N, P, Q, K):
         raise ValueError(f"dy has shape {tuple(dy.shape)}, expected {(N, P, Q, K)}")
-    dx = torch.empty((N, H, W, C), dtype=torch.bfloat16, device=dy.device)
+    dx = dy.new_empty((N, H, W, C))
     w_t = torch.empty_like(w)
-    check(_lib.lib().osog_conv2d_backward_data(ctypes.byref(s), _ptr(dy), _ptr(w), _ptr(x_act),
+    check(_lib.lib().osog_conv2d_backward_data(s, _ptr(dy), _ptr(w), _ptr(x_act),
                                                _ptr(dx), _ptr(w_t), _stream(dy.device)),
           "osog_conv2d_backward_data")
     return dx
@@ -113,12 +112,12 @@ def conv2d_backward_filter(dy, x, w_shape, stride: int, pad: int, ws=None):
     if tuple(dy.shape) != (N, P, Q, K):
         raise ValueError(f"dy has shape {tuple(dy.shape)}, expected {(N, P, Q, K)}")
     L = _lib.lib()
-    need = L.osog_conv2d_backward_filter_workspace(ctypes.byref(s))
+    need = L.osog_conv2d_backward_filter_workspace(s)
     if ws is None or ws.numel() < need:
         ws = torch.empty(max(need, 16), dtype=torch.uint8, device=dy.device)
     dw = torch.empty((K, R, S, C), dtype=torch.float32, device=dy.device)
     db = torch.empty((K,), dtype=torch.float32, device=dy.device)
-    check(L.osog_conv2d_backward_filter(ctypes.byref(s), _ptr(dy), _ptr(x), _ptr(dw), _ptr(db),
+    check(L.osog_conv2d_backward_filter(s, _ptr(dy), _ptr(x), _ptr(dw), _ptr(db),
                                         _ptr(ws), ws.numel(), _stream(dy.device)),
           "osog_conv2d_backward_filter")
     return dw, db
@@ -133,7 +132,7 @@ def use_tcgen05(enable: bool) -> None:
 def sync_status(device=None) -> int:
     """Synchronise and return (and clear) a latched convolution error."""
     dev = torch.device(device or "cuda")
-    return int(_lib.lib().osog_conv_sync_status(_stream(dev)))
+    return int(_lib.lib().osog_conv_sync_status(torch.cuda.current_stream(dev).cuda_stream))
 
 
 def relu_backward(dy, act):

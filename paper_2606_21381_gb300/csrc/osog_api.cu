@@ -243,9 +243,7 @@ int enqueue_group(osog_plan *p, const float *soa, int64_t ld, const int32_t *cou
         return fail(OSOG_ERR_INVALID_ARG, "band_rows must be a multiple of the strip height "
                                           "dividing H into at most 64 bands");
     const int pairs_per_particle = opt.ppp;
-    GroupDev gd{};
-    gd.S = S;
-    gd.K = K;
+    GroupDev gd = group_dev(S, K, 0);
     int64_t n = 0, chunks = 0, pairs = 0;
     for (int s = 0; s < S; ++s) {
         SceneDev sc = scene_dev(optics[s]);
@@ -312,12 +310,7 @@ int enqueue_group(osog_plan *p, const float *soa, int64_t ld, const int32_t *cou
     sa.opd_out = reinterpret_cast<float2 *>(opd_out);
     sa.S = S;
     for (int s = 0; s < S; ++s) sa.sc[s] = gd.sc[s];
-    ColumnArgs ca{};
-    ca.geo = geo;
-    ca.w = w;
-    ca.tw = p->tw_h;
-    ca.S = S;
-    ca.K = K;
+    ColumnArgs ca = column_args(geo, w, p->tw_h, S, K);
     for (int s = 0; s < S; ++s)
         for (int k = 0; k < K; ++k) ca.md[s][k] = gd.md[s][k];
     ca.wait_polls = opt.wait_polls;
@@ -415,10 +408,7 @@ int bwd_setup(osog_plan *p, const float *soa, int64_t ld, int32_t n, const osog_
     b.bl = make_bwd_layout(p->geo, n, b.chunks, b.K, ppp);
     rc = check_ws(ws, b.bl.total, ws_bytes);
     if (rc) return rc;
-    b.gd = GroupDev{};
-    b.gd.S = 1;
-    b.gd.K = b.K;
-    b.gd.nchunks = (int32_t)b.chunks;
+    b.gd = group_dev(1, b.K, (int)b.chunks);
     b.sc = scene_dev(*optics);
     b.sc.p0 = 0;
     b.sc.n = n;
@@ -472,12 +462,7 @@ int bwd_forward(osog_plan *p, const float *soa, int64_t ld, const BwdState &b, f
     sa.sc[0] = b.sc;
     rc = raster_and_strip(p, sa, st);
     if (rc) return rc;
-    ColumnArgs ca{};
-    ca.geo = geo;
-    ca.w = b.w;
-    ca.tw = p->tw_h;
-    ca.S = 1;
-    ca.K = b.K;
+    ColumnArgs ca = column_args(geo, b.w, p->tw_h, 1, b.K);
     for (int k = 0; k < b.K; ++k) ca.md[0][k] = b.gd.md[0][k];
     rc = run_kernel(p, OSOG_KERNEL_COLUMN, st, [&] { return launch_column(ca, st); });
     if (rc || !image) return rc;
@@ -507,13 +492,7 @@ int bwd_adjoint(osog_plan *p, const BwdState &b, const float *grad_image, float 
     ra.K = b.K;
     int rc = run_kernel(p, OSOG_KERNEL_BWD_ROWS, st, [&] { return launch_bwd_rows(ra, st); });
     if (rc) return rc;
-    BwdColumnArgs bc{};
-    bc.geo = geo;
-    bc.w = b.w;
-    bc.tw = p->tw_h;
-    bc.opart = b.opart;
-    bc.S = 1;
-    bc.K = b.K;
+    BwdColumnArgs bc = bwd_column_args(geo, b.w, p->tw_h, b.opart, 1, b.K);
     for (int k = 0; k < b.K; ++k) bc.md[0][k] = b.gd.md[0][k];
     rc = run_kernel(p, OSOG_KERNEL_BWD_COLUMN, st, [&] { return launch_bwd_column(bc, st); });
     if (rc) return rc;
@@ -722,21 +701,14 @@ int osog_render_dic_incoherent(osog_plan_t *p, const float *soa, int64_t ld, int
     float *J = reinterpret_cast<float *>(static_cast<char *>(ws) + dl.img);
     float2 *otf = reinterpret_cast<float2 *>(static_cast<char *>(ws) + dl.otf);
 
-    GroupDev gd{};
-    gd.S = 1;
-    gd.K = 1;
+    GroupDev gd = group_dev(1, 1, 0);
     gd.sc[0] = scene_dev(*optics);  // no particles until step 3
     StripArgs sa{};
     sa.geo = geo;
     sa.w = w;
     sa.tw = p->tw_w;
     sa.S = 1;
-    ColumnArgs ca{};
-    ca.geo = geo;
-    ca.w = w;
-    ca.tw = p->tw_h;
-    ca.S = 1;
-    ca.K = 1;
+    ColumnArgs ca = column_args(geo, w, p->tw_h, 1, 1);
     InverseArgs ia{};
     ia.geo = geo;
     ia.w = w;
@@ -1146,12 +1118,7 @@ static int loss_passes(osog_plan *p, const float *images, int K, ModeDev md, flo
     sa.tw = p->tw_w;
     sa.opd_att = reinterpret_cast<const float2 *>(images);
     sa.S = K;
-    ColumnArgs ca{};
-    ca.geo = geo;
-    ca.w = w;
-    ca.tw = p->tw_h;
-    ca.S = K;
-    ca.K = 1;
+    ColumnArgs ca = column_args(geo, w, p->tw_h, K, 1);
     if (loss) ca.loss = *loss;
     for (int s = 0; s < K; ++s) {
         md.tab = tab + (size_t)s * geo.H * geo.W;

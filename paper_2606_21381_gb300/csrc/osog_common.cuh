@@ -271,9 +271,15 @@ __device__ __forceinline__ void pdl_enter() {
 // latency-bound launches (one scene), while for grids of many waves (the
 // batched path) the early dispatch measured slower.
 constexpr long kPdlMaxCtas = 1024;
-template <typename... KArgs, typename... Args>
+// The arguments are handed over by address: the launch structs of a group of
+// scenes are up to 20 KB, and the runtime copies them once.
+template <typename T>
+struct KernelArg {
+    using type = T;
+};
+template <typename... KArgs>
 inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
-                                cudaStream_t st, Args &&...args) {
+                                cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -284,7 +290,8 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, 
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = (long)grid.x * grid.y * grid.z <= kPdlMaxCtas ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Args &&>(args)...);
+    void *ptrs[] = {const_cast<void *>(static_cast<const void *>(&args))...};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), ptrs);
     if (e != cudaSuccess) (void)cudaGetLastError();  // reported once, by the return value
     return e;
 }

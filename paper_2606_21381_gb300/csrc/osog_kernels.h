@@ -114,6 +114,40 @@ struct BwdReduceArgs {  // fixed-order sums into the particle and optics gradien
     SceneDev sc[kMaxScenes];
 };
 
+// Host: a launch struct with everything set but its per-scene arrays (the
+// entries of the launch's scenes are filled in by the caller; the others, up
+// to 19 KB of them, are never read).
+inline ColumnArgs column_args(const Geometry &geo, const Work &w, const float2 *tw, int S, int K) {
+    ColumnArgs a;
+    a.geo = geo;
+    a.w = w;
+    a.tw = tw;
+    a.S = S;
+    a.K = K;
+    a.unit_input = a.wait_polls = a.wait_extra = 0;
+    a.loss = LossDev{};
+    return a;
+}
+inline BwdColumnArgs bwd_column_args(const Geometry &geo, const Work &w, const float2 *tw, float *opart,
+                                     int S, int K) {
+    BwdColumnArgs a;
+    a.geo = geo;
+    a.w = w;
+    a.tw = tw;
+    a.opart = opart;
+    a.S = S;
+    a.K = K;
+    return a;
+}
+inline GroupDev group_dev(int S, int K, int nchunks) {
+    GroupDev g;
+    g.S = S;
+    g.K = K;
+    g.nchunks = nchunks;
+    g.pad_ = 0;
+    return g;
+}
+
 // Host: the scene constants of one optics struct (the caller fills in the
 // launch fields p0, n, chunk0, pair0 and pair_cap), and the transfer-
 // function constants of one modality bit, in double precision rounded

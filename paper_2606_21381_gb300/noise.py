@@ -2,12 +2,11 @@
 plus Gaussian read noise, computed by libosog's osog_sensor_noise."""
 from __future__ import annotations
 
-import ctypes
-
 import torch
 
 from . import _lib
 from ._lib import check
+from ._stream import raw_stream
 
 
 def sensor_noise(image: torch.Tensor, photons_per_unit: float, read_sigma: float, seed: int,
@@ -18,10 +17,9 @@ def sensor_noise(image: torch.Tensor, photons_per_unit: float, read_sigma: float
         raise ValueError("image must be a contiguous CUDA float32 tensor")
     if out is None:
         out = torch.empty_like(image)
-    stream = torch.cuda.current_stream(image.device).cuda_stream
-    check(_lib.lib().osog_sensor_noise(ctypes.c_void_p(image.data_ptr()), image.numel(),
+    check(_lib.lib().osog_sensor_noise(image.data_ptr(), image.numel(),
                                        float(photons_per_unit), float(read_sigma),
-                                       int(seed) & 0xFFFFFFFFFFFFFFFF,
-                                       ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(stream)),
+                                       int(seed) & 0xFFFFFFFFFFFFFFFF, out.data_ptr(),
+                                       raw_stream(image.device.index)),
           "osog_sensor_noise")
     return out

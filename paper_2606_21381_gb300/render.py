@@ -14,19 +14,19 @@ import torch
 
 from . import _lib
 from ._lib import LossParams, OsogError, Optics, Tuning, check, optics_struct
+from ._stream import raw_stream
 
 
 def n_modes(optics: dict) -> int:
     return bin(int(optics["modes"]) & 7).count("1")
 
 
-def _ptr(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: torch.Tensor | None) -> int | None:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    return raw_stream() if stream is None else stream.cuda_stream
 
 
 class Renderer:
@@ -69,7 +69,7 @@ class Renderer:
         return self._ws
 
     def _check_soa(self, soa: torch.Tensor) -> None:
-        if soa.device.type != "cuda" or soa.dtype != torch.float32 or soa.dim() != 2 \
+        if not soa.is_cuda or soa.dtype != torch.float32 or soa.dim() != 2 \
                 or soa.shape[0] != 9 or not soa.is_contiguous():
             raise ValueError("soa must be a contiguous cuda float32 tensor of shape (9, ld)")
 
