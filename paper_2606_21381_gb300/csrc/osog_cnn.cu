@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(NT) k_conv_gemm(const __grid_constant__ Args a
     auto Bs = [&](int buf, int row, int k) -> __nv_bfloat16 * {
         return T ? smB + buf * BK * LDT + k * LDT + row : smB + buf * BN * LDS + row * LDS + k;
     };
+    pdl_enter();
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
     int kbeg = 0, kend = a.Kred;
     if constexpr (PASS == kWgrad) {
@@ -419,6 +420,7 @@ __global__ void __launch_bounds__(kC8Threads, 3) k_conv_c8(const __grid_constant
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) unsigned char out[kC8Threads / 32][16 * 80];
     __shared__ __align__(16) uint4 zero;
+    pdl_enter();
     const Geo &g = a.g;
     const PatchC8 p = patch_c8(g, kC8Rows);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -520,6 +522,7 @@ k_wgrad_c8(const __grid_constant__ Args a, int splits) {
     constexpr int KP = MT * 16, VECS = KP / 8, kPix = kC8W * kC8GradRows;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) uint4 zero;
+    pdl_enter();
     const Geo &g = a.g;
     const PatchC8 p = patch_c8(g, kC8GradRows);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -655,8 +658,7 @@ cudaError_t launch_conv_c8(const Args &a, cudaStream_t st) {
         cudaFuncSetAttribute(k_conv_c8, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     if (opt_in != cudaSuccess) return opt_in;
     const dim3 grid(g.N * ((g.Q + kC8W - 1) / kC8W) * ((g.P + kC8Rows - 1) / kC8Rows), (g.K + 31) / 32);
-    k_conv_c8<<<grid, kC8Threads, p.pitch * p.ph * 16, st>>>(a);
-    return cudaGetLastError();
+    return launch_conv(k_conv_c8, grid, kC8Threads, p.pitch * p.ph * 16, st, a);
 }
 
 template <int MT>
@@ -669,8 +671,7 @@ cudaError_t launch_wgrad_c8(const Args &a, cudaStream_t st) {
         cudaFuncSetAttribute(k_wgrad_c8<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (opt_in != cudaSuccess) return opt_in;
     const int splits = splits_c8(a.g);
-    k_wgrad_c8<MT><<<splits, kC8Threads, smem, st>>>(a, splits);
-    return cudaGetLastError();
+    return launch_conv(k_wgrad_c8<MT>, dim3(splits), kC8Threads, smem, st, a, splits);
 }
 
 // Sum of the filter-gradient partial tiles over the pixel splits, in split
@@ -849,8 +850,7 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
     }
     if (!y_f32 && fits_c8(a.g)) return status_of(launch_conv_c8(a, st));
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
-    k_conv_gemm<kFwd><<<grid, NT, 0, st>>>(a);
-    return status_of(cudaGetLastError());
+    return status_of(launch_conv(k_conv_gemm<kFwd>, grid, NT, 0, st, a));
 }
 
 int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy,

@@ -278,8 +278,8 @@ struct KernelArg {
     using type = T;
 };
 template <typename... KArgs>
-inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
-                                cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), bool early, dim3 grid, int block, size_t smem,
+                              cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -289,11 +289,17 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, 
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = (long)grid.x * grid.y * grid.z <= kPdlMaxCtas ? 1 : 0;
+    cfg.numAttrs = early ? 1 : 0;
     void *ptrs[] = {const_cast<void *>(static_cast<const void *>(&args))...};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), ptrs);
     if (e != cudaSuccess) (void)cudaGetLastError();  // reported once, by the return value
     return e;
+}
+template <typename... KArgs>
+inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
+                                cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
+    return launch_pdl(kernel, (long)grid.x * grid.y * grid.z <= kPdlMaxCtas, grid, block, smem, st,
+                      args...);
 }
 
 // ---------------------------------------------------------------- status

@@ -36,6 +36,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "osog_common.cuh"
 #include "osog_conv_tma.h"
 
 namespace osog {
@@ -258,6 +259,7 @@ k_conv_patch(const __grid_constant__ CUtensorMap src, const __grid_constant__ CU
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    pdl_enter();  // after the allocation: see launch_conv
     const int tile = blockIdx.x % (a.tiles_x * a.tiles_y), img = blockIdx.x / (a.tiles_x * a.tiles_y);
     const int oy0 = (tile / a.tiles_x) * a.ty * kTileH, ox0 = (tile % a.tiles_x) * a.tx * kTileW;
     const int n0 = blockIdx.y * a.bn;
@@ -546,6 +548,7 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    pdl_enter();
     const uint32_t base = smem_addr(smem);
     const int dy_bytes = a.k64 * kTileW * kTileH * 128;
     const uint32_t planes = a.planes[group];
@@ -720,6 +723,7 @@ __global__ void __launch_bounds__(32 * kSumLanes)
 k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, float4 *out,
             float4 *out2) {
     __shared__ float4 red[kSumLanes][32];
+    pdl_enter();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * 32 + lane, row = count4 + extra4;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -886,8 +890,7 @@ cudaError_t launch_patch_ch(const CUtensorMap &src, const CUtensorMap &flt, cons
         k_conv_patch<FWD, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
     if (opt_in != cudaSuccess) return opt_in;
     const dim3 grid(images * a.tiles_x * a.tiles_y, ceil_div(a.ncols, a.bn));
-    k_conv_patch<FWD, CH><<<grid, kCtaThreads, patch_smem(a), st>>>(src, flt, a);
-    return cudaGetLastError();
+    return launch_conv(k_conv_patch<FWD, CH>, grid, kCtaThreads, patch_smem(a), st, src, flt, a);
 }
 
 template <bool FWD>
@@ -1100,8 +1103,7 @@ cudaError_t launch_wgrad(const CUtensorMap &mdy, const CUtensorMap &mx, const Wg
         k_wgrad_patch<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
     if (opt_in != cudaSuccess) return opt_in;
     const dim3 grid(ceil_div(a.K, 128) * a.cblocks * a.groups, a.splits);
-    k_wgrad_patch<CH><<<grid, kCtaThreads, wgrad_smem(a), st>>>(mdy, mx, a);
-    return cudaGetLastError();
+    return launch_conv(k_wgrad_patch<CH>, grid, kCtaThreads, wgrad_smem(a), st, mdy, mx, a);
 }
 
 }  // namespace
@@ -1137,10 +1139,9 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
 cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
                            cudaStream_t st) {
     const int64_t count4 = (int64_t)g.K * g.R * g.S * g.C / 4, extra4 = g.K / 4;
-    k_sum_parts<<<(unsigned)((count4 + extra4 + 31) / 32), 32 * kSumLanes, 0, st>>>(
-        reinterpret_cast<const float4 *>(part), splits, count4, extra4, reinterpret_cast<float4 *>(dw),
-        reinterpret_cast<float4 *>(dbias));
-    return cudaGetLastError();
+    return launch_conv(k_sum_parts, dim3((unsigned)((count4 + extra4 + 31) / 32)), 32 * kSumLanes, 0, st,
+                       reinterpret_cast<const float4 *>(part), splits, count4, extra4,
+                       reinterpret_cast<float4 *>(dw), reinterpret_cast<float4 *>(dbias));
 }
 
 cudaError_t conv_tma_take_status(int *timed_out) {

@@ -5,8 +5,23 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "osog_common.cuh"
+
 namespace osog {
 namespace cnn {
+
+// Launch of a convolution kernel with programmatic stream serialization: it is
+// dispatched and sets itself up while the kernel before it finishes.  Such a
+// kernel calls pdl_enter() before anything it reads or writes in global memory,
+// and after its tensor memory is allocated: the next kernel's CTAs may come as
+// soon as every CTA of this one has let them, and one that took the tensor
+// memory of an SM before a CTA of this kernel had its own would wait for this
+// kernel, which would wait for it.
+template <typename... KArgs>
+inline cudaError_t launch_conv(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
+                               cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
+    return launch_pdl(kernel, true, grid, block, smem, st, args...);
+}
 
 struct Geo {
     int N, H, W, C, K, R, S, stride, pad, P, Q;
