@@ -29,13 +29,12 @@ constexpr int kRounds = 64;            // attempts cap (2 per round)
 __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32_t k1) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c[0]), lo0 = 0xD2511F53u * c[0];
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c[2]), lo1 = 0xCD9E8D57u * c[2];
-        const uint32_t n0 = hi1 ^ c[1] ^ k0, n2 = hi0 ^ c[3] ^ k1;
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c[0], p1 = (uint64_t)0xCD9E8D57u * c[2];
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c[1] ^ k0, n2 = (uint32_t)(p0 >> 32) ^ c[3] ^ k1;
         c[0] = n0;
-        c[1] = lo1;
+        c[1] = (uint32_t)p1;
         c[2] = n2;
-        c[3] = lo0;
+        c[3] = (uint32_t)p0;
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
     }
@@ -109,57 +108,166 @@ struct NoiseArgs {
     int32_t fast;
 };
 
-// One element on the FP32 pipes; false when a decision is left open.
-__device__ __forceinline__ bool draw_fast(const NoiseArgs &a, float v, int64_t i, float *out) {
-    uint32_t c[4] = {(uint32_t)(uint64_t)i, (uint32_t)((uint64_t)i >> 32), 0u, kTag};
-    philox4x32_10(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
-    ff z = {0.f, 0.f};
-    if (a.sigma_ff.h > 0.f) {
-        if (c[0] == 0u) return false;
-        z = normal_ff(c[0], c[1]);
+// An element whose first rejection attempt was not accepted at once: its
+// candidate (n = 0: rejected already), its rate, sigma z and place in the tile.
+struct Pending {
+    float k;
+    uint32_t n, xv;
+    ff lam, noise;
+    uint32_t at;
+};
+
+// The attempts of the rounds after the first one: kYes with the count or
+// kUndecided.
+__device__ __forceinline__ int more_attempts(const NoiseArgs &a, ff lam, int64_t i, float *k) {
+    const Ptrs p = ptrs_of(lam);
+    int s = kNo;
+    for (uint32_t r = 1; s == kNo && r < kRounds; ++r) {
+        uint32_t c[4] = {(uint32_t)(uint64_t)i, (uint32_t)((uint64_t)i >> 32), r, kTag};
+        philox4x32_10(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+        s = ptrs_attempt(p, c[0], c[1], k);
+        if (s == kNo) s = ptrs_attempt(p, c[2], c[3], k);
     }
-    float k = 0.f;
-    if (v > 0.f) {
-        ff lam = two_prod(a.g_ff.h, v);
-        lam = fast_two_sum(lam.h, f_fma(a.g_ff.l, v, lam.l));
-        // below 10 inverts; the rate is exact when the gain has 24 bits
-        const float side = f_add(f_sub(lam.h, 10.f), lam.l);
-        if (a.g_ff.l != 0.f && fabsf(side) < 1e-10f) return false;
-        if (side < 0.f) {
-            if (poisson_small(lam.h, c[2], &k) != kYes) return false;
-        } else {
-            if (!(lam.h < 4194304.f)) return false;
-            const Ptrs p = ptrs_of(lam);
-            int s = ptrs_attempt(p, c[2], c[3], &k);
-            for (uint32_t r = 1; s == kNo; ++r) {
-                if (r == kRounds) return false;
-                c[0] = (uint32_t)(uint64_t)i;
-                c[1] = (uint32_t)((uint64_t)i >> 32);
-                c[2] = r;
-                c[3] = kTag;
-                philox4x32_10(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
-                s = ptrs_attempt(p, c[0], c[1], &k);
-                if (s == kNo) s = ptrs_attempt(p, c[2], c[3], &k);
-            }
-            if (s != kYes) return false;
-        }
-    }
-    return noisy_value(k, a.sigma_ff, z, a.inv_g, out);
+    return s == kNo ? kUndecided : s;
 }
 
-// Bound by instruction issue: about 900 warp instructions per 32 elements
-// (Philox 100 a round, the normal 155, about 80 per rejection attempt, and a
-// warp runs as many attempts as its unluckiest lane needs).  All of it in
-// double precision was bound by the FP64 pipe, 11.54 ms for 16 images of
-// 1024 x 1024 at 1,000 photons; this kernel takes 0.574 ms, with the same bits.
-__global__ void __launch_bounds__(256) k_sensor_noise(const __grid_constant__ NoiseArgs a) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float v = a.img[i];
-        float y;
-        if (!(a.fast && draw_fast(a, v, i, &y))) y = draw_exact(v, i, a.g, a.sigma, a.seed);
-        a.out[i] = y;
+constexpr int kNoiseThreads = 256, kPerThread = 4, kTile = kNoiseThreads * kPerThread;
+constexpr int kNoiseCtas = 4;  // resident on an SM
+
+// A CTA draws tiles of kTile elements in three sweeps.  Every element gets its
+// normal and the quick part of its first attempt (about 68% of rates above ten
+// end there); the others queue up in shared memory and take their acceptance
+// test as full warps; those it rejects queue up again for further attempts.  A
+// warp would otherwise run every step for its unluckiest lane.  Undecided
+// elements collect over the tiles and are drawn in double precision by the CTA
+// together.
+//
+// Bound by instruction issue.  16 images of 1024 x 1024 at 1,000 photons (the
+// same bits): all in double precision 11.54 ms, bound by the FP64 pipe; on the
+// FP32 pipes without queues 0.560 ms, about 1,000 warp instructions per 32
+// elements; this kernel 0.45 ms, about 740.
+__global__ void __launch_bounds__(kNoiseThreads, kNoiseCtas)
+k_sensor_noise(const __grid_constant__ NoiseArgs a) {
+    __shared__ Pending queue[kTile];
+    __shared__ uint16_t again[kTile];
+    __shared__ int64_t open[kTile + kNoiseThreads];
+    __shared__ int npend, nagain, nopen;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    if (threadIdx.x == 0) npend = nagain = nopen = 0;
+    __syncthreads();
+    // a warp's lanes with `take` reserve consecutive places of a list
+    auto reserve = [&](int *count, bool take) {
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(count, __popc(m));
+        return __shfl_sync(0xffffffffu, base, 0) + __popc(m & below);
+    };
+    const int64_t tiles = (a.count + kTile - 1) / kTile;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t i0 = tile * kTile;
+        for (int u = 0; u < kPerThread; ++u) {
+            const int at = u * kNoiseThreads + threadIdx.x;
+            const int64_t i = i0 + at;
+            Pending e;
+            bool pend = false, undecided = false;
+            if (i < a.count) {
+                const float v = a.img[i];
+                uint32_t c[4] = {(uint32_t)(uint64_t)i, (uint32_t)((uint64_t)i >> 32), 0u, kTag};
+                philox4x32_10(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+                e.noise = {0.f, 0.f};
+                undecided = !a.fast;
+                if (a.sigma_ff.h > 0.f) {
+                    undecided = undecided || c[0] == 0u;
+                    e.noise = mul_lazy(a.sigma_ff, normal_ff(c[0], c[1]));
+                }
+                e.k = 0.f;
+                if (v > 0.f) {
+                    e.lam = two_prod(a.g_ff.h, v);
+                    e.lam = fast_two_sum(e.lam.h, f_fma(a.g_ff.l, v, e.lam.l));
+                    // below 10 inverts; the rate is exact when the gain has 24 bits
+                    const float side = f_add(f_sub(e.lam.h, 10.f), e.lam.l);
+                    if (a.g_ff.l != 0.f && fabsf(side) < 1e-10f) undecided = true;
+                    if (side < 0.f) {
+                        if (!undecided) undecided = poisson_small(e.lam.h, c[2], &e.k) != kYes;
+                    } else if (!(e.lam.h < 4194304.f)) {
+                        undecided = true;
+                    } else {
+                        const Ptrs p = ptrs_of(e.lam);
+                        e.n = 0u;
+                        e.xv = c[3];
+                        int s = ptrs_candidate(p, c[2], c[3], &e.k, &e.n);
+                        if (s == kYes) s = ptrs_quick(p, e.n, c[3]);
+                        pend = s == kNo;
+                        undecided = undecided || s == kUndecided;
+                    }
+                }
+                if (undecided) {
+                    pend = false;
+                } else if (!pend) {
+                    float y;
+                    undecided = !noisy_value(e.k, e.noise, a.inv_g, &y);
+                    if (!undecided) a.out[i] = y;
+                }
+                e.at = (uint32_t)at;
+            }
+            const int q = reserve(&npend, pend);
+            if (pend) queue[q] = e;
+            if (__any_sync(0xffffffffu, undecided)) {
+                const int o = reserve(&nopen, undecided);
+                if (undecided) open[o] = i;
+            }
+        }
+        __syncthreads();
+        const int np = npend;
+        for (int q = threadIdx.x; q - lane < np; q += kNoiseThreads) {
+            int s = kYes;
+            int64_t i = 0;
+            if (q < np) {
+                const Pending e = queue[q];
+                i = i0 + e.at;
+                s = e.n ? ptrs_accept_float(e.lam, e.k, e.n, e.xv) : kNo;
+                if (s == kYes) {
+                    float y;
+                    if (noisy_value(e.k, e.noise, a.inv_g, &y))
+                        a.out[i] = y;
+                    else
+                        s = kUndecided;
+                }
+            }
+            const int r = reserve(&nagain, s == kNo);
+            if (s == kNo) again[r] = (uint16_t)q;
+            const int o = reserve(&nopen, s == kUndecided);
+            if (s == kUndecided) open[o] = i;
+        }
+        __syncthreads();
+        const int na = nagain;
+        for (int q = threadIdx.x; q - lane < na; q += kNoiseThreads) {
+            bool undecided = false;
+            int64_t i = 0;
+            if (q < na) {
+                const Pending e = queue[again[q]];
+                i = i0 + e.at;
+                float k, y;
+                undecided = more_attempts(a, e.lam, i, &k) != kYes || !noisy_value(k, e.noise, a.inv_g, &y);
+                if (!undecided) a.out[i] = y;
+            }
+            const int o = reserve(&nopen, undecided);
+            if (undecided) open[o] = i;
+        }
+        __syncthreads();
+        // room for a whole tile stays in the list of undecided elements
+        if (nopen >= kNoiseThreads) {
+            for (int o = threadIdx.x; o < nopen; o += kNoiseThreads)
+                a.out[open[o]] = draw_exact(a.img[open[o]], open[o], a.g, a.sigma, a.seed);
+            __syncthreads();
+            if (threadIdx.x == 0) nopen = 0;
+        }
+        if (threadIdx.x == 0) npend = nagain = 0;
+        __syncthreads();
     }
+    for (int o = threadIdx.x; o < nopen; o += kNoiseThreads)
+        a.out[open[o]] = draw_exact(a.img[open[o]], open[o], a.g, a.sigma, a.seed);
 }
 
 }  // namespace
@@ -178,8 +286,6 @@ extern "C" int osog_sensor_noise(const float *image, int64_t count, double photo
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return OSOG_ERR_CUDA;
-    const int64_t want = (count + 255) / 256;
-    const int blocks = (int)(want < (int64_t)sms * 8 ? want : (int64_t)sms * 8);
     osog::noise::NoiseArgs a;
     a.img = image;
     a.out = out;
@@ -192,6 +298,10 @@ extern "C" int osog_sensor_noise(const float *image, int64_t count, double photo
     a.g_ff = osog::noise::split(photons_per_unit);
     a.inv_g = osog::noise::split(1.0 / photons_per_unit);
     a.sigma_ff = osog::noise::split(read_sigma);
-    osog::noise::k_sensor_noise<<<blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+    const int64_t tiles = (count + osog::noise::kTile - 1) / osog::noise::kTile;
+    const int blocks = (int)(tiles < (int64_t)sms * osog::noise::kNoiseCtas
+                                 ? tiles
+                                 : (int64_t)sms * osog::noise::kNoiseCtas);
+    osog::noise::k_sensor_noise<<<blocks, osog::noise::kNoiseThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
     return cudaGetLastError() == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA;
 }

@@ -24,9 +24,22 @@ namespace osog {
 namespace noise {
 
 #if defined(__CUDA_ARCH__)
-OSOG_HD float fast_rcp(float a) { return __fdividef(1.0f, a); }
-OSOG_HD float fast_rsqrt(float a) { return rsqrtf(a); }
-OSOG_HD float fast_log(float a) { return __logf(a); }
+// (the plain approximations: no scaling of denormals, which do not occur here)
+OSOG_HD float fast_rcp(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+OSOG_HD float fast_rsqrt(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+OSOG_HD float fast_log(float a) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r * 0.693147181f;
+}
 OSOG_HD int count_lz(uint32_t x) { return __clz((int)x); }
 #else
 OSOG_HD float fast_rcp(float a) { return 1.0f / a; }
@@ -183,8 +196,8 @@ OSOG_HD Ptrs ptrs_of(ff lam) {
     c.lam = lam;
     const ff s = fast_root(lam);
     ff b = mul_lazy(s, ff{PtrsB1::h, PtrsB1::l});
-    c.b = ff_add(b, ff{PtrsB0::h, PtrsB0::l});
-    const ff a = ff_add(mul_lazy(c.b, ff{PtrsA1::h, PtrsA1::l}), ff{PtrsA0::h, PtrsA0::l});
+    c.b = add_small(b, ff{PtrsB0::h, PtrsB0::l});  // 2.53 s >= 8
+    const ff a = add_small(mul_lazy(c.b, ff{PtrsA1::h, PtrsA1::l}), ff{PtrsA0::h, PtrsA0::l});
     c.a2 = ff{f_add(a.h, a.h), f_add(a.l, a.l)};
     c.inv_alpha = f_fma(1.1328f, fast_rcp(f_sub(c.b.h, 3.4f)), 1.1239f);
     c.vr = f_fma(-3.6224f, fast_rcp(f_sub(c.b.h, 2.0f)), 0.9277f);
@@ -227,21 +240,19 @@ OSOG_HD float log_density(ff lam, float k) {
 constexpr uint32_t kUs007 = 601295422u;   // smallest n with n 2^-33 >= 0.07
 constexpr uint32_t kUs0013 = 111669150u;  // smallest n with n 2^-33 >= 0.013
 
-// One attempt of PTRS from the words of U and V: kYes with *k_out, kNo
-// (rejected) or kUndecided.
-OSOG_HD int ptrs_attempt(const Ptrs &c, uint32_t xu, uint32_t xv, float *k_out) {
+// The candidate of one attempt of PTRS from the word of U (xv, the word of V,
+// settles the rejection of slim tails): kYes with k = floor((2 a / us + b) U +
+// lam + 0.43) and us = n 2^-33, kNo (rejected whatever k is) or kUndecided.
+OSOG_HD int ptrs_candidate(const Ptrs &c, uint32_t xu, uint32_t xv, float *k_out, uint32_t *n_out) {
     // U = -+ m 2^-33, us = 1/2 - |U| = n 2^-33, m = 2^32 - n
     const bool neg = xu < 0x80000000u;
     const uint32_t n = neg ? 2u * xu + 1u : 0u - (2u * xu + 1u);
     const uint32_t m = 0u - n;
-    const bool slim = n < kUs0013;
+    // us < 0.013 and V > us: rejected (the quick acceptance needs us >= 0.07;
+    // k < 0 is rejected too, so k is not needed)
+    if (n < kUs0013 && xv > (n >> 1)) return kNo;
     const ff nf = {(float)(n & 0xFFFFFF00u), (float)(n & 0xFFu)};
     const ff mf = {(float)(m & 0xFFFFFF00u), (float)(m & 0xFFu)};
-    if (slim && (xv > (n >> 1))) {
-        // V > us: rejected, unless the quick acceptance (us >= 0.07) took it,
-        // which slim excludes; k < 0 is rejected too, so k is not needed
-        return kNo;
-    }
     // X = -+ (2 a m / n + b m 2^-33) + lam + 0.43
     const float r = fast_rcp(f_add(nf.h, nf.l));
     const float q0 = f_mul(f_add(mf.h, mf.l), r);
@@ -253,44 +264,76 @@ OSOG_HD int ptrs_attempt(const Ptrs &c, uint32_t xu, uint32_t xv, float *k_out) 
                                f_mul(mf.l, 1.1641532182693481e-10f));
     const ff t2 = mul_lazy(c.b, mu);
     const float sg = neg ? -1.0f : 1.0f;
-    const ff t = ff_add(t1, t2);
-    const ff base = ff_add(c.lam, ff{PtrsShift::h, PtrsShift::l});
-    const ff X = ff_add(ff{f_mul(sg, t.h), f_mul(sg, t.l)}, base);
+    ff t = two_sum(t1.h, t2.h);
+    t.l = f_add(t.l, f_add(t1.l, t2.l));
+    const ff base = add_small(c.lam, ff{PtrsShift::h, PtrsShift::l});
+    ff X = two_sum(f_mul(sg, t.h), base.h);
+    X.l = f_add(X.l, f_fma(sg, t.l, base.l));  // |X.l| stays within a few ulps
     // 2^-39 of the largest term bounds the error of X
     const float err = f_mul(f_add(f_add(t.h, c.lam.h), 1.0f), 1.8189894035458565e-12f);
     if (X.h < -1.0f) return kNo;      // k < 0 (us is below 0.07 then)
     if (!(X.h < 4194304.0f)) return kUndecided;
     float k = floorf(X.h);
     float fr = f_add(f_sub(X.h, k), X.l);
-    if (fr < 0.0f) {
-        k = f_sub(k, 1.0f);
-        fr = f_add(fr, 1.0f);
-    }
+    const float carry = fr < 0.0f ? -1.0f : fr >= 1.0f ? 1.0f : 0.0f;
+    k = f_add(k, carry);
+    fr = f_sub(fr, carry);
     if (fr < err || fr > f_sub(1.0f, err) - 1.2e-7f) return kUndecided;
     *k_out = k;
-    const float V = f_mul((float)(xv >> 8) + (float)(xv & 0xFFu) * 0.00390625f + 0.001953125f,
-                          5.9604644775390625e-08f);
-    if (n >= kUs007) {
-        const float dv = f_sub(c.vr, V);
-        if (fabsf(dv) < 2e-6f) return kUndecided;
-        if (dv > 0.0f) return kYes;
-    }
+    *n_out = n;
+    return kYes;
+}
+
+OSOG_HD float ptrs_v(uint32_t xv) {  // V = (xv + 1/2) 2^-32
+    return f_mul((float)(xv >> 8) + (float)(xv & 0xFFu) * 0.00390625f + 0.001953125f,
+                 5.9604644775390625e-08f);
+}
+
+// The quick acceptance of a candidate: kYes, kUndecided, or kNo: not accepted by
+// it (ptrs_accept decides).
+OSOG_HD int ptrs_quick(const Ptrs &c, uint32_t n, uint32_t xv) {
+    const float dv = f_sub(c.vr, ptrs_v(xv));
+    if (n < kUs007 || dv < -2e-6f) return kNo;
+    return dv < 2e-6f ? kUndecided : kYes;
+}
+
+// The acceptance test of a candidate k that the quick one left: b and a2 of the
+// rate in float are enough.
+OSOG_HD int ptrs_accept(ff lam, float b, float a2, float inv_alpha, float k, uint32_t n, uint32_t xv) {
     if (k < 0.0f) return kNo;
     const float us = f_mul((float)n, 1.1641532182693481e-10f);
-    const float lhs = fast_log(f_mul(f_mul(V, c.inv_alpha),
-                                     fast_rcp(f_fma(f_mul(0.5f, c.a2.h), fast_rcp(f_mul(us, us)),
-                                                    c.b.h))));
-    const float rhs = log_density(c.lam, k);
+    const float lhs = fast_log(f_mul(f_mul(ptrs_v(xv), inv_alpha),
+                                     fast_rcp(f_fma(f_mul(0.5f, a2), fast_rcp(f_mul(us, us)), b))));
+    const float rhs = log_density(lam, k);
     const float gap = f_sub(rhs, lhs);
     const float tol = f_fma(fabsf(rhs), 1e-5f, 4e-5f);
     if (!(fabsf(gap) >= tol)) return kUndecided;
     return gap > 0.0f ? kYes : kNo;
 }
 
+// ptrs_accept with the constants of the rate taken in float (b to a few 1e-7
+// relative, well inside its tolerance).
+OSOG_HD int ptrs_accept_float(ff lam, float k, uint32_t n, uint32_t xv) {
+    const float b = f_fma(2.53f, f_mul(lam.h, fast_rsqrt(lam.h)), 0.931f);
+    const float a2 = 2.0f * f_fma(0.02483f, b, -0.059f);
+    return ptrs_accept(lam, b, a2, f_fma(1.1328f, fast_rcp(f_sub(b, 3.4f)), 1.1239f), k, n, xv);
+}
+
+// One attempt of PTRS from the words of U and V: kYes with *k_out, kNo
+// (rejected) or kUndecided.
+OSOG_HD int ptrs_attempt(const Ptrs &c, uint32_t xu, uint32_t xv, float *k_out) {
+    uint32_t n;
+    float k;
+    int s = ptrs_candidate(c, xu, xv, &k, &n);
+    if (s != kYes) return s;
+    *k_out = k;
+    s = ptrs_quick(c, n, xv);
+    return s != kNo ? s : ptrs_accept(c.lam, c.b.h, c.a2.h, c.inv_alpha, k, n, xv);
+}
+
 // (k + sigma z) / g rounded to float: true with *out when the error bounds of
-// the parts decide the rounding.  inv_g = 1 / g and sigma as float-float.
-OSOG_HD bool noisy_value(float k, ff sigma, ff z, ff inv_g, float *out) {
-    const ff sz = mul_lazy(sigma, z);
+// the parts decide the rounding.  sz = sigma z and inv_g = 1 / g as float-float.
+OSOG_HD bool noisy_value(float k, ff sz, ff inv_g, float *out) {
     ff T = two_sum(k, sz.h);
     T = fast_two_sum(T.h, f_add(T.l, sz.l));
     const ff y = ff_mul(T, inv_g);

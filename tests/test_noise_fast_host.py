@@ -61,6 +61,13 @@ int main(int, char **argv) {
                         -lam + kk * std::log(lam) - std::lgamma(kk + 1.0) ? kYes : kNo;
             if (r == kUndecided) ++open;
             else if (r != want || (r == kYes && (double)k != kk)) ++wrong;
+            // the test with the rate's constants in float
+            float kc = 0.f;
+            uint32_t m = 0;
+            if (ptrs_candidate(ptrs_of(lf), a, b, &kc, &m) == kYes && !(us >= 0.07 && V <= vr)) {
+                const int s = ptrs_accept_float(lf, kc, m, b);
+                if (s != kUndecided && s != want) ++wrong;
+            }
         } else {  // the rounded output for counts up to 2^22
             if (a == 0u) continue;
             const float k = i % 7 ? (float)(rng() % (1u << (1 + rng() % 22))) : 0.f;
@@ -68,8 +75,8 @@ int main(int, char **argv) {
             const double z = std::sqrt(-2.0 * std::log(unit(a))) *
                              std::cos(6.283185307179586476925286766559 * unit(b));
             float got;
-            const bool ok = noisy_value(k, split(sigma), sigma > 0 ? normal_ff(a, b) : ff{0.f, 0.f},
-                                        split(1.0 / p), &got);
+            const ff sz = sigma > 0 ? mul_lazy(split(sigma), normal_ff(a, b)) : ff{0.f, 0.f};
+            const bool ok = noisy_value(k, sz, split(1.0 / p), &got);
             if (!ok) ++open;
             else if (got != (float)(((double)k + sigma * z) / p)) ++wrong;
         }
