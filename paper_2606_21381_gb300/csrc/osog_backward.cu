@@ -31,6 +31,29 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// The sums of eight values over the lanes of a warp: lanes exchange halves of
+// the values while they add (nine shuffles instead of forty), in a fixed order.
+// Lane l ends with the sum of value (l >> 2) & 7 as 4 b4 + 2 b3 + b2 of its bits.
+__device__ __forceinline__ float warp_sum8(float (&v)[8], int lane) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool up = lane & 16;
+        const float give = up ? v[i] : v[i + 4], keep = up ? v[i + 4] : v[i];
+        v[i] = keep + __shfl_xor_sync(kFull, give, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const bool up = lane & 8;
+        const float give = up ? v[i] : v[i + 2], keep = up ? v[i + 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(kFull, give, 8);
+    }
+    const bool up = lane & 4;
+    const float give = up ? v[0] : v[1], keep = up ? v[1] : v[0];
+    float s = keep + __shfl_xor_sync(kFull, give, 4);
+    s += __shfl_xor_sync(kFull, s, 2);
+    return s + __shfl_xor_sync(kFull, s, 1);
+}
+
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1) k_bwd_rows(const __grid_constant__ BwdRowsArgs a) {
     pdl_enter();
@@ -158,7 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_strip(const __grid_constant
     float2 *bufG = reinterpret_cast<float2 *>(smem_raw);
     float2 *bufO = bufG + L * LS;
     PRec *srec = reinterpret_cast<PRec *>(bufO + L * LS);
-    Rect *srect = reinterpret_cast<Rect *>(srec + kThreads);
+    RRec *srrec = reinterpret_cast<RRec *>(srec + kThreads);
+    Rect *srect = reinterpret_cast<Rect *>(srrec + kThreads);
     int *sslot = reinterpret_cast<int *>(srect + kThreads);
     int *wsum = sslot + kThreads;
     const Geometry &geo = a.geo;
@@ -222,45 +246,74 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_strip(const __grid_constant
             const int slot = before + __popc(m & lt);
             srect[slot] = q;
             srec[slot] = a.w.rec[id];
+            srrec[slot] = a.w.rrec[id];
             sslot[slot] = i;
         }
         __syncthreads();
         for (int k = warp; k < nl; k += NW) {
             const PRec r = srec[k];
+            const RRec rr = srrec[k];
             const Rect rq = srect[k];
-            const int xa = rq.x0, xb = rq.x1;
             const int ya = max((int)rq.y0, y0), yb = min((int)rq.y1, ylast);
-            const int bh = yb - ya + 1;
-            const int lyn = bh >= 32 ? 32 : (bh <= 1 ? 1 : 1 << (32 - __clz(bh - 1)));
+            const int bh = yb - ya + 1;  // at most R <= 32 rows
+            const int lyn = bh <= 1 ? 1 : 1 << (32 - __clz(bh - 1));
             const int lxn = 32 / lyn, shx = ilog2(lxn);
             const int lx = lane & (lxn - 1), ly = lane >> shx;
+            // lane l finds the span of row ya + l (as in the raster); a pixel's
+            // lanes take it from there
+            RowItem it;
+            it.hdr = 0u;
+            it.f[0] = it.f[1] = it.f[2] = it.f[3] = 0.f;
+            if (lane >= bh || !make_row_item<kAccPhase>(rr, rq.x0, rq.x1, ya + lane, 0, 1.f, it))
+                it.hdr = 0u;
+            const uint32_t hdr = __shfl_sync(kFull, it.hdr, ly);
+            const int yy = ya + ly;
+            const float ey = (float)yy + 0.5f - r.cy;
+            const int xe = (int)(hdr & 0xFFFu) + (int)((hdr >> 12) & 0xFFFu);
+            const float2 *row = bufO + (min(yy, ylast) - y0) * LS;
             float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            for (int yy = ya + ly; yy <= yb; yy += lyn) {
-                const float2 *row = bufO + (yy - y0) * LS;
-                for (int xx = xa + lx; xx <= xb; xx += lxn) {
+            if (rr.kind == 0) {
+                const float xlh = __shfl_sync(kFull, it.f[0], ly), xll = __shfl_sync(kFull, it.f[1], ly);
+                const float xrh = __shfl_sync(kFull, it.f[2], ly), xrl = __shfl_sync(kFull, it.f[3], ly);
+                const EllipseGrad e = ellipse_grad(r, rr.p[2]);
+                for (int xx = (int)(hdr & 0xFFFu) + lx; xx < xe; xx += lxn) {
+                    const float X = (float)xx + 0.5f;
+                    const float ep = __fadd_rn(__fsub_rn(xrh, X), xrl);
+                    const float en = __fsub_rn(__fsub_rn(X, xlh), xll);
+                    const float qq = __fmul_rn(ep, en);
+                    if (qq > 1e-30f) {
+                        const float2 g = row[pad16(xx)];
+                        ellipse_pixel_grad(r, e, qq, X - r.cx, ey, g.x, g.y, acc);
+                    }
+                }
+            } else {
+                for (int xx = (int)(hdr & 0xFFFu) + lx; xx < xe; xx += lxn) {
                     const float2 g = row[pad16(xx)];
-                    thickness_grad(r, (float)xx + 0.5f, (float)yy + 0.5f, g.x, g.y, acc);
+                    prism_grad(r, (float)xx + 0.5f - r.cx, ey, g.x, g.y, acc);
                 }
             }
+            const float v = warp_sum8(acc, lane);
             float *dst = a.part + ((size_t)(sc.pair0 + sslot[k]) * spb + kstrip) * 8;
-#pragma unroll
-            for (int f = 0; f < 8; ++f) {
-                const float v = warp_sum(acc[f]);
-                if (lane == f) dst[f] = v;
-            }
+            if ((lane & 3) == 0) dst[((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = v;
         }
         __syncthreads();
     }
 }
 
+// Eight lanes per particle, one per field, kReduceParticles particles per CTA:
+// lane f adds entry f of the particle's partials (a 32-byte line) in band and
+// strip order, loading eight partials at a time before it adds them.
+constexpr int kReduceParticles = kChunk / 8;
+
 __global__ void __launch_bounds__(kChunk) k_bwd_reduce(const __grid_constant__ BwdReduceArgs a) {
     pdl_enter();
     const Geometry &geo = a.geo;
-    if ((int)blockIdx.x >= a.nchunks) {  // optics: sum the per-block partials
+    const int pblocks = a.nchunks * (kChunk / kReduceParticles);
+    if ((int)blockIdx.x >= pblocks) {  // optics: sum the per-block partials
         // Warp f sums component f: lane l adds blocks l, l + 32, ... in
         // double, then a fixed butterfly combines the lanes (same order on
         // every run).
-        const int s = blockIdx.x - a.nchunks;
+        const int s = blockIdx.x - pblocks;
         const int f = threadIdx.x >> 5, lane = threadIdx.x & 31;
         if (f < 4) {
             double v = 0.0;
@@ -272,51 +325,41 @@ __global__ void __launch_bounds__(kChunk) k_bwd_reduce(const __grid_constant__ B
         }
         return;
     }
+    const int chunk = blockIdx.x / (kChunk / kReduceParticles);
     int s = 0;
     for (int t = 1; t < a.S; ++t)
-        if (a.sc[t].chunk0 <= (int)blockIdx.x) s = t;
+        if (a.sc[t].chunk0 <= chunk) s = t;
     const SceneDev &sc = a.sc[s];
-    const int local = ((int)blockIdx.x - sc.chunk0) * kChunk + threadIdx.x;
+    const int f = threadIdx.x & 7;
+    const int local = (chunk - sc.chunk0) * kChunk +
+                      (blockIdx.x % (kChunk / kReduceParticles)) * kReduceParticles + (threadIdx.x >> 3);
     if (local >= sc.n) return;
     const int p = sc.p0 + local;
     const Rect q = a.w.rect[p];
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float acc = 0.f;
     if (q.x0 <= q.x1 && q.y0 <= q.y1) {
-        // The particle's band slots, 8 at a time: all slot loads first, then
-        // the partials of every (slot, strip) in band and strip order.
         const int spb = geo.BH / geo.R;
         const int b0 = q.y0 / geo.BH;
         const int nb = min(q.y1 / geo.BH - b0 + 1, a.w.slotmap_ppp);
         const int32_t *sm = a.w.slotmap + (size_t)p * a.w.slotmap_ppp;
-        for (int j0 = 0; j0 < nb; j0 += 8) {
-            int slot[8];
+        for (int e0 = 0; e0 < nb * spb; e0 += 8) {
+            float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) slot[j] = j0 + j < nb ? sm[j0 + j] : -1;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (slot[j] < 0) continue;
-                const int b = b0 + j0 + j;
-                const float4 *src =
-                    reinterpret_cast<const float4 *>(a.part + (size_t)(sc.pair0 + slot[j]) * spb * 8);
-                for (int k = 0; k < spb; ++k) {
-                    const int r0 = b * geo.BH + k * geo.R;
-                    if (r0 > q.y1 || r0 + geo.R - 1 < q.y0) continue;
-                    const float4 u = src[2 * k], v = src[2 * k + 1];
-                    acc[0] += u.x;
-                    acc[1] += u.y;
-                    acc[2] += u.z;
-                    acc[3] += u.w;
-                    acc[4] += v.x;
-                    acc[5] += v.y;
-                    acc[6] += v.z;
-                    acc[7] += v.w;
+            for (int i = 0; i < 8; ++i) {
+                const int e = e0 + i, j = e / spb, k = e - j * spb;
+                const int r0 = (b0 + j) * geo.BH + k * geo.R;
+                v[i] = 0.f;
+                if (e < nb * spb && r0 <= q.y1 && r0 + geo.R - 1 >= q.y0) {
+                    const int slot = sm[j];
+                    if (slot >= 0) v[i] = a.part[((size_t)(sc.pair0 + slot) * spb + k) * 8 + f];
                 }
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc += v[i];
         }
     }
-#pragma unroll
-    for (int f = 0; f < 8; ++f) a.grad_soa[(int64_t)f * a.ld + p] = acc[f];
-    a.grad_soa[(int64_t)8 * a.ld + p] = 0.f;
+    a.grad_soa[(int64_t)f * a.ld + p] = acc;
+    if (f == 0) a.grad_soa[(int64_t)8 * a.ld + p] = 0.f;
 }
 
 template <int N>
@@ -373,7 +416,7 @@ size_t bwd_column_smem(int H) {
 
 size_t bwd_strip_smem(int W) {
     const int L = set_elems(W) / W;
-    const size_t gather = kThreads * (sizeof(PRec) + sizeof(Rect) + sizeof(int)) + 64;
+    const size_t gather = kThreads * (sizeof(PRec) + sizeof(RRec) + sizeof(Rect) + sizeof(int)) + 64;
     return (size_t)2 * L * line_stride(W) * sizeof(float2) +
            (gather > raster_smem<kThreads>() ? gather : raster_smem<kThreads>());
 }
@@ -395,7 +438,7 @@ cudaError_t launch_bwd_strip(const BwdStripArgs &a, cudaStream_t st) {
     return dispatch_n<BwdStrip>(a.geo.W, a, st);
 }
 cudaError_t launch_bwd_reduce(const BwdReduceArgs &a, cudaStream_t st) {
-    return launch_chain(k_bwd_reduce, dim3(a.nchunks + a.S), kChunk, 0, st, a);
+    return launch_chain(k_bwd_reduce, dim3(a.nchunks * (kChunk / kReduceParticles) + a.S), kChunk, 0, st, a);
 }
 
 }  // namespace osog

@@ -76,7 +76,6 @@ __device__ bool setup_planes(const Work &w, int off, int m, double c, double s, 
 // Setup of one particle: validation, float-float record, bounding rect.
 __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneDev &sc,
                                const Geometry &geo, const Work &w) {
-    PRec *rec = w.rec;
     int32_t *status = w.status;
     float f[9];
 #pragma unroll
@@ -125,12 +124,11 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
     r.cx = cx;
     r.cy = cy;
     r.ch = cf.h;
-    r.cl = cf.l;
     r.sh = sf.h;
-    r.sl = sf.l;
     r.T = T;
     r.dn = f[6];
     r.mu = f[7];
+    r.pad_[0] = r.pad_[1] = 0.f;
     float ex, ey;
     const float c = fabsf(r.ch), s = fabsf(r.sh);
     RRec rr;
@@ -145,10 +143,7 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
             latch(status, OSOG_ERR_NONFINITE_INPUT);
             return empty;
         }
-        r.p0h = __int_as_float(poff);
-        r.p0l = 0.f;
-        r.p1h = __int_as_float(pcnt);
-        r.p1l = 0.f;
+        r.p0h = r.p1h = 0.f;
         r.g = -1.f;  // marks a general polyhedron
         ex = ey = a;  // circumscribed radius of the footprint (px)
         rr.p[0] = __int_as_float(poff);
@@ -157,9 +152,7 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
         rr.kind = 2;
     } else if (kind == 1.f) {
         r.p0h = a;
-        r.p0l = 0.f;
         r.p1h = b;
-        r.p1l = 0.f;
         r.g = sc.prism_g;
         ex = a * c + b * s;
         ey = a * s + b * c;
@@ -171,11 +164,8 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
         rr.p[5] = T;
         rr.kind = 1;
     } else {
-        const ff ia = ff_recip(a), ib = ff_recip(b);
-        r.p0h = ia.h;
-        r.p0l = ia.l;
-        r.p1h = ib.h;
-        r.p1l = ib.l;
+        r.p0h = f_rcp(a);
+        r.p1h = f_rcp(b);
         r.g = 0.f;
         ex = sqrtf(a * a * c * c + b * b * s * s);
         ey = sqrtf(a * a * s * s + b * b * c * c);
@@ -190,7 +180,7 @@ __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneD
         rr.tsa = f_fma(T, q.sqrt_alpha.l, f_mul(T, q.sqrt_alpha.h));
         rr.kind = 0;
     }
-    rec[p] = r;
+    if (w.slotmap) w.rec[p] = r;
     w.rrec[p] = rr;
     // Pixel centres j + 0.5 inside [cx - ex, cx + ex], widened by one pixel
     // on each side; the thickness is exactly zero on the extra pixels.

@@ -62,19 +62,17 @@ __host__ inline Geometry make_geometry(int H, int W) {
     return g;
 }
 
-// Per-particle record written by the setup pass (64 bytes).  Angles and
-// inverse semi-axes are stored as float-float pairs (hi + lo), computed in
-// float-float arithmetic (cos, sin to 2^-47, reciprocals to 2^-47) so that
-// the ellipsoid rim can be evaluated with ~2^-44 relative error (see
-// ellipse_delta_ff()).
+// Per-particle record of the adjoint (48 bytes), written by the setup pass when
+// the adjoint follows (Work.slotmap set).
 struct __align__(16) PRec {
     float cx, cy;
-    float ch, cl, sh, sl;     // cos(theta), sin(theta) hi/lo
-    float p0h, p0l, p1h, p1l; // ellipsoid: 1/a, 1/b hi/lo; prism: hx, hy, -, -
+    float ch, sh;             // cos(theta), sin(theta)
+    float p0h, p1h;           // ellipsoid: 1/a, 1/b; prism: hx, hy
     float T, dn, mu;
     float g;                  // 0 for an ellipsoid, 2 s_b dx for a prism
+    float pad_[2];
 };
-static_assert(sizeof(PRec) == 64, "PRec is 64 bytes");
+static_assert(sizeof(PRec) == 48, "PRec is 48 bytes");
 
 // Per-particle constants of the row-span raster (48 bytes), written by the
 // setup pass beside PRec.  For an ellipsoid the chord through pixel centre
@@ -322,29 +320,5 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {  // a * conj(b)
 
 // ---------------------------------------------------------------- float-float
 // struct ff and its error-free transformations: osog_ff.h.
-
-// ---------------------------------------------------------------- geometry
-// 1 - rho^2 of an ellipsoid at pixel centre (x, y) in float-float, from the
-// float-float record: u = c ex + s ey, v = -s ex + c ey, rho^2 = (u/a)^2 +
-// (v/b)^2 with ex = x - cx taken exactly (TwoSum).  Used where the float32
-// value of 1 - rho^2 is small: there the float32 rounding of rho^2 (~2e-7)
-// would put an error of order T sqrt(2e-7) on the thickness T sqrt(1 - rho^2).
-__device__ __forceinline__ float ellipse_delta_ff(const PRec &r, float x, float y) {
-    ff exf = two_sum(x, -r.cx);
-    ff eyf = two_sum(y, -r.cy);
-    ff c = {r.ch, r.cl}, s = {r.sh, r.sl};
-    ff uf = ff_add(ff_mul(c, exf), ff_mul(s, eyf));
-    ff vf = ff_add(ff_mul(c, eyf), ff_neg(ff_mul(s, exf)));
-    ff uaf = ff_mul(uf, ff{r.p0h, r.p0l});
-    ff vbf = ff_mul(vf, ff{r.p1h, r.p1l});
-    ff rho2 = ff_add(ff_mul(uaf, uaf), ff_mul(vbf, vbf));
-    ff d = ff_add(ff{1.f, 0.f}, ff_neg(rho2));
-    return d.h + d.l;
-}
-
-// Band of 1 - rho^2 (float32) inside which the ellipsoid is re-evaluated in
-// float-float.  Outside it the float32 error of the thickness is below
-// T * 5e-7 / (2 sqrt(4e-3)) ~ 4e-6 T.
-constexpr float kRimBand = 4e-3f;
 
 }  // namespace osog

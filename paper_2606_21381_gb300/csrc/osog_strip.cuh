@@ -626,63 +626,76 @@ __device__ __forceinline__ void transfer_grad(const ModeDev &md, int fx, int fy,
 //   ellipsoid: t = T sqrt(delta), delta = 1 - u'^2 - v'^2, u' = u/a,
 //     v' = v/b; d delta/d(cx, cy) = 2 (u' c/a - v' s/b, u' s/a + v' c/b),
 //     d delta/d theta = 2 u' v' (a/b - b/a), d delta/d(a, b) = 2 (u'^2/a,
-//     v'^2/b); delta comes from float-float inside the rim band.
+//     v'^2/b); delta = qq alpha with qq = (xr - x)(x - xl) from the row's
+//     chord ends, which keeps its relative error at a rounding even at the
+//     rim (see item_chord);
 //   prism: t = clamp(g d, 0, T), d = min(hx - |u|, hy - |v|): on the ramp
 //     dt = g dd with dd/d(hx or hy) = 1 and the chain through |u| or |v|;
 //     on the plateau dt/dT = 1.
-__device__ __forceinline__ void thickness_grad(const PRec &r, float xc, float yc, float go,
-                                               float ga, float acc[8]) {
-    const float ex = xc - r.cx, ey = yc - r.cy;
+__device__ __forceinline__ void prism_grad(const PRec &r, float ex, float ey, float go, float ga,
+                                           float acc[8]) {
     const float wgt = fmaf(r.dn, go, r.mu * ga);
-    if (r.g > 0.f) {
-        const float u = fmaf(r.ch, ex, r.sh * ey);
-        const float v = fmaf(-r.sh, ex, r.ch * ey);
-        const float du = r.p0h - fabsf(u), dv = r.p1h - fabsf(v);
-        const float gd = r.g * fminf(du, dv);
-        if (!(gd > 0.f)) return;
-        const float t = fminf(gd, r.T);
-        acc[6] = fmaf(go, t, acc[6]);
-        acc[7] = fmaf(ga, t, acc[7]);
-        if (gd >= r.T) {
-            acc[5] += wgt;
-            return;
-        }
-        const float q = wgt * r.g;
-        if (du <= dv) {
-            const float sq = u >= 0.f ? q : -q;
-            acc[0] = fmaf(sq, r.ch, acc[0]);
-            acc[1] = fmaf(sq, r.sh, acc[1]);
-            acc[2] = fmaf(-sq, v, acc[2]);
-            acc[3] += q;
-        } else {
-            const float sq = v >= 0.f ? q : -q;
-            acc[0] = fmaf(-sq, r.sh, acc[0]);
-            acc[1] = fmaf(sq, r.ch, acc[1]);
-            acc[2] = fmaf(sq, u, acc[2]);
-            acc[4] += q;
-        }
+    const float u = fmaf(r.ch, ex, r.sh * ey);
+    const float v = fmaf(-r.sh, ex, r.ch * ey);
+    const float du = r.p0h - fabsf(u), dv = r.p1h - fabsf(v);
+    const float gd = r.g * fminf(du, dv);
+    if (!(gd > 0.f)) return;
+    const float t = fminf(gd, r.T);
+    acc[6] = fmaf(go, t, acc[6]);
+    acc[7] = fmaf(ga, t, acc[7]);
+    if (gd >= r.T) {
+        acc[5] += wgt;
         return;
     }
-    const float cia = r.ch * r.p0h, sia = r.sh * r.p0h;
-    const float cib = r.ch * r.p1h, sib = r.sh * r.p1h;
-    const float ua = fmaf(cia, ex, sia * ey);
-    const float vb = fmaf(-sib, ex, cib * ey);
-    float delta = 1.f - fmaf(ua, ua, vb * vb);
-    if (delta < kRimBand) {
-        if (delta <= -kRimBand) return;
-        delta = ellipse_delta_ff(r, xc, yc);
-        if (!(delta > 0.f)) return;
+    const float q = wgt * r.g;
+    if (du <= dv) {
+        const float sq = u >= 0.f ? q : -q;
+        acc[0] = fmaf(sq, r.ch, acc[0]);
+        acc[1] = fmaf(sq, r.sh, acc[1]);
+        acc[2] = fmaf(-sq, v, acc[2]);
+        acc[3] += q;
+    } else {
+        const float sq = v >= 0.f ? q : -q;
+        acc[0] = fmaf(-sq, r.sh, acc[0]);
+        acc[1] = fmaf(sq, r.ch, acc[1]);
+        acc[2] = fmaf(sq, u, acc[2]);
+        acc[4] += q;
     }
-    const float rs = rsqrtf(delta);
-    const float sq = delta * rs;
+}
+
+// Constants of one ellipsoid's gradients.
+struct EllipseGrad {
+    float cia, sia, cib, sib;  // c / a, s / a, c / b, s / b
+    float sa, inv_sa;          // sqrt(alpha), 1 / sqrt(alpha)
+    float ratio;               // a / b - b / a
+};
+__device__ __forceinline__ EllipseGrad ellipse_grad(const PRec &r, float inv_alpha) {
+    EllipseGrad e;
+    e.cia = r.ch * r.p0h;
+    e.sia = r.sh * r.p0h;
+    e.cib = r.ch * r.p1h;
+    e.sib = r.sh * r.p1h;
+    e.sa = rsqrtf(inv_alpha);
+    e.inv_sa = inv_alpha * e.sa;
+    e.ratio = r.p1h / r.p0h - r.p0h / r.p1h;
+    return e;
+}
+__device__ __forceinline__ void ellipse_pixel_grad(const PRec &r, const EllipseGrad &e, float qq,
+                                                   float ex, float ey, float go, float ga,
+                                                   float acc[8]) {
+    const float wgt = fmaf(r.dn, go, r.mu * ga);
+    const float ua = fmaf(e.cia, ex, e.sia * ey);
+    const float vb = fmaf(-e.sib, ex, e.cib * ey);
+    const float rq = rsqrtf(qq);
+    const float sq = qq * rq * e.sa;  // sqrt(delta)
     const float t = r.T * sq;
     acc[6] = fmaf(go, t, acc[6]);
     acc[7] = fmaf(ga, t, acc[7]);
     acc[5] = fmaf(wgt, sq, acc[5]);
-    const float q = wgt * r.T * rs;  // 2 * wgt * dt/ddelta
-    acc[0] = fmaf(q, fmaf(ua, cia, -vb * sib), acc[0]);
-    acc[1] = fmaf(q, fmaf(ua, sia, vb * cib), acc[1]);
-    acc[2] = fmaf(q * ua * vb, r.p1h / r.p0h - r.p0h / r.p1h, acc[2]);
+    const float q = wgt * r.T * (rq * e.inv_sa);  // 2 wgt dt/ddelta
+    acc[0] = fmaf(q, fmaf(ua, e.cia, -vb * e.sib), acc[0]);
+    acc[1] = fmaf(q, fmaf(ua, e.sia, vb * e.cib), acc[1]);
+    acc[2] = fmaf(q * ua * vb, e.ratio, acc[2]);
     acc[3] = fmaf(q * ua * ua, r.p0h, acc[3]);
     acc[4] = fmaf(q * vb * vb, r.p1h, acc[4]);
 }
