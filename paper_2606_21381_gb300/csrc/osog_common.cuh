@@ -20,6 +20,8 @@ namespace osog {
 constexpr int kMaxSetElems = 8192;
 constexpr int kSetLines = 4;
 constexpr int kThreads = 512;          // threads of every FFT-bearing CTA
+constexpr int kWideThreads = 1024;     // of a strip CTA that has an SM to itself
+constexpr int kSms = 152;              // GB300
 __host__ __device__ constexpr int set_elems(int n) {
     return n >= 1024 ? kMaxSetElems : kSetLines * n < kThreads ? kThreads : kSetLines * n;
 }

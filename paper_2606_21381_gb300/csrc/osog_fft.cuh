@@ -146,6 +146,19 @@ __device__ __forceinline__ void line_sync(int l) {
     }
 }
 
+// How the threads of a pass synchronise: the whole CTA, the group of a line
+// (line_sync), or the first kThreads threads of a larger CTA.
+enum FftSync { kSyncCta = 0, kSyncLine = 1, kSyncThreads = 2 };
+template <int G, int L>
+__device__ __forceinline__ void pass_sync(int l) {
+    if constexpr (G == kSyncLine)
+        line_sync<L>(l);
+    else if constexpr (G == kSyncThreads)
+        asm volatile("bar.sync 15, %0;" ::"n"(kThreads) : "memory");
+    else
+        __syncthreads();
+}
+
 // True when the passes of an N-point transform can run with one thread
 // group per line: every pass has at least one butterfly per thread of the
 // group (sets of 8192 samples, N >= 1024).
@@ -156,9 +169,9 @@ __host__ __device__ constexpr bool fft_grouped(int n) {
 // Butterfly q of this thread in a pass of NB butterflies per line over L
 // lines: grouped, the threads [l TPL, (l + 1) TPL) take line l; otherwise
 // consecutive threads take consecutive butterflies of the whole set.
-template <int L, int NB, bool G>
+template <int L, int NB, bool LINE>
 __device__ __forceinline__ void butterfly_of(int q, int &l, int &j) {
-    if constexpr (G) {
+    if constexpr (LINE) {
         constexpr int TPL = kThreads / L;
         l = threadIdx.x / TPL;
         j = threadIdx.x % TPL + q * TPL;
@@ -218,21 +231,21 @@ __device__ __forceinline__ void apply_twiddles(float2 *v, const float2 *__restri
 
 // One Stockham pass over L lines of N points.  G: one thread group per line
 // (fft_grouped(N)); the pass then synchronises only the line's group.
-template <int N, int L, int P, int NS, bool INV, bool G = false>
+template <int N, int L, int P, int NS, bool INV, int G = kSyncCta>
 __device__ __forceinline__ void stockham_pass(float2 *buf, const float2 *__restrict__ tw) {
     static_assert(NS == 1 || NS == 8 || NS % 16 == 0, "unsupported Stockham stride");
     constexpr int NB = N / P;
     constexpr int TOT = L * NB;
     constexpr int PER = (TOT + kThreads - 1) / kThreads;
     constexpr int LS = line_stride(N);
-    static_assert(!G || (NB % (kThreads / L) == 0 && kThreads % L == 0), "grouped pass");
+    static_assert(G != kSyncLine || (NB % (kThreads / L) == 0 && kThreads % L == 0), "grouped pass");
     float2 v[PER][P];
     int l = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G>(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             if constexpr (NB % 16 == 0) {
                 const float2 *src = buf + l * LS + pad16(j);
 #pragma unroll
@@ -244,12 +257,12 @@ __device__ __forceinline__ void stockham_pass(float2 *buf, const float2 *__restr
             }
         }
     }
-    if constexpr (G) line_sync<L>(l); else __syncthreads();
+    pass_sync<G, L>(l);
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G>(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             const int k = j & (NS - 1);
             if constexpr (NS > 1) apply_twiddles<P, INV, NS>(v[q], tw + k);  // entries [r - 1][k]
             dft<P, INV>(v[q]);
@@ -258,24 +271,24 @@ __device__ __forceinline__ void stockham_pass(float2 *buf, const float2 *__restr
             for (int r = 0; r < P; ++r) dst[stride_off(NS, r)] = v[q][r];
         }
     }
-    if constexpr (G) line_sync<L>(l); else __syncthreads();
+    pass_sync<G, L>(l);
 }
 
 // Full FFT of the L lines (forward: exp(-2 pi i jk/N); inverse: conjugate,
 // unnormalised), following the radix plan above.  tw is the N-point
 // transform's table block.
-template <int N, int L, bool INV, int PASS = 0>
+template <int N, int L, bool INV, int G = kSyncCta, int PASS = 0>
 __device__ __forceinline__ void fft_lines(float2 *buf, const float2 *__restrict__ tw) {
     if constexpr (PASS < fft_passes(N)) {
-        stockham_pass<N, L, fft_radix(N, PASS), fft_ns(N, PASS), INV>(buf,
-                                                                      tw + fft_twoff(N, PASS));
-        fft_lines<N, L, INV, PASS + 1>(buf, tw);
+        stockham_pass<N, L, fft_radix(N, PASS), fft_ns(N, PASS), INV, G>(buf,
+                                                                         tw + fft_twoff(N, PASS));
+        fft_lines<N, L, INV, G, PASS + 1>(buf, tw);
     }
 }
 
 // Passes [PASS, END) of the radix plan, each an in-place Stockham pass
 // (G: grouped, see stockham_pass).
-template <int N, int L, bool INV, int PASS, int END, bool G = false>
+template <int N, int L, bool INV, int PASS, int END, int G = kSyncCta>
 __device__ __forceinline__ void fft_pass_range(float2 *buf, const float2 *__restrict__ tw) {
     if constexpr (PASS < END) {
         stockham_pass<N, L, fft_radix(N, PASS), fft_ns(N, PASS), INV, G>(buf,
@@ -292,40 +305,40 @@ __device__ __forceinline__ void fft_pass_range(float2 *buf, const float2 *__rest
 // IN_PLACE: ld reads buf itself, and the threads synchronise between the
 // loads and the writes.  G: grouped (see stockham_pass); ld(l, i) may then
 // read only line l of buf.  Ends with a barrier (the line's, grouped).
-template <int N, int L, bool INV, bool IN_PLACE, bool G, class Ld>
+template <int N, int L, bool INV, bool IN_PLACE, int G, class Ld>
 __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
     constexpr int P = fft_radix(N, 0);
     constexpr int NB = N / P;
     constexpr int TOT = L * NB;
     constexpr int PER = (TOT + kThreads - 1) / kThreads;
     constexpr int LS = line_stride(N);
-    static_assert(!G || (NB % (kThreads / L) == 0 && kThreads % L == 0), "grouped pass");
+    static_assert(G != kSyncLine || (NB % (kThreads / L) == 0 && kThreads % L == 0), "grouped pass");
     float2 v[PER][P];
     int l = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G>(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
 #pragma unroll
             for (int r = 0; r < P; ++r) v[q][r] = ld(l, j + r * NB);
         }
     }
     if constexpr (IN_PLACE) {
-        if constexpr (G) line_sync<L>(l); else __syncthreads();
+        pass_sync<G, L>(l);
     }
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G>(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             dft<P, INV>(v[q]);
             float2 *dst = buf + l * LS + pad16(j * P);
 #pragma unroll
             for (int r = 0; r < P; ++r) dst[r] = v[q][r];
         }
     }
-    if constexpr (G) line_sync<L>(l); else __syncthreads();
+    pass_sync<G, L>(l);
 }
 
 // The last pass of the plan with its outputs handed to st(l, i, value),
@@ -335,13 +348,13 @@ __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
 // block, interleaved in global memory; the pass before must end with a CTA
 // barrier); G: grouped (see stockham_pass); else consecutive butterflies of
 // the whole set.  buf is only read, so there is no barrier.
-template <int N, int L, bool INV, bool LINE_FAST, bool G, class St>
+template <int N, int L, bool INV, bool LINE_FAST, int G, class St>
 __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *__restrict__ tw,
                                               St st) {
     constexpr int PASS = fft_passes(N) - 1;
     constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS);
     static_assert(NS * P == N && NS > 1, "the last pass of the plan");
-    static_assert(!(LINE_FAST && G), "one thread mapping");
+    static_assert(!(LINE_FAST && G == kSyncLine), "one thread mapping");
     constexpr int NB = N / P;
     constexpr int TOT = L * NB;
     constexpr int PER = (TOT + kThreads - 1) / kThreads;
@@ -354,14 +367,14 @@ __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *_
             l = b % L;
             j = b / L;
         } else {
-            butterfly_of<L, NB, G>(q, l, j);
+            butterfly_of<L, NB, G == kSyncLine>(q, l, j);
         }
     };
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int l, j;
         which(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             if constexpr (NB % 16 == 0) {
                 const float2 *src = buf + l * LS + pad16(j);
 #pragma unroll
@@ -377,7 +390,7 @@ __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *_
     for (int q = 0; q < PER; ++q) {
         int l, j;
         which(q, l, j);
-        if (G || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             apply_twiddles<P, INV, NS>(v[q], t + j);
             dft<P, INV>(v[q]);
 #pragma unroll

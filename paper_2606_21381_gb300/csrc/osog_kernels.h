@@ -249,7 +249,6 @@ size_t persistent_smem(int N, int K);
 cudaError_t launch_persistent(const PersistArgs &a, cudaStream_t st);
 
 size_t bwd_column_smem(int H);
-size_t bwd_strip_smem(int W);
 cudaError_t prepare_backward(int H, int W);
 cudaError_t launch_bwd_rows(const BwdRowsArgs &a, cudaStream_t st);
 cudaError_t launch_bwd_column(const BwdColumnArgs &a, cudaStream_t st);

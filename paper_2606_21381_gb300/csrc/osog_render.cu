@@ -27,8 +27,9 @@ namespace {
 // line (named barriers) instead of CTA-wide barriers.
 constexpr bool kGroupFft = true;
 
-// One strip (rows [strip R, strip R + R)) of scene s.
-template <int N, int MODE, bool SQ = false>
+// One strip (rows [strip R, strip R + R)) of scene s.  NT: threads of the CTA;
+// those past kThreads only rasterise.
+template <int N, int MODE, bool SQ = false, int NT = kThreads>
 __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, int strip,
                                                    unsigned char *smem_raw) {
     constexpr int L = set_elems(N) / N;
@@ -83,16 +84,18 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
     } else {
         float4 *b4 = reinterpret_cast<float4 *>(buf);
         const int n4 = (ACC == kAccOpd ? 2 : 1) * R * LS / 2;
-        for (int i = threadIdx.x; i < n4; i += kThreads) b4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = threadIdx.x; i < n4; i += NT) b4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
-        raster_strip<N, ACC>(a.geo, a.w, a.sc[s], s, y0, R, smem_raw, scratch);
+        raster_strip<N, ACC, NT>(a.geo, a.w, a.sc[s], s, y0, R, smem_raw, scratch);
+        // (ends with a CTA barrier; later ones count the threads that are left)
+        if (NT > kThreads && threadIdx.x >= kThreads) return;
     }
     __syncthreads();
     if constexpr (MODE == kStripRender) {
         // the exit wave of the accumulated words is formed as the first FFT
         // pass loads them, and the last pass stores G (column-blocked, only
         // the columns some pupil passes)
-        constexpr bool GRP = kGroupFft && fft_grouped(N);
+        constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
         fft_first_pass<N, L, false, true, GRP>(buf, [&](int l, int x) -> float2 {
             return l < R ? exit_wave_fixed(*reinterpret_cast<const uint2 *>(buf + l * LS + pad16(x)))
                          : make_float2(0.f, 0.f);
@@ -188,11 +191,16 @@ __global__ void __launch_bounds__(kRThreads, 4) k_raster_tiles(const __grid_cons
         dst[(size_t)(i >> lw) * (geo.W / 2) + (i & (TW / 2 - 1))] = a4[i];
 }
 
-template <int N, int MODE, bool SQ>
-__global__ void __launch_bounds__(kThreads, 2) k_strip_forward(const __grid_constant__ StripArgs a) {
+// WIDE: 1024 threads rasterise the strip, for launches of at most one CTA per
+// SM, where 16 warps leave the raster waiting for its loads and shuffles (two
+// CTAs of 512 threads share an SM otherwise): one dense 1024 x 1024 image 23.5 ->
+// 20.2 us, 512 x 1024 with 1,501 particles 15.0 -> 11.7 us.
+template <int N, int MODE, bool SQ, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? kWideThreads : kThreads, WIDE ? 1 : 2)
+k_strip_forward(const __grid_constant__ StripArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_enter();
-    strip_forward_item<N, MODE, SQ>(a, blockIdx.y, blockIdx.x, smem_raw);
+    strip_forward_item<N, MODE, SQ, WIDE ? kWideThreads : kThreads>(a, blockIdx.y, blockIdx.x, smem_raw);
 }
 
 // The image losses of inverse rendering on one column block of image s
@@ -362,7 +370,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
     static_assert(!BULK || (SQ && N >= 1024), "bulk staging needs full column blocks");
     __shared__ uint64_t bar;  // completes the bulk copy (BULK)
     const bool bulk = BULK && !a.unit_input;
-    constexpr bool GRP = kGroupFft && fft_grouped(N);
+    constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
     if (bulk) {
         if constexpr (BULK)
             if (threadIdx.x == 0)
@@ -403,7 +411,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
             bulk_wait(&bar, a.w.status, a.wait_polls);
             first_pass_from_block<N, false>(buf0, live);
             fft_pass_range<N, L, false, 1, fft_passes(N), GRP>(buf0, a.tw);
-            if constexpr (GRP) __syncthreads();  // every line done before any thread reads another's
+            if constexpr (GRP == kSyncLine) __syncthreads();  // every line done before any thread reads another's
         }
     } else if (!a.unit_input) {
         fft_lines<N, L, false>(buf0, a.tw);
@@ -459,7 +467,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
             fft_pass_range<N, L, true, 0, 1>(buf1, a.tw);
         }
         fft_pass_range<N, L, true, 1, fft_passes(N) - 1, GRP>(buf1, a.tw);
-        if constexpr (GRP) __syncthreads();
+        if constexpr (GRP == kSyncLine) __syncthreads();
         // the last pass stores Q; consecutive threads take the block's
         // columns, so a warp writes whole rows of the block
         fft_last_pass<N, L, true, true, false>(buf1, a.tw, [&](int c, int y, float2 v) {
@@ -493,7 +501,7 @@ __device__ __forceinline__ void inverse_item(const InverseArgs &a, int sm, int s
     // the first pass reads the strip's rows of Q straight from global memory
     // (columns that no pupil passes, and lines past the strip, read as zero);
     // the last pass writes the intensity rows
-    constexpr bool GRP = kGroupFft && fft_grouped(N);
+    constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
     fft_first_pass<N, L, true, false, GRP>(buf, [&](int l, int kx) -> float2 {
         const int fx = kx < N / 2 ? kx : kx - N;
         return l < R && fx >= cr.x && fx <= cr.y
@@ -639,7 +647,13 @@ struct StripFwdLaunch {
         dim3 grid(a.geo.nstrips, a.S);
         const size_t smem = strip_forward_smem(N), smem_opd = strip_forward_smem(N, true);
         const size_t smem_fft = strip_inverse_smem(N);  // the set alone: no raster
-        if (mode == kStripRender && a.geo.H == a.geo.W)
+        const bool wide = (int)(grid.x * grid.y) <= kSms;
+        const size_t smem_wide = strip_forward_smem(N) + raster_smem<kWideThreads>() - raster_smem<kThreads>();
+        if (mode == kStripRender && wide && a.geo.H == a.geo.W)
+            return launch_chain(k_strip_forward<N, kStripRender, true, true>, grid, kWideThreads, smem_wide, st, a);
+        else if (mode == kStripRender && wide)
+            return launch_chain(k_strip_forward<N, kStripRender, false, true>, grid, kWideThreads, smem_wide, st, a);
+        else if (mode == kStripRender && a.geo.H == a.geo.W)
             return launch_chain(k_strip_forward<N, kStripRender, true>, grid, kThreads, smem, st, a);
         else if (mode == kStripRender)
             return launch_chain(k_strip_forward<N, kStripRender, false>, grid, kThreads, smem, st, a);
@@ -670,6 +684,11 @@ struct StripFwdLaunch {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripFromReal, false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const int smem_wide = smem + (int)(raster_smem<kWideThreads>() - raster_smem<kThreads>());
+        for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
+            e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripRender, true, true>
+                                        : k_strip_forward<N, kStripRender, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem_wide);
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
             e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripFromPhase, true>
                                         : k_strip_forward<N, kStripFromPhase, false>,

@@ -428,7 +428,7 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
 
 // The strip [y0, y0 + R) of scene s rasterised into the padded FFT lines of
 // an N-point set (the adjoint's re-raster; osog_render_opd in OPD mode).
-template <int N, int ACC>
+template <int N, int ACC, int NT = kThreads>
 __device__ void raster_strip(const Geometry &geo, const Work &w, const SceneDev &sc, int s,
                              int y0, int R, void *acc, unsigned char *scratch) {
     constexpr int LS = line_stride(N);
@@ -441,7 +441,7 @@ __device__ void raster_strip(const Geometry &geo, const Work &w, const SceneDev 
     auto slot = [base](int row, int x) -> uint32_t {
         return base + (uint32_t)(row * LS + pad16(x)) * (ACC == kAccPhase ? 8u : 16u);
     };
-    raster_region<kThreads, ACC>(w, w.pairs + sc.pair0, w.pair_rect ? w.pair_rect + sc.pair0 : nullptr,
+    raster_region<NT, ACC>(w, w.pairs + sc.pair0, w.pair_rect ? w.pair_rect + sc.pair0 : nullptr,
                                  lo, hi, y0, R, 0, geo.W - 1, 0.5f * sc.two_over_lambda, slot,
                                  scratch);
 }
