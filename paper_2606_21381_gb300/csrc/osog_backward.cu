@@ -54,37 +54,51 @@ __device__ __forceinline__ float warp_sum8(float (&v)[8], int lane) {
     return s + __shfl_xor_sync(kFull, s, 1);
 }
 
+// The thread groups of the passes (see fft_grouped).
 template <int N>
-__global__ void __launch_bounds__(kThreads, 1) k_bwd_rows(const __grid_constant__ BwdRowsArgs a) {
+constexpr int kGroup = fft_grouped(N) ? kSyncLine : kSyncCta;
+
+// Rows: the inverse transform's first pass takes Q from global memory and its
+// last hands 2 gI E to a second set, whose forward transform stores the result
+// over Q from its last pass.
+template <int N>
+__global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant__ BwdRowsArgs a) {
     pdl_enter();
-    constexpr int L = set_elems(N) / N;
-    constexpr int LS = line_stride(N);
+    constexpr int L = set_elems(N) / N, LS = line_stride(N), G = kGroup<N>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *buf = reinterpret_cast<float2 *>(smem_raw);
+    float2 *bufE = reinterpret_cast<float2 *>(smem_raw), *bufQ = bufE + L * LS;
     const Geometry &geo = a.geo;
-    const int sm = blockIdx.y, K = a.K;
-    const int y0 = blockIdx.x * geo.R;
-    const int RN = geo.R * N;
-    float2 *Qm = a.w.Q + (size_t)sm * geo.nblocks * geo.H * geo.B;
+    const int sm = blockIdx.y, K = a.K, R = geo.R, B = geo.B, lb = ilog2(B), H = geo.H;
+    const int y0 = blockIdx.x * R;
+    float2 *Qm = a.w.Q + (size_t)sm * geo.nblocks * H * B;
     const int2 cr = a.w.hull[sm / K];
-    load_strip_blocked<N>(buf, Qm, geo, y0, cr);
-    __syncthreads();
-    fft_lines<N, L, true>(buf, a.tw);  // E_m rows
-    const float *gI = a.grad_image + ((size_t)sm * geo.H + y0) * N;
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        if (e < RN) {
-            float2 *v = buf + (e / N) * LS + pad16(e % N);
-            const float g2 = 2.f * gI[e];
-            *v = make_float2(g2 * v->x, g2 * v->y);
-        }
-    }
-    __syncthreads();
-    fft_lines<N, L, false>(buf, a.tw);  // adjoint of the inverse row DFT
-    store_strip_blocked<N>(buf, Qm, geo, y0, cr);
+    fft_first_pass<N, L, true, false, G>(bufE, [&](int l, int kx) -> float2 {
+        const int fx = kx < N / 2 ? kx : kx - N;
+        return l < R && fx >= cr.x && fx <= cr.y
+                   ? Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))]
+                   : make_float2(0.f, 0.f);
+    });
+    fft_pass_range<N, L, true, 1, fft_passes(N) - 1, G>(bufE, a.tw);  // E_m rows
+    const float *gI = a.grad_image + ((size_t)sm * H + y0) * N;
+    fft_last_pass<N, L, true, false, G>(bufE, a.tw, [&](int l, int x, float2 v) {
+        const float g2 = l < R ? 2.f * gI[(size_t)l * N + x] : 0.f;
+        bufQ[l * LS + pad16(x)] = make_float2(g2 * v.x, g2 * v.y);
+    });
+    if constexpr (G == kSyncLine)
+        line_sync<L>(threadIdx.x / (kThreads / L));
+    else
+        __syncthreads();
+    // adjoint of the inverse row DFT
+    fft_pass_range<N, L, false, 0, fft_passes(N) - 1, G>(bufQ, a.tw);
+    fft_last_pass<N, L, false, false, G>(bufQ, a.tw, [&](int l, int kx, float2 v) {
+        const int fx = kx < N / 2 ? kx : kx - N;
+        if (l < R && fx >= cr.x && fx <= cr.y)
+            Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))] = v;
+    });
 }
 
+// Columns: the last pass of each modality's transform hands dL/dZ_m to the
+// accumulation in registers, and the last of the inverse one stores over G.
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constant__ BwdColumnArgs a) {
     pdl_enter();
@@ -108,56 +122,60 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
     }
     float2 *Gb = a.w.G + ((size_t)s * geo.nblocks + bk) * N * B;
     load_block<N>(bufE, Gb, geo, bk, cr);
+    load_block<N>(bufZ, a.w.Q + (((size_t)s * K) * geo.nblocks + bk) * N * B, geo, bk, cr);
     for (int j = threadIdx.x; j < K * B; j += kThreads) {  // this block's chords
         const int m = j >> lb, c = j & (B - 1), kx = bk * B + c;
         chords[m * L + c] = mode_chord(a.md[s][m], kx < half ? kx : kx - geo.W, N);
     }
     __syncthreads();
     fft_lines<N, L, false>(bufE, a.tw);  // E^ of the block's columns
-    float2 acc[ept(N)];
+    constexpr int OUT = fft_last_outputs<N, L>();
+    float2 acc[OUT];
 #pragma unroll
-    for (int i = 0; i < ept(N); ++i) acc[i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < OUT; ++i) acc[i] = make_float2(0.f, 0.f);
     float po[4] = {0.f, 0.f, 0.f, 0.f};
     for (int m = 0; m < K; ++m) {
         const ModeDev md = live_mode(a.md[s][m]);
-        const float2 *Qb = a.w.Q + (((size_t)s * K + m) * geo.nblocks + bk) * N * B;
-        load_block<N>(bufZ, Qb, geo, bk, cr);
-        __syncthreads();
-        fft_lines<N, L, false>(bufZ, a.tw);  // dL/dZ_m (adjoint of the inverse column DFT)
-#pragma unroll 4
-        for (int i = 0; i < ept(N); ++i) {
-            const int e = threadIdx.x + i * kThreads;  // line-major: consecutive rows
-            const int c = e / N, y = e % N;
-            if (c < B) {
-                const int kx = bk * B + c;
-                const int fx = kx < half ? kx : kx - geo.W;
-                const int fy = y < N / 2 ? y : y - N;
-                const int2 ch = chords[m * L + c];
-                if (fy >= ch.x && fy <= ch.y) {
-                    float2 h, dh[4];
-                    transfer_grad(md, fx, fy, h, dh);
-                    const float2 gz = bufZ[c * LS + pad16(y)];
-                    const float2 eh = bufE[c * LS + pad16(y)];
-                    acc[i] = cadd(acc[i], cmulc(gz, h));  // conj(H) dL/dZ
+        if (m > 0) {
+            __syncthreads();  // the modality before has read bufZ
+            load_block<N>(bufZ, a.w.Q + (((size_t)s * K + m) * geo.nblocks + bk) * N * B, geo, bk, cr);
+            __syncthreads();
+        }
+        // dL/dZ_m (adjoint of the inverse column DFT)
+        fft_pass_range<N, L, false, 0, fft_passes(N) - 1>(bufZ, a.tw);
+        fft_last_pass<N, L, false, false, kSyncCta>(bufZ, a.tw, [&](int c, int y, float2 gz, int i) {
+            if (c >= B) return;
+            const int kx = bk * B + c;
+            const int fx = kx < half ? kx : kx - geo.W;
+            const int fy = y < N / 2 ? y : y - N;
+            const int2 ch = chords[m * L + c];
+            if (fy >= ch.x && fy <= ch.y) {
+                float2 h, dh[4];
+                transfer_grad(md, fx, fy, h, dh);
+                const float2 eh = bufE[c * LS + pad16(y)];
+                acc[i] = cadd(acc[i], cmulc(gz, h));  // conj(H) dL/dZ
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float2 w = cmul(eh, dh[k]);
-                        po[k] = fmaf(gz.x, w.x, fmaf(gz.y, w.y, po[k]));
-                    }
+                for (int k = 0; k < 4; ++k) {
+                    const float2 w = cmul(eh, dh[k]);
+                    po[k] = fmaf(gz.x, w.x, fmaf(gz.y, w.y, po[k]));
                 }
             }
-        }
-        __syncthreads();
+        });
     }
+    // acc to bufE (read by its own outputs' threads only), in the same places
+    constexpr int P = fft_radix(N, fft_passes(N) - 1), NBF = N / P;
 #pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        const int c = e / N, y = e % N;
-        if (c < B) bufZ[c * LS + pad16(y)] = acc[i];
+    for (int i = 0; i < OUT; ++i) {
+        int l, j;
+        butterfly_of<L, NBF, false>(i / P, l, j);
+        if (l < B) bufE[l * LS + pad16(j + (i % P) * NBF)] = acc[i];
     }
     __syncthreads();
-    fft_lines<N, L, true>(bufZ, a.tw);  // dL/dG (adjoint of the forward column DFT)
-    store_block<N>(bufZ, Gb, geo);
+    // dL/dG (adjoint of the forward column DFT)
+    fft_pass_range<N, L, true, 0, fft_passes(N) - 1>(bufE, a.tw);
+    fft_last_pass<N, L, true, true, kSyncCta>(bufE, a.tw, [&](int c, int y, float2 v) {
+        if (c < B) Gb[(size_t)y * B + c] = v;
+    });
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float v = warp_sum(po[k]);
@@ -384,7 +402,7 @@ template <int N>
 struct BwdLaunch {
     static cudaError_t rows(const BwdRowsArgs &a, cudaStream_t st) {
         return launch_chain(k_bwd_rows<N>, dim3(a.geo.nstrips, a.S * a.K), kThreads,
-                            strip_inverse_smem(N), st, a);
+                            2 * strip_inverse_smem(N), st, a);
     }
     static cudaError_t column(const BwdColumnArgs &a, cudaStream_t st) {
         return launch_chain(k_bwd_column<N>, dim3(a.geo.nblocks, a.S), kThreads, bwd_column_smem(N),
@@ -401,7 +419,7 @@ struct BwdLaunch {
     static cudaError_t prepare(int which) {
         if (which == 0)
             return cudaFuncSetAttribute(k_bwd_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)strip_inverse_smem(N));
+                                        2 * (int)strip_inverse_smem(N));
         if (which == 1)
             return cudaFuncSetAttribute(k_bwd_column<N>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -24,6 +24,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "osog_common.cuh"
 
 namespace osog {
@@ -347,7 +349,14 @@ __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
 // consecutive threads take consecutive lines (the columns of a column
 // block, interleaved in global memory; the pass before must end with a CTA
 // barrier); G: grouped (see stockham_pass); else consecutive butterflies of
-// the whole set.  buf is only read, so there is no barrier.
+// the whole set.  buf is only read, so there is no barrier.  st may take a
+// fourth argument, the number of the output among the thread's own (a constant
+// once the loops are unrolled; fft_last_outputs of them).
+template <int N, int L>
+__host__ __device__ constexpr int fft_last_outputs() {
+    constexpr int P = fft_radix(N, fft_passes(N) - 1);
+    return (L * (N / P) + kThreads - 1) / kThreads * P;
+}
 template <int N, int L, bool INV, bool LINE_FAST, int G, class St>
 __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *__restrict__ tw,
                                               St st) {
@@ -394,7 +403,12 @@ __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *_
             apply_twiddles<P, INV, NS>(v[q], t + j);
             dft<P, INV>(v[q]);
 #pragma unroll
-            for (int r = 0; r < P; ++r) st(l, j + r * NS, v[q][r]);
+            for (int r = 0; r < P; ++r) {
+                if constexpr (std::is_invocable_v<St, int, int, float2, int>)
+                    st(l, j + r * NS, v[q][r], q * P + r);
+                else
+                    st(l, j + r * NS, v[q][r]);
+            }
         }
     }
 }

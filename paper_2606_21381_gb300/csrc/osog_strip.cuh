@@ -505,9 +505,8 @@ __device__ __forceinline__ float2 transfer(const ModeDev &md, int fx, int fy) {
 
 // ---------------------------------------------------------------- layouts
 // A row-strip [y0, y0 + R) of a column-blocked array [W/B][H][B] (complex)
-// to and from the padded shared lines of an N = W point set.  Columns whose
-// signed frequency lies outside [cr.x, cr.y] (no pupil passes them) are
-// neither read (zero-filled) nor written.
+// to the padded shared lines of an N = W point set.  Columns whose signed
+// frequency lies outside [cr.x, cr.y] (no pupil passes them) load as zero.
 template <int N, bool SQ = false>
 __device__ __forceinline__ void load_strip_blocked(float2 *buf, const float2 *src,
                                                    const Geometry &geo, int y0, int2 cr) {
@@ -532,25 +531,8 @@ __device__ __forceinline__ void load_strip_blocked(float2 *buf, const float2 *sr
     }
 }
 
-template <int N, bool SQ = false>
-__device__ __forceinline__ void store_strip_blocked(const float2 *buf, float2 *dst,
-                                                    const Geometry &geo, int y0, int2 cr) {
-    constexpr int LS = line_stride(N);
-    const int R = SQ ? sq_rb(N) : geo.R, B = SQ ? sq_rb(N) : geo.B;
-    const int lb = SQ ? clog2(sq_rb(N)) : ilog2(B), lr = SQ ? clog2(sq_rb(N)) : ilog2(R);
-    const int RN = R * N, H = SQ ? N : geo.H;
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        const int c = e & (B - 1), r = (e >> lb) & (R - 1), bk = e >> (lb + lr);
-        const int kx = bk * B + c, fx = kx < N / 2 ? kx : kx - N;
-        if (e < RN && fx >= cr.x && fx <= cr.y)
-            dst[((size_t)bk * H + y0 + r) * B + c] = buf[r * LS + pad16(kx)];
-    }
-}
-
-// A column block (B columns, N = H rows, contiguous [H][B]) to and from the
-// padded shared lines (line c = column c).  Inactive columns load as zero.
+// A column block (B columns, N = H rows, contiguous [H][B]) to the padded
+// shared lines (line c = column c).  Inactive columns load as zero.
 template <int N>
 __device__ __forceinline__ void load_block(float2 *buf, const float2 *src, const Geometry &geo,
                                            int bk, int2 cr) {
@@ -567,17 +549,6 @@ __device__ __forceinline__ void load_block(float2 *buf, const float2 *src, const
     for (int i = 0; i < ept(N); ++i) {
         const int e = threadIdx.x + i * kThreads;
         if (e < NB) buf[(e & (B - 1)) * LS + pad16(e >> lb)] = v[i];
-    }
-}
-
-template <int N>
-__device__ __forceinline__ void store_block(const float2 *buf, float2 *dst, const Geometry &geo) {
-    constexpr int LS = line_stride(N);
-    const int B = geo.B, lb = ilog2(B), NB = N * B;
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        if (e < NB) dst[e] = buf[(e & (B - 1)) * LS + pad16(e >> lb)];
     }
 }
 
