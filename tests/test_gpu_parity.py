@@ -304,3 +304,22 @@ def test_single_chunk_binning_equals_the_three_passes():
                    tuning={"use_graph": 0}).clone()
     assert r.sync_status() == 0
     assert torch.equal(alone, both[0])
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+def test_row_spans_end_at_the_last_covered_pixel_centre(kind):
+    # chord ends a hair inside and outside pixel centres (by 2^-4 to 2^-18 px, at
+    # turns of 0 and pi / 2), then edges nearly along the rows and columns: the
+    # spans hold every covered centre and no other contributes
+    rows = []
+    for i in range(16):
+        cx, cy = 12.5 + 30.0 * (i % 8), 20.5 + 60.0 * (i // 8)
+        eps = (1.0 if i % 2 else -1.0) * 2.0 ** -(4 + i % 15)
+        rows.append((cx, cy, 0.0 if i < 8 else math.pi / 2, 7.0 + eps, 9.0 - eps))
+    for i, tilt in enumerate([0.9e-6, 1.1e-6, 3e-6, 1e-5, 1e-4, 1e-3, 1e-2, -1e-5]):
+        rows.append((13.0 + 30.0 * i, 140.25, tilt, 8.0, 11.0))
+        rows.append((13.5 + 30.0 * i, 200.5, math.pi / 2 + tilt, 9.0, 7.5))
+    soa = np.zeros((9, len(rows)), dtype=np.float32)
+    soa[:5] = np.array(rows).T
+    soa[5], soa[6], soa[7], soa[8] = 2.0, 0.04, 0.02, kind
+    assert_opd_close(soa, scenes.optics(256, 256))
