@@ -49,7 +49,7 @@ struct __align__(16) RowItem {
     float f[8];     // ellipsoid: left and right chord ends (hi, lo each), T sqrt(alpha)
                     // prism: cx, g s ey, g c ey, g cos, g sin, g hx, g hy, T
                     // polyhedron: cx, ey, plane offset, plane count (int bits)
-    int32_t row;    // row in the rasterised region
+    int32_t row;    // row in the rasterised region (bits 0-15), number of its first chunk (16-31)
     float dn;       // kAccPhase: dn / lambda (cycles per um); kAccOpd: dn
     float mu;       // kAccPhase: mu in units of 2^-20 per um; kAccOpd: mu
 };
@@ -262,18 +262,17 @@ __device__ __forceinline__ int warp_incl_scan(int v) {
     return v;
 }
 
-// The lane whose range of a warp prefix holds key: the number of lanes whose
-// inclusive prefix (field (inc >> sh) & mask, non-decreasing over the lanes)
-// is at most key.  Every lane of the warp takes part; the result is at most
-// 31, and it is the owning lane whenever key is below lane 31's prefix.
-__device__ __forceinline__ int warp_owner(int inc, int key, int sh, int mask) {
-    int e = 0;
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        const int t = (__shfl_sync(kFull, inc, e + s - 1) >> sh) & mask;
-        if (t <= key) e += s;
-    }
-    return e;
+// Lanes' ranges laid end to end (first the start of a lane's own, ascending over
+// the ranges; INT32_MAX for none), read 32 at a time: the number of the range that
+// holds position at + lane, for at ascending by 32 with `before` (0 at the start)
+// the ranges that start below it.  A reduction and a population count, against
+// five dependent shuffles of a search over the lanes.
+__device__ __forceinline__ int range_of(int first, int at, int &before) {
+    const unsigned d = (unsigned)(first - at);
+    const unsigned starts = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
+    const int r = before + __popc(starts & (2u * lanemask_lt() + 1u)) - 1;
+    before += __popc(starts);
+    return r;
 }
 
 // Pixels of one chunk of a row item.
@@ -299,8 +298,8 @@ __host__ __device__ constexpr size_t raster_smem() {
 //      ellipsoids first, the region rows each covers, and a warp prefix sum
 //      of those row counts;
 //   2. waves of 32 (particle, row) items, one per lane (the owning entry
-//      found by a search over the prefix), built from the particle's
-//      row-span constants into the warp's item slots;
+//      found by range_of), built from the particle's row-span constants into
+//      the warp's item slots;
 //   3. the wave's pixels cut into chunks of up to kChunkPx, ellipsoid items'
 //      chunks first so that most passes run one chord formula; lane l of a
 //      pass takes chunk l and evaluates its pixels as independent unrolled
@@ -322,6 +321,7 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
     const int gsz = min(32, max(1, (hi - lo + NW - 1) / NW));
     if (threadIdx.x == 0) *next = lo + NW * gsz;
     __syncthreads();
+    const unsigned lt = lanemask_lt();
     int base = lo + warp * gsz;
     while (base < hi) {
         int nb = 0;
@@ -351,7 +351,6 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
                 if (nr > 0 && !prect) kind = w.rrec[id].kind;
                 ell = nr > 0 && kind == 0;
             }
-            const unsigned lt = lanemask_lt();
             const unsigned me = __ballot_sync(kFull, ell), mo = __ballot_sync(kFull, nr > 0 && !ell);
             const int ne = __popc(me);
             int4 *tmp = reinterpret_cast<int4 *>(items);
@@ -378,9 +377,11 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
         const int ex = inc - nr;
         const int total = __shfl_sync(kFull, inc, 31);
         // 2. waves of 32 (particle, row) items
+        const int first = nr > 0 ? ex : INT32_MAX;
+        int before = 0;
         for (int jb = 0; jb < total; jb += 32) {
             const int j = jb + lane;
-            const int e = warp_owner(inc, j, 0, -1);
+            const int e = range_of(first, jb, before);
             const int ide = __shfl_sync(kFull, id, e);
             const int ye = __shfl_sync(kFull, ry0, e) + j - __shfl_sync(kFull, ex, e);
             const int c0 = __shfl_sync(kFull, rx0, e), c1 = __shfl_sync(kFull, rx1, e);
@@ -389,27 +390,32 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
             if (j < total)
                 valid = make_row_item<ACC>(w.rrec[ide], c0, c1, ye, ye - ty0, inv_lambda, it);
             // 3. chunks: ellipsoid items' count in the low half-word, the
-            //    other kinds' in the high one
+            //    other kinds' in the high one; the items in that order
+            const bool ell = valid && ((it.hdr >> 24) & 3u) == 0;
             const int nch = valid ? (int)((((it.hdr >> 12) & 0xFFFu) + kChunkPx - 1) / kChunkPx) : 0;
-            const int mine = valid && ((it.hdr >> 24) & 3u) == 0 ? nch : nch << 16;
+            const int mine = ell ? nch : nch << 16;
             const int cinc = warp_incl_scan(mine);
             const int cex = cinc - mine;
             const int ctot = __shfl_sync(kFull, cinc, 31);
             const int TE = ctot & 0xFFFF, TC = TE + (ctot >> 16);
-            if (valid) items[lane] = it;
+            const unsigned me = __ballot_sync(kFull, ell), mo = __ballot_sync(kFull, valid && !ell);
+            const int c0th = !valid ? INT32_MAX : ell ? cex & 0xFFFF : TE + (cex >> 16);
+            if (valid) {
+                it.row |= c0th << 16;
+                items[ell ? __popc(me & lt) : __popc(me) + __popc(mo & lt)] = it;
+            }
             __syncwarp();
+            int cbefore = 0;
             for (int cb = 0; cb < TC; cb += 32) {
                 const int c = cb + lane;
-                const int sh = c < TE ? 0 : 16;
-                const int key = c < TE ? c : c - TE;
-                const int k = warp_owner(cinc, key, sh, 0xFFFF);
-                const int kex = (__shfl_sync(kFull, cex, k) >> sh) & 0xFFFF;
+                const int k = range_of(c0th, cb, cbefore);
                 if (c < TC) {
                     const RowItem rit = items[k];  // registers: the reductions below may not alias it
                     const uint32_t h = rit.hdr;
                     const int j0 = (int)(h & 0xFFFu), cnt = (int)((h >> 12) & 0xFFFu);
                     const int kind = (int)((h >> 24) & 3u);
-                    const int k0 = (key - kex) * kChunkPx;
+                    const int row = rit.row & 0xFFFF;
+                    const int k0 = (c - (int)((uint32_t)rit.row >> 16)) * kChunkPx;
                     const int len = min(kChunkPx, cnt - k0);
                     const int x0 = j0 + k0;
                     float t[kChunkPx];
@@ -432,7 +438,7 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
 #pragma unroll
                     for (int u = 0; u < kChunkPx; ++u) {
                         const bool on = u < len && t[u] > 0.f;
-                        deposit<ACC>(slot(rit.row, on ? x0 + u : x0), on ? t[u] : 0.f, rit.dn, rit.mu);
+                        deposit<ACC>(slot(row, on ? x0 + u : x0), on ? t[u] : 0.f, rit.dn, rit.mu);
                     }
                 }
             }
