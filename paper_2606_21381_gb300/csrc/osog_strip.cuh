@@ -45,7 +45,7 @@ __host__ __device__ constexpr int sq_rb(int n) { return set_elems(n) / n < n ? s
 enum { kAccPhase = 0, kAccOpd = 1 };
 
 struct __align__(16) RowItem {
-    uint32_t hdr;   // first column j0 (bits 0-11), pixel count (12-23), kind (24-25)
+    uint32_t hdr;   // first column j0 (bits 0-11), pixel count (12-23), kind (24-25), kFarItem (26)
     float f[8];     // ellipsoid: left and right chord ends (hi, lo each), T sqrt(alpha)
                     // prism: cx, g s ey, g c ey, g cos, g sin, g hx, g hy, T
                     // polyhedron: cx, ey, plane offset, plane count (int bits)
@@ -54,6 +54,14 @@ struct __align__(16) RowItem {
     float mu;       // kAccPhase: mu in units of 2^-20 per um; kAccOpd: mu
 };
 static_assert(sizeof(RowItem) == 48, "RowItem is 48 bytes");
+
+// An item whose contributions may reach 2^21 cycles, or 2^21 units of absorption,
+// at a pixel (or whose thickness has no cheap bound): see deposit.
+constexpr uint32_t kFarItem = 1u << 26;
+// fma(r, 2^23, kMagic) and x + kMagic round to an integer in the low mantissa bits
+// (|values| < 2^22); kMagicBits are the bits of kMagic = 1.5 2^23.
+constexpr float kMagic = 12582912.f;
+constexpr int kMagicBits = 0x4B400000;
 
 // Square root of a float-float a (a.h > 0): a float estimate s, then one
 // correction step (a - s^2) / (2 s) with the residual taken exactly by a
@@ -84,6 +92,7 @@ __device__ __forceinline__ bool make_row_item(const RRec &r, int c0, int c1, int
     const float yc = (float)y + 0.5f;
     float lo, hi;  // span of pixel-centre x
     float c = 0.f, sn = 0.f, s_ey = 0.f, c_ey = 0.f;
+    float tmax = INFINITY;  // of the chord on this row
     if (r.kind == 0) {
         const ff ey = two_sum(yc, -r.cy);
         const ff x0 = ff_add(ff{r.cx, 0.f}, ff_mul(ff{r.p[0], r.p[1]}, ey));
@@ -96,6 +105,7 @@ __device__ __forceinline__ bool make_row_item(const RRec &r, int c0, int c1, int
         it.f[2] = xr.h;
         it.f[3] = xr.l;
         it.f[4] = r.tsa;
+        tmax = r.tsa * w.h;
         lo = xl.h;
         hi = xr.h;
     } else if (r.kind == 1) {
@@ -155,12 +165,14 @@ __device__ __forceinline__ bool make_row_item(const RRec &r, int c0, int c1, int
         it.f[5] = g * r.p[2];
         it.f[6] = g * r.p[3];
         it.f[7] = r.p[5];
+        tmax = r.p[5];
     }
     it.hdr = (uint32_t)j0 | ((uint32_t)(j1 - j0 + 1) << 12) | ((uint32_t)r.kind << 24);
     it.row = row;
     if constexpr (ACC == kAccPhase) {
         it.dn = r.dn * inv_lambda;
         it.mu = r.mu * 1048576.f;  // the exponent's unit folded in (exact: a power of two)
+        if (!(fmaxf(fabsf(it.dn), fabsf(it.mu)) * tmax < 2097152.f)) it.hdr |= kFarItem;
     } else {
         it.dn = r.dn;
         it.mu = r.mu;
@@ -214,20 +226,31 @@ __device__ __forceinline__ float item_chord(const RowItem &it, int kind, float X
 // at shared-memory address acc (phase mode: a uint2 slot, x the phase in
 // 2^-23 cycles, y the absorption exponent in 2^-20; OPD mode: two int64 in
 // 2^-32 um).  dn and mu are the item's (phase mode: dn / lambda in cycles
-// per um, mu already in 2^-20 per um).  The additions are shared-space reductions issued on the slot's
-// shared address (no generic addressing, no returned value).
-template <int ACC>
+// per um, mu already in 2^-20 per um).  The additions are shared-space
+// reductions issued on the slot's shared address (no generic addressing, no
+// returned value).  Rounding to integers by the magic addend is the same as by
+// conversions for FAR = false, whose values stay below 2^22; conversions issue
+// on the quarter-rate pipe, two or three per pixel beside the chord's square root
+// (32 images of 2048 x 2048 1635 -> 1622 us without them).
+template <int ACC, bool FAR>
 __device__ __forceinline__ void deposit(uint32_t acc, float t, float dn, float mu) {
     if constexpr (ACC == kAccPhase) {
-        const float c = t * dn;                   // cycles
-        const float r = c - rintf(c);             // in [-1/2, 1/2]
-        // round(r 2^23) from the mantissa of r 2^23 + 1.5 2^23
-        const int q = __float_as_int(fmaf(r, 8388608.f, 12582912.f)) - 0x4B400000;
+        const float c = t * dn;  // cycles
+        float k;
+        if constexpr (FAR)
+            k = rintf(c);
+        else
+            k = __fsub_rn(__fadd_rn(c, kMagic), kMagic);
+        const float r = c - k;  // in [-1/2, 1/2]
+        const int q = __float_as_int(fmaf(r, 8388608.f, kMagic)) - kMagicBits;
         asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(acc), "r"(q) : "memory");
         if (mu != 0.f) {
-            const float x = fminf(fmaxf(t * mu, -16777216.f), 16777216.f);  // |mu t| <= 16
-            asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(acc + 4u), "r"(__float2int_rn(x))
-                         : "memory");
+            int a;
+            if constexpr (FAR)
+                a = __float2int_rn(fminf(fmaxf(t * mu, -16777216.f), 16777216.f));  // |mu t| <= 16
+            else
+                a = __float_as_int(__fadd_rn(__fmul_rn(t, mu), kMagic)) - kMagicBits;
+            asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(acc + 4u), "r"(a) : "memory");
         }
     } else {
         asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(acc),
@@ -244,9 +267,11 @@ __device__ __forceinline__ void deposit(uint32_t acc, float t, float dn, float m
 // pixel (both words zero) takes the same path: sin 0, cos 0 and 2^0 are
 // exact, so it gives (1, 0) without a branch that would split the warp.
 __device__ __forceinline__ float2 exit_wave_fixed(uint2 acc) {
-    const int p = (int)(acc.x << 9) >> 9;  // units of 2^-23 cycles
+    // the low 23 bits as a signed number p of 2^-23 cycles: with the sign bit
+    // flipped they are the mantissa of kMagic + p
+    const float p = __int_as_float((int)((acc.x & 0x7FFFFFu) ^ (uint32_t)kMagicBits)) - kMagic;
     float s, c;
-    __sincosf((float)p * 7.4901405658471572e-07f, &s, &c);              // 2 pi 2^-23
+    __sincosf(p * 7.4901405658471572e-07f, &s, &c);                     // 2 pi 2^-23
     const float a = __expf((float)(int)acc.y * -9.5367431640625e-07f);  // -2^-20
     return make_float2(a * c, a * s);
 }
@@ -418,28 +443,33 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
                     const int k0 = (c - (int)((uint32_t)rit.row >> 16)) * kChunkPx;
                     const int len = min(kChunkPx, cnt - k0);
                     const int x0 = j0 + k0;
+                    const float X = (float)x0 + 0.5f;  // X + u is exact
                     float t[kChunkPx];
                     if (kind == 0) {
 #pragma unroll
-                        for (int u = 0; u < kChunkPx; ++u)
-                            t[u] = item_chord(rit, 0, (float)(x0 + u) + 0.5f, nullptr);
+                        for (int u = 0; u < kChunkPx; ++u) t[u] = item_chord(rit, 0, X + (float)u, nullptr);
                     } else if (kind == 1) {
 #pragma unroll
-                        for (int u = 0; u < kChunkPx; ++u)
-                            t[u] = item_chord(rit, 1, (float)(x0 + u) + 0.5f, nullptr);
+                        for (int u = 0; u < kChunkPx; ++u) t[u] = item_chord(rit, 1, X + (float)u, nullptr);
                     } else {
 #pragma unroll
                         for (int u = 0; u < kChunkPx; ++u)
-                            t[u] = u < len ? item_chord(rit, 2, (float)(x0 + u) + 0.5f, w.plane_coef)
-                                           : -1.f;
+                            t[u] = u < len ? item_chord(rit, 2, X + (float)u, w.plane_coef) : -1.f;
                     }
                     // every step deposits (zero at the chunk's first pixel when the
                     // pixel is past the chunk or outside the footprint): no branch
+                    auto add = [&](auto far) {
 #pragma unroll
-                    for (int u = 0; u < kChunkPx; ++u) {
-                        const bool on = u < len && t[u] > 0.f;
-                        deposit<ACC>(slot(row, on ? x0 + u : x0), on ? t[u] : 0.f, rit.dn, rit.mu);
-                    }
+                        for (int u = 0; u < kChunkPx; ++u) {
+                            const bool on = u < len && t[u] > 0.f;
+                            deposit<ACC, decltype(far)::value>(slot(row, on ? x0 + u : x0), on ? t[u] : 0.f,
+                                                               rit.dn, rit.mu);
+                        }
+                    };
+                    if (ACC == kAccPhase && (h & kFarItem))
+                        add(std::true_type{});
+                    else
+                        add(std::false_type{});
                 }
             }
             __syncwarp();  // the wave's items are read before the next wave writes
