@@ -231,9 +231,9 @@ k_bwd_strip(const __grid_constant__ BwdStripArgs a) {
         {
             const int idx = (e / N) * LS + pad16(e % N);
             const float2 g = bufG[idx];
-            const float2 E = exit_wave_fixed(reinterpret_cast<const uint2 *>(bufO)[idx]);
+            const float2 E = exit_wave_fixed(PhaseSlot<N>::load(bufO, e / N, e % N));
             const float ex = E.x, ey = E.y;
-            bufO[idx] = make_float2(k2pi * fmaf(g.y, ex, -g.x * ey), -fmaf(g.x, ex, g.y * ey));
+            bufG[idx] = make_float2(k2pi * fmaf(g.y, ex, -g.x * ey), -fmaf(g.x, ex, g.y * ey));
         }
     }
     __syncthreads();
@@ -293,7 +293,7 @@ k_bwd_strip(const __grid_constant__ BwdStripArgs a) {
             const int yy = ya + ly;
             const float ey = (float)yy + 0.5f - r.cy;
             const int xe = (int)(hdr & 0xFFFu) + (int)((hdr >> 12) & 0xFFFu);
-            const float2 *row = bufO + (min(yy, ylast) - y0) * LS;
+            const float2 *row = bufG + (min(yy, ylast) - y0) * LS;
             float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             if (rr.kind == 0) {
                 const float xlh = __shfl_sync(kFull, it.f[0], ly), xll = __shfl_sync(kFull, it.f[1], ly);

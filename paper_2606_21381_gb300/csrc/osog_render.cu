@@ -97,7 +97,7 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
         // the columns some pupil passes)
         constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
         fft_first_pass<N, L, false, true, GRP>(buf, [&](int l, int x) -> float2 {
-            return l < R ? exit_wave_fixed(*reinterpret_cast<const uint2 *>(buf + l * LS + pad16(x)))
+            return l < R ? exit_wave_fixed(PhaseSlot<N>::load(buf, l, x))
                          : make_float2(0.f, 0.f);
         });
         fft_pass_range<N, L, false, 1, fft_passes(N) - 1, GRP>(buf, a.tw);
@@ -160,6 +160,16 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
 // ------------------------------------------------------------ tile raster
 constexpr int kRThreads = 256;
 
+// Accumulators of a tile: (phase, absorption) pairs, as they are stored.
+struct TileSlot {
+    static constexpr uint32_t att = 4u;
+    uint32_t base;
+    int TW, tx0;
+    __device__ __forceinline__ uint32_t operator()(int row, int x, int u, bool on) const {
+        return base + (uint32_t)(row * TW + ((on ? x + u : x) - tx0)) * 8u;
+    }
+};
+
 __global__ void __launch_bounds__(kRThreads, 4) k_raster_tiles(const __grid_constant__ RasterArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_enter();
@@ -177,9 +187,7 @@ __global__ void __launch_bounds__(kRThreads, 4) k_raster_tiles(const __grid_cons
     const int hi = min(off[band + 1], sc.pair_cap);
     const int lo = min(off[band], hi);
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(acc);
-    auto slot = [base, TW, tx0](int row, int x) -> uint32_t {
-        return base + (uint32_t)(row * TW + (x - tx0)) * 8u;
-    };
+    const TileSlot slot{base, TW, tx0};
     raster_region<kRThreads, kAccPhase>(a.w, a.w.pairs + sc.pair0,
                                         a.w.pair_rect ? a.w.pair_rect + sc.pair0 : nullptr, lo, hi, ty0, TH, tx0,
                                         tx0 + TW - 1, 0.5f * sc.two_over_lambda, slot, scratch);

@@ -222,18 +222,18 @@ __device__ __forceinline__ float item_chord(const RowItem &it, int kind, float X
     return inside && zhi > zlo ? zhi - zlo : -1.f;
 }
 
-// Adds one particle's contribution at chord t > 0 to the pixel's accumulators
-// at shared-memory address acc (phase mode: a uint2 slot, x the phase in
-// 2^-23 cycles, y the absorption exponent in 2^-20; OPD mode: two int64 in
-// 2^-32 um).  dn and mu are the item's (phase mode: dn / lambda in cycles
+// Adds one particle's contribution at chord t >= 0 to the pixel's
+// accumulators at shared-memory addresses acc and acc + att (phase mode: 32-bit
+// words, the phase in 2^-23 cycles and the absorption exponent in 2^-20; OPD
+// mode: int64 in 2^-32 um).  dn and mu are the item's (phase mode: dn / lambda in cycles
 // per um, mu already in 2^-20 per um).  The additions are shared-space
-// reductions issued on the slot's shared address (no generic addressing, no
-// returned value).  Rounding to integers by the magic addend is the same as by
+// reductions issued on the shared address (no generic addressing, no returned
+// value).  Rounding to integers by the magic addend is the same as by
 // conversions for FAR = false, whose values stay below 2^22; conversions issue
 // on the quarter-rate pipe, two or three per pixel beside the chord's square root
 // (32 images of 2048 x 2048 1635 -> 1622 us without them).
 template <int ACC, bool FAR>
-__device__ __forceinline__ void deposit(uint32_t acc, float t, float dn, float mu) {
+__device__ __forceinline__ void deposit(uint32_t acc, uint32_t att, float t, float dn, float mu) {
     if constexpr (ACC == kAccPhase) {
         const float c = t * dn;  // cycles
         float k;
@@ -250,13 +250,13 @@ __device__ __forceinline__ void deposit(uint32_t acc, float t, float dn, float m
                 a = __float2int_rn(fminf(fmaxf(t * mu, -16777216.f), 16777216.f));  // |mu t| <= 16
             else
                 a = __float_as_int(__fadd_rn(__fmul_rn(t, mu), kMagic)) - kMagicBits;
-            asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(acc + 4u), "r"(a) : "memory");
+            asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(acc + att), "r"(a) : "memory");
         }
     } else {
         asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(acc),
                      "l"((unsigned long long)__float2ll_rn(t * dn * 4294967296.f)) : "memory");
         if (mu != 0.f)
-            asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(acc + 8u),
+            asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(acc + att),
                          "l"((unsigned long long)__float2ll_rn(t * mu * 4294967296.f)) : "memory");
     }
 }
@@ -313,8 +313,10 @@ __host__ __device__ constexpr size_t raster_smem() {
 // OPD and ATT of the region rows [ty0, ty0 + nrows) x columns [tx0, tx1]
 // of scene s from the band list entries [lo, hi) (ids of the scene's
 // records; prect, when not null, the entries' rectangles with their kinds,
-// else they are gathered by id), added into the accumulators that slot(row, x) addresses (zeroed
-// by the caller; kAccPhase: uint2, kAccOpd: two int64).  Each warp works on
+// else they are gathered by id), added into the accumulators at the shared
+// addresses slot(row, x, u, on) of column x + u, where slot.att bytes further the
+// absorption is (zeroed by the caller; kAccPhase: 32-bit, kAccOpd: int64; where
+// !on, any accumulators that zeros may be added to).  Each warp works on
 // its own groups of 32 list entries (fewer when the list is short, so that
 // every warp gets a group; the first NT / 32 groups in warp order, the rest
 // handed out by a shared counter as warps finish), with no CTA barrier
@@ -330,7 +332,7 @@ __host__ __device__ constexpr size_t raster_smem() {
 //      pass takes chunk l and evaluates its pixels as independent unrolled
 //      chains, adding each covered pixel with integer shared-memory
 //      reductions (a step past the chunk or outside the footprint adds zero,
-//      so the pass has no branch around them).
+//      so the pass has no branch around them; predicated reductions took longer).
 // Every thread of the CTA must call it; it ends with a CTA barrier.
 template <int NT, int ACC, typename Slot>
 __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *prect, int lo,
@@ -456,13 +458,11 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
                         for (int u = 0; u < kChunkPx; ++u)
                             t[u] = u < len ? item_chord(rit, 2, X + (float)u, w.plane_coef) : -1.f;
                     }
-                    // every step deposits (zero at the chunk's first pixel when the
-                    // pixel is past the chunk or outside the footprint): no branch
                     auto add = [&](auto far) {
 #pragma unroll
                         for (int u = 0; u < kChunkPx; ++u) {
                             const bool on = u < len && t[u] > 0.f;
-                            deposit<ACC, decltype(far)::value>(slot(row, on ? x0 + u : x0), on ? t[u] : 0.f,
+                            deposit<ACC, decltype(far)::value>(slot(row, x0, u, on), slot.att, on ? t[u] : 0.f,
                                                                rit.dn, rit.mu);
                         }
                     };
@@ -479,21 +479,50 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
     __syncthreads();
 }
 
-// The strip [y0, y0 + R) of scene s rasterised into the padded FFT lines of
-// an N-point set (the adjoint's re-raster; osog_render_opd in OPD mode).
+// Accumulators of a strip in the memory of its padded FFT lines of N points.
+// Phase mode: line l holds the row's N phase words, then its N absorption words,
+// shifted by some words per row within the line's padding.  Lanes of a raster pass
+// are four pixels apart in a row and in neighbouring rows of a particle; with
+// (phase, absorption) pairs at the samples' own places they fell on a quarter of
+// the banks (3.7 wavefronts a reduction; the planes' shift puts the next row's
+// pixels 13 banks on, 2.4), and a chunk's pixels are at constant offsets, the ones
+// past a row's end in the next words of its line: 32 images of 2048 x 2048 1622 ->
+// 1604 us.  OPD mode: pairs of int64 at the samples' places.
+template <int N>
+struct PhaseSlot {
+    static constexpr int kLine = 2 * line_stride(N), kShift = N >= 256 ? 5 : 1;
+    static_assert(2 * N + 7 * kShift + kChunkPx - 1 <= kLine, "a row's words stay in its line");
+    static constexpr uint32_t att = 4u * N;
+    __host__ __device__ static constexpr int word(int row, int x) { return row * kLine + kShift * (row & 7) + x; }
+    uint32_t base;
+    __device__ __forceinline__ uint32_t operator()(int row, int x, int u, bool) const {
+        return base + 4u * (uint32_t)word(row, x) + 4u * (uint32_t)u;
+    }
+    static __device__ __forceinline__ uint2 load(const void *acc, int row, int x) {
+        const uint32_t *p = static_cast<const uint32_t *>(acc) + word(row, x);
+        return make_uint2(p[0], p[N]);
+    }
+};
+template <int N>
+struct OpdSlot {
+    static constexpr uint32_t att = 8u;
+    uint32_t base;
+    __device__ __forceinline__ uint32_t operator()(int row, int x, int u, bool on) const {
+        return base + 16u * (uint32_t)(row * line_stride(N) + pad16(on ? x + u : x));
+    }
+};
+
+// The strip [y0, y0 + R) of scene s rasterised into accumulators in the memory
+// of N-point FFT lines (PhaseSlot; OpdSlot for osog_render_opd).
 template <int N, int ACC, int NT = kThreads>
 __device__ void raster_strip(const Geometry &geo, const Work &w, const SceneDev &sc, int s,
                              int y0, int R, void *acc, unsigned char *scratch) {
-    constexpr int LS = line_stride(N);
     const int band = y0 / geo.BH;
     const int32_t *off = w.band_off + (size_t)s * (geo.nbands + 1);
     const int hi = min(off[band + 1], sc.pair_cap);
     const int lo = min(off[band], hi);
-    // shared address of the (row, x) slot: uint2 (phase) or two int64 (OPD)
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(acc);
-    auto slot = [base](int row, int x) -> uint32_t {
-        return base + (uint32_t)(row * LS + pad16(x)) * (ACC == kAccPhase ? 8u : 16u);
-    };
+    using Slot = std::conditional_t<ACC == kAccPhase, PhaseSlot<N>, OpdSlot<N>>;
+    const Slot slot{(uint32_t)__cvta_generic_to_shared(acc)};
     raster_region<NT, ACC>(w, w.pairs + sc.pair0, w.pair_rect ? w.pair_rect + sc.pair0 : nullptr,
                                  lo, hi, y0, R, 0, geo.W - 1, 0.5f * sc.two_over_lambda, slot,
                                  scratch);
