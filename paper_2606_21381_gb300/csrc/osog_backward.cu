@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant_
     const int y0 = blockIdx.x * R;
     float2 *Qm = a.w.Q + (size_t)sm * geo.nblocks * H * B;
     const int2 cr = a.w.hull[sm / K];
-    fft_first_pass<N, L, true, false, G>(bufE, [&](int l, int kx) -> float2 {
+    fft_first_pass<N, L, true, false, kSyncCta, kRowFast>(bufE, [&](int l, int kx) -> float2 {
         const int fx = kx < N / 2 ? kx : kx - N;
         return l < R && fx >= cr.x && fx <= cr.y
                    ? Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))]
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant_
     });
     fft_pass_range<N, L, true, 1, fft_passes(N) - 1, G>(bufE, a.tw);  // E_m rows
     const float *gI = a.grad_image + ((size_t)sm * H + y0) * N;
-    fft_last_pass<N, L, true, false, G>(bufE, a.tw, [&](int l, int x, float2 v) {
+    fft_last_pass<N, L, true, 0, G>(bufE, a.tw, [&](int l, int x, float2 v) {
         const float g2 = l < R ? 2.f * gI[(size_t)l * N + x] : 0.f;
         bufQ[l * LS + pad16(x)] = make_float2(g2 * v.x, g2 * v.y);
     });
@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant_
         __syncthreads();
     // adjoint of the inverse row DFT
     fft_pass_range<N, L, false, 0, fft_passes(N) - 1, G>(bufQ, a.tw);
-    fft_last_pass<N, L, false, false, G>(bufQ, a.tw, [&](int l, int kx, float2 v) {
+    if constexpr (G == kSyncLine) __syncthreads();
+    fft_last_pass<N, L, false, kRowFast, kSyncCta>(bufQ, a.tw, [&](int l, int kx, float2 v) {
         const int fx = kx < N / 2 ? kx : kx - N;
         if (l < R && fx >= cr.x && fx <= cr.y)
             Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))] = v;
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
         }
         // dL/dZ_m (adjoint of the inverse column DFT)
         fft_pass_range<N, L, false, 0, fft_passes(N) - 1>(bufZ, a.tw);
-        fft_last_pass<N, L, false, false, kSyncCta>(bufZ, a.tw, [&](int c, int y, float2 gz, int i) {
+        fft_last_pass<N, L, false, 0, kSyncCta>(bufZ, a.tw, [&](int c, int y, float2 gz, int i) {
             if (c >= B) return;
             const int kx = bk * B + c;
             const int fx = kx < half ? kx : kx - geo.W;
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
     __syncthreads();
     // dL/dG (adjoint of the forward column DFT)
     fft_pass_range<N, L, true, 0, fft_passes(N) - 1>(bufE, a.tw);
-    fft_last_pass<N, L, true, true, kSyncCta>(bufE, a.tw, [&](int c, int y, float2 v) {
+    fft_last_pass<N, L, true, L, kSyncCta>(bufE, a.tw, [&](int c, int y, float2 v) {
         if (c < B) Gb[(size_t)y * B + c] = v;
     });
 #pragma unroll

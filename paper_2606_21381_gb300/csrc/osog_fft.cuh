@@ -184,6 +184,28 @@ __device__ __forceinline__ void butterfly_of(int q, int &l, int &j) {
     }
 }
 
+// The same for the passes that read or write global memory; FAST > 0: consecutive
+// threads take FAST consecutive lines, then the butterflies of those lines.
+template <int L, int NB, int G, int FAST>
+__device__ __forceinline__ void line_butterfly(int q, int &l, int &j) {
+    if constexpr (FAST > 0) {
+        static_assert(L % FAST == 0, "whole groups of lines");
+        const int b = threadIdx.x + q * kThreads;
+        l = b % FAST + b / (FAST * NB) * FAST;
+        j = b / FAST % NB;
+    } else {
+        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+    }
+}
+
+// Row strips read and write column-blocked arrays, whose block of one strip is R x B
+// samples end to end.  Consecutive threads over four lines cover 128 bytes of 4 x 4
+// samples and more; along one line they would take 32 or 64 bytes of every block
+// (inverse rows of a 2048 x 2048 image 11.6 -> 10.6 us; 32 whole images 1607 -> 1550,
+// twelve DIC images of 1024 x 1024 305 -> 303).  Four lines are also as many as lie
+// on different banks (line_stride).
+constexpr int kRowFast = 4;
+
 // Largest radix whose twiddles are formed as products (0: all read from the
 // table).  A radix-P pass needs w^{r k}, r = 1..P-1: the table entries at
 // r = 1, 2, 4 (and 8) are read and the others formed as products of two of
@@ -306,8 +328,9 @@ __device__ __forceinline__ void fft_pass_range(float2 *buf, const float2 *__rest
 // operation are those of stockham_pass, so the results are bitwise the same.
 // IN_PLACE: ld reads buf itself, and the threads synchronise between the
 // loads and the writes.  G: grouped (see stockham_pass); ld(l, i) may then
-// read only line l of buf.  Ends with a barrier (the line's, grouped).
-template <int N, int L, bool INV, bool IN_PLACE, int G, class Ld>
+// read only line l of buf.  FAST: as in fft_last_pass.  Ends with a barrier
+// (the line's, grouped).
+template <int N, int L, bool INV, bool IN_PLACE, int G, int FAST = 0, class Ld>
 __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
     constexpr int P = fft_radix(N, 0);
     constexpr int NB = N / P;
@@ -315,12 +338,13 @@ __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
     constexpr int PER = (TOT + kThreads - 1) / kThreads;
     constexpr int LS = line_stride(N);
     static_assert(G != kSyncLine || (NB % (kThreads / L) == 0 && kThreads % L == 0), "grouped pass");
+    static_assert(!(FAST > 0 && G == kSyncLine), "one thread mapping");
     float2 v[PER][P];
     int l = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        line_butterfly<L, NB, G, FAST>(q, l, j);
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
 #pragma unroll
             for (int r = 0; r < P; ++r) v[q][r] = ld(l, j + r * NB);
@@ -332,7 +356,7 @@ __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int j;
-        butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+        line_butterfly<L, NB, G, FAST>(q, l, j);
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             dft<P, INV>(v[q]);
             float2 *dst = buf + l * LS + pad16(j * P);
@@ -345,9 +369,9 @@ __device__ __forceinline__ void fft_first_pass(float2 *buf, Ld ld) {
 
 // The last pass of the plan with its outputs handed to st(l, i, value),
 // sample i of line l, instead of written back to buf (the kernels store
-// straight to global memory).  Arithmetic as in stockham_pass.  LINE_FAST:
-// consecutive threads take consecutive lines (the columns of a column
-// block, interleaved in global memory; the pass before must end with a CTA
+// straight to global memory).  Arithmetic as in stockham_pass.  FAST > 0:
+// consecutive threads take FAST consecutive lines (columns of a block, rows of a
+// strip, interleaved in global memory; the pass before must end with a CTA
 // barrier); G: grouped (see stockham_pass); else consecutive butterflies of
 // the whole set.  buf is only read, so there is no barrier.  st may take a
 // fourth argument, the number of the output among the thread's own (a constant
@@ -357,32 +381,23 @@ __host__ __device__ constexpr int fft_last_outputs() {
     constexpr int P = fft_radix(N, fft_passes(N) - 1);
     return (L * (N / P) + kThreads - 1) / kThreads * P;
 }
-template <int N, int L, bool INV, bool LINE_FAST, int G, class St>
+template <int N, int L, bool INV, int FAST, int G, class St>
 __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *__restrict__ tw,
                                               St st) {
     constexpr int PASS = fft_passes(N) - 1;
     constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS);
     static_assert(NS * P == N && NS > 1, "the last pass of the plan");
-    static_assert(!(LINE_FAST && G == kSyncLine), "one thread mapping");
+    static_assert(!(FAST > 0 && G == kSyncLine), "one thread mapping");
     constexpr int NB = N / P;
     constexpr int TOT = L * NB;
     constexpr int PER = (TOT + kThreads - 1) / kThreads;
     constexpr int LS = line_stride(N);
     const float2 *__restrict__ t = tw + fft_twoff(N, PASS);
     float2 v[PER][P];
-    auto which = [](int q, int &l, int &j) {
-        if constexpr (LINE_FAST) {
-            const int b = threadIdx.x + q * kThreads;
-            l = b % L;
-            j = b / L;
-        } else {
-            butterfly_of<L, NB, G == kSyncLine>(q, l, j);
-        }
-    };
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int l, j;
-        which(q, l, j);
+        line_butterfly<L, NB, G, FAST>(q, l, j);
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             if constexpr (NB % 16 == 0) {
                 const float2 *src = buf + l * LS + pad16(j);
@@ -398,7 +413,7 @@ __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *_
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
         int l, j;
-        which(q, l, j);
+        line_butterfly<L, NB, G, FAST>(q, l, j);
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             apply_twiddles<P, INV, NS>(v[q], t + j);
             dft<P, INV>(v[q]);

@@ -106,7 +106,8 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
         const int H = SQ ? N : geo.H;
         float2 *G = a.w.G + (size_t)s * H * N;
         const int2 cr = a.w.hull[s];
-        fft_last_pass<N, L, false, false, GRP>(buf, a.tw, [&](int l, int kx, float2 v) {
+        if constexpr (GRP == kSyncLine) __syncthreads();
+        fft_last_pass<N, L, false, kRowFast, kSyncCta>(buf, a.tw, [&](int l, int kx, float2 v) {
             const int fx = kx < N / 2 ? kx : kx - N;
             if (l < R && fx >= cr.x && fx <= cr.y)  // columns outside every pupil are never read
                 G[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))] = v;
@@ -478,7 +479,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
         if constexpr (GRP == kSyncLine) __syncthreads();
         // the last pass stores Q; consecutive threads take the block's
         // columns, so a warp writes whole rows of the block
-        fft_last_pass<N, L, true, true, false>(buf1, a.tw, [&](int c, int y, float2 v) {
+        fft_last_pass<N, L, true, L, kSyncCta>(buf1, a.tw, [&](int c, int y, float2 v) {
             if (c < B) Qm[(size_t)y * B + c] = v;
         });
         __syncthreads();
@@ -510,7 +511,7 @@ __device__ __forceinline__ void inverse_item(const InverseArgs &a, int sm, int s
     // (columns that no pupil passes, and lines past the strip, read as zero);
     // the last pass writes the intensity rows
     constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
-    fft_first_pass<N, L, true, false, GRP>(buf, [&](int l, int kx) -> float2 {
+    fft_first_pass<N, L, true, false, kSyncCta, kRowFast>(buf, [&](int l, int kx) -> float2 {
         const int fx = kx < N / 2 ? kx : kx - N;
         return l < R && fx >= cr.x && fx <= cr.y
                    ? Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))]
@@ -519,7 +520,7 @@ __device__ __forceinline__ void inverse_item(const InverseArgs &a, int sm, int s
     fft_pass_range<N, L, true, 1, fft_passes(N) - 1, GRP>(buf, a.tw);
     float *img = a.images + ((size_t)sm * H + y0) * N;
     const int real_out = a.real_out;
-    fft_last_pass<N, L, true, false, GRP>(buf, a.tw, [&](int l, int x, float2 v) {
+    fft_last_pass<N, L, true, 0, GRP>(buf, a.tw, [&](int l, int x, float2 v) {
         if (l < R) img[(size_t)l * N + x] = real_out ? v.x : fmaf(v.x, v.x, __fmul_rn(v.y, v.y));
     });
 }
