@@ -428,6 +428,138 @@ __device__ __forceinline__ void fft_last_pass(const float2 *buf, const float2 *_
     }
 }
 
+// ------------------------------------------------------- transposed passes
+// The DFT matrix is symmetric, so the plan's passes transposed and in reverse order
+// are the same transform: pass p loads from where the pass above stores, transforms,
+// multiplies by the same twiddles and stores to where that pass loads from.  Its first
+// pass takes samples j + r NS of the plan's last, which are the outputs a thread of
+// fft_last_pass holds: what follows a transform (a product with a transfer function)
+// and the transform back need no pass over shared memory in between, and the slots
+// are the thread's own, so no barrier either.
+template <int N, int L, int PASS, bool LOAD>
+__device__ __forceinline__ void line_slots(float2 *buf, int l, int j, float2 *v) {
+    constexpr int P = fft_radix(N, PASS), NB = N / P;  // samples j + r NB of line l
+    float2 *b = buf + l * line_stride(N) + (NB % 16 == 0 ? pad16(j) : 0);
+#pragma unroll
+    for (int r = 0; r < P; ++r) {
+        float2 &x = b[NB % 16 == 0 ? r * (NB + NB / 16) : pad16(j + r * NB)];
+        if constexpr (LOAD)
+            v[r] = x;
+        else
+            x = v[r];
+    }
+}
+
+// First transposed pass, inputs from ld(l, i); ld may read any memory but other
+// threads' slots of buf.  Ends with a barrier (the line's, grouped).
+template <int N, int L, bool INV, int G, class Ld>
+__device__ __forceinline__ void fft_t_first_pass(float2 *buf, const float2 *__restrict__ tw, Ld ld) {
+    constexpr int PASS = fft_passes(N) - 1;
+    constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS);
+    constexpr int TOT = L * NS, PER = (TOT + kThreads - 1) / kThreads;
+    const float2 *__restrict__ t = tw + fft_twoff(N, PASS);
+    int l = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        int j;
+        butterfly_of<L, NS, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+            float2 v[P];
+#pragma unroll
+            for (int r = 0; r < P; ++r) v[r] = ld(l, j + r * NS);
+            dft<P, INV>(v);
+            apply_twiddles<P, INV, NS>(v, t + j);
+            line_slots<N, L, PASS, false>(buf, l, j, v);
+        }
+    }
+    pass_sync<G, L>(l);
+}
+
+// The plan's last pass (forward), f(l, i, value) on its outputs, and the first
+// transposed pass of the inverse transform, in registers.
+template <int N, int L, int G, class F>
+__device__ __forceinline__ void fft_turn_pass(float2 *buf, const float2 *__restrict__ tw, F f) {
+    constexpr int PASS = fft_passes(N) - 1;
+    constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS);
+    constexpr int TOT = L * NS, PER = (TOT + kThreads - 1) / kThreads;
+    const float2 *__restrict__ t = tw + fft_twoff(N, PASS);
+    int l = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        int j;
+        butterfly_of<L, NS, G == kSyncLine>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+            float2 v[P];
+            line_slots<N, L, PASS, true>(buf, l, j, v);
+            apply_twiddles<P, false, NS>(v, t + j);
+            dft<P, false>(v);
+#pragma unroll
+            for (int r = 0; r < P; ++r) v[r] = f(l, j + r * NS, v[r]);
+            dft<P, true>(v);
+            apply_twiddles<P, true, NS>(v, t + j);
+            line_slots<N, L, PASS, false>(buf, l, j, v);
+        }
+    }
+    pass_sync<G, L>(l);
+}
+
+// The transposed passes between the first and the last.
+template <int N, int L, bool INV, int G, int PASS = fft_passes(N) - 2>
+__device__ __forceinline__ void fft_t_mid_passes(float2 *buf, const float2 *__restrict__ tw) {
+    if constexpr (PASS >= 1) {
+        constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS), NB = N / P;
+        constexpr int TOT = L * NB, PER = (TOT + kThreads - 1) / kThreads;
+        float2 v[PER][P];
+        int l = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            int j;
+            butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+            if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+                const int k = j & (NS - 1);
+                const float2 *src = buf + l * line_stride(N) + pad16((j - k) * P + k);
+#pragma unroll
+                for (int r = 0; r < P; ++r) v[q][r] = src[stride_off(NS, r)];
+            }
+        }
+        pass_sync<G, L>(l);
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            int j;
+            butterfly_of<L, NB, G == kSyncLine>(q, l, j);
+            if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+                dft<P, INV>(v[q]);
+                apply_twiddles<P, INV, NS>(v[q], tw + fft_twoff(N, PASS) + (j & (NS - 1)));
+                line_slots<N, L, PASS, false>(buf, l, j, v[q]);
+            }
+        }
+        pass_sync<G, L>(l);
+        fft_t_mid_passes<N, L, INV, G, PASS - 1>(buf, tw);
+    }
+}
+
+// The last transposed pass, outputs to st(l, i, value); FAST, G as in fft_last_pass.
+template <int N, int L, bool INV, int FAST, int G, class St>
+__device__ __forceinline__ void fft_t_last_pass(const float2 *buf, St st) {
+    constexpr int P = fft_radix(N, 0), NB = N / P;
+    constexpr int TOT = L * NB, PER = (TOT + kThreads - 1) / kThreads;
+    static_assert(!(FAST > 0 && G == kSyncLine), "one thread mapping");
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        int l, j;
+        line_butterfly<L, NB, G, FAST>(q, l, j);
+        if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
+            float2 v[P];
+            const float2 *src = buf + l * line_stride(N) + pad16(j * P);
+#pragma unroll
+            for (int r = 0; r < P; ++r) v[r] = src[r];
+            dft<P, INV>(v);
+#pragma unroll
+            for (int r = 0; r < P; ++r) st(l, j + r * NB, v[r]);
+        }
+    }
+}
+
 // Host: the twiddle tables of an n-point transform, n entries, in double
 // precision rounded once to float: pass p's block holds
 // exp(-2 pi i r k / (Ns P)) at [(r - 1) Ns + k], r = 1..P-1, k = 0..Ns-1.

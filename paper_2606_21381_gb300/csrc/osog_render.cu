@@ -380,6 +380,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
     __shared__ uint64_t bar;  // completes the bulk copy (BULK)
     const bool bulk = BULK && !a.unit_input;
     constexpr int GRP = kGroupFft && fft_grouped(N) ? kSyncLine : kSyncCta;
+    constexpr int LAST = fft_passes(N) - 1;
     if (bulk) {
         if constexpr (BULK)
             if (threadIdx.x == 0)
@@ -419,11 +420,17 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
             }
             bulk_wait(&bar, a.w.status, a.wait_polls);
             first_pass_from_block<N, false>(buf0, live);
-            fft_pass_range<N, L, false, 1, fft_passes(N), GRP>(buf0, a.tw);
-            if constexpr (GRP == kSyncLine) __syncthreads();  // every line done before any thread reads another's
+            fft_pass_range<N, L, false, 1, LAST, GRP>(buf0, a.tw);
         }
     } else if (!a.unit_input) {
-        fft_lines<N, L, false>(buf0, a.tw);
+        fft_pass_range<N, L, false, 0, LAST, GRP>(buf0, a.tw);
+    }
+    // a single pupil's transform, product and transform back meet in one pass;
+    // otherwise the spectrum is left in buf0
+    const bool turn = !MULTI && !a.unit_input && (a.md[s][0].op == kOpPupil || a.md[s][0].op == kOpAllPass);
+    if (!turn && !a.unit_input) {
+        fft_pass_range<N, L, false, LAST, LAST + 1, GRP>(buf0, a.tw);
+        if constexpr (GRP == kSyncLine) __syncthreads();  // every line done before any thread reads another's
     }
     for (int m = 0; m < K; ++m) {
         const ModeDev md = live_mode(a.md[s][m]);
@@ -441,20 +448,23 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
         }
         float2 *Qm = a.w.Q + (((size_t)s * K + m) * geo.nblocks + bk) * N * B;
         if (md.op == kOpPupil || md.op == kOpAllPass) {
-            // the transfer function is applied as the first inverse pass
-            // loads the spectrum (in place when buf1 is buf0)
-            auto ld = [&](int c, int y) -> float2 {
+            auto filter = [&](int c, int y, float2 v) -> float2 {
                 if (c < B) {
                     const int2 ch = chords[m * L + c];
                     const int fy = y < N / 2 ? y : y - N;
                     if (fy >= ch.x && fy <= ch.y) {
                         const int kx = bk * B + c;
-                        return cmul(buf0[c * LS + pad16(y)], transfer(md, kx < half ? kx : kx - W, fy));
+                        return cmul(v, transfer(md, kx < half ? kx : kx - W, fy));
                     }
                 }
                 return make_float2(0.f, 0.f);
             };
-            fft_first_pass<N, L, true, !MULTI, GRP>(buf1, ld);
+            if (!MULTI && turn)
+                fft_turn_pass<N, L, GRP>(buf1, a.tw, filter);
+            else
+                fft_t_first_pass<N, L, true, GRP>(buf1, a.tw, [&](int c, int y) -> float2 {
+                    return filter(c, y, buf0[c * LS + pad16(y)]);
+                });
         } else {
             if (md.op == kOpLoss) {
                 loss_columns<N>(a, s, bk, B, W, buf0, buf1);
@@ -473,13 +483,14 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
                 }
             }
             __syncthreads();
-            fft_pass_range<N, L, true, 0, 1>(buf1, a.tw);
+            fft_t_first_pass<N, L, true, GRP>(
+                buf1, a.tw, [&](int c, int y) -> float2 { return buf1[c * LS + pad16(y)]; });
         }
-        fft_pass_range<N, L, true, 1, fft_passes(N) - 1, GRP>(buf1, a.tw);
+        fft_t_mid_passes<N, L, true, GRP>(buf1, a.tw);
         if constexpr (GRP == kSyncLine) __syncthreads();
         // the last pass stores Q; consecutive threads take the block's
         // columns, so a warp writes whole rows of the block
-        fft_last_pass<N, L, true, L, kSyncCta>(buf1, a.tw, [&](int c, int y, float2 v) {
+        fft_t_last_pass<N, L, true, L, kSyncCta>(buf1, [&](int c, int y, float2 v) {
             if (c < B) Qm[(size_t)y * B + c] = v;
         });
         __syncthreads();
