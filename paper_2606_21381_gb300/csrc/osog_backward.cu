@@ -58,15 +58,15 @@ __device__ __forceinline__ float warp_sum8(float (&v)[8], int lane) {
 template <int N>
 constexpr int kGroup = fft_grouped(N) ? kSyncLine : kSyncCta;
 
-// Rows: the inverse transform's first pass takes Q from global memory and its
-// last hands 2 gI E to a second set, whose forward transform stores the result
-// over Q from its last pass.
+// Rows: the inverse transform's first pass takes Q from global memory, its last
+// multiplies by 2 gI and goes on as the first (transposed) pass of the forward
+// transform, whose last stores the result over Q.
 template <int N>
 __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant__ BwdRowsArgs a) {
     pdl_enter();
-    constexpr int L = set_elems(N) / N, LS = line_stride(N), G = kGroup<N>;
+    constexpr int L = set_elems(N) / N, G = kGroup<N>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *bufE = reinterpret_cast<float2 *>(smem_raw), *bufQ = bufE + L * LS;
+    float2 *bufE = reinterpret_cast<float2 *>(smem_raw);
     const Geometry &geo = a.geo;
     const int sm = blockIdx.y, K = a.K, R = geo.R, B = geo.B, lb = ilog2(B), H = geo.H;
     const int y0 = blockIdx.x * R;
@@ -80,18 +80,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant_
     });
     fft_pass_range<N, L, true, 1, fft_passes(N) - 1, G>(bufE, a.tw);  // E_m rows
     const float *gI = a.grad_image + ((size_t)sm * H + y0) * N;
-    fft_last_pass<N, L, true, 0, G>(bufE, a.tw, [&](int l, int x, float2 v) {
+    fft_turn_pass<N, L, true, G>(bufE, a.tw, [&](int l, int x, float2 v) {
         const float g2 = l < R ? 2.f * gI[(size_t)l * N + x] : 0.f;
-        bufQ[l * LS + pad16(x)] = make_float2(g2 * v.x, g2 * v.y);
+        return make_float2(g2 * v.x, g2 * v.y);
     });
-    if constexpr (G == kSyncLine)
-        line_sync<L>(threadIdx.x / (kThreads / L));
-    else
-        __syncthreads();
-    // adjoint of the inverse row DFT
-    fft_pass_range<N, L, false, 0, fft_passes(N) - 1, G>(bufQ, a.tw);
+    fft_t_mid_passes<N, L, false, G>(bufE, a.tw);  // adjoint of the inverse row DFT
     if constexpr (G == kSyncLine) __syncthreads();
-    fft_last_pass<N, L, false, kRowFast, kSyncCta>(bufQ, a.tw, [&](int l, int kx, float2 v) {
+    fft_t_last_pass<N, L, false, kRowFast, kSyncCta>(bufE, [&](int l, int kx, float2 v) {
         const int fx = kx < N / 2 ? kx : kx - N;
         if (l < R && fx >= cr.x && fx <= cr.y)
             Qm[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))] = v;
@@ -163,18 +158,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
             }
         });
     }
-    // acc to bufE (read by its own outputs' threads only), in the same places
-    constexpr int P = fft_radix(N, fft_passes(N) - 1), NBF = N / P;
-#pragma unroll
-    for (int i = 0; i < OUT; ++i) {
-        int l, j;
-        butterfly_of<L, NBF, false>(i / P, l, j);
-        if (l < B) bufE[l * LS + pad16(j + (i % P) * NBF)] = acc[i];
-    }
-    __syncthreads();
-    // dL/dG (adjoint of the forward column DFT)
-    fft_pass_range<N, L, true, 0, fft_passes(N) - 1>(bufE, a.tw);
-    fft_last_pass<N, L, true, L, kSyncCta>(bufE, a.tw, [&](int c, int y, float2 v) {
+    // dL/dG (adjoint of the forward column DFT), from acc's own places
+    fft_t_first_pass<N, L, true, kSyncCta>(bufE, a.tw, [&](int, int, int i) { return acc[i]; });
+    fft_t_mid_passes<N, L, true, kSyncCta>(bufE, a.tw);
+    fft_t_last_pass<N, L, true, L, kSyncCta>(bufE, [&](int c, int y, float2 v) {
         if (c < B) Gb[(size_t)y * B + c] = v;
     });
 #pragma unroll
@@ -402,8 +389,8 @@ constexpr bool bwd_strip_wide(int W) { return W >= 1024; }
 template <int N>
 struct BwdLaunch {
     static cudaError_t rows(const BwdRowsArgs &a, cudaStream_t st) {
-        return launch_chain(k_bwd_rows<N>, dim3(a.geo.nstrips, a.S * a.K), kThreads,
-                            2 * strip_inverse_smem(N), st, a);
+        const dim3 grid(a.geo.nstrips, a.S * a.K);
+        return launch_chain(k_bwd_rows<N>, grid, kThreads, solo_smem<N>(grid, strip_inverse_smem(N)), st, a);
     }
     static cudaError_t column(const BwdColumnArgs &a, cudaStream_t st) {
         return launch_chain(k_bwd_column<N>, dim3(a.geo.nblocks, a.S), kThreads, bwd_column_smem(N),
@@ -414,24 +401,25 @@ struct BwdLaunch {
         if constexpr (bwd_strip_wide(N))
             if ((int)(grid.x * grid.y) <= kSms)
                 return launch_chain(k_bwd_strip<N, true>, grid, kWideThreads,
-                                    bwd_strip_smem(N, kWideThreads), st, a);
-        return launch_chain(k_bwd_strip<N, false>, grid, kThreads, bwd_strip_smem(N, kThreads), st, a);
+                                    solo_smem<N>(grid, bwd_strip_smem(N, kWideThreads)), st, a);
+        return launch_chain(k_bwd_strip<N, false>, grid, kThreads,
+                            solo_smem<N>(grid, bwd_strip_smem(N, kThreads)), st, a);
     }
     static cudaError_t prepare(int which) {
         if (which == 0)
             return cudaFuncSetAttribute(k_bwd_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        2 * (int)strip_inverse_smem(N));
+                                        prepared_smem<N>(strip_inverse_smem(N)));
         if (which == 1)
             return cudaFuncSetAttribute(k_bwd_column<N>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)bwd_column_smem(N));
         cudaError_t e = cudaFuncSetAttribute(k_bwd_strip<N, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bwd_strip_smem(N, kThreads));
+                                             prepared_smem<N>(bwd_strip_smem(N, kThreads)));
         if constexpr (bwd_strip_wide(N))
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k_bwd_strip<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bwd_strip_smem(N, kWideThreads));
+                                         prepared_smem<N>(bwd_strip_smem(N, kWideThreads)));
         return e;
     }
 };

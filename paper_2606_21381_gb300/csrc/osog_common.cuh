@@ -295,6 +295,24 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), bool early, dim3 grid, i
     if (e != cudaSuccess) (void)cudaGetLastError();  // reported once, by the return value
     return e;
 }
+// A grid of at most one CTA per SM, and more than half as many, whose CTAs would fit
+// in pairs asks for more than half of an SM's shared memory: dispatched while the
+// kernel before it still runs, its CTAs otherwise pair up on the SMs that come free
+// first and leave the others idle (one dense 1024 x 1024 image, loss and adjoint:
+// 114.9 -> 107.2 us of GPU time; 512 x 512, two modalities: 52.9 -> 51.1).  Kernels of
+// sets of 512 points and more: a raised limit alone (prepared_smem) took 0.6 us from
+// the four kernels of a 256 x 256 image, whose 64 CTAs have nothing to gain.
+constexpr size_t kSoloSmem = 116 * 1024;
+template <int N>
+inline int prepared_smem(size_t need) {
+    return (int)(N >= 512 && need < kSoloSmem ? kSoloSmem : need);
+}
+template <int N>
+inline size_t solo_smem(dim3 grid, size_t need) {
+    const long ctas = (long)grid.x * grid.y;
+    return ctas > kSms / 2 && ctas <= kSms ? (size_t)prepared_smem<N>(need) : need;
+}
+
 template <typename... KArgs>
 inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
                                 cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {

@@ -450,7 +450,8 @@ __device__ __forceinline__ void line_slots(float2 *buf, int l, int j, float2 *v)
     }
 }
 
-// First transposed pass, inputs from ld(l, i); ld may read any memory but other
+// First transposed pass, inputs from ld(l, i), or ld(l, i, the number of the input
+// among the thread's own: as in fft_last_pass); ld may read any memory but other
 // threads' slots of buf.  Ends with a barrier (the line's, grouped).
 template <int N, int L, bool INV, int G, class Ld>
 __device__ __forceinline__ void fft_t_first_pass(float2 *buf, const float2 *__restrict__ tw, Ld ld) {
@@ -466,7 +467,12 @@ __device__ __forceinline__ void fft_t_first_pass(float2 *buf, const float2 *__re
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             float2 v[P];
 #pragma unroll
-            for (int r = 0; r < P; ++r) v[r] = ld(l, j + r * NS);
+            for (int r = 0; r < P; ++r) {
+                if constexpr (std::is_invocable_v<Ld, int, int, int>)
+                    v[r] = ld(l, j + r * NS, q * P + r);
+                else
+                    v[r] = ld(l, j + r * NS);
+            }
             dft<P, INV>(v);
             apply_twiddles<P, INV, NS>(v, t + j);
             line_slots<N, L, PASS, false>(buf, l, j, v);
@@ -475,9 +481,9 @@ __device__ __forceinline__ void fft_t_first_pass(float2 *buf, const float2 *__re
     pass_sync<G, L>(l);
 }
 
-// The plan's last pass (forward), f(l, i, value) on its outputs, and the first
-// transposed pass of the inverse transform, in registers.
-template <int N, int L, int G, class F>
+// The plan's last pass, f(l, i, value) on its outputs, and the first transposed
+// pass of the transform back, in registers (INV: the first one is the inverse).
+template <int N, int L, bool INV, int G, class F>
 __device__ __forceinline__ void fft_turn_pass(float2 *buf, const float2 *__restrict__ tw, F f) {
     constexpr int PASS = fft_passes(N) - 1;
     constexpr int P = fft_radix(N, PASS), NS = fft_ns(N, PASS);
@@ -491,12 +497,12 @@ __device__ __forceinline__ void fft_turn_pass(float2 *buf, const float2 *__restr
         if (G == kSyncLine || TOT % kThreads == 0 || threadIdx.x + q * kThreads < TOT) {
             float2 v[P];
             line_slots<N, L, PASS, true>(buf, l, j, v);
-            apply_twiddles<P, false, NS>(v, t + j);
-            dft<P, false>(v);
+            apply_twiddles<P, INV, NS>(v, t + j);
+            dft<P, INV>(v);
 #pragma unroll
             for (int r = 0; r < P; ++r) v[r] = f(l, j + r * NS, v[r]);
-            dft<P, true>(v);
-            apply_twiddles<P, true, NS>(v, t + j);
+            dft<P, !INV>(v);
+            apply_twiddles<P, !INV, NS>(v, t + j);
             line_slots<N, L, PASS, false>(buf, l, j, v);
         }
     }

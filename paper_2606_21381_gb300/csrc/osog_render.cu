@@ -460,7 +460,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
                 return make_float2(0.f, 0.f);
             };
             if (!MULTI && turn)
-                fft_turn_pass<N, L, GRP>(buf1, a.tw, filter);
+                fft_turn_pass<N, L, false, GRP>(buf1, a.tw, filter);
             else
                 fft_t_first_pass<N, L, true, GRP>(buf1, a.tw, [&](int c, int y) -> float2 {
                     return filter(c, y, buf0[c * LS + pad16(y)]);
@@ -665,10 +665,12 @@ template <int N>
 struct StripFwdLaunch {
     static cudaError_t run(const StripArgs &a, StripMode mode, cudaStream_t st) {
         dim3 grid(a.geo.nstrips, a.S);
-        const size_t smem = strip_forward_smem(N), smem_opd = strip_forward_smem(N, true);
-        const size_t smem_fft = strip_inverse_smem(N);  // the set alone: no raster
+        const size_t smem = solo_smem<N>(grid, strip_forward_smem(N));
+        const size_t smem_opd = solo_smem<N>(grid, strip_forward_smem(N, true));
+        const size_t smem_fft = solo_smem<N>(grid, strip_inverse_smem(N));  // the set alone: no raster
         const bool wide = (int)(grid.x * grid.y) <= kSms;
-        const size_t smem_wide = strip_forward_smem(N) + raster_smem<kWideThreads>() - raster_smem<kThreads>();
+        const size_t smem_wide = solo_smem<N>(
+            grid, strip_forward_smem(N) + raster_smem<kWideThreads>() - raster_smem<kThreads>());
         if (mode == kStripRender && wide && a.geo.H == a.geo.W)
             return launch_chain(k_strip_forward<N, kStripRender, true, true>, grid, kWideThreads, smem_wide, st, a);
         else if (mode == kStripRender && wide)
@@ -691,29 +693,29 @@ struct StripFwdLaunch {
     static cudaError_t prepare() {
         const int smem = (int)strip_forward_smem(N), smem_opd = (int)strip_forward_smem(N, true);
         cudaError_t e = cudaFuncSetAttribute(k_strip_forward<N, kStripRender, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripRender, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripOpdOnly, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem_opd);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem_opd));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripFromMap, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripFromReal, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         const int smem_wide = smem + (int)(raster_smem<kWideThreads>() - raster_smem<kThreads>());
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
             e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripRender, true, true>
                                         : k_strip_forward<N, kStripRender, false, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem_wide);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem_wide));
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
             e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripFromPhase, true>
                                         : k_strip_forward<N, kStripFromPhase, false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)strip_inverse_smem(N));
+                                     prepared_smem<N>(strip_inverse_smem(N)));
         return e;
     }
 };
@@ -722,6 +724,7 @@ template <int N>
 struct ColumnLaunch {
     static cudaError_t run(const ColumnArgs &a, cudaStream_t st, size_t smem) {
         dim3 grid(a.geo.nblocks, a.S);
+        smem = solo_smem<N>(grid, smem);
         const bool sq = a.geo.H == a.geo.W;
         if (a.K > 1 && sq)
             return launch_chain(k_column<N, true, true>, grid, kThreads, smem, st, a);
@@ -736,10 +739,10 @@ struct ColumnLaunch {
         cudaError_t e = cudaSuccess;
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq) {
             e = cudaFuncSetAttribute(sq ? k_column<N, false, true> : k_column<N, false, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem1));
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(sq ? k_column<N, true, true> : k_column<N, true, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem2));
         }
         return e;
     }
@@ -749,6 +752,7 @@ template <int N>
 struct InverseLaunch {
     static cudaError_t run(const InverseArgs &a, cudaStream_t st, size_t smem) {
         dim3 grid(a.geo.nstrips, a.S * a.K);
+        smem = solo_smem<N>(grid, smem);
         if (a.geo.H == a.geo.W)
             return launch_chain(k_strip_inverse<N, true>, grid, kThreads, smem, st, a);
         else
@@ -756,10 +760,10 @@ struct InverseLaunch {
     }
     static cudaError_t prepare(size_t smem) {
         cudaError_t e = cudaFuncSetAttribute(k_strip_inverse<N, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_inverse<N, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
         return e;
     }
 };
