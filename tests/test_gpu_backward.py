@@ -261,3 +261,10 @@ def test_more_live_differentiable_renders_than_the_plan_remembers():
     for x, w in zip(xs, ws):
         gs, _ = r.backward(x.detach(), None, o, w)
         assert torch.equal(x.grad, gs)
+
+
+@pytest.mark.parametrize("H,W,modes", [(32, 32, 1), (32, 512, 3), (512, 32, 4), (64, 1024, 1), (1024, 64, 2),
+                                       (32, 2048, 1), (2048, 32, 1)])
+def test_backward_at_every_transform_length(H, W, modes):
+    # rows and columns of every plan, and grids on both sides of 76 and 152 CTAs
+    test_backward_matches_oracle_adjoint(H, W, modes)

@@ -323,3 +323,18 @@ def test_row_spans_end_at_the_last_covered_pixel_centre(kind):
     soa[:5] = np.array(rows).T
     soa[5], soa[6], soa[7], soa[8] = 2.0, 0.04, 0.02, kind
     assert_opd_close(soa, scenes.optics(256, 256))
+
+
+@pytest.mark.parametrize("H", [32, 64, 128, 256, 512, 1024, 2048])
+def test_single_modality_columns_at_every_plan(H):
+    # one modality's columns turn in registers, several go through shared memory:
+    # against the oracle, and bit for bit the same image either way
+    W = 32 if H > 64 else 64
+    rng = np.random.default_rng(H)
+    soa = scenes.draw_particles(rng, 12, H, W, mu=(0.0, 0.02))
+    o = scenes.optics(H, W, modes=2, NA=0.5, defocus=0.7)
+    ref = oracle.render(soa, soa.shape[1], oracle.make_optics(**o))["images"]
+    one = gpu_render(soa, o)
+    assert_images_close(one, ref, o)
+    both = gpu_render(soa, {**o, "modes": 3})
+    assert np.array_equal(both[1], one[0])
