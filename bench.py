@@ -144,7 +144,8 @@ def ncu_traffic(kernel: str):
 
 
 RENDER_SOURCES = ("osog_api.cu", "osog_bin.cu", "osog_render.cu", "osog_common.cuh",
-                  "osog_fft.cuh", "osog_strip.cuh", "osog_kernels.h")
+                  "osog_fft.cuh", "osog_strip.cuh", "osog_kernels.h", "osog_ff.h",
+                  "osog_pupil.h")
 
 
 def ncu_instructions(kernel: str):

@@ -73,7 +73,7 @@ __device__ bool setup_planes(const Work &w, int off, int m, double c, double s, 
     return true;
 }
 
-// Setup of one particle: validation, float-float record, bounding rect.
+// Setup of one particle: validation, records, bounding rect.
 __device__ Rect setup_particle(const float *soa, int64_t ld, int p, const SceneDev &sc,
                                const Geometry &geo, const Work &w) {
     int32_t *status = w.status;

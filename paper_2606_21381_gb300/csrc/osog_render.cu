@@ -36,7 +36,7 @@ __device__ __forceinline__ void strip_forward_item(const StripArgs &a, int s, in
     constexpr int LS = line_stride(N);
     constexpr int ACC = MODE == kStripOpdOnly ? kAccOpd : kAccPhase;
     float2 *buf = reinterpret_cast<float2 *>(smem_raw);
-    // accumulators: one uint2 per padded slot (phase mode) or two int64 (OPD mode)
+    // accumulators: two 32-bit words (PhaseSlot) or two int64 (OpdSlot) per pixel
     unsigned char *scratch = smem_raw + (ACC == kAccOpd ? 2 : 1) * L * LS * sizeof(float2);
     const Geometry &geo = a.geo;
     const int R = SQ ? sq_rb(N) : geo.R;
