@@ -117,14 +117,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
         return;
     }
     float2 *Gb = a.w.G + ((size_t)s * geo.nblocks + bk) * N * B;
-    load_block<N>(bufE, Gb, geo, bk, cr);
-    load_block<N>(bufZ, a.w.Q + (((size_t)s * K) * geo.nblocks + bk) * N * B, geo, bk, cr);
+    // The first pass of a block's columns, read from its global layout: as a copy to
+    // shared memory and a pass the kernel took 19.3 us on a 1024 x 1024 image and the
+    // whole adjoint 106.2 us; so 104.8 (107.4 with the strips' copy of G, too).
+    auto first_pass = [&](float2 *buf, const float2 *src) {
+        fft_first_pass<N, L, false, false, kSyncCta, L>(buf, [&](int c, int y) -> float2 {
+            const int kx = bk * B + c, fx = kx < half ? kx : kx - geo.W;
+            return c < B && fx >= cr.x && fx <= cr.y ? src[(size_t)y * B + c] : make_float2(0.f, 0.f);
+        });
+    };
     for (int j = threadIdx.x; j < K * B; j += kThreads) {  // this block's chords
         const int m = j >> lb, c = j & (B - 1), kx = bk * B + c;
         chords[m * L + c] = mode_chord(a.md[s][m], kx < half ? kx : kx - geo.W, N);
     }
-    __syncthreads();
-    fft_lines<N, L, false>(bufE, a.tw);  // E^ of the block's columns
+    first_pass(bufE, Gb);
+    first_pass(bufZ, a.w.Q + (((size_t)s * K) * geo.nblocks + bk) * N * B);
+    fft_pass_range<N, L, false, 1, fft_passes(N)>(bufE, a.tw);  // E^ of the block's columns
     constexpr int OUT = fft_last_outputs<N, L>();
     float2 acc[OUT];
 #pragma unroll
@@ -134,11 +142,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constan
         const ModeDev md = live_mode(a.md[s][m]);
         if (m > 0) {
             __syncthreads();  // the modality before has read bufZ
-            load_block<N>(bufZ, a.w.Q + (((size_t)s * K + m) * geo.nblocks + bk) * N * B, geo, bk, cr);
-            __syncthreads();
+            first_pass(bufZ, a.w.Q + (((size_t)s * K + m) * geo.nblocks + bk) * N * B);
         }
         // dL/dZ_m (adjoint of the inverse column DFT)
-        fft_pass_range<N, L, false, 0, fft_passes(N) - 1>(bufZ, a.tw);
+        fft_pass_range<N, L, false, 1, fft_passes(N) - 1>(bufZ, a.tw);
         fft_last_pass<N, L, false, 0, kSyncCta>(bufZ, a.tw, [&](int c, int y, float2 gz, int i) {
             if (c >= B) return;
             const int kx = bk * B + c;
@@ -202,13 +209,20 @@ k_bwd_strip(const __grid_constant__ BwdStripArgs a) {
     const SceneDev &sc = a.sc[s];
     const int2 cr = a.w.hull[s];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (!WIDE || threadIdx.x < kThreads)
-        load_strip_blocked<N>(bufG, a.w.G + (size_t)s * geo.H * N, geo, y0, cr);
     float4 *o4 = reinterpret_cast<float4 *>(bufO);
     for (int i = threadIdx.x; i < geo.R * LS / 2; i += NT) o4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    if (!WIDE || threadIdx.x < kThreads)
-        fft_lines<N, L, true, WIDE ? kSyncThreads : kSyncCta>(bufG, a.tw);  // dL/dE
+    if (!WIDE || threadIdx.x < kThreads) {  // dL/dE (the raster's barriers order it and the zeros)
+        constexpr int G = WIDE ? kSyncThreads : kSyncCta;
+        const int B = geo.B, lb = ilog2(B), H = geo.H, R = geo.R;
+        const float2 *Gs = a.w.G + (size_t)s * H * N;
+        fft_first_pass<N, L, true, false, G, kRowFast>(bufG, [&](int l, int kx) -> float2 {
+            const int fx = kx < N / 2 ? kx : kx - N;
+            return l < R && fx >= cr.x && fx <= cr.y
+                       ? Gs[((size_t)(kx >> lb) * H + y0 + l) * B + (kx & (B - 1))]
+                       : make_float2(0.f, 0.f);
+        });
+        fft_pass_range<N, L, true, 1, fft_passes(N), G>(bufG, a.tw);
+    }
     // OPD and ATT as fixed-point accumulators in bufO (its staging shares
     // the gather's staging area below, used only after the raster)
     raster_strip<N, kAccPhase, NT>(geo, a.w, sc, s, y0, geo.R, bufO,

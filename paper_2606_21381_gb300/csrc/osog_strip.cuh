@@ -586,54 +586,6 @@ __device__ __forceinline__ float2 transfer(const ModeDev &md, int fx, int fy) {
 }
 
 // ---------------------------------------------------------------- layouts
-// A row-strip [y0, y0 + R) of a column-blocked array [W/B][H][B] (complex)
-// to the padded shared lines of an N = W point set.  Columns whose signed
-// frequency lies outside [cr.x, cr.y] (no pupil passes them) load as zero.
-template <int N, bool SQ = false>
-__device__ __forceinline__ void load_strip_blocked(float2 *buf, const float2 *src,
-                                                   const Geometry &geo, int y0, int2 cr) {
-    constexpr int LS = line_stride(N);
-    const int R = SQ ? sq_rb(N) : geo.R, B = SQ ? sq_rb(N) : geo.B;
-    const int lb = SQ ? clog2(sq_rb(N)) : ilog2(B), lr = SQ ? clog2(sq_rb(N)) : ilog2(R);
-    const int RN = R * N, H = SQ ? N : geo.H;
-    float2 v[ept(N)];
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        const int c = e & (B - 1), r = (e >> lb) & (R - 1), bk = e >> (lb + lr);
-        const int kx = bk * B + c, fx = kx < N / 2 ? kx : kx - N;
-        v[i] = e < RN && fx >= cr.x && fx <= cr.y ? src[((size_t)bk * H + y0 + r) * B + c]
-                                                  : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        const int c = e & (B - 1), r = (e >> lb) & (R - 1), bk = e >> (lb + lr);
-        if (e < RN) buf[r * LS + pad16(bk * B + c)] = v[i];
-    }
-}
-
-// A column block (B columns, N = H rows, contiguous [H][B]) to the padded
-// shared lines (line c = column c).  Inactive columns load as zero.
-template <int N>
-__device__ __forceinline__ void load_block(float2 *buf, const float2 *src, const Geometry &geo,
-                                           int bk, int2 cr) {
-    constexpr int LS = line_stride(N);
-    const int B = geo.B, lb = ilog2(B), NB = N * B, half = geo.W / 2;
-    float2 v[ept(N)];
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        const int kx = bk * B + (e & (B - 1)), fx = kx < half ? kx : kx - geo.W;
-        v[i] = e < NB && fx >= cr.x && fx <= cr.y ? src[e] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int i = 0; i < ept(N); ++i) {
-        const int e = threadIdx.x + i * kThreads;
-        if (e < NB) buf[(e & (B - 1)) * LS + pad16(e >> lb)] = v[i];
-    }
-}
-
 // True if some column of block bk has a signed frequency inside cr.
 __device__ __forceinline__ bool block_active(const Geometry &geo, int bk, int2 cr) {
     const int u0 = bk * geo.B, u1 = u0 + geo.B - 1, half = geo.W / 2;
