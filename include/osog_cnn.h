@@ -17,7 +17,7 @@
  * (H + 2 pad - R) / stride + 1.  The matrix products run on the tensor cores
  * in BF16 with FP32 accumulation; every reduction runs in a fixed order.
  * All calls are asynchronous on `stream` and return OSOG_OK or
- * OSOG_ERR_INVALID_ARG (bad shape or NULL pointer) / OSOG_ERR_WORKSPACE /
+ * OSOG_ERR_INVALID_ARG (bad shape, NULL or misaligned pointer) / OSOG_ERR_WORKSPACE /
  * OSOG_ERR_CUDA.
  */
 #ifndef OSOG_CNN_H
@@ -44,7 +44,8 @@ int32_t osog_conv_out_w(const osog_conv_shape_t *shape);
 
 /* y = act(conv(x, w) + bias); relu = 1 applies max(0, .).  y is bf16 NHWC
  * [N][P][Q][K]; when y_f32 is not NULL the same values are also written as
- * fp32 (before rounding to bf16). */
+ * fp32 (before rounding to bf16).  x and w are 16-byte aligned, y at least 4-
+ * and y_f32 8-byte aligned (16 for the fastest kernels). */
 int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const uint16_t *w,
                         const float *bias, int32_t relu, uint16_t *y, float *y_f32,
                         osog_stream_t stream);

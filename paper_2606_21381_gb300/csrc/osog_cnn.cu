@@ -17,6 +17,8 @@
 // in a fixed order, so every result is bitwise reproducible.
 #include <cuda_bf16.h>
 
+#include <initializer_list>
+
 #include "osog_cnn.h"
 #include "osog_conv_tma.h"
 
@@ -816,6 +818,13 @@ int status_of(cudaError_t e) { return e == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA
 // (1, default) or the warp-level MMA kernel (0).
 int g_use_tcgen05 = 1;
 
+// True if every pointer is a multiple of `bytes` (a NULL is).
+bool aligned(uintptr_t bytes, std::initializer_list<const void *> ptrs) {
+    uintptr_t any = 0;
+    for (const void *p : ptrs) any |= reinterpret_cast<uintptr_t>(p);
+    return any % bytes == 0;
+}
+
 const __nv_bfloat16 *bf(const uint16_t *p) { return reinterpret_cast<const __nv_bfloat16 *>(p); }
 __nv_bfloat16 *bf(uint16_t *p) { return reinterpret_cast<__nv_bfloat16 *>(p); }
 
@@ -829,7 +838,7 @@ int32_t osog_conv_out_w(const osog_conv_shape_t *s) { return shape_ok(s) ? geo_o
 int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const uint16_t *w,
                         const float *bias, int32_t relu, uint16_t *y, float *y_f32,
                         osog_stream_t stream) {
-    if (!shape_ok(shape) || !x || !w || !bias || !y) return OSOG_ERR_INVALID_ARG;
+    if (!shape_ok(shape) || !x || !w || !bias || !y || !aligned(16, {x})) return OSOG_ERR_INVALID_ARG;
     Args a{};
     a.g = geo_of(shape);
     a.x = bf(x);
@@ -843,12 +852,15 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
     a.Kred = a.g.R * a.g.S * a.g.C;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // reductions shorter than 128 stay on the warp-level MMA (the 8-channel
-    // first layer and the 1 x 1 head)
-    if (g_use_tcgen05 && a.Kred >= 128) {
+    // first layer and the 1 x 1 head).  The patch kernels store 16-byte vectors;
+    // k_conv_gemm takes the outputs that are not so aligned (pairs of columns).
+    if (g_use_tcgen05 && a.Kred >= 128 && aligned(16, {w, y, y_f32})) {
         const cudaError_t e = conv_forward_tma(a.g, x, w, bias, relu != 0, y, y_f32, st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
-    if (!y_f32 && fits_c8(a.g)) return status_of(launch_conv_c8(a, st));
+    if (!y_f32 && fits_c8(a.g) && aligned(16, {y}) && aligned(4, {w}))
+        return status_of(launch_conv_c8(a, st));
+    if (!aligned(16, {w}) || !aligned(4, {y}) || !aligned(8, {y_f32})) return OSOG_ERR_INVALID_ARG;
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN);
     return status_of(launch_conv(k_conv_gemm<kFwd>, grid, NT, 0, st, a));
 }

@@ -74,3 +74,18 @@ def test_optics_struct_mirrors_header_layout():
     assert ctypes.sizeof(_lib.Optics) == 8 + 5 * 8 + 8 + 6 * 8
     assert _lib.Optics.modes.offset == 48
     assert _lib.Optics.oblique_frac.offset == 56
+
+
+@pytest.mark.parametrize("shape", [(2, 20, 20, 8, 16, 3, 3, 1, 1), (2, 20, 20, 32, 16, 3, 3, 1, 1),
+                                   (2, 20, 20, 16, 16, 1, 1, 1, 0)])
+def test_conv_forward_refuses_misaligned_pointers_on_the_host(L, shape):
+    # what no kernel can read or write as it is aligned is refused before any
+    # launch (the addresses are never touched)
+    s, ok = _lib.ConvShape(*shape), 0x10000
+    good = dict(x=ok, w=ok, bias=ok, y=ok, y32=ok)
+    for name, off in (("x", 8), ("w", 2), ("y", 2), ("y32", 4)):
+        p = {**good, name: ok + off}
+        if name == "w":
+            p["y"] = ok + 4  # neither 16-byte vectors of filters nor of outputs
+        assert L.osog_conv2d_forward(ctypes.byref(s), p["x"], p["w"], p["bias"], 0, p["y"],
+                                     p["y32"], None) == 1, name

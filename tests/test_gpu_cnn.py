@@ -221,3 +221,36 @@ def test_forward_without_the_fp32_copy_gives_the_same_bits(cnn, shape):
     bd = torch.from_numpy(b).to(dev)
     y, _ = cnn.conv2d(xd, wd, bd, shape[7], shape[8], True, want_f32=True)
     assert torch.equal(cnn.conv2d(xd, wd, bd, shape[7], shape[8], True), y)
+
+
+def _at(shape, dtype, offset):
+    """A contiguous CUDA tensor `offset` elements past a 16-byte boundary."""
+    flat = torch.empty(int(np.prod(shape)) + 16, dtype=dtype, device="cuda")
+    return flat[offset:offset + int(np.prod(shape))].view(shape)
+
+
+@pytest.mark.parametrize("shape", [
+    (1, 20, 33, 8, 24, 3, 3, 1, 1),   # eight channels, nine taps
+    (1, 20, 18, 32, 40, 3, 3, 1, 1),  # tcgen05
+    (1, 9, 13, 32, 8, 1, 1, 1, 0),    # a short reduction
+])
+def test_forward_into_outputs_that_are_only_pair_aligned(cnn, shape):
+    # y 4-byte and y_f32 8-byte aligned: no kernel that stores 16-byte vectors
+    from paper_2606_21381_gb300 import _lib
+    dev = torch.device("cuda")
+    x, w, b, _ = _inputs(shape, 1)
+    xd, x64 = _bf16(x, dev)
+    wd, w64 = _bf16(w, dev)
+    bd = torch.from_numpy(b).to(dev)
+    want = ref.conv_forward(x64, w64, b.astype(np.float64), shape[7], shape[8], True)
+    scale = np.abs(want).max()
+    s = cnn.conv_shape(xd, wd, shape[7], shape[8])
+    for want32 in (False, True):
+        y = _at(want.shape, torch.bfloat16, 2)
+        y32 = _at(want.shape, torch.float32, 2) if want32 else None
+        assert _lib.lib().osog_conv2d_forward(s, cnn._ptr(xd), cnn._ptr(wd), cnn._ptr(bd), 1, cnn._ptr(y),
+                                              cnn._ptr(y32), cnn._stream(dev)) == 0
+        got = y.to(torch.float32).cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
+        if want32:
+            assert np.abs(y32.cpu().numpy() - want).max() <= 1e-5 * scale
