@@ -55,7 +55,10 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
  * gradient at the convolution's output (after its own ReLU derivative).
  * w_t is a workspace of R*S*K*C bf16 for this call's use (the warp-level MMA
  * engine reorders the filters to [C][R][S][K] in it; the tcgen05 engine reads
- * them as they are and leaves it untouched). */
+ * them as they are and leaves it untouched).  dy is 16-byte aligned, x_act and
+ * dx at least 4-byte aligned and w at any address; with w, x_act or dx not
+ * 16-byte aligned the call runs on the warp-level MMA engine, whose w_t is
+ * 16-byte aligned. */
 int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy,
                               const uint16_t *w, const uint16_t *x_act, uint16_t *dx,
                               uint16_t *w_t, osog_stream_t stream);

@@ -868,13 +868,16 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
 int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy,
                               const uint16_t *w, const uint16_t *x_act, uint16_t *dx,
                               uint16_t *w_t, osog_stream_t stream) {
-    if (!shape_ok(shape) || !dy || !w || !dx || !w_t) return OSOG_ERR_INVALID_ARG;
+    if (!shape_ok(shape) || !dy || !w || !dx || !w_t || !aligned(16, {dy})) return OSOG_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const Geo g = geo_of(shape);
-    if (g_use_tcgen05) {  // reads the filters in place: w_t stays untouched
+    // reads the filters in place, by TMA: w_t stays untouched.  Filters at any
+    // address are transposed element by element into w_t below.
+    if (g_use_tcgen05 && aligned(16, {w, x_act, dx})) {
         const cudaError_t e = conv_dgrad_tma(g, dy, w, x_act, dx, st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
+    if (!aligned(16, {w_t}) || !aligned(4, {x_act, dx})) return OSOG_ERR_INVALID_ARG;
     const int64_t nw = (int64_t)g.K * g.R * g.S * g.C;
     k_filter_transpose<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(bf(w), g.K, g.R * g.S, g.C, bf(w_t));
     Args a{};

@@ -89,3 +89,15 @@ def test_conv_forward_refuses_misaligned_pointers_on_the_host(L, shape):
             p["y"] = ok + 4  # neither 16-byte vectors of filters nor of outputs
         assert L.osog_conv2d_forward(ctypes.byref(s), p["x"], p["w"], p["bias"], 0, p["y"],
                                      p["y32"], None) == 1, name
+
+
+@pytest.mark.parametrize("shape", [(2, 20, 20, 32, 16, 3, 3, 1, 1), (2, 20, 20, 16, 16, 3, 3, 2, 1)])
+def test_conv_backward_data_refuses_misaligned_pointers_on_the_host(L, shape):
+    s, ok = _lib.ConvShape(*shape), 0x10000
+    good = dict(dy=ok, w=ok, x_act=ok, dx=ok, w_t=ok)
+    for name, off in (("dy", 8), ("x_act", 2), ("dx", 2), ("w_t", 8)):
+        p = {**good, name: ok + off}
+        if name == "w_t":
+            p["w"] = ok + 2  # the engine that transposes the filters
+        assert L.osog_conv2d_backward_data(ctypes.byref(s), p["dy"], p["w"], p["x_act"], p["dx"],
+                                           p["w_t"], None) == 1, name

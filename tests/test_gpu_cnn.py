@@ -254,3 +254,30 @@ def test_forward_into_outputs_that_are_only_pair_aligned(cnn, shape):
         assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * scale)
         if want32:
             assert np.abs(y32.cpu().numpy() - want).max() <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("shape", [(1, 21, 18, 40, 24, 3, 3, 1, 1), (2, 15, 17, 16, 40, 3, 3, 2, 1)])
+@pytest.mark.parametrize("what", ["w", "x_act", "dx"])
+def test_backward_data_of_operands_that_are_not_16_byte_aligned(cnn, shape, what):
+    # filters 2 bytes, the mask and the result 4 bytes past a 16-byte boundary
+    from paper_2606_21381_gb300 import _lib
+    dev = torch.device("cuda")
+    x, w, b, dy = _inputs(shape, 2)
+    xd, x64 = _bf16(x, dev)
+    wd, w64 = _bf16(w, dev)
+    dyd, dy64 = _bf16(dy, dev)
+    want, _, _ = ref.conv_grads(x64, w64, b.astype(np.float64), shape[7], shape[8], dy64)
+    want = want * (x64 > 0)
+    dx = torch.empty_like(xd)
+    if what == "w":
+        wd = _at(wd.shape, torch.bfloat16, 1).copy_(wd)
+    elif what == "x_act":
+        xd = _at(xd.shape, torch.bfloat16, 2).copy_(xd)
+    else:
+        dx = _at(xd.shape, torch.bfloat16, 2)
+    s = cnn.conv_shape(xd, wd, shape[7], shape[8])
+    w_t = torch.empty(wd.numel(), dtype=torch.bfloat16, device=dev)
+    assert _lib.lib().osog_conv2d_backward_data(s, cnn._ptr(dyd), cnn._ptr(wd), cnn._ptr(xd), cnn._ptr(dx),
+                                                cnn._ptr(w_t), cnn._stream(dev)) == 0
+    got = dx.to(torch.float32).cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * np.abs(want).max())
