@@ -66,7 +66,8 @@ int osog_conv2d_backward_data(const osog_conv_shape_t *shape, const uint16_t *dy
 /* dw = sum over pixels of dy (x) and dbias = sum of dy, by a split
  * reduction over pixel chunks followed by a fixed-order sum.  ws must hold
  * osog_conv2d_backward_filter_workspace(shape) bytes (enough for either
- * engine, see osog_conv_use_tcgen05). */
+ * engine, see osog_conv_use_tcgen05).  dy and x are 16-byte aligned, ws at
+ * least 8- and dw and dbias 4-byte aligned (16 for the fastest kernels). */
 size_t osog_conv2d_backward_filter_workspace(const osog_conv_shape_t *shape);
 int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *dy,
                                 const uint16_t *x, float *dw, float *dbias, void *ws,

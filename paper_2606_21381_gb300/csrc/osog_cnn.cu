@@ -935,7 +935,7 @@ size_t osog_conv2d_backward_filter_workspace(const osog_conv_shape_t *shape) {
 int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *dy,
                                 const uint16_t *x, float *dw, float *dbias, void *ws,
                                 size_t ws_bytes, osog_stream_t stream) {
-    if (!shape_ok(shape) || !dy || !x || !dw || !dbias) return OSOG_ERR_INVALID_ARG;
+    if (!shape_ok(shape) || !dy || !x || !dw || !dbias || !aligned(16, {dy, x})) return OSOG_ERR_INVALID_ARG;
     if (!ws || ws_bytes < osog_conv2d_backward_filter_workspace(shape)) return OSOG_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const Geo g = geo_of(shape);
@@ -947,17 +947,17 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     a.M = g.K;
     a.Ncols = g.R * g.S * g.C;
     a.Kred = g.N * g.P * g.Q;
-    const bool aligned = ((reinterpret_cast<uintptr_t>(ws) | reinterpret_cast<uintptr_t>(dw) |
-                           reinterpret_cast<uintptr_t>(dbias)) & 15) == 0;  // of k_sum_parts
-    if (aligned && fits_c8(g) && g.K <= 64) {
+    const bool vectors = aligned(16, {ws, dw, dbias});  // of k_sum_parts
+    if (vectors && fits_c8(g) && g.K <= 64) {
         cudaError_t e = g.K <= 32 ? launch_wgrad_c8<2>(a, st) : launch_wgrad_c8<4>(a, st);
         if (e == cudaSuccess) e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, st);
         return status_of(e);
     }
-    if (g_use_tcgen05 && aligned) {
+    if (g_use_tcgen05 && vectors) {
         const cudaError_t e = conv_wgrad_tma(g, dy, x, dw, dbias, static_cast<float *>(ws), st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
+    if (!aligned(8, {ws}) || !aligned(4, {dw, dbias})) return OSOG_ERR_INVALID_ARG;
     const int splits = splits_of(g);
     dim3 grid((a.M + BM - 1) / BM, (a.Ncols + BN - 1) / BN, splits);
     k_conv_gemm<kWgrad><<<grid, NT, 0, st>>>(a);

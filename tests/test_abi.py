@@ -101,3 +101,14 @@ def test_conv_backward_data_refuses_misaligned_pointers_on_the_host(L, shape):
             p["w"] = ok + 2  # the engine that transposes the filters
         assert L.osog_conv2d_backward_data(ctypes.byref(s), p["dy"], p["w"], p["x_act"], p["dx"],
                                            p["w_t"], None) == 1, name
+
+
+@pytest.mark.parametrize("shape", [(2, 20, 20, 8, 16, 3, 3, 1, 1), (2, 20, 20, 32, 16, 3, 3, 1, 1)])
+def test_conv_backward_filter_refuses_misaligned_pointers_on_the_host(L, shape):
+    s, ok = _lib.ConvShape(*shape), 0x10000
+    need = L.osog_conv2d_backward_filter_workspace(ctypes.byref(s))
+    good = dict(dy=ok, x=ok, dw=ok, db=ok, ws=ok)
+    for name, off in (("dy", 8), ("x", 8), ("dw", 2), ("db", 2), ("ws", 4)):
+        p = {**good, name: ok + off}
+        assert L.osog_conv2d_backward_filter(ctypes.byref(s), p["dy"], p["x"], p["dw"], p["db"],
+                                             p["ws"], need, None) == 1, name
