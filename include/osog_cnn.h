@@ -82,10 +82,8 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
  * tcgen05 selected, forward convolutions whose reduction R S C is below 128
  * still run on the warp-level MMA, and so do filter gradients whose ws, dw or
  * dbias is not 16-byte aligned; layers of 8 input channels and nine or ten
- * taps run on the warp-level MMA in either case.  (Filter gradients pair output
- * pixels past the image, as zeros, with the activations there: an infinite
- * activation at the image's edge can make further entries of dw NaN.)  The
- * switch also covers osog_conv2d_backward_filter. */
+ * taps run on the warp-level MMA in either case.  The switch also covers
+ * osog_conv2d_backward_filter. */
 void osog_conv_use_tcgen05(int32_t enable);
 
 /* Synchronise `stream` and report a latched device error of the

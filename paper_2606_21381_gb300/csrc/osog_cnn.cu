@@ -950,7 +950,9 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
     const bool vectors = aligned(16, {ws, dw, dbias});  // of k_sum_parts
     if (vectors && fits_c8(g) && g.K <= 64) {
         cudaError_t e = g.K <= 32 ? launch_wgrad_c8<2>(a, st) : launch_wgrad_c8<4>(a, st);
-        if (e == cudaSuccess) e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, st);
+        const bool ragged = g.P % kC8GradRows || g.Q % kC8W;
+        if (e == cudaSuccess)
+            e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, ragged ? dy : nullptr, x, st);
         return status_of(e);
     }
     if (g_use_tcgen05 && vectors) {

@@ -714,14 +714,73 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
                      : "memory");
 }
 
-// out[i] = sum over z of part[z][i], i < count (out = dw) or count <= i < count
-// + extra (out2 = dbias), four outputs per thread (count and extra are
-// multiples of 8), the splits in order within each of kSumLanes interleaved
-// partial sums, which are then added in order.
+// Sums over the splits, out[i] = sum over z of part[z][i], i < count (out = dw) or
+// count <= i < count + extra (out2 = dbias), four outputs per thread (count and
+// extra are multiples of 8), the splits in order within each of kSumLanes
+// interleaved partial sums, which are then added in order.
+//
+// Tiles that reach past the image pair its missing output pixels, zeros of dY, with
+// whatever X holds there for other taps: 0 inf is NaN, in entries that those pixels
+// are no part of.  Only a product of a zero can do that, and only to make an entry
+// NaN; so where tiles are ragged (fix.dy set) a CTA that finds a NaN among its 128
+// entries adds them up again over the existing pixels alone, and keeps the new values
+// of the NaN ones (an entry whose own products give NaN stays so).  Sums without a
+// NaN, all but those of a diverged network, pay one vote; with them the pass takes
+// as long as a plain loop over dY and X.
 constexpr int kSumLanes = 8;
+struct EdgeFix {
+    const __nv_bfloat16 *dy, *x;  // dy NULL: no ragged tiles
+    Geo g;
+};
+__device__ __noinline__ float4 sum_of_pixels(const EdgeFix &f, int64_t i4, float4 (*red)[32]) {
+    const Geo &g = f.g;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t e = 4 * i4;
+    const int c = (int)(e % g.C), t = (int)(e / g.C), rs = t % (g.R * g.S), k = t / (g.R * g.S);
+    const int dh = rs / g.S - g.pad, dw = rs % g.S - g.pad;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int row = w; k < g.K && row < g.N * g.P; row += kSumLanes) {
+        const int n = row / g.P, h = (row - n * g.P) * g.stride + dh;
+        const __nv_bfloat16 *dy = f.dy + (size_t)row * g.Q * g.K + k;
+        const __nv_bfloat16 *x = f.x + ((size_t)n * g.H + h) * g.W * g.C + c;
+        const bool in = h >= 0 && h < g.H;
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < g.Q; ++q) {
+            const int v = q * g.stride + dw;
+            const float d = __bfloat162float(dy[(size_t)q * g.K]);
+            float2 a = make_float2(0.f, 0.f), b = a;  // padding
+            if (in && v >= 0 && v < g.W) {
+                const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(x + (size_t)v * g.C);
+                a = __bfloat1622float2(p[0]);
+                b = __bfloat1622float2(p[1]);
+            }
+            u.x = fmaf(d, a.x, u.x);
+            u.y = fmaf(d, a.y, u.y);
+            u.z = fmaf(d, b.x, u.z);
+            u.w = fmaf(d, b.y, u.w);
+        }
+        s.x += u.x;
+        s.y += u.y;
+        s.z += u.z;
+        s.w += u.w;
+    }
+    __syncthreads();  // red is read
+    red[w][lane] = s;
+    __syncthreads();
+    s = red[0][lane];
+    for (int l = 1; l < kSumLanes; ++l) {
+        const float4 v = red[l][lane];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    return s;
+}
+
 __global__ void __launch_bounds__(32 * kSumLanes)
 k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, float4 *out,
-            float4 *out2) {
+            float4 *out2, const __grid_constant__ EdgeFix fix) {
     __shared__ float4 red[kSumLanes][32];
     pdl_enter();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -747,6 +806,18 @@ k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, floa
             s.z += v.z;
             s.w += v.w;
         }
+    }
+    if (fix.dy) {
+        const bool nan = w == 0 && i < count4 && (isnan(s.x) || isnan(s.y) || isnan(s.z) || isnan(s.w));
+        if (__syncthreads_or(nan)) {
+            const float4 v = sum_of_pixels(fix, i, red);
+            s.x = isnan(s.x) ? v.x : s.x;
+            s.y = isnan(s.y) ? v.y : s.y;
+            s.z = isnan(s.z) ? v.z : s.z;
+            s.w = isnan(s.w) ? v.w : s.w;
+        }
+    }
+    if (w == 0 && i < row) {
         if (i < count4)
             out[i] = s;
         else
@@ -1133,15 +1204,18 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
     if (e != cudaSuccess) return e;
     e = ch == 64 ? launch_wgrad<64>(mdy, mx, a, st) : launch_wgrad<32>(mdy, mx, a, st);
     if (e != cudaSuccess) return e;
-    return conv_sum_parts(g, a.splits, ws, dw, dbias, st);
+    const bool ragged = g.P % kTileH || g.Q % kTileW;
+    return conv_sum_parts(g, a.splits, ws, dw, dbias, ragged ? dy : nullptr, x, st);
 }
 
 cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
-                           cudaStream_t st) {
+                           const uint16_t *ragged_dy, const uint16_t *x, cudaStream_t st) {
     const int64_t count4 = (int64_t)g.K * g.R * g.S * g.C / 4, extra4 = g.K / 4;
     return launch_conv(k_sum_parts, dim3((unsigned)((count4 + extra4 + 31) / 32)), 32 * kSumLanes, 0, st,
                        reinterpret_cast<const float4 *>(part), splits, count4, extra4,
-                       reinterpret_cast<float4 *>(dw), reinterpret_cast<float4 *>(dbias));
+                       reinterpret_cast<float4 *>(dw), reinterpret_cast<float4 *>(dbias),
+                       EdgeFix{reinterpret_cast<const __nv_bfloat16 *>(ragged_dy),
+                               reinterpret_cast<const __nv_bfloat16 *>(x), g});
 }
 
 cudaError_t conv_tma_take_status(int *timed_out) {

@@ -42,9 +42,10 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
                            float *dbias, float *ws, cudaStream_t st);
 
 // dw, dbias = the sums over the splits of part [splits][K R S C + K], in order
-// (all 16-byte aligned).
+// (all 16-byte aligned).  ragged_dy: dY when the tiles that the partial sums come
+// from reach past the image, else NULL (see k_sum_parts).
 cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
-                           cudaStream_t st);
+                           const uint16_t *ragged_dy, const uint16_t *x, cudaStream_t st);
 
 // Latched status of the bounded waits (read and cleared), and the
 // failure-detection hook (osog_conv_test_wait_limit).

@@ -281,3 +281,33 @@ def test_backward_data_of_operands_that_are_not_16_byte_aligned(cnn, shape, what
                                                 cnn._ptr(w_t), cnn._stream(dev)) == 0
     got = dx.to(torch.float32).cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-5 * np.abs(want).max())
+
+
+@pytest.mark.parametrize("shape", [
+    (1, 21, 18, 40, 24, 3, 3, 1, 1),
+    (2, 40, 37, 16, 136, 3, 3, 2, 1),
+    (1, 9, 30, 72, 16, 5, 2, 1, 2),
+    (2, 35, 70, 8, 40, 3, 3, 1, 1),  # eight channels, nine taps
+    (1, 67, 41, 8, 24, 3, 3, 2, 1),
+    (1, 32, 16, 24, 16, 3, 3, 1, 1),  # whole tiles
+])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_filter_gradient_of_activations_that_are_not_finite(cnn, shape, value):
+    # at the corners and edges of the image: exactly the entries that such a pixel
+    # is a factor of are not finite, the others are as accurate as ever
+    dev = torch.device("cuda")
+    x, w, b, dy = _inputs(shape, 3)
+    H, W = shape[1:3]
+    for c, (h, v) in enumerate([(0, 0), (H - 1, W - 1), (H - 1, W // 2), (H // 2, W - 1), (H - 2, W - 2)]):
+        x[0, h, v, c] = value
+    xd, x64 = _bf16(x, dev)
+    _, w64 = _bf16(w, dev)
+    dyd, dy64 = _bf16(dy, dev)
+    dw, db = cnn.conv2d_backward_filter(dyd, xd, w.shape, shape[7], shape[8])
+    _, want_w, want_b = ref.conv_grads(x64, w64, b.astype(np.float64), shape[7], shape[8], dy64)
+    got_w = dw.cpu().numpy().astype(np.float64)
+    fin = np.isfinite(want_w)
+    assert np.array_equal(np.isfinite(got_w), fin)
+    np.testing.assert_array_equal(got_w[~fin], want_w[~fin])
+    assert np.abs(got_w[fin] - want_w[fin]).max() <= 1e-5 * np.abs(want_w[fin]).max() * np.sqrt(dy.size / dy.shape[-1])
+    assert np.abs(db.cpu().numpy() - want_b).max() <= 1e-5 * np.abs(dy64).sum(axis=(0, 1, 2)).max()
