@@ -952,7 +952,8 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
         cudaError_t e = g.K <= 32 ? launch_wgrad_c8<2>(a, st) : launch_wgrad_c8<4>(a, st);
         const bool ragged = g.P % kC8GradRows || g.Q % kC8W;
         if (e == cudaSuccess)
-            e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, ragged ? dy : nullptr, x, st);
+            e = conv_sum_parts(g, splits_c8(g), a.part, dw, dbias, ragged ? dy : nullptr, x, kC8GradRows,
+                               kC8W, st);
         return status_of(e);
     }
     if (g_use_tcgen05 && vectors) {

@@ -721,64 +721,81 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
 //
 // Tiles that reach past the image pair its missing output pixels, zeros of dY, with
 // whatever X holds there for other taps: 0 inf is NaN, in entries that those pixels
-// are no part of.  Only a product of a zero can do that, and only to make an entry
-// NaN; so where tiles are ragged (fix.dy set) a CTA that finds a NaN among its 128
-// entries adds them up again over the existing pixels alone, and keeps the new values
-// of the NaN ones (an entry whose own products give NaN stays so).  Sums without a
-// NaN, all but those of a diverged network, pay one vote; with them the pass takes
-// as long as a plain loop over dY and X.
+// are no part of.  Only a product of a zero can do that, and only to make a partial
+// sum NaN; so where tiles are ragged (RAGGED) a warp whose sum is NaN adds its splits
+// again, and takes the NaN entries of a split from the existing pixels of the
+// split's tiles (an entry whose own products give NaN stays so, and ends the loop).
+// Sums without a NaN, all but those of a diverged network, keep their bits and pay one
+// vote (33 images of 63 x 61, stride 2, 40 -> 72: 20.5 us with its products; all of X
+// NaN 152.  8 images of 255 x 249, 64 -> 64: 75.7; all NaN 142, one pixel infinite in
+// every channel 1360: its split's 3,300 pixels are walked by a warp for each 32 x 4
+// entries).
 constexpr int kSumLanes = 8;
 struct EdgeFix {
-    const __nv_bfloat16 *dy, *x;  // dy NULL: no ragged tiles
+    const __nv_bfloat16 *dy, *x;
     Geo g;
+    int tile_h, tile_w;
 };
-__device__ __noinline__ float4 sum_of_pixels(const EdgeFix &f, int64_t i4, float4 (*red)[32]) {
+__device__ __forceinline__ bool any_nan(float4 v) {
+    return isnan(v.x) || isnan(v.y) || isnan(v.z) || isnan(v.w);
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+// The entries e .. e + 3 of split z's partial sum v, the NaN ones (bad: this lane has
+// any) added up from the existing pixels.
+__device__ float4 split_of_pixels(const EdgeFix &f, int z, int splits, int64_t e, float4 v, bool bad) {
     const Geo &g = f.g;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t e = 4 * i4;
     const int c = (int)(e % g.C), t = (int)(e / g.C), rs = t % (g.R * g.S), k = t / (g.R * g.S);
     const int dh = rs / g.S - g.pad, dw = rs % g.S - g.pad;
+    const int tx = (g.Q + f.tile_w - 1) / f.tile_w, ty = (g.P + f.tile_h - 1) / f.tile_h;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int row = w; k < g.K && row < g.N * g.P; row += kSumLanes) {
-        const int n = row / g.P, h = (row - n * g.P) * g.stride + dh;
-        const __nv_bfloat16 *dy = f.dy + (size_t)row * g.Q * g.K + k;
-        const __nv_bfloat16 *x = f.x + ((size_t)n * g.H + h) * g.W * g.C + c;
-        const bool in = h >= 0 && h < g.H;
-        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int q = 0; q < g.Q; ++q) {
-            const int v = q * g.stride + dw;
-            const float d = __bfloat162float(dy[(size_t)q * g.K]);
-            float2 a = make_float2(0.f, 0.f), b = a;  // padding
-            if (in && v >= 0 && v < g.W) {
-                const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(x + (size_t)v * g.C);
-                a = __bfloat1622float2(p[0]);
-                b = __bfloat1622float2(p[1]);
+    bool open = bad;
+    for (int tile = z; tile < g.N * tx * ty && __any_sync(0xffffffffu, open); tile += splits) {
+        const int n = tile / (tx * ty), p0 = tile % (tx * ty) / tx * f.tile_h, q0 = tile % tx * f.tile_w;
+        for (int p = p0; p < min(p0 + f.tile_h, g.P); ++p) {
+            if (!open) continue;
+            const int h = p * g.stride + dh;
+            const __nv_bfloat16 *dy = f.dy + ((size_t)n * g.P + p) * g.Q * g.K + k;
+            const __nv_bfloat16 *x = f.x + ((size_t)n * g.H + h) * g.W * g.C + c;
+#pragma unroll 4
+            for (int q = q0; q < min(q0 + f.tile_w, g.Q); ++q) {
+                const int u = q * g.stride + dw;
+                const float d = __bfloat162float(dy[(size_t)q * g.K]);
+                float2 a = make_float2(0.f, 0.f), b = a;  // padding
+                if (h >= 0 && h < g.H && u >= 0 && u < g.W) {
+                    const __nv_bfloat162 *px = reinterpret_cast<const __nv_bfloat162 *>(x + (size_t)u * g.C);
+                    a = __bfloat1622float2(px[0]);
+                    b = __bfloat1622float2(px[1]);
+                }
+                s.x = fmaf(d, a.x, s.x);
+                s.y = fmaf(d, a.y, s.y);
+                s.z = fmaf(d, b.x, s.z);
+                s.w = fmaf(d, b.y, s.w);
             }
-            u.x = fmaf(d, a.x, u.x);
-            u.y = fmaf(d, a.y, u.y);
-            u.z = fmaf(d, b.x, u.z);
-            u.w = fmaf(d, b.y, u.w);
+            open = (isnan(v.x) && !isnan(s.x)) || (isnan(v.y) && !isnan(s.y)) ||
+                   (isnan(v.z) && !isnan(s.z)) || (isnan(v.w) && !isnan(s.w));
         }
-        s.x += u.x;
-        s.y += u.y;
-        s.z += u.z;
-        s.w += u.w;
     }
-    __syncthreads();  // red is read
-    red[w][lane] = s;
-    __syncthreads();
-    s = red[0][lane];
-    for (int l = 1; l < kSumLanes; ++l) {
-        const float4 v = red[l][lane];
-        s.x += v.x;
-        s.y += v.y;
-        s.z += v.z;
-        s.w += v.w;
+    return make_float4(isnan(v.x) ? s.x : v.x, isnan(v.y) ? s.y : v.y, isnan(v.z) ? s.z : v.z,
+                       isnan(v.w) ? s.w : v.w);
+}
+// This warp's splits w, w + kSumLanes, ... of the entries 4 i .. 4 i + 3 (live: they
+// are entries of dw).
+__device__ __noinline__ float4 sum_with_edges(const EdgeFix &f, const float4 *part, int splits, int64_t row,
+                                              int64_t i, bool live, int w) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int z = w; z < splits; z += kSumLanes) {
+        float4 v = live ? __ldg(part + (size_t)z * row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool bad = any_nan(v);
+        if (__any_sync(0xffffffffu, bad)) v = split_of_pixels(f, z, splits, live ? 4 * i : 0, v, bad);
+        s = add4(s, v);
     }
     return s;
 }
 
-__global__ void __launch_bounds__(32 * kSumLanes)
+template <bool RAGGED>
+__global__ void __launch_bounds__(32 * kSumLanes, RAGGED ? 4 : 8)
 k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, float4 *out,
             float4 *out2, const __grid_constant__ EdgeFix fix) {
     __shared__ float4 red[kSumLanes][32];
@@ -788,36 +805,19 @@ k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, floa
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < row) {
 #pragma unroll 4
-        for (int z = w; z < splits; z += kSumLanes) {
-            const float4 v = __ldg(part + (size_t)z * row + i);
-            s.x += v.x;
-            s.y += v.y;
-            s.z += v.z;
-            s.w += v.w;
+        for (int z = w; z < splits; z += kSumLanes) s = add4(s, __ldg(part + (size_t)z * row + i));
+    }
+    if constexpr (RAGGED) {
+        const bool bad = i < count4 && any_nan(s);
+        if (__any_sync(0xffffffffu, bad)) {
+            const float4 v = sum_with_edges(fix, part, splits, row, i, i < count4, w);
+            if (bad) s = v;
         }
     }
     red[w][lane] = s;
     __syncthreads();
     if (w == 0 && i < row) {
-        for (int l = 1; l < kSumLanes; ++l) {
-            const float4 v = red[l][lane];
-            s.x += v.x;
-            s.y += v.y;
-            s.z += v.z;
-            s.w += v.w;
-        }
-    }
-    if (fix.dy) {
-        const bool nan = w == 0 && i < count4 && (isnan(s.x) || isnan(s.y) || isnan(s.z) || isnan(s.w));
-        if (__syncthreads_or(nan)) {
-            const float4 v = sum_of_pixels(fix, i, red);
-            s.x = isnan(s.x) ? v.x : s.x;
-            s.y = isnan(s.y) ? v.y : s.y;
-            s.z = isnan(s.z) ? v.z : s.z;
-            s.w = isnan(s.w) ? v.w : s.w;
-        }
-    }
-    if (w == 0 && i < row) {
+        for (int l = 1; l < kSumLanes; ++l) s = add4(s, red[l][lane]);
         if (i < count4)
             out[i] = s;
         else
@@ -1205,17 +1205,19 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
     e = ch == 64 ? launch_wgrad<64>(mdy, mx, a, st) : launch_wgrad<32>(mdy, mx, a, st);
     if (e != cudaSuccess) return e;
     const bool ragged = g.P % kTileH || g.Q % kTileW;
-    return conv_sum_parts(g, a.splits, ws, dw, dbias, ragged ? dy : nullptr, x, st);
+    return conv_sum_parts(g, a.splits, ws, dw, dbias, ragged ? dy : nullptr, x, kTileH, kTileW, st);
 }
 
 cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
-                           const uint16_t *ragged_dy, const uint16_t *x, cudaStream_t st) {
+                           const uint16_t *ragged_dy, const uint16_t *x, int tile_h, int tile_w,
+                           cudaStream_t st) {
     const int64_t count4 = (int64_t)g.K * g.R * g.S * g.C / 4, extra4 = g.K / 4;
-    return launch_conv(k_sum_parts, dim3((unsigned)((count4 + extra4 + 31) / 32)), 32 * kSumLanes, 0, st,
+    return launch_conv(ragged_dy ? k_sum_parts<true> : k_sum_parts<false>,
+                       dim3((unsigned)((count4 + extra4 + 31) / 32)), 32 * kSumLanes, 0, st,
                        reinterpret_cast<const float4 *>(part), splits, count4, extra4,
                        reinterpret_cast<float4 *>(dw), reinterpret_cast<float4 *>(dbias),
                        EdgeFix{reinterpret_cast<const __nv_bfloat16 *>(ragged_dy),
-                               reinterpret_cast<const __nv_bfloat16 *>(x), g});
+                               reinterpret_cast<const __nv_bfloat16 *>(x), g, tile_h, tile_w});
 }
 
 cudaError_t conv_tma_take_status(int *timed_out) {

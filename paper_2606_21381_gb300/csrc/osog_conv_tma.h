@@ -42,10 +42,12 @@ cudaError_t conv_wgrad_tma(const Geo &g, const uint16_t *dy, const uint16_t *x, 
                            float *dbias, float *ws, cudaStream_t st);
 
 // dw, dbias = the sums over the splits of part [splits][K R S C + K], in order
-// (all 16-byte aligned).  ragged_dy: dY when the tiles that the partial sums come
-// from reach past the image, else NULL (see k_sum_parts).
+// (all 16-byte aligned).  Split z added the tiles z, z + splits, ... of tile_h x tile_w
+// output pixels; ragged_dy: dY when tiles reach past the image, else NULL (see
+// k_sum_parts).
 cudaError_t conv_sum_parts(const Geo &g, int splits, const float *part, float *dw, float *dbias,
-                           const uint16_t *ragged_dy, const uint16_t *x, cudaStream_t st);
+                           const uint16_t *ragged_dy, const uint16_t *x, int tile_h, int tile_w,
+                           cudaStream_t st);
 
 // Latched status of the bounded waits (read and cleared), and the
 // failure-detection hook (osog_conv_test_wait_limit).
