@@ -28,7 +28,6 @@ namespace {
 
 constexpr int BM = 64, BN = 64, BK = 32, LDS = BK + 8;  // smem row: 40 bf16 = 80 bytes
 constexpr int NT = 128;
-constexpr int kSplitPixels = 2048;  // pixels per CTA in the filter-gradient reduction
 
 // kDgrad2: the data gradient of a stride-2 convolution for the input
 // pixels of one parity class (h mod 2, w mod 2), reduced over the taps that
@@ -522,6 +521,7 @@ template <int MT>
 __global__ void __launch_bounds__(kC8Threads, MT == 2 ? 2 : 1)
 k_wgrad_c8(const __grid_constant__ Args a, int splits) {
     constexpr int KP = MT * 16, VECS = KP / 8, kPix = kC8W * kC8GradRows;
+    static_assert(kPix == kC8Threads, "a thread sums VECS vectors of a tile");
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) uint4 zero;
     pdl_enter();
@@ -593,18 +593,21 @@ k_wgrad_c8(const __grid_constant__ Args a, int splits) {
                 }
             }
         }
-        // bias: thread u sums vector u % VECS over the pixels u / VECS, ...
+        // bias: thread u sums vector u % VECS over the pixels u / VECS, ... of the tile,
+        // then adds that to the tiles before
         const uint4 *d = reinterpret_cast<const uint4 *>(smem + buf * stage);
+        uint4 v[VECS];
 #pragma unroll
-        for (int px = threadIdx.x / VECS; px < kPix; px += kC8Threads / VECS) {
-            const uint4 v = d[at(px, threadIdx.x % VECS)];
-            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+        for (int i = 0; i < VECS; ++i)
+            v[i] = d[at(threadIdx.x / VECS + i * (kC8Threads / VECS), threadIdx.x % VECS)];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __bfloat1622float2(h[j]);
-                sum[2 * j] += f.x;
-                sum[2 * j + 1] += f.y;
-            }
+        for (int j = 0; j < 4; ++j) {
+            float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < VECS; ++i)
+                t = cadd(t, __bfloat1622float2(reinterpret_cast<const __nv_bfloat162 *>(&v[i])[j]));
+            sum[2 * j] += t.x;
+            sum[2 * j + 1] += t.y;
         }
         __syncthreads();
         buf ^= 1;
@@ -650,7 +653,12 @@ bool fits_c8(const Geo &g) {
 }
 int splits_c8(const Geo &g) {
     const int64_t tiles = (int64_t)g.N * ((g.Q + kC8W - 1) / kC8W) * ((g.P + kC8GradRows - 1) / kC8GradRows);
-    return (int)(tiles < 304 ? tiles : 304);  // two CTAs on each of 152 SMs
+    // two CTAs on each SM, and more where one of a CTA's eight warps would add more
+    // than kSplitPixels pixels
+    const int64_t fill = 2 * kSms, warps = kC8Threads / 32 * kSplitPixels;
+    const int64_t least = ((int64_t)g.N * g.P * g.Q + warps - 1) / warps;
+    const int64_t splits = fill > least ? fill : least;
+    return (int)(tiles < splits ? tiles : splits);
 }
 
 cudaError_t launch_conv_c8(const Args &a, cudaStream_t st) {

@@ -494,6 +494,15 @@ k_conv_patch(const __grid_constant__ CUtensorMap src, const __grid_constant__ CU
 // before / now): 128 -> 128, 32 x 32: 123 / 23; 64 -> 128, stride 2: 116 / 20;
 // 32 -> 64, stride 2: 138 / 37 (bound by the reads of dY from shared memory, 4 KB
 // per product however few its columns); 128 -> 64: 96 / 21.
+//
+// The accumulators round (to FP32, towards zero) at every 16 pixels, so the error of a
+// sum grows with their number; a split has at most about kSplitPixels pixels of one
+// accumulator, whatever the layer and however many images.  Without that limit the
+// 3 x 3 layer of 256 -> 256 channels on 64 images of 64 x 64 added 21,800 pixels: its
+// error was 3.2e-5 of the gradient's norm, now 1.8e-6 (the general kernel's 2.0e-6), for
+// 314 us instead of 200 (1,461 with the copies through cp.async); the network's layers
+// have shorter chains anyway.  The bias gradient is summed tile by tile for the same
+// reason.
 struct WgradArgs {
     int tiles_x, tiles, splits;        // tiles of all images
     int tiles_y;
@@ -525,9 +534,9 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t full = smem_addr(bars), empty = full + 8u * kMaxRing,
                    all_done = empty + 8u * kMaxRing, probe = all_done + 8u;
-    const int group = blockIdx.x % a.groups, blk = blockIdx.x / a.groups;
+    const int blocks = gridDim.x / a.splits, z = blockIdx.x / blocks;
+    const int group = blockIdx.x % blocks % a.groups, blk = blockIdx.x % blocks / a.groups;
     const int c0 = (blk % a.cblocks) * a.cblk, k0 = (blk / a.cblocks) * 128;
-    const int z = blockIdx.y;
     const bool sums_bias = group == 0 && c0 == 0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
@@ -637,16 +646,19 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
             if (!ok) break;
             const unsigned char *src = smem + (size_t)st * a.stage_bytes +
                                        (vec >> 3) * (kTileW * kTileH * 128);
+            float part[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             for (int p = p0; p < kTileW * kTileH; p += lanes) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(src + p * 128 + (((vec ^ p) & 7) << 4));
                 const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float2 f = __bfloat1622float2(h[j]);
-                    sum[2 * j] += f.x;
-                    sum[2 * j + 1] += f.y;
+                    part[2 * j] += f.x;
+                    part[2 * j + 1] += f.y;
                 }
             }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum[j] += part[j];
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(empty + 8u * st) : "memory");
@@ -1148,10 +1160,14 @@ bool wgrad_plan(const Geo &g, WgradArgs &a, int &ch) {
         if (a.ring > kMaxRing) a.ring = kMaxRing;
         if (a.ring < 1) continue;
         a.tmem_cols = tmem_columns((each - 1) * a.bn + round_up(a.bn, 32));
+        // a CTA per SM, and more where a split would add more pixels in one accumulator
+        // than kSplitPixels less a tile
+        constexpr int kMost = kSplitPixels - kTileW * kTileH;
+        const int64_t pixels = (int64_t)g.N * g.P * g.Q;
         const int blocks = ceil_div(g.K, 128) * a.cblocks * a.groups;
-        int splits = 152 / blocks;
-        splits = splits < 1 ? 1 : splits;
-        a.splits = splits < a.tiles ? splits : a.tiles;
+        const int fill = kSms / blocks, least = (int)((pixels + kMost - 1) / kMost);
+        a.splits = fill > least ? fill : least;
+        if (a.splits > a.tiles) a.splits = a.tiles;
         return true;
     }
     return false;
@@ -1173,7 +1189,8 @@ cudaError_t launch_wgrad(const CUtensorMap &mdy, const CUtensorMap &mx, const Wg
     static const cudaError_t opt_in = cudaFuncSetAttribute(
         k_wgrad_patch<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
     if (opt_in != cudaSuccess) return opt_in;
-    const dim3 grid(ceil_div(a.K, 128) * a.cblocks * a.groups, a.splits);
+    // (one dimension: the others end at 65,535, which the splits may pass)
+    const dim3 grid(ceil_div(a.K, 128) * a.cblocks * a.groups * a.splits);
     return launch_conv(k_wgrad_patch<CH>, grid, kCtaThreads, wgrad_smem(a), st, mdy, mx, a);
 }
 

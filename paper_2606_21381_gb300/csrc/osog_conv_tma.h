@@ -23,6 +23,10 @@ inline cudaError_t launch_conv(void (*kernel)(KArgs...), dim3 grid, int block, s
     return launch_pdl(kernel, true, grid, block, smem, st, args...);
 }
 
+// Most pixels that a filter gradient adds in one accumulator before it sums the
+// partial results of its splits.
+constexpr int kSplitPixels = 2048;
+
 struct Geo {
     int N, H, W, C, K, R, S, stride, pad, P, Q;
 };

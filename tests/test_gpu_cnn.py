@@ -311,3 +311,22 @@ def test_filter_gradient_of_activations_that_are_not_finite(cnn, shape, value):
     np.testing.assert_array_equal(got_w[~fin], want_w[~fin])
     assert np.abs(got_w[fin] - want_w[fin]).max() <= 1e-5 * np.abs(want_w[fin]).max() * np.sqrt(dy.size / dy.shape[-1])
     assert np.abs(db.cpu().numpy() - want_b).max() <= 1e-5 * np.abs(dy64).sum(axis=(0, 1, 2)).max()
+
+
+def test_long_filter_gradients_are_as_accurate_as_the_general_kernel():
+    # 131,072 pixels in a layer wide enough to fill the chip with nine splits: the
+    # accumulators' rounding grows with the pixels added in one (2048 in the general
+    # kernel), so the norm of the error stays below its, but for the order of the
+    # products (a quarter at most)
+    from paper_2606_21381_gb300 import cnn as m
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((32, 64, 64, 512), generator=g, device="cuda").clamp_(min=0).to(torch.bfloat16)
+    dy = (torch.randn((32, 64, 64, 512), generator=g, device="cuda") + 0.5).to(torch.bfloat16)
+    want = dy.reshape(-1, 512).double().t() @ x.reshape(-1, 512).double()
+    err = []
+    for engine in (False, True):
+        m.use_tcgen05(engine)
+        dw, db = m.conv2d_backward_filter(dy, x, (512, 1, 1, 512), 1, 0)
+        err.append((dw.reshape(512, 512).double() - want).norm().item())
+        assert (db.double() - dy.double().sum((0, 1, 2))).abs().max() <= 2e-6 * dy.double().abs().sum((0, 1, 2)).max()
+    assert err[1] <= 1.25 * err[0]
