@@ -63,7 +63,7 @@ constexpr int kGroup = fft_grouped(N) ? kSyncLine : kSyncCta;
 // transform, whose last stores the result over Q.
 template <int N>
 __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant__ BwdRowsArgs a) {
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     constexpr int L = set_elems(N) / N, G = kGroup<N>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *bufE = reinterpret_cast<float2 *>(smem_raw);
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(const __grid_constant_
 // accumulation in registers, and the last of the inverse one stores over G.
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1) k_bwd_column(const __grid_constant__ BwdColumnArgs a) {
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     constexpr int L = set_elems(N) / N;
     constexpr int LS = line_stride(N);
     constexpr int NW = kThreads / 32;
@@ -190,7 +190,7 @@ template <int N, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? kWideThreads : kThreads, 1)
 k_bwd_strip(const __grid_constant__ BwdStripArgs a) {
     constexpr int NT = WIDE ? kWideThreads : kThreads;
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     constexpr int L = set_elems(N) / N;
     constexpr int LS = line_stride(N);
     constexpr int NW = NT / 32;
@@ -404,7 +404,7 @@ template <int N>
 struct BwdLaunch {
     static cudaError_t rows(const BwdRowsArgs &a, cudaStream_t st) {
         const dim3 grid(a.geo.nstrips, a.S * a.K);
-        return launch_chain(k_bwd_rows<N>, grid, kThreads, solo_smem<N>(grid, strip_inverse_smem(N)), st, a);
+        return launch_chain(k_bwd_rows<N>, grid, kThreads, strip_inverse_smem(N), st, a);
     }
     static cudaError_t column(const BwdColumnArgs &a, cudaStream_t st) {
         return launch_chain(k_bwd_column<N>, dim3(a.geo.nblocks, a.S), kThreads, bwd_column_smem(N),
@@ -415,25 +415,24 @@ struct BwdLaunch {
         if constexpr (bwd_strip_wide(N))
             if ((int)(grid.x * grid.y) <= kSms)
                 return launch_chain(k_bwd_strip<N, true>, grid, kWideThreads,
-                                    solo_smem<N>(grid, bwd_strip_smem(N, kWideThreads)), st, a);
-        return launch_chain(k_bwd_strip<N, false>, grid, kThreads,
-                            solo_smem<N>(grid, bwd_strip_smem(N, kThreads)), st, a);
+                                    bwd_strip_smem(N, kWideThreads), st, a);
+        return launch_chain(k_bwd_strip<N, false>, grid, kThreads, bwd_strip_smem(N, kThreads), st, a);
     }
     static cudaError_t prepare(int which) {
         if (which == 0)
             return cudaFuncSetAttribute(k_bwd_rows<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        prepared_smem<N>(strip_inverse_smem(N)));
+                                        (int)strip_inverse_smem(N));
         if (which == 1)
             return cudaFuncSetAttribute(k_bwd_column<N>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)bwd_column_smem(N));
         cudaError_t e = cudaFuncSetAttribute(k_bwd_strip<N, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             prepared_smem<N>(bwd_strip_smem(N, kThreads)));
+                                             (int)bwd_strip_smem(N, kThreads));
         if constexpr (bwd_strip_wide(N))
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k_bwd_strip<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         prepared_smem<N>(bwd_strip_smem(N, kWideThreads)));
+                                         (int)bwd_strip_smem(N, kWideThreads));
         return e;
     }
 };

@@ -253,16 +253,31 @@ __device__ __forceinline__ int2 mode_chord(const ModeDev &md, int fx, int H) {
 }
 
 // ---------------------------------------------------------------- launches
-// Programmatic dependent launch.  Every kernel of the render and adjoint
-// chains starts with pdl_enter(): it first lets the next kernel of the
-// stream be dispatched (once all CTAs of this grid have done the same), then
-// waits until the kernels before it in the stream have completed and their
+// Programmatic dependent launch.  The small kernels of the render and adjoint
+// chains (binning, sums) start with pdl_enter(): it first lets the next kernel
+// of the stream be dispatched (once all CTAs of this grid have done the same),
+// then waits until the kernels before it in the stream have completed and their
 // writes are visible.  Nothing is read from global memory before the wait,
 // so the overlap covers launch and CTA dispatch only.  Launched without the
 // attribute (launch_chain), or after other stream work, the wait returns at
 // once.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// The kernels that transform strips and column blocks (of S scenes) let the next one
+// in as their CTAs finish, unless all of them have more than two CTAs per SM: a last
+// wave leaves SMs idle, which the next kernel's CTAs then fill (five images of 1024 x
+// 1024 114 us, 119 without).  CTAs of a single wave, dispatched while the grid before
+// them still runs, find every SM half taken, pair up on the few that come free first
+// and leave the rest idle.  Asking for the whole SM's shared memory prevents the pairs,
+// too (what these kernels did before), but keeps the CTAs of other streams out as well.
+// GPU time of one image, early / whole SM / as it is: 512 x 512, 200 particles, with its
+// adjoint 52.9 / 50.7 / 46.5 us; four such images on four streams, rendered only, 32.9 /
+// 38.5 / 25.9.
+__device__ __forceinline__ void pdl_enter_spread(const Geometry &geo, int S) {
+    if ((geo.nstrips < geo.nblocks ? geo.nstrips : geo.nblocks) * S > 2 * kSms)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -295,24 +310,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), bool early, dim3 grid, i
     if (e != cudaSuccess) (void)cudaGetLastError();  // reported once, by the return value
     return e;
 }
-// A grid of at most one CTA per SM, and more than half as many, whose CTAs would fit
-// in pairs asks for more than half of an SM's shared memory: dispatched while the
-// kernel before it still runs, its CTAs otherwise pair up on the SMs that come free
-// first and leave the others idle (one dense 1024 x 1024 image, loss and adjoint:
-// 114.9 -> 107.2 us of GPU time; 512 x 512, two modalities: 52.9 -> 51.1).  Kernels of
-// sets of 512 points and more: a raised limit alone (prepared_smem) took 0.6 us from
-// the four kernels of a 256 x 256 image, whose 64 CTAs have nothing to gain.
-constexpr size_t kSoloSmem = 116 * 1024;
-template <int N>
-inline int prepared_smem(size_t need) {
-    return (int)(N >= 512 && need < kSoloSmem ? kSoloSmem : need);
-}
-template <int N>
-inline size_t solo_smem(dim3 grid, size_t need) {
-    const long ctas = (long)grid.x * grid.y;
-    return ctas > kSms / 2 && ctas <= kSms ? (size_t)prepared_smem<N>(need) : need;
-}
-
 template <typename... KArgs>
 inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
                                 cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {

@@ -200,15 +200,17 @@ __global__ void __launch_bounds__(kRThreads, 4) k_raster_tiles(const __grid_cons
         dst[(size_t)(i >> lw) * (geo.W / 2) + (i & (TW / 2 - 1))] = a4[i];
 }
 
-// WIDE: 1024 threads rasterise the strip, for launches of at most one CTA per
-// SM, where 16 warps leave the raster waiting for its loads and shuffles (two
-// CTAs of 512 threads share an SM otherwise): one dense 1024 x 1024 image 23.5 ->
-// 20.2 us, 512 x 1024 with 1,501 particles 15.0 -> 11.7 us.
+// WIDE: 1024 threads rasterise the strip, for launches that would leave an SM with
+// 16 warps, too few for the raster's loads and shuffles (one dense 1024 x 1024 image
+// 23.5 -> 20.2 us, 512 x 1024 with 1,501 particles 15.0 -> 11.7).  Such a CTA takes an
+// SM's registers whole, so grids of 77 to 152 CTAs use it from 1024 pixels a row only,
+// where it pays (adjoint of that dense image 108.7 -> 100.6 us): eight images of 512 x
+// 512 rendered on eight streams took 57.8 us with it, 42.9 without.
 template <int N, int MODE, bool SQ, bool WIDE = false>
 __global__ void __launch_bounds__(WIDE ? kWideThreads : kThreads, WIDE ? 1 : 2)
 k_strip_forward(const __grid_constant__ StripArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     strip_forward_item<N, MODE, SQ, WIDE ? kWideThreads : kThreads>(a, blockIdx.y, blockIdx.x, smem_raw);
 }
 
@@ -500,7 +502,7 @@ __device__ __forceinline__ void column_item(const ColumnArgs &a, int s, int bk,
 template <int N, bool MULTI, bool SQ>
 __global__ void __launch_bounds__(kThreads, 2) k_column(const __grid_constant__ ColumnArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     column_item<N, MULTI, SQ, SQ && N >= 1024>(a, blockIdx.y, blockIdx.x, smem_raw);
 }
 
@@ -539,7 +541,7 @@ __device__ __forceinline__ void inverse_item(const InverseArgs &a, int sm, int s
 template <int N, bool SQ>
 __global__ void __launch_bounds__(kThreads, 2) k_strip_inverse(const __grid_constant__ InverseArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_enter();
+    pdl_enter_spread(a.geo, a.S);
     inverse_item<N, SQ>(a, blockIdx.y, blockIdx.x, smem_raw);
 }
 
@@ -665,12 +667,11 @@ template <int N>
 struct StripFwdLaunch {
     static cudaError_t run(const StripArgs &a, StripMode mode, cudaStream_t st) {
         dim3 grid(a.geo.nstrips, a.S);
-        const size_t smem = solo_smem<N>(grid, strip_forward_smem(N));
-        const size_t smem_opd = solo_smem<N>(grid, strip_forward_smem(N, true));
-        const size_t smem_fft = solo_smem<N>(grid, strip_inverse_smem(N));  // the set alone: no raster
-        const bool wide = (int)(grid.x * grid.y) <= kSms;
-        const size_t smem_wide = solo_smem<N>(
-            grid, strip_forward_smem(N) + raster_smem<kWideThreads>() - raster_smem<kThreads>());
+        const size_t smem = strip_forward_smem(N), smem_opd = strip_forward_smem(N, true);
+        const size_t smem_fft = strip_inverse_smem(N);  // the set alone: no raster
+        const int ctas = (int)(grid.x * grid.y);
+        const bool wide = ctas <= kSms / 2 || (N >= 1024 && ctas <= kSms);  // see k_strip_forward
+        const size_t smem_wide = smem + raster_smem<kWideThreads>() - raster_smem<kThreads>();
         if (mode == kStripRender && wide && a.geo.H == a.geo.W)
             return launch_chain(k_strip_forward<N, kStripRender, true, true>, grid, kWideThreads, smem_wide, st, a);
         else if (mode == kStripRender && wide)
@@ -693,29 +694,29 @@ struct StripFwdLaunch {
     static cudaError_t prepare() {
         const int smem = (int)strip_forward_smem(N), smem_opd = (int)strip_forward_smem(N, true);
         cudaError_t e = cudaFuncSetAttribute(k_strip_forward<N, kStripRender, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripRender, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripOpdOnly, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem_opd));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem_opd);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripFromMap, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_forward<N, kStripFromReal, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         const int smem_wide = smem + (int)(raster_smem<kWideThreads>() - raster_smem<kThreads>());
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
             e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripRender, true, true>
                                         : k_strip_forward<N, kStripRender, false, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem_wide));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem_wide);
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq)
             e = cudaFuncSetAttribute(sq ? k_strip_forward<N, kStripFromPhase, true>
                                         : k_strip_forward<N, kStripFromPhase, false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     prepared_smem<N>(strip_inverse_smem(N)));
+                                     (int)strip_inverse_smem(N));
         return e;
     }
 };
@@ -724,7 +725,6 @@ template <int N>
 struct ColumnLaunch {
     static cudaError_t run(const ColumnArgs &a, cudaStream_t st, size_t smem) {
         dim3 grid(a.geo.nblocks, a.S);
-        smem = solo_smem<N>(grid, smem);
         const bool sq = a.geo.H == a.geo.W;
         if (a.K > 1 && sq)
             return launch_chain(k_column<N, true, true>, grid, kThreads, smem, st, a);
@@ -739,10 +739,10 @@ struct ColumnLaunch {
         cudaError_t e = cudaSuccess;
         for (int sq = 0; sq < 2 && e == cudaSuccess; ++sq) {
             e = cudaFuncSetAttribute(sq ? k_column<N, false, true> : k_column<N, false, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem1));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(sq ? k_column<N, true, true> : k_column<N, true, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem2));
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
         }
         return e;
     }
@@ -752,7 +752,6 @@ template <int N>
 struct InverseLaunch {
     static cudaError_t run(const InverseArgs &a, cudaStream_t st, size_t smem) {
         dim3 grid(a.geo.nstrips, a.S * a.K);
-        smem = solo_smem<N>(grid, smem);
         if (a.geo.H == a.geo.W)
             return launch_chain(k_strip_inverse<N, true>, grid, kThreads, smem, st, a);
         else
@@ -760,10 +759,10 @@ struct InverseLaunch {
     }
     static cudaError_t prepare(size_t smem) {
         cudaError_t e = cudaFuncSetAttribute(k_strip_inverse<N, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_strip_inverse<N, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, prepared_smem<N>(smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         return e;
     }
 };

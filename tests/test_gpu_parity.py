@@ -338,3 +338,31 @@ def test_single_modality_columns_at_every_plan(H):
     assert_images_close(one, ref, o)
     both = gpu_render(soa, {**o, "modes": 3})
     assert np.array_equal(both[1], one[0])
+
+
+@pytest.mark.parametrize("size,modes", [(256, 3), (512, 1), (1024, 4)])
+def test_images_and_adjoints_on_several_streams_at_once(size, modes):
+    # four renderers on four streams, their kernels in flight together (grids of 64 and
+    # 128 CTAs, of 512 and 1024 threads): bit for bit what each gives alone
+    rng = np.random.default_rng(size)
+    o = scenes.optics(size, size, modes=modes, defocus=0.3)
+    K = bin(modes).count("1")
+    work = []
+    for _ in range(4):
+        soa = torch.from_numpy(scenes.draw_particles(rng, 300, size, size, mu=(0.0, 0.02))).cuda()
+        grad = torch.from_numpy(rng.standard_normal((K, size, size)).astype(np.float32)).cuda()
+        work.append((type(renderer(size, size))(size, size), soa, grad, torch.cuda.Stream()))
+    alone = []
+    for r, soa, grad, _ in work:
+        alone.append((r.render(soa, None, o).clone(), *(g.clone() for g in r.backward(soa, None, o, grad))))
+        torch.cuda.synchronize()
+    got = [[] for _ in work]
+    for _ in range(5):
+        for i, (r, soa, grad, st) in enumerate(work):
+            with torch.cuda.stream(st):
+                got[i].append((r.render(soa, None, o), *r.backward(soa, None, o, grad)))
+    torch.cuda.synchronize()
+    for (r, *_), want, runs in zip(work, alone, got):
+        assert r.sync_status() == 0
+        for run in runs:
+            assert all(torch.equal(a, b) for a, b in zip(run, want))
