@@ -96,8 +96,7 @@ __device__ __noinline__ float draw_exact(float v, int64_t i, double g, double si
 }
 
 // Gain and read noise of a launch: in double precision, and as float-float
-// for the FP32 draw (fast = 0: outside its range, every element is drawn in
-// double precision).
+// for the FP32 draw.
 struct NoiseArgs {
     const float *img;
     float *out;
@@ -105,8 +104,14 @@ struct NoiseArgs {
     uint64_t seed;
     double g, sigma;
     ff g_ff, inv_g, sigma_ff;
-    int32_t fast;
 };
+
+// Gains and read noises outside the FP32 draw's range: every element in double
+// precision.
+__global__ void __launch_bounds__(256) k_sensor_noise_exact(const __grid_constant__ NoiseArgs a) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.count; i += (int64_t)gridDim.x * 256)
+        a.out[i] = draw_exact(a.img[i], i, a.g, a.sigma, a.seed);
+}
 
 // An element whose first rejection attempt was not accepted at once: its
 // candidate (n = 0: rejected already), its rate, sigma z and place in the tile.
@@ -131,23 +136,31 @@ __device__ __forceinline__ int more_attempts(const NoiseArgs &a, ff lam, int64_t
     return s == kNo ? kUndecided : s;
 }
 
-constexpr int kNoiseThreads = 256, kPerThread = 4, kTile = kNoiseThreads * kPerThread;
+constexpr int kNoiseThreads = 256, kPerThread = 4;
 constexpr int kNoiseCtas = 4;  // resident on an SM
 
-// A CTA draws tiles of kTile elements in three sweeps.  Every element gets its
+// A CTA draws tiles of PER elements a thread in three sweeps.  Every element gets its
 // normal and the quick part of its first attempt (about 68% of rates above ten
 // end there); the others queue up in shared memory and take their acceptance
 // test as full warps; those it rejects queue up again for further attempts.  A
 // warp would otherwise run every step for its unluckiest lane.  Undecided
 // elements collect over the tiles and are drawn in double precision by the CTA
-// together.
+// together, as are rates from 2^22 (of 1,048,576 such pixels 830 us; a thread per element,
+// as in k_sensor_noise_exact, 739).
+//
+// PER = kPerThread, or 1 where every such tile has a place on the chip: an element
+// drawn in double precision costs as much as a hundred others, and 4,096 of 10^8
+// photons took 114 us in four tiles, 33 in sixteen; 65,536 at 1,000 photons 23.0 and
+// 20.1.
 //
 // Bound by instruction issue.  16 images of 1024 x 1024 at 1,000 photons (the
 // same bits): all in double precision 11.54 ms, bound by the FP64 pipe; on the
 // FP32 pipes without queues 0.560 ms, about 1,000 warp instructions per 32
 // elements; this kernel 0.45 ms, about 740.
+template <int PER>
 __global__ void __launch_bounds__(kNoiseThreads, kNoiseCtas)
 k_sensor_noise(const __grid_constant__ NoiseArgs a) {
+    constexpr int kTile = kNoiseThreads * PER;
     __shared__ Pending queue[kTile];
     __shared__ uint16_t again[kTile];
     __shared__ int64_t open[kTile + kNoiseThreads];
@@ -166,7 +179,7 @@ k_sensor_noise(const __grid_constant__ NoiseArgs a) {
     const int64_t tiles = (a.count + kTile - 1) / kTile;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int64_t i0 = tile * kTile;
-        for (int u = 0; u < kPerThread; ++u) {
+        for (int u = 0; u < PER; ++u) {
             const int at = u * kNoiseThreads + threadIdx.x;
             const int64_t i = i0 + at;
             Pending e;
@@ -176,7 +189,6 @@ k_sensor_noise(const __grid_constant__ NoiseArgs a) {
                 uint32_t c[4] = {(uint32_t)(uint64_t)i, (uint32_t)((uint64_t)i >> 32), 0u, kTag};
                 philox4x32_10(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
                 e.noise = {0.f, 0.f};
-                undecided = !a.fast;
                 if (a.sigma_ff.h > 0.f) {
                     undecided = undecided || c[0] == 0u;
                     e.noise = mul_lazy(a.sigma_ff, normal_ff(c[0], c[1]));
@@ -293,15 +305,25 @@ extern "C" int osog_sensor_noise(const float *image, int64_t count, double photo
     a.seed = seed;
     a.g = photons_per_unit;
     a.sigma = read_sigma;
+    const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const int64_t rows = (count + osog::noise::kNoiseThreads - 1) / osog::noise::kNoiseThreads;
     // the range where no float-float part under- or overflows
-    a.fast = photons_per_unit >= 1e-6 && (read_sigma == 0.0 || (read_sigma >= 1e-6 && read_sigma <= 1e6));
+    const bool fast = photons_per_unit >= 1e-6 && (read_sigma == 0.0 || (read_sigma >= 1e-6 && read_sigma <= 1e6));
     a.g_ff = osog::noise::split(photons_per_unit);
     a.inv_g = osog::noise::split(1.0 / photons_per_unit);
     a.sigma_ff = osog::noise::split(read_sigma);
-    const int64_t tiles = (count + osog::noise::kTile - 1) / osog::noise::kTile;
-    const int blocks = (int)(tiles < (int64_t)sms * osog::noise::kNoiseCtas
-                                 ? tiles
-                                 : (int64_t)sms * osog::noise::kNoiseCtas);
-    osog::noise::k_sensor_noise<<<blocks, osog::noise::kNoiseThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+    if (!fast) {
+        const int64_t most = (int64_t)sms * 8;
+        osog::noise::k_sensor_noise_exact<<<(unsigned)(rows < most ? rows : most), 256, 0, st>>>(a);
+        return cudaGetLastError() == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA;
+    }
+    const int64_t ctas = (int64_t)sms * osog::noise::kNoiseCtas;
+    if (rows <= ctas) {
+        osog::noise::k_sensor_noise<1><<<(unsigned)rows, osog::noise::kNoiseThreads, 0, st>>>(a);
+    } else {
+        const int64_t tiles = (rows + osog::noise::kPerThread - 1) / osog::noise::kPerThread;
+        osog::noise::k_sensor_noise<osog::noise::kPerThread>
+            <<<(unsigned)(tiles < ctas ? tiles : ctas), osog::noise::kNoiseThreads, 0, st>>>(a);
+    }
     return cudaGetLastError() == cudaSuccess ? OSOG_OK : OSOG_ERR_CUDA;
 }

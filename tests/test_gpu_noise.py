@@ -73,3 +73,25 @@ def test_boundaries_of_the_fp32_draw(g, sigma, level):
     want = oracle.sensor_noise(np.nan_to_num(x), g, sigma, 99)
     got = sensor_noise(torch.from_numpy(x).cuda(), g, sigma, 99).cpu().numpy()
     np.testing.assert_allclose(got, want, rtol=2e-7, atol=1e-9)
+
+
+# tiles of one to four elements a thread, whole and ragged, up to several tiles a CTA
+@pytest.mark.parametrize("n", [1, 31, 255, 257, 1023, 155_648, 155_649, 311_297, 466_945, 622_593, 700_001])
+@pytest.mark.parametrize("g", [3.0, 1000.0])
+def test_draws_do_not_depend_on_the_size_of_the_launch(n, g):
+    from paper_2606_21381_gb300.noise import sensor_noise
+    x = torch.rand(1_400_000, generator=torch.Generator().manual_seed(n)).cuda() * 4.0
+    want = sensor_noise(x, g, 1.5, 11)
+    assert torch.equal(sensor_noise(x[:n], g, 1.5, 11), want[:n])
+
+
+@pytest.mark.parametrize("g,run", [(4e6, 1), (4e6, 64), (1e-7, 64), (1e8, 64)])
+def test_warps_in_and_out_of_the_fp32_draws_range(g, run):
+    # runs of pixels brighter and darker than 2^22 photons, of one lane and of two
+    # warps, and gains that no pixel's or every pixel's FP32 draw takes
+    from paper_2606_21381_gb300.noise import sensor_noise
+    x = np.where((np.arange(5000) // run) % 2 == 0, 0.5, 1.5).astype(np.float32)
+    x[17::301] = 0.0
+    want = oracle.sensor_noise(x, g, 2.0, 7)
+    got = sensor_noise(torch.from_numpy(x).cuda(), g, 2.0, 7).cpu().numpy()
+    np.testing.assert_allclose(got, want, rtol=2e-7, atol=1e-9)
