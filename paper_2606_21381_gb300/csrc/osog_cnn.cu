@@ -664,9 +664,9 @@ int splits_c8(const Geo &g) {
 cudaError_t launch_conv_c8(const Args &a, cudaStream_t st) {
     const Geo &g = a.g;
     const PatchC8 p = patch_c8(g, kC8Rows);
-    static const cudaError_t opt_in =
-        cudaFuncSetAttribute(k_conv_c8, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (opt_in != cudaSuccess) return opt_in;
+    static osog::DeviceOnce once;
+    const cudaError_t e = opt_in_smem(once, k_conv_c8, 96 * 1024);
+    if (e != cudaSuccess) return e;
     const dim3 grid(g.N * ((g.Q + kC8W - 1) / kC8W) * ((g.P + kC8Rows - 1) / kC8Rows), (g.K + 31) / 32);
     return launch_conv(k_conv_c8, grid, kC8Threads, p.pitch * p.ph * 16, st, a);
 }
@@ -677,9 +677,9 @@ cudaError_t launch_wgrad_c8(const Args &a, cudaStream_t st) {
     const int red = (MT * 16 * kC8Taps * 8 + kC8Threads * 8) * 4;
     int smem = 2 * (kC8W * kC8GradRows * MT * 32 + p.pitch * p.ph * 16);
     if (smem < red) smem = red;
-    static const cudaError_t opt_in =
-        cudaFuncSetAttribute(k_wgrad_c8<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (opt_in != cudaSuccess) return opt_in;
+    static osog::DeviceOnce once;
+    const cudaError_t e = opt_in_smem(once, k_wgrad_c8<MT>, 200 * 1024);
+    if (e != cudaSuccess) return e;
     const int splits = splits_c8(a.g);
     return launch_conv(k_wgrad_c8<MT>, dim3(splits), kC8Threads, smem, st, a, splits);
 }

@@ -969,9 +969,9 @@ bool conv_patch_plan(PatchArgs &a, int images, int oh, int ow, int reach_y, int 
 template <bool FWD, int CH>
 cudaError_t launch_patch_ch(const CUtensorMap &src, const CUtensorMap &flt, const PatchArgs &a,
                             int images, cudaStream_t st) {
-    static const cudaError_t opt_in = cudaFuncSetAttribute(
-        k_conv_patch<FWD, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
-    if (opt_in != cudaSuccess) return opt_in;
+    static DeviceOnce once;
+    const cudaError_t e = opt_in_smem(once, k_conv_patch<FWD, CH>, kSmemMax - 2048);
+    if (e != cudaSuccess) return e;
     const dim3 grid(images * a.tiles_x * a.tiles_y, ceil_div(a.ncols, a.bn));
     return launch_conv(k_conv_patch<FWD, CH>, grid, kCtaThreads, patch_smem(a), st, src, flt, a);
 }
@@ -1186,9 +1186,9 @@ int wgrad_smem(const WgradArgs &a) {
 template <int CH>
 cudaError_t launch_wgrad(const CUtensorMap &mdy, const CUtensorMap &mx, const WgradArgs &a,
                          cudaStream_t st) {
-    static const cudaError_t opt_in = cudaFuncSetAttribute(
-        k_wgrad_patch<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048);
-    if (opt_in != cudaSuccess) return opt_in;
+    static DeviceOnce once;
+    const cudaError_t e = opt_in_smem(once, k_wgrad_patch<CH>, kSmemMax - 2048);
+    if (e != cudaSuccess) return e;
     // (one dimension: the others end at 65,535, which the splits may pass)
     const dim3 grid(ceil_div(a.K, 128) * a.cblocks * a.groups * a.splits);
     return launch_conv(k_wgrad_patch<CH>, grid, kCtaThreads, wgrad_smem(a), st, mdy, mx, a);

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "osog_common.cuh"
+#include "osog_device_once.h"
 
 namespace osog {
 namespace cnn {
@@ -21,6 +22,16 @@ template <typename... KArgs>
 inline cudaError_t launch_conv(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem,
                                cudaStream_t st, const typename KernelArg<KArgs>::type &...args) {
     return launch_pdl(kernel, true, grid, block, smem, st, args...);
+}
+
+// Opt-in of a kernel to `bytes` of dynamic shared memory on the current device
+// (`once` is the kernel's own).
+template <typename... KArgs>
+inline cudaError_t opt_in_smem(DeviceOnce &once, void (*kernel)(KArgs...), int bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return once(dev, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 // Most pixels that a filter gradient adds in one accumulator before it sums the
