@@ -735,79 +735,51 @@ k_wgrad_patch(const __grid_constant__ CUtensorMap mdy, const __grid_constant__ C
 // whatever X holds there for other taps: 0 inf is NaN, in entries that those pixels
 // are no part of.  Only a product of a zero can do that, and only to make a partial
 // sum NaN; so where tiles are ragged (RAGGED) a warp whose sum is NaN adds its splits
-// again, and takes the NaN entries of a split from the existing pixels of the
-// split's tiles (an entry whose own products give NaN stays so, and ends the loop).
+// again, and takes the NaN entries of a split from the existing pixels of the split's
+// tiles (an entry whose own products give NaN stays so, and is left at that).
 // Sums without a NaN, all but those of a diverged network, keep their bits and pay one
-// vote (33 images of 63 x 61, stride 2, 40 -> 72: 20.5 us with its products; all of X
-// NaN 152.  8 images of 255 x 249, 64 -> 64: 75.7; all NaN 142, one pixel infinite in
-// every channel 1360: its split's 3,300 pixels are walked by a warp for each 32 x 4
-// entries).
+// vote; the other path goes entry by entry, so that the kernel keeps its 32 registers
+// (8 images of 255 x 249, 64 -> 64: 99 us; all of X NaN 261, one pixel infinite in every
+// channel 1,170).
 constexpr int kSumLanes = 8;
 struct EdgeFix {
     const __nv_bfloat16 *dy, *x;
     Geo g;
     int tile_h, tile_w;
 };
-__device__ __forceinline__ bool any_nan(float4 v) {
-    return isnan(v.x) || isnan(v.y) || isnan(v.z) || isnan(v.w);
-}
 __device__ __forceinline__ float4 add4(float4 a, float4 b) {
     return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
-// The entries e .. e + 3 of split z's partial sum v, the NaN ones (bad: this lane has
-// any) added up from the existing pixels.
-__device__ float4 split_of_pixels(const EdgeFix &f, int z, int splits, int64_t e, float4 v, bool bad) {
+
+// Entry e of split z's partial sum from the existing pixels (of the lanes that want it;
+// all lanes of the warp call it).
+__device__ __forceinline__ float split_of_pixels(const EdgeFix &f, int z, int splits, int64_t e, bool want) {
     const Geo &g = f.g;
     const int c = (int)(e % g.C), t = (int)(e / g.C), rs = t % (g.R * g.S), k = t / (g.R * g.S);
     const int dh = rs / g.S - g.pad, dw = rs % g.S - g.pad;
     const int tx = (g.Q + f.tile_w - 1) / f.tile_w, ty = (g.P + f.tile_h - 1) / f.tile_h;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    bool open = bad;
-    for (int tile = z; tile < g.N * tx * ty && __any_sync(0xffffffffu, open); tile += splits) {
+    float s = 0.f;
+    for (int tile = z; tile < g.N * tx * ty && __any_sync(0xffffffffu, want); tile += splits) {
         const int n = tile / (tx * ty), p0 = tile % (tx * ty) / tx * f.tile_h, q0 = tile % tx * f.tile_w;
         for (int p = p0; p < min(p0 + f.tile_h, g.P); ++p) {
-            if (!open) continue;
+            if (!want) continue;
             const int h = p * g.stride + dh;
             const __nv_bfloat16 *dy = f.dy + ((size_t)n * g.P + p) * g.Q * g.K + k;
             const __nv_bfloat16 *x = f.x + ((size_t)n * g.H + h) * g.W * g.C + c;
 #pragma unroll 4
             for (int q = q0; q < min(q0 + f.tile_w, g.Q); ++q) {
                 const int u = q * g.stride + dw;
-                const float d = __bfloat162float(dy[(size_t)q * g.K]);
-                float2 a = make_float2(0.f, 0.f), b = a;  // padding
-                if (h >= 0 && h < g.H && u >= 0 && u < g.W) {
-                    const __nv_bfloat162 *px = reinterpret_cast<const __nv_bfloat162 *>(x + (size_t)u * g.C);
-                    a = __bfloat1622float2(px[0]);
-                    b = __bfloat1622float2(px[1]);
-                }
-                s.x = fmaf(d, a.x, s.x);
-                s.y = fmaf(d, a.y, s.y);
-                s.z = fmaf(d, b.x, s.z);
-                s.w = fmaf(d, b.y, s.w);
+                const bool in = h >= 0 && h < g.H && u >= 0 && u < g.W;  // else padding
+                s = fmaf(__bfloat162float(dy[(size_t)q * g.K]), in ? __bfloat162float(x[(size_t)u * g.C]) : 0.f, s);
             }
-            open = (isnan(v.x) && !isnan(s.x)) || (isnan(v.y) && !isnan(s.y)) ||
-                   (isnan(v.z) && !isnan(s.z)) || (isnan(v.w) && !isnan(s.w));
+            want = !isnan(s);
         }
-    }
-    return make_float4(isnan(v.x) ? s.x : v.x, isnan(v.y) ? s.y : v.y, isnan(v.z) ? s.z : v.z,
-                       isnan(v.w) ? s.w : v.w);
-}
-// This warp's splits w, w + kSumLanes, ... of the entries 4 i .. 4 i + 3 (live: they
-// are entries of dw).
-__device__ __noinline__ float4 sum_with_edges(const EdgeFix &f, const float4 *part, int splits, int64_t row,
-                                              int64_t i, bool live, int w) {
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int z = w; z < splits; z += kSumLanes) {
-        float4 v = live ? __ldg(part + (size_t)z * row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const bool bad = any_nan(v);
-        if (__any_sync(0xffffffffu, bad)) v = split_of_pixels(f, z, splits, live ? 4 * i : 0, v, bad);
-        s = add4(s, v);
     }
     return s;
 }
 
 template <bool RAGGED>
-__global__ void __launch_bounds__(32 * kSumLanes, RAGGED ? 4 : 8)
+__global__ void __launch_bounds__(32 * kSumLanes, 8)
 k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, float4 *out,
             float4 *out2, const __grid_constant__ EdgeFix fix) {
     __shared__ float4 red[kSumLanes][32];
@@ -819,16 +791,29 @@ k_sum_parts(const float4 *part, int splits, int64_t count4, int64_t extra4, floa
 #pragma unroll 4
         for (int z = w; z < splits; z += kSumLanes) s = add4(s, __ldg(part + (size_t)z * row + i));
     }
+    red[w][lane] = s;
     if constexpr (RAGGED) {
-        const bool bad = i < count4 && any_nan(s);
-        if (__any_sync(0xffffffffu, bad)) {
-            const float4 v = sum_with_edges(fix, part, splits, row, i, i < count4, w);
-            if (bad) s = v;
+        if (__any_sync(0xffffffffu, i < count4 && isnan(s.x + s.y + s.z + s.w))) {
+            for (int j = 0; j < 4; ++j) {
+                float *mine = &red[w][lane].x + j;
+                const bool bad = i < count4 && isnan(*mine);
+                float t = 0.f;
+                for (int z = w; z < splits; z += kSumLanes) {
+                    float v = bad ? reinterpret_cast<const float *>(part + (size_t)z * row + i)[j] : 0.f;
+                    const bool want = isnan(v) && !isnan(t);
+                    if (__any_sync(0xffffffffu, want)) {
+                        const float u = split_of_pixels(fix, z, splits, want ? 4 * i + j : 0, want);
+                        if (want) v = u;
+                    }
+                    t += v;
+                }
+                if (bad) *mine = t;
+            }
         }
     }
-    red[w][lane] = s;
     __syncthreads();
     if (w == 0 && i < row) {
+        s = red[0][lane];
         for (int l = 1; l < kSumLanes; ++l) s = add4(s, red[l][lane]);
         if (i < count4)
             out[i] = s;
