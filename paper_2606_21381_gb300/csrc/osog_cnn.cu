@@ -860,9 +860,14 @@ int osog_conv2d_forward(const osog_conv_shape_t *shape, const uint16_t *x, const
     a.Kred = a.g.R * a.g.S * a.g.C;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // reductions shorter than 128 stay on the warp-level MMA (the 8-channel
-    // first layer and the 1 x 1 head).  The patch kernels store 16-byte vectors;
-    // k_conv_gemm takes the outputs that are not so aligned (pairs of columns).
-    if (g_use_tcgen05 && a.Kred >= 128 && aligned(16, {w, y, y_f32})) {
+    // first layer and the 1 x 1 head), and so do 8 channels up to 25 taps: the patch
+    // kernel spends a product of 16 on each tap's 8 and a TMA row on each of its
+    // filters' 16 bytes (81 x 154, 8 -> 216, 4 x 4: 21.6 us, k_conv_gemm 11.6; 16 images
+    // of 23 x 42, 8 -> 24, 5 x 5: 14.9 and 14.1; at 49 taps 19.5 and 21.1).  The patch
+    // kernels store 16-byte vectors; k_conv_gemm takes the outputs that are not so
+    // aligned (pairs of columns).
+    const bool deep = a.g.C == 8 ? a.Kred > 200 : a.Kred >= 128;
+    if (g_use_tcgen05 && deep && aligned(16, {w, y, y_f32})) {
         const cudaError_t e = conv_forward_tma(a.g, x, w, bias, relu != 0, y, y_f32, st);
         if (e != cudaErrorNotSupported) return status_of(e);
     }
