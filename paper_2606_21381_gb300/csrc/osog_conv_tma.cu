@@ -1162,7 +1162,10 @@ bool wgrad_plan(const Geo &g, WgradArgs &a, int &ch) {
         const int64_t pixels = (int64_t)g.N * g.P * g.Q;
         const int blocks = ceil_div(g.K, 128) * a.cblocks * a.groups;
         const int fill = kSms / blocks, least = (int)((pixels + kMost - 1) / kMost);
-        a.splits = fill > least ? fill : least;
+        // (the last of several waves is filled, too: 64 images of 44 x 67, 8 -> 8, 7 x 7
+        // 175 -> 126 us)
+        const int waves = (least * blocks + kSms - 1) / kSms;
+        a.splits = fill > least ? fill : waves * kSms / blocks > least ? waves * kSms / blocks : least;
         if (a.splits > a.tiles) a.splits = a.tiles;
         return true;
     }
