@@ -330,3 +330,44 @@ def test_long_filter_gradients_are_as_accurate_as_the_general_kernel():
         err.append((dw.reshape(512, 512).double() - want).norm().item())
         assert (db.double() - dy.double().sum((0, 1, 2))).abs().max() <= 2e-6 * dy.double().abs().sum((0, 1, 2)).max()
     assert err[1] <= 1.25 * err[0]
+
+
+# filter gradients whose CTAs add several tiles, with the blocks (of output and input
+# channels and of taps) that share the 152 SMs: stages are used again (two of them; one,
+# for wide filters on stride 2), accumulators go on over tiles, and CTAs with and without
+# the bias gradient run side by side
+MANY_TILES = [
+    ((6, 48, 40, 136, 264, 3, 3, 1, 1), 18, (16, 8)),
+    ((9, 70, 66, 72, 16, 7, 7, 2, 3), 9, (16, 8)),
+    ((20, 50, 50, 32, 64, 3, 3, 1, 1), 1, (16, 8)),
+    ((3, 200, 400, 8, 16, 3, 3, 1, 1), 0, (8, 32)),  # eight channels, nine taps: 304 CTAs
+    ((3, 200, 400, 8, 64, 3, 3, 1, 1), 0, (8, 32)),
+]
+
+
+@pytest.mark.parametrize("shape,blocks,tile", MANY_TILES)
+def test_filter_gradients_of_several_tiles_a_cta(cnn, shape, blocks, tile):
+    N, H, W, _, _, R, S, stride, pad = shape
+    P, Q = (H + 2 * pad - R) // stride + 1, (W + 2 * pad - S) // stride + 1
+    tiles = N * -(-P // tile[0]) * -(-Q // tile[1])
+    splits = max(152 // blocks, -(-N * P * Q // 1920)) if blocks else 304
+    assert tiles >= 2.4 * splits
+    test_conv_backward_filter_matches_reference(cnn, shape)
+
+
+# both sides of the forward kernels' dispatch and of the column blocks: eight channels
+# with 16, 25 and 28 taps, 136 and 200 output channels
+@pytest.mark.parametrize("shape", [
+    (1, 20, 18, 8, 24, 4, 4, 1, 2), (2, 15, 17, 8, 40, 5, 5, 2, 2), (1, 20, 18, 8, 24, 4, 7, 1, 3),
+    (1, 18, 20, 16, 136, 3, 3, 1, 1), (2, 9, 21, 72, 200, 3, 3, 2, 1),
+])
+def test_forward_routes_match_reference(cnn, shape):
+    test_conv_forward_matches_reference(cnn, shape, True)
+    test_forward_without_the_fp32_copy_gives_the_same_bits(cnn, shape)
+
+
+# few tiles: the taps spread over the idle SMs, one to a CTA and several
+@pytest.mark.parametrize("shape", [(1, 7, 10, 8, 24, 7, 7, 2, 7), (2, 12, 7, 16, 48, 5, 5, 1, 0),
+                                   (1, 30, 22, 40, 136, 8, 3, 1, 2)])
+def test_filter_gradients_of_a_few_tiles(cnn, shape):
+    test_conv_backward_filter_matches_reference(cnn, shape)
