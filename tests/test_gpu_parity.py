@@ -366,3 +366,18 @@ def test_images_and_adjoints_on_several_streams_at_once(size, modes):
         assert r.sync_status() == 0
         for run in runs:
             assert all(torch.equal(a, b) for a, b in zip(run, want))
+
+
+# particles of 1.9 to 40 absorption lengths: below and above the 2 from which a
+# contribution is rounded by conversion, and past the 16 where a particle's is clamped
+# (e^-16 of the amplitude is 1e-7)
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("depth", [1.9, 2.1, 10.0, 40.0])
+def test_opaque_particles(kind, depth):
+    rng = np.random.default_rng(int(10 * depth) + kind)
+    soa = scenes.draw_particles(rng, 24, 128, 256, thickness=(1.0, 2.0))
+    soa[7] = depth / soa[5]
+    soa[8] = kind
+    o = scenes.optics(128, 256, modes=7, defocus=0.4)
+    ref = oracle.render(soa, soa.shape[1], oracle.make_optics(**o))["images"]
+    assert_images_close(gpu_render(soa, o), ref, o)
