@@ -113,3 +113,14 @@ def test_decided_draws_are_those_of_double_precision(harness, what, low, high, m
     assert wrong == 0
     # rates past 2^22 are left to double precision by design
     assert undecided <= most * n or high > 4e6
+
+
+# the shares above, of all rates below 2^22 and of all counts (none is left to double
+# precision by design there)
+@pytest.mark.parametrize("what,low,high,most", [(1, 3e4, 4e6, 2e-3), (2, 1e5, 1e12, 5e-4)])
+def test_few_draws_of_large_rates_and_gains_stay_open(harness, what, low, high, most):
+    out = subprocess.run([str(harness), str(what), repr(low), repr(high)], check=True,
+                         capture_output=True, text=True).stdout
+    n, undecided, wrong = (int(v) for v in out.split())
+    assert wrong == 0
+    assert undecided <= most * n
