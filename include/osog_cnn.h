@@ -79,11 +79,10 @@ int osog_conv2d_backward_filter(const osog_conv_shape_t *shape, const uint16_t *
  * (tcgen05.mma with the accumulator in tensor memory), 0 the warp-level
  * MMA (mma.sync).  Both compute the same products in BF16 with FP32
  * accumulation; summation order inside the tensor core differs.  With
- * tcgen05 selected, forward convolutions whose reduction R S C is below 128
- * still run on the warp-level MMA, and so do filter gradients whose ws, dw or
- * dbias is not 16-byte aligned; layers of 8 input channels and nine or ten
- * taps run on the warp-level MMA in either case.  The switch also covers
- * osog_conv2d_backward_filter. */
+ * tcgen05 selected, these still run on the warp-level MMA: forward
+ * convolutions whose reduction R S C is below 128 or that have 8 input
+ * channels and at most 25 taps, filter gradients of 8 input channels and nine
+ * or ten taps, and calls whose operands or results are not 16-byte aligned. */
 void osog_conv_use_tcgen05(int32_t enable);
 
 /* Synchronise `stream` and report a latched device error of the

@@ -236,8 +236,7 @@ k_bin_count(const float *__restrict__ soa, int64_t ld, const __grid_constant__ G
 }
 
 // Scan of one scene's band counts (CTA s): for every band the exclusive
-// prefix over the scene's chunks, in place; then the bands' starts and the
-// scene's column hull.  The counts are laid out [chunk][band], so a band's
+// prefix over the scene's chunks, in place; then the bands' starts.  The counts are laid out [chunk][band], so a band's
 // column is strided: the CTA moves tiles of kScanTile chunks x all bands
 // between global memory and shared memory with coalesced accesses (one
 // 128-byte line per 32 counts instead of one line per count) and scans the

@@ -915,7 +915,7 @@ bool conv_patch_plan(PatchArgs &a, int images, int oh, int ow, int reach_y, int 
         t.plane_bytes = round_up(t.pw * t.ph * 2 * t.ch, 1024);
         t.tiles_x = ceil_div(ow, t.tx * kTileW);
         t.tiles_y = ceil_div(oh, t.ty * kTileH);
-        const double per_sm_ctas = (double)images * t.tiles_x * t.tiles_y * col_blocks / 152.0;
+        const double per_sm_ctas = (double)images * t.tiles_x * t.tiles_y * col_blocks / kSms;
         const int steps = t.taps * t.chunks;
         const double mma = (double)steps * (t.ch / 16) * t.bn / 2.0 * subs;
         const double units = (t.classes * subs * ceil_div(t.bn, 64) + 1) / 2;

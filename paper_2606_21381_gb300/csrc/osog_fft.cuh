@@ -202,7 +202,7 @@ __device__ __forceinline__ void line_butterfly(int q, int &l, int &j) {
 // samples end to end.  Consecutive threads over four lines cover 128 bytes of 4 x 4
 // samples and more; along one line they would take 32 or 64 bytes of every block
 // (inverse rows of a 2048 x 2048 image 11.6 -> 10.6 us; 32 whole images 1607 -> 1550,
-// twelve DIC images of 1024 x 1024 305 -> 303).  Four lines are also as many as lie
+// sixteen DIC images of 1024 x 1024 305 -> 303).  Four lines are also as many as lie
 // on different banks (line_stride).
 constexpr int kRowFast = 4;
 

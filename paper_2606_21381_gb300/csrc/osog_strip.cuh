@@ -151,7 +151,7 @@ __device__ __forceinline__ bool make_row_item(const RRec &r, int c0, int c1, int
     // for that end is negative there.  A prism's carry the slack above.  (A row of
     // a particle is some eleven pixels, and spans a column or two wider on each
     // side for the rounding had four more, a quarter of the chunks: 32 images of
-    // 2048 x 2048 1682 -> 1642 us, one with 40,000 particles 110.8 -> 105.8.)
+    // 2048 x 2048 1702 -> 1660 us a call, one with 40,000 particles 112.6 -> 107.5.)
     const int j0 = max(c0, (int)ceilf(fmaxf(lo - 0.5f, -2.f)));
     const int j1 = min(c1, (int)floorf(fminf(hi - 0.5f, 4096.f)));
     if (j1 < j0) return false;
@@ -487,7 +487,7 @@ __device__ void raster_region(const Work &w, const int32_t *ids, const Rect *pre
 // the banks (3.7 wavefronts a reduction; the planes' shift puts the next row's
 // pixels 13 banks on, 2.4), and a chunk's pixels are at constant offsets, the ones
 // past a row's end in the next words of its line: 32 images of 2048 x 2048 1622 ->
-// 1604 us.  OPD mode: pairs of int64 at the samples' places.
+// 1607 us.  OPD mode: pairs of int64 at the samples' places.
 template <int N>
 struct PhaseSlot {
     static constexpr int kLine = 2 * line_stride(N), kShift = N >= 256 ? 5 : 1;
